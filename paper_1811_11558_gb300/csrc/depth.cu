@@ -7,25 +7,35 @@
 // with w_h the piecewise-linear interpolant of the nodal coefficients (Sec. 3.2).
 //
 // GB300 formulation (the paper's element integrals, evaluated exactly, reorganised):
-// * Frame: the tensors are rotated so that q lies along x1; with Delta(-q) = (-i, 0, 0)
-//   every kernel coefficient of Table 1 becomes a constant and the contraction of the
-//   4th-order kernels with w collapses to five rotated components of w plus one scalar
-//   (Delta^+-.w.Delta^+-) per branch; the in-plane component perpendicular to q has no
-//   strain (eps_pp = 0).
-// * Depth integral: the g0/g1 kernels are exponentials exp(-q|y3 - x3|) times
-//   polynomials, so the integrals over all elements above (g^- branch) and below (g^+
-//   branch) of node i follow from those of node i-1 / i+1 by the exact one-element
-//   recursions  M0 <- e^{-qh} M0 + element,  M1 <- e^{-qh}(M1 -+ qh M0) + element,
-//   with the linear-element integrals of Eq. (int_g0)/(int_g1) in closed form.  This
-//   replaces the cutoff of Sec. 3.2 (no approximation) and costs O(Nz) per mode.
-// * Parallelism: a CTA holds KT consecutive k1 columns (one k2) for all depth nodes in
-//   shared memory; the depth range is cut into chunks of C nodes, one thread per
-//   (chunk, k1).  Each chunk first computes its local contribution (from zero), the
-//   carries of the two recursions are folded across chunks in shared memory, then every
-//   chunk re-runs its recursion from the exact carries and writes its nodes.
-// * Image term: the surface traction of the full-space field needs the + branch at
-//   x3 = 0, i.e. the fully folded carry; the cancelling Boussinesq field is then a
-//   closed form exp(-q z)(P + q z Q) in the rotated frame.
+// * Frame: the tensors are rotated so that q lies along x1; with Delta(-q) = (-i, 0, 0) every
+//   kernel coefficient of Table 1 becomes a constant.  In that frame the contraction of the
+//   kernels with w has rank three per branch: with the nodal sources
+//     n = w_33 - w_qq -+ 2i w_q3,   m = (2 nu - 1)(w_qq + w_33),   a = w_qp +- i w_p3
+//   (upper sign: the branch A of the elements above the node, lower: P, below), every strain
+//   and stress component is a fixed combination of three moments per branch,
+//     n = int g0 n,   a = int g0 a,   v = int g0 m -+ int g1 n.
+//   (The generic form carries five rotated components and one contraction per branch, and
+//   evaluates the image field per node: 457 warp instructions per warp of nodes, measured on
+//   512 x 512 x 64 FP32.  Depth kernel, ms, generic form -> this one: 512 x 512 x 64 FP32 0.204
+//   -> 0.146, 1024 x 1024 x 32 (C = 2) 0.642 -> 0.465, 256 x 128 x 57 refined 0.043 -> 0.027,
+//   128 x 128 x 126 FP64 1.163 -> 0.385.)
+// * Depth integral: the g0/g1 kernels are exponentials exp(-q|y3 - x3|) times polynomials, so
+//   the moments follow from those of the neighbouring node by exact one-element steps,
+//     v <- e^{-qh}(v - qh n) + ...,  n <- e^{-qh} n + ...,  a <- e^{-qh} a + ...,
+//   with the linear-element integrals of Eq. (int_g0)/(int_g1) in closed form.  This replaces
+//   the cutoff of Sec. 3.2 (no approximation) and costs O(Nz) per mode.
+// * Image term: the Boussinesq field that cancels the surface traction of the full-space field
+//   has the form of the A branch of a source at the surface, so it is the starting value of
+//   the A recursion there: A(0) = (n_P + 2 v_P, -v_P, a_P) with P = P(0) the complete moments
+//   of the branch below.  The surface displacement is u3(0) = v_P / (2 mu).
+// * In the stress the local terms of the 33, 23 and 13 components cancel exactly (the
+//   traction is continuous across the layer), and those of the others are w_33 nu / (1 - nu) - w.
+// * Parallelism: a CTA holds KT consecutive k1 columns (one k2) for all depth nodes; the depth
+//   range is cut into chunks of C nodes, one thread per (chunk, k1).  Each chunk computes its
+//   own moments at every node and the carry it hands to its neighbours (both recursions from
+//   zero); 4 KT threads then run the chunk recurrences of the carries (two branches, the
+//   coupled pair (n, v) and a apart), in chunk order: a log-depth scan by all threads cost more
+//   instructions than everything else at C = 2; then every thread adds the propagated carries.
 // * q = 0 (mode k = 0): laminate solution (sigma_i3 = 0, eps_ab = 0).  k2 = N2/2
 //   (not in Z^2_N): no operator term, so sigma_hat = -w_hat (stress) or 0 (strain).
 #include <string.h>
@@ -63,15 +73,29 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned long lo
   return false;
 }
 
-// Linear-element integrals of Eq. (int_g0)/(int_g1): with a = q h,
-//   I_n(a) = int_0^1 s^n exp(-a s) ds,  n = 0, 1, 2,
-// closed form for a above a threshold, Taylor series below it (no cancellation).
-template <typename T> struct Elem {
-  T E, a, h, hI0mI1, hI1, ahI1mI2, ahI2;
-};
 
-template <typename T> __device__ __forceinline__ Elem<T> elem_coef(T q, T h) {
-  Elem<T> c;
+// ---- moments and element coefficients ------------------------------------------------
+// One branch of the depth integral at a node (rank-three form, see the head of the file).
+template <typename V> struct Br {
+  V n, v, a;
+};
+template <typename V> __device__ __forceinline__ Br<V> br_zero() {
+  Br<V> s;
+  s.n = s.v = s.a = mk<V>(0, 0);
+  return s;
+}
+
+// One element: with a = q h and I_n(a) = int_0^1 s^n exp(-a s) ds (Eq. (int_g0)/(int_g1)),
+// E = e^{-a}; b0, d0 weight the source of the node the step arrives at (h (I0 - I1), a h (I1 - I2)),
+// b1, d1 that of the node it leaves (h I1, a h I2).
+template <typename T> struct El {
+  T E, a, b0, b1, d0, d1;
+};
+constexpr int EL_N = 6;
+
+// closed form for a above a threshold, Taylor series below it (no cancellation)
+template <typename T> __device__ __forceinline__ El<T> elem_coef(T q, T h) {
+  El<T> c;
   const T a = q * h;
   const T E = dexp<T>(-a);
   T I0, I1, I2;
@@ -96,189 +120,169 @@ template <typename T> __device__ __forceinline__ Elem<T> elem_coef(T q, T h) {
   }
   c.E = E;
   c.a = a;
-  c.h = h;
-  c.hI0mI1 = h * (I0 - I1);
-  c.hI1 = h * I1;
-  c.ahI1mI2 = a * h * (I1 - I2);
-  c.ahI2 = a * h * I2;
+  c.b0 = h * (I0 - I1);
+  c.b1 = h * I1;
+  c.d0 = a * h * (I1 - I2);
+  c.d1 = a * h * I2;
+  return c;
+}
+// the coefficients of one element and column in shared memory: p[j * KT], j < EL_N
+template <typename T, int KT> __device__ __forceinline__ void el_put(T* p, const El<T>& c) {
+  p[0] = c.E; p[KT] = c.a; p[2 * KT] = c.b0; p[3 * KT] = c.b1; p[4 * KT] = c.d0; p[5 * KT] = c.d1;
+}
+template <typename T, int KT> __device__ __forceinline__ El<T> el_get(const T* p) {
+  El<T> c;
+  c.E = p[0]; c.a = p[KT]; c.b0 = p[2 * KT]; c.b1 = p[3 * KT]; c.d0 = p[4 * KT]; c.d1 = p[5 * KT];
   return c;
 }
 
-// moments of one branch: m = int g0 w_h for the rotated components
-// (qq, 33, p3, q3, qp); n = int g1 (D.w_h.D) with D = Delta^{+-}(-q) in the rotated frame
-template <typename V> struct Mom {
-  V m[5];
-  V n;
+// one step of a branch: arriving at a node (its source weighted b0, d0), and leaving it across
+// the next element (propagation, its source weighted b1, d1)
+template <typename T, typename V>
+__device__ __forceinline__ void br_arrive(Br<V>& s, const El<T>& c, V n, V m, V a) {
+  s.n = caxpy(s.n, c.b0, n);
+  s.v = caxpy(caxpy(s.v, c.b0, m), -c.d0, n);
+  s.a = caxpy(s.a, c.b0, a);
+}
+template <typename T, typename V>
+__device__ __forceinline__ void br_leave(Br<V>& s, const El<T>& c, V n, V m, V a) {
+  V v = cscale(caxpy(s.v, -c.a, s.n), c.E);
+  s.v = caxpy(caxpy(v, c.b1, m), -c.d1, n);
+  s.n = caxpy(cscale(s.n, c.E), c.b1, n);
+  s.a = caxpy(cscale(s.a, c.E), c.b1, a);
+}
+// d += c propagated over a distance with E = e^{-x}, xE = x e^{-x}, x = q times the distance
+template <typename T, typename V>
+__device__ __forceinline__ void br_add_prop(Br<V>& d, const Br<V>& c, T E, T xE) {
+  d.n = caxpy(d.n, E, c.n);
+  d.v = caxpy(caxpy(d.v, E, c.v), -xE, c.n);
+  d.a = caxpy(d.a, E, c.a);
+}
+
+// Direction cosines and their products for the rotation into the (q, p, 3) frame.
+template <typename T> struct Rot {
+  T c, s, cc, ss, cs, c2;
+  __device__ __forceinline__ Rot(T c_, T s_) : c(c_), s(s_), cc(c_ * c_), ss(s_ * s_), cs(c_ * s_), c2(c_ * c_ - s_ * s_) {}
 };
-
-// rotated storage order: 0 qq, 1 pp, 2 33, 3 p3, 4 q3, 5 qp; moment j -> rotated j ? j + 1 : 0
-
-template <typename V> __device__ __forceinline__ void mom_zero(Mom<V>& M) {
-#pragma unroll
-  for (int j = 0; j < 5; ++j) M.m[j] = mk<V>(0, 0);
-  M.n = mk<V>(0, 0);
-}
-
-// scalar Delta^-.X.Delta^- (A branch, sgn = -1) or Delta^+.X.Delta^+ (P branch, sgn = +1)
-// for the rotated components qq, 33, q3:  -X_qq + X_33 + sgn 2i X_q3
-template <typename V> __device__ __forceinline__ V nscal(V qq, V z33, V q3, int sgn) {
-  const V r = csub(z33, qq);
-  return caxpy_i(r, sgn > 0 ? (decltype(V::x))2 : (decltype(V::x))-2, q3);
-}
-
-// forward step of the g^- moments from node i to node i+1 over element [i, i+1]
+// nodal sources of both branches from w (11, 22, 33, 23, 13, 12)
+template <typename V> struct Src {
+  V nA, nP, m, aA, aP;
+};
 template <typename T, typename V>
-__device__ __forceinline__ void stepA(Mom<V>& A, const Elem<T>& c, const V* wi, const V* wj) {
-  const V n_old = nscal(A.m[0], A.m[1], A.m[3], -1);
+__device__ __forceinline__ Src<V> node_source(const V* x, const Rot<T>& r, T m_scale) {
+  const V qq = caxpy(caxpy(cscale(x[0], r.cc), r.ss, x[1]), (T)2 * r.cs, x[5]);
+  const V qp = caxpy(cscale(csub(x[1], x[0]), r.cs), r.c2, x[5]);
+  const V q3 = caxpy(cscale(x[4], r.c), r.s, x[3]);
+  const V p3 = caxpy(cscale(x[3], r.c), -r.s, x[4]);
+  const V d = csub(x[2], qq);
+  Src<V> o;
+  o.nA = caxpy_i(d, (T)-2, q3);
+  o.nP = caxpy_i(d, (T)2, q3);
+  o.m = cscale(cadd(x[2], qq), m_scale);
+  o.aA = caxpy_i(qp, (T)1, p3);
+  o.aP = caxpy_i(qp, (T)-1, p3);
+  return o;
+}
+template <typename T, typename V> __device__ __forceinline__ void hooke_mode(V* x, T lam, T mu) {
+  const V tr = cadd(cadd(x[0], x[1]), x[2]);
 #pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    const int r = (j == 0) ? 0 : j + 1;
-    V v = cscale(A.m[j], c.E);
-    v = caxpy(v, c.hI1, wi[r]);
-    v = caxpy(v, c.hI0mI1, wj[r]);
-    A.m[j] = v;
+  for (int cc = 0; cc < 6; ++cc) x[cc] = cscale(x[cc], (T)2 * mu);
+#pragma unroll
+  for (int cc = 0; cc < 3; ++cc) x[cc] = caxpy(x[cc], lam, tr);
+}
+
+// Output of a node from the complete moments of both branches: with kappa = q / (4 (1 - nu)),
+//   sigma_33 = kappa (v_A + v_P),             sigma_q3 = -i kappa (v_A - v_P + n_A - n_P),
+//   sigma_qq = -kappa (v_A + v_P + 2 (n_A + n_P)),   sigma_pp = -2 nu kappa (n_A + n_P),
+//   sigma_p3 = i q/2 (a_A - a_P),             sigma_qp = q/2 (a_A + a_P)
+// plus the local terms; the strain is the same with 2 - 2 nu for the factor 2 of qq, 2 nu (n_A
+// + n_P) added to 33, no pp component, all over 2 mu.  The constants of the rotation back are
+// folded into the combinations.
+template <typename T> struct OutC {
+  T w, t, k11w, k22w, k12w, k11n, k22n, k12n, k11a, k12a, k33, cy, sy, cz, sz;
+  __device__ __forceinline__ OutC(const Rot<T>& r, T q, T mu, T nu, bool stress) {
+    const T sc = stress ? (T)1 : (T)1 / ((T)2 * mu);
+    const T kap = sc * q / ((T)4 * ((T)1 - nu)), q2 = sc * (T)0.5 * q;
+    const T p = stress ? (T)-2 * nu * kap : (T)0;
+    w = stress ? (T)2 : (T)2 - (T)2 * nu;
+    t = stress ? (T)0 : (T)2 * nu;
+    k11w = -kap * r.cc; k22w = -kap * r.ss; k12w = -kap * r.cs;
+    k11n = p * r.ss; k22n = p * r.cc; k12n = -p * r.cs;
+    k11a = (T)-2 * q2 * r.cs; k12a = q2 * r.c2;
+    k33 = kap;
+    cy = kap * r.c; sy = kap * r.s; cz = q2 * r.c; sz = q2 * r.s;
   }
-  const V ni = nscal(wi[0], wi[2], wi[4], -1);
-  const V nj = nscal(wj[0], wj[2], wj[4], -1);
-  V v = cscale(caxpy(A.n, -c.a, n_old), c.E);
-  v = caxpy(v, -c.ahI2, ni);
-  v = caxpy(v, -c.ahI1mI2, nj);
-  A.n = v;
-}
-
-// backward step of the g^+ moments from node i+1 to node i over element [i, i+1]
+};
+// L: local terms (stress: 11, 22, 12; strain: 33, 23, 13)
 template <typename T, typename V>
-__device__ __forceinline__ void stepP(Mom<V>& P, const Elem<T>& c, const V* wi, const V* wj) {
-  const V n_old = nscal(P.m[0], P.m[1], P.m[3], +1);
-#pragma unroll
-  for (int j = 0; j < 5; ++j) {
-    const int r = (j == 0) ? 0 : j + 1;
-    V v = cscale(P.m[j], c.E);
-    v = caxpy(v, c.hI0mI1, wi[r]);
-    v = caxpy(v, c.hI1, wj[r]);
-    P.m[j] = v;
+__device__ __forceinline__ void node_out(V* o, const Br<V>& A, const Br<V>& P, const V* L, const OutC<T>& k,
+                                         bool stress) {
+  const V N = cadd(A.n, P.n), Vv = cadd(A.v, P.v), z = csub(A.a, P.a), sa = cadd(A.a, P.a);
+  const V y = cadd(csub(A.v, P.v), csub(A.n, P.n));
+  const V W = caxpy(Vv, k.w, N);
+  const V g = caxpy(cscale(y, k.cy), k.sz, z);   // 13 = -i g
+  const V h = caxpy(cscale(z, k.cz), -k.sy, y);  // 23 = i h
+  if (stress) {
+    o[0] = caxpy(caxpy(caxpy(L[0], k.k11w, W), k.k11n, N), k.k11a, sa);
+    o[1] = caxpy(caxpy(caxpy(L[1], k.k22w, W), k.k22n, N), -k.k11a, sa);
+    o[2] = cscale(Vv, k.k33);
+    o[3] = mk<V>(-h.y, h.x);
+    o[4] = mk<V>(g.y, -g.x);
+    o[5] = caxpy(caxpy(caxpy(L[2], k.k12w, W), k.k12n, N), k.k12a, sa);
+  } else {
+    o[0] = caxpy(cscale(W, k.k11w), k.k11a, sa);
+    o[1] = caxpy(cscale(W, k.k22w), -k.k11a, sa);
+    o[2] = caxpy(L[0], k.k33, caxpy(Vv, k.t, N));
+    o[3] = mk<V>(L[1].x - h.y, L[1].y + h.x);
+    o[4] = mk<V>(L[2].x + g.y, L[2].y - g.x);
+    o[5] = caxpy(cscale(W, k.k12w), k.k12a, sa);
   }
-  const V ni = nscal(wi[0], wi[2], wi[4], +1);
-  const V nj = nscal(wj[0], wj[2], wj[4], +1);
-  V v = cscale(caxpy(P.n, c.a, n_old), c.E);
-  v = caxpy(v, c.ahI1mI2, ni);
-  v = caxpy(v, c.ahI2, nj);
-  P.n = v;
 }
-
-// propagate a branch across a depth span with a = q * span (no source inside)
+// local terms of a node from w: stress nu / (1 - nu) w_33 - w_11, .. - w_22, -w_12 (the others
+// cancel); strain w_33 / (lam + 2 mu), w_23 / (2 mu), w_13 / (2 mu)
+template <typename T> struct LocC {
+  T a, b;
+  __device__ __forceinline__ LocC(T lam, T mu, T nu, bool stress)
+      : a(stress ? nu / ((T)1 - nu) : (T)1 / (lam + (T)2 * mu)), b((T)1 / ((T)2 * mu)) {}
+};
 template <typename T, typename V>
-__device__ __forceinline__ void propA(Mom<V>& A, T a) {
-  const T E = dexp<T>(-a);
-  const V n0 = nscal(A.m[0], A.m[1], A.m[3], -1);
-  A.n = cscale(caxpy(A.n, -a, n0), E);
+__device__ __forceinline__ void node_local(V* L, const V* x, const LocC<T>& k, bool stress) {
+  if (stress) {
+    const V t = cscale(x[2], k.a);
+    L[0] = csub(t, x[0]);
+    L[1] = csub(t, x[1]);
+    L[2] = mk<V>(-x[5].x, -x[5].y);
+  } else {
+    L[0] = cscale(x[2], k.a);
+    L[1] = cscale(x[3], k.b);
+    L[2] = cscale(x[4], k.b);
+  }
+}
+// output of a node of a mode without depth recursion: k = 0 (laminate) or outside Z^2_N (nyq)
+template <typename T, typename V>
+__device__ __forceinline__ void node_special(V* o, const V* w, bool nyq, T lam, T mu, bool stress) {
+  if (nyq) {
 #pragma unroll
-  for (int j = 0; j < 5; ++j) A.m[j] = cscale(A.m[j], E);
-}
-// with E = e^{-a} given
-template <typename T, typename V>
-__device__ __forceinline__ void propP_E(Mom<V>& P, T a, T E) {
-  const V n0 = nscal(P.m[0], P.m[1], P.m[3], +1);
-  P.n = cscale(caxpy(P.n, a, n0), E);
+    for (int cc = 0; cc < 6; ++cc) o[cc] = stress ? cscale(w[cc], (T)-1) : mk<V>(0, 0);
+    return;
+  }
+  // laminate: eps_33 = w_33/(lam+2mu), eps_a3 = w_a3/(2mu), eps_ab = 0
+  V e[6];
+  e[0] = e[1] = e[5] = mk<V>(0, 0);
+  e[2] = cscale(w[2], (T)1 / (lam + (T)2 * mu));
+  e[3] = cscale(w[3], (T)1 / ((T)2 * mu));
+  e[4] = cscale(w[4], (T)1 / ((T)2 * mu));
+  if (!stress) {
 #pragma unroll
-  for (int j = 0; j < 5; ++j) P.m[j] = cscale(P.m[j], E);
-}
-template <typename T, typename V>
-__device__ __forceinline__ void propP(Mom<V>& P, T a) {
-  propP_E(P, a, dexp<T>(-a));
-}
-template <typename V> __device__ __forceinline__ void mom_add(Mom<V>& a, const Mom<V>& b) {
+    for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
+    return;
+  }
+  const V trc = e[2];
 #pragma unroll
-  for (int j = 0; j < 5; ++j) a.m[j] = cadd(a.m[j], b.m[j]);
-  a.n = cadd(a.n, b.n);
-}
-
-// Kelvin part of the strain (full-space field, Eq. 2gradient + Eq. jump) in the rotated
-// frame from the two branch moments and the nodal eigenstress w (rotated, 6 comps).
-template <typename T, typename V>
-__device__ __forceinline__ void kelvin_strain(const Mom<V>& A, const Mom<V>& P, const V* w, T q, T nu, T mu,
-                                              V* e) {
-  const T K = (T)1 / ((T)8 * mu * (nu - (T)1));
-  const V S0 = cadd(A.m[0], P.m[0]), S2 = cadd(A.m[1], P.m[1]), S3 = cadd(A.m[2], P.m[2]);
-  const V S4 = cadd(A.m[3], P.m[3]), S5 = cadd(A.m[4], P.m[4]);
-  const V D0 = csub(A.m[0], P.m[0]), D2 = csub(A.m[1], P.m[1]), D3 = csub(A.m[2], P.m[2]);
-  const V D4 = csub(A.m[3], P.m[3]), D5 = csub(A.m[4], P.m[4]);
-  const V An = A.n, Pn = P.n;
-  // eps_qq = q K [(4nu-3) S0 + S2 + 4i(nu-1) D4 + An - Pn]
-  V t = cscale(S0, (T)4 * nu - (T)3);
-  t = cadd(t, S2);
-  t = caxpy_i(t, (T)4 * (nu - (T)1), D4);
-  t = cadd(t, csub(An, Pn));
-  e[0] = cscale(t, q * K);
-  e[1] = mk<V>(0, 0);
-  // eps_33 = K [q (S0 - (4nu-1) S2 + 4i nu D4 - An + Pn) + 4(2nu-1) w33]
-  t = caxpy(S0, -((T)4 * nu - (T)1), S2);
-  t = caxpy_i(t, (T)4 * nu, D4);
-  t = cadd(t, csub(Pn, An));
-  t = cscale(t, q);
-  t = caxpy(t, (T)4 * ((T)2 * nu - (T)1), w[2]);
-  e[2] = cscale(t, K);
-  // eps_p3 = (q(-S3 + i D5) + 2 w_p3) / (4 mu)
-  t = caxpy_i(cscale(S3, (T)-1), (T)1, D5);
-  t = cscale(t, q);
-  t = caxpy(t, (T)2, w[3]);
-  e[3] = cscale(t, (T)1 / ((T)4 * mu));
-  // eps_q3 = K [q(i(2(nu-1) D0 + 2 nu D2 + An + Pn) + 2 S4) + 4(nu-1) w_q3]
-  V u = cscale(D0, (T)2 * (nu - (T)1));
-  u = caxpy(u, (T)2 * nu, D2);
-  u = cadd(u, cadd(An, Pn));
-  t = caxpy_i(cscale(S4, (T)2), (T)1, u);
-  t = cscale(t, q);
-  t = caxpy(t, (T)4 * (nu - (T)1), w[4]);
-  e[4] = cscale(t, K);
-  // eps_qp = q (i D3 + S5) / (4 mu)
-  t = caxpy_i(S5, (T)1, D3);
-  e[5] = cscale(t, q / ((T)4 * mu));
-}
-
-// strain of the Boussinesq-Cerruti field of a surface traction t (rotated frame, force on
-// the body per unit area, Eq. B:fourier with its gradient recurrence) at zeta = q z
-template <typename T, typename V>
-__device__ __forceinline__ void bous_strain_add(const V* tr, T zeta, T ex, T nu, T imu, V* e) {
-  // ex = exp(-zeta), imu = 1 / mu
-  const T c1 = ex * imu, c2 = (T)0.5 * ex * imu;
-  const V t0 = tr[0], t1 = tr[1], t2 = tr[2];
-  // qq: ((1-nu) i t0 + (nu - 1/2) t2 + zeta(-i t0/2 + t2/2)) / mu
-  //   = ((1 - nu) - zeta/2) i t0 + ((nu - 1/2) + zeta/2) t2
-  V v = caxpy_i(cscale(t2, nu - (T)0.5 + (T)0.5 * zeta), (T)1 - nu - (T)0.5 * zeta, t0);
-  e[0] = caxpy(e[0], c1, v);
-  // 33: (-2 i nu t0 + (2nu-1) t2 + zeta (i t0 - t2)) / (2 mu)
-  //   = (zeta - 2 nu) i t0 + ((2 nu - 1) - zeta) t2
-  v = caxpy_i(cscale(t2, (T)2 * nu - (T)1 - zeta), zeta - (T)2 * nu, t0);
-  e[2] = caxpy(e[2], c2, v);
-  // p3: -t1 / (2 mu) ; qp: i t1 / (2 mu)
-  e[3] = caxpy(e[3], -c2, t1);
-  e[5] = caxpy_i(e[5], c2, t1);
-  // q3: (-t0 + zeta (t0 + i t2)) / (2 mu) = (zeta - 1) t0 + zeta i t2
-  v = caxpy_i(cscale(t0, zeta - (T)1), zeta, t2);
-  e[4] = caxpy(e[4], c2, v);
-}
-
-// rotate a symmetric tensor (11,22,33,23,13,12) into the (q, p, 3) frame and back
-template <typename T, typename V>
-__device__ __forceinline__ void rotate_in(V* x, T c, T s) {
-  const V X11 = x[0], X22 = x[1], X23 = x[3], X13 = x[4], X12 = x[5];
-  const T cc = c * c, ss = s * s, cs = c * s;
-  x[0] = caxpy(caxpy(cscale(X11, cc), ss, X22), (T)2 * cs, X12);
-  x[1] = caxpy(caxpy(cscale(X11, ss), cc, X22), (T)-2 * cs, X12);
-  x[3] = caxpy(cscale(X13, -s), c, X23);
-  x[4] = caxpy(cscale(X13, c), s, X23);
-  x[5] = caxpy(caxpy(cscale(X11, -cs), cs, X22), cc - ss, X12);
-}
-template <typename T, typename V>
-__device__ __forceinline__ void rotate_out(V* y, T c, T s) {
-  const V qq = y[0], pp = y[1], p3 = y[3], q3 = y[4], qp = y[5];
-  const T cc = c * c, ss = s * s, cs = c * s;
-  y[0] = caxpy(caxpy(cscale(qq, cc), ss, pp), (T)-2 * cs, qp);
-  y[1] = caxpy(caxpy(cscale(qq, ss), cc, pp), (T)2 * cs, qp);
-  y[3] = caxpy(cscale(q3, s), c, p3);
-  y[4] = caxpy(cscale(q3, c), -s, p3);
-  y[5] = caxpy(caxpy(cscale(qq, cs), -cs, pp), cc - ss, qp);
+  for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
+  o[0] = caxpy(o[0], lam, trc);
+  o[1] = caxpy(o[1], lam, trc);
+  o[2] = caxpy(o[2], lam, trc);
 }
 
 template <typename T> struct ModeGeom {
@@ -305,21 +309,110 @@ __device__ __forceinline__ ModeGeom<T> mode_geom(int k1, int k2, int n1, int n2,
   return g;
 }
 
-// ----------------------------------------------------------------------------------
-// Mindlin depth kernel
-// grid: (h1 / KT, n2); block: KT * nch threads, thread = (chunk, k1 column)
-// smem: W[nz][6][KT] (rotated in place) + Pst[max(nz, 2 nch + 1)][6][KT]
-// ----------------------------------------------------------------------------------
-template <typename T, int KT, bool EIN>
-__global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
-                                const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int C, int nch, int prow, T w1,
-                                T w2, T lam, T mu, T nu, int out_kind, int want_u3, int uniform, T hz,
-                                const int* __restrict__ zr) {
+// Chunk exchange area of a tile (values per column): the carries S of the A branch and T of the
+// P branch, [nch][3] each; slot R: the P moments of node 0 without their carry; slot I: the
+// image field at the surface.
+template <typename V, int KT> struct Xch {
+  V *A, *P, *R, *I;
+  __device__ __forceinline__ Xch(V* base, int nch) : A(base), P(base + (size_t)nch * 3 * KT),
+      R(base + (size_t)nch * 6 * KT), I(base + (size_t)nch * 6 * KT + 3 * KT) {}
+  static __host__ __device__ size_t count(int nch) { return (size_t)(6 * nch + 6) * KT; }
+};
+template <typename V, int KT> __device__ __forceinline__ void br_put(V* p, const Br<V>& s) {
+  p[0] = s.n; p[KT] = s.v; p[2 * KT] = s.a;
+}
+template <typename V, int KT> __device__ __forceinline__ Br<V> br_get(const V* p) {
+  Br<V> s;
+  s.n = p[0]; s.v = p[KT]; s.a = p[2 * KT];
+  return s;
+}
+
+// Carries into every chunk, in place over the chunks' own ones (A: arriving at the chunk's first
+// node, P: at its last), then the complete P moments of node 0, the image field and the surface
+// displacement.  Work item t = role KT + column, roles 0: P (n, v), 1: A (n, v), 2: P a, 3: A a.
+// The column of item t is that of the calling thread (KT divides both thread counts).  local: a
+// chunk's carry is its neighbour's own one (cutoff).
+template <typename T, int KT>
+__device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& X, const T* zs, int tid, int nthr, int C,
+                                              int nch, int nz, T q, bool uniform, T hz, bool local, bool live,
+                                              typename Cx<T>::t* u3, T u3_scale) {
   typedef typename Cx<T>::t V;
+  const int col = tid & (KT - 1);
+  T Eu = 0, xu = 0;
+  if (uniform) {
+    xu = q * hz * (T)C;
+    Eu = dexp<T>(-xu);
+  }
+  for (int t = tid; t < 4 * KT; t += nthr) {
+    const bool isA = (t / KT) & 1, isa = t / KT >= 2;
+    const int step = isA ? 3 * KT : -3 * KT;
+    V* p = (isA ? X.A : X.P + (size_t)(nch - 1) * 3 * KT) + col + (isa ? 2 * KT : 0);
+    V rn = mk<V>(0, 0), rv = mk<V>(0, 0);
+    V sn = p[0], sv = isa ? rv : p[KT];
+    for (int jj = 0; jj < nch; ++jj) {
+      V* pn = p + step;
+      V nn = rn, nv = rv;
+      if (jj + 1 < nch) {   // the next chunk's own carry, ahead of the recurrence
+        nn = pn[0];
+        if (!isa) nv = pn[KT];
+      }
+      p[0] = rn;
+      if (!isa) p[KT] = rv;
+      T E = Eu, x = xu;
+      if (!uniform) {
+        const int n0 = (isA ? jj : nch - 1 - jj) * C;
+        const int lo = isA ? n0 : max(n0 - 1, 0);
+        const int hi = min(isA ? n0 + C : n0 + C - 1, nz - 1);
+        x = q * (zs[hi] - zs[lo]);
+        E = dexp<T>(-x);
+      }
+      if (local) E = (T)0;
+      rv = caxpy(sv, E, caxpy(rv, -x, rn));
+      rn = caxpy(sn, E, rn);
+      sn = nn;
+      sv = nv;
+      p = pn;
+    }
+    if (!isA && live) {
+      const T x = q * (zs[min(C - 1, nz - 1)] - zs[0]);
+      const T E = dexp<T>(-x);
+      if (isa) {
+        X.I[2 * KT + col] = caxpy(X.R[2 * KT + col], E, X.P[2 * KT + col]);
+      } else {
+        const V dn = X.P[col], dv = X.P[KT + col];
+        const V n = caxpy(X.R[col], E, dn);
+        const V v = caxpy(X.R[KT + col], E, caxpy(dv, -x, dn));
+        X.I[col] = caxpy(n, (T)2, v);
+        X.I[KT + col] = mk<V>(-v.x, -v.y);
+        if (u3) *u3 = cscale(v, u3_scale);
+      }
+    }
+  }
+}
+
+// ----------------------------------------------------------------------------------
+// Mindlin depth kernel, shared-memory variant (FP64, deep grids, narrow grids, long chunks)
+// grid: (h1 / KT, n2); block: KT * nch threads, thread = (chunk, k1 column)
+// smem: W[nz][6][KT] (input, then the chunk's own moments in place; LS false: [nz][9][KT] with the
+// local terms), exchange area, element coefficients, depth nodes.
+// LS: at most 8 nodes per chunk, their local terms in registers.
+// Bound by the FP64 pipe in FP64 (two multiply-adds per clock and SM): 1163 -> 385 us at
+// 128 x 128 x 126 when the moments went from six to three per branch.
+// ----------------------------------------------------------------------------------
+template <typename T, int KT, bool LS>
+__global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
+                                const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int C, int nch, T w1,
+                                T w2, T lam, T mu, T nu, int out_kind, int want_u3, int uniform, T hz,
+                                const int* __restrict__ zr, int ein) {
+  typedef typename Cx<T>::t V;
+  constexpr int SL = LS ? 6 : 9, CM = LS ? 8 : 1;
   extern __shared__ __align__(128) unsigned char smraw[];  // one alignment for every kernel of this file
-  V* W = reinterpret_cast<V*>(smraw);                 // [nz][6][KT]
-  V* Pst = W + (size_t)nz * 6 * KT;                   // [max(nz, 2 nch + 1)][6][KT]
-  T* zs = reinterpret_cast<T*>(Pst + (size_t)prow * KT * 6);  // [nz] depth nodes
+  V* W = reinterpret_cast<V*>(smraw);                      // [nz][SL][KT]
+  V* xbase = W + (size_t)nz * SL * KT;
+  const Xch<V, KT> X(xbase, nch);
+  T* el = reinterpret_cast<T*>(xbase + Xch<V, KT>::count(nch));  // [uniform ? 1 : nz][6][KT]
+  T* pr = el + (size_t)(uniform ? 1 : nz) * EL_N * KT;     // [uniform ? C : nz][KT] propagators
+  T* zs = pr + (size_t)(uniform ? C : nz) * KT;            // [nz] depth nodes
   const int kt = threadIdx.x & (KT - 1);
   const int ch = threadIdx.x / KT;
   const int k1 = blockIdx.x * KT + kt;
@@ -330,609 +423,389 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   // 1. load the tile (coalesced KT-wide rows, every copy in flight before one wait) and
   //    the depth nodes
   // (layers outside zr hold no input: their spectrum was not computed and reads as zero)
-  if (!zr) {
-    for (int idx = threadIdx.x; idx < nz * 6 * KT; idx += blockDim.x) {
-      const int zc = idx / KT, j = idx & (KT - 1);
-      cp_async_cx(W + idx, spec + (size_t)zc * plane + colofs + j);
-    }
-  } else {
-    const int zlo = zr[0], zhi = zr[1];
-    for (int idx = threadIdx.x; idx < nz * 6 * KT; idx += blockDim.x) {
-      const int zc = idx / KT, j = idx & (KT - 1);
-      const int zl = zc / 6;
-      if (zl >= zlo && zl < zhi) cp_async_cx(W + idx, spec + (size_t)zc * plane + colofs + j);
-      else W[idx] = mk<V>(0, 0);
-    }
+  const int zlo = zr ? zr[0] : 0, zhi = zr ? zr[1] : nz;
+  for (int idx = threadIdx.x; idx < nz * 6 * KT; idx += blockDim.x) {
+    const int zc = idx / KT, j = idx & (KT - 1);
+    const int zl = zc / 6;
+    V* dst = W + ((size_t)zl * SL + (zc - zl * 6)) * KT + j;
+    if (zl >= zlo && zl < zhi) cp_async_cx(dst, spec + (size_t)zc * plane + colofs + j);
+    else *dst = mk<V>(0, 0);
   }
   for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
+  const ModeGeom<T> g = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2);
+  const bool special = g.zero || g.nyq;
+  const bool stress = out_kind == FVIM_STRESS;
+  const int n0 = ch * C;
+  const int nend = min(n0 + C, nz);
+  const bool active = n0 < nz;
+  const bool work = active && !special;
+  // element coefficients while the tile is in flight: element e below node e; none below the
+  // last node (zero)
+  if (uniform) {
+    // and the powers E^0 .. E^(C-1) of a uniform grid's propagator
+    if (threadIdx.x < KT) {
+      const El<T> c = elem_coef<T>(g.q, hz);
+      el_put<T, KT>(el + kt, c);
+      T p = 1;
+      for (int k = 0; k < C; ++k, p *= c.E) pr[k * KT + kt] = p;
+    }
+  } else {
+    for (int e = n0; e < nend; ++e) {
+      El<T> c = {0, 0, 0, 0, 0, 0};
+      if (e + 1 < nz) c = elem_coef<T>(g.q, zn[e + 1] - zn[e]);
+      el_put<T, KT>(el + (size_t)e * EL_N * KT + kt, c);
+    }
+  }
   cp_async_wait_all();
   __syncthreads();
 
-  const ModeGeom<T> g = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2);
-  const bool special = g.zero || g.nyq;
-  const int n0 = ch * C;
-  const int nend = min(n0 + C, nz);
-  const int e1 = min(n0 + C, nz - 1);  // elements [n0, e1)
-  const bool active = n0 < nz;
-
-  // 2. (eps_p input: w = C:eps_p per mode) rotate own nodes into the (q, p, 3) frame
-  if (active && (EIN || !special)) {
-    for (int i = n0; i < nend; ++i) {
+  const Rot<T> rot(g.c, g.s);
+  El<T> ec = {0, 0, 0, 0, 0, 0};
+  if (uniform) ec = el_get<T, KT>(el + kt);
+  const LocC<T> lc(lam, mu, nu, stress);
+  const T ms = (T)2 * nu - (T)1;
+  V L[CM][3];
+  // 2. own moments of the chunk: A forward (slots 0..2), the P sources kept in slots 3..5 and
+  //    then replaced by the P moments, backward
+  if (work) {
+    Br<V> s = br_zero<V>();
+    auto fwd = [&](int i, V* Li) {
+      V* w = W + (size_t)i * SL * KT + kt;
       V x[6];
 #pragma unroll
-      for (int cc = 0; cc < 6; ++cc) x[cc] = W[(i * 6 + cc) * KT + kt];
-      if (EIN) {
-        const V tr = cadd(cadd(x[0], x[1]), x[2]);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) x[cc] = cscale(x[cc], (T)2 * mu);
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) x[cc] = caxpy(x[cc], lam, tr);
+      for (int cc = 0; cc < 6; ++cc) x[cc] = w[cc * KT];
+      if (ein) hooke_mode(x, lam, mu);
+      const Src<V> o = node_source(x, rot, ms);
+      node_local(Li, x, lc, stress);
+      if (uniform) {
+        if (i > 0) br_arrive(s, ec, o.nA, o.m, o.aA);
+        br_put<V, KT>(w, s);
+        br_leave(s, ec, o.nA, o.m, o.aA);
+      } else {
+        if (i > 0) br_arrive(s, el_get<T, KT>(el + (size_t)(i - 1) * EL_N * KT + kt), o.nA, o.m, o.aA);
+        br_put<V, KT>(w, s);
+        br_leave(s, el_get<T, KT>(el + (size_t)i * EL_N * KT + kt), o.nA, o.m, o.aA);
       }
-      if (!special) rotate_in(x, g.c, g.s);
+      w[3 * KT] = o.nP;
+      w[4 * KT] = o.m;
+      w[5 * KT] = o.aP;
+    };
+    if constexpr (LS) {
 #pragma unroll
-      for (int cc = 0; cc < 6; ++cc) W[(i * 6 + cc) * KT + kt] = x[cc];
+      for (int l = 0; l < CM; ++l)
+        if (l < nend - n0) fwd(n0 + l, L[l]);
+    } else {
+      for (int i = n0; i < nend; ++i) {
+        fwd(i, L[0]);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) W[((size_t)i * SL + 6 + j) * KT + kt] = L[0][j];
+      }
     }
+    br_put<V, KT>(X.A + (size_t)ch * 3 * KT + kt, s);
+    s = br_zero<V>();
+    T ep = 1;  // propagator from node i to the chunk's last node
+    for (int i = nend - 1; i >= n0; --i) {
+      V* w = W + (size_t)i * SL * KT + kt;
+      const V n = w[3 * KT], m = w[4 * KT], a = w[5 * KT];
+      if (!uniform) {
+        ec = el_get<T, KT>(el + (size_t)i * EL_N * KT + kt);
+        if (i + 1 < nend) ep *= ec.E;
+        pr[i * KT + kt] = ep;
+      }
+      if (i + 1 < nz) br_arrive(s, ec, n, m, a);
+      br_put<V, KT>(w + 3 * KT, s);
+      if (i == 0) br_put<V, KT>(X.R + kt, s);
+      if (!uniform) ec = el_get<T, KT>(el + (size_t)max(i - 1, 0) * EL_N * KT + kt);
+      br_leave(s, ec, n, m, a);
+    }
+    br_put<V, KT>(X.P + (size_t)ch * 3 * KT + kt, s);
+  } else if (active) {
+    br_put<V, KT>(X.A + (size_t)ch * 3 * KT + kt, br_zero<V>());
+    br_put<V, KT>(X.P + (size_t)ch * 3 * KT + kt, br_zero<V>());
   }
   __syncthreads();
 
-  Elem<T> ec;
-  if (uniform) ec = elem_coef<T>(g.q, hz);
-
-  // 3. local summaries of both recursions over the chunk's elements, from zero
-  Mom<V>* SP = reinterpret_cast<Mom<V>*>(Pst);          // [nch][KT]
-  Mom<V>* SA = SP + (size_t)nch * KT;                   // [nch][KT]
-  if (active && !special) {
-    Mom<V> A, P;
-    mom_zero(A);
-    mom_zero(P);
-    for (int e = n0; e < e1; ++e) {
-      if (!uniform) ec = elem_coef<T>(g.q, zs[e + 1] - zs[e]);
-      V wi[6], wj[6];
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) {
-        wi[cc] = W[(e * 6 + cc) * KT + kt];
-        wj[cc] = W[((e + 1) * 6 + cc) * KT + kt];
-      }
-      stepA(A, ec, wi, wj);
-    }
-    for (int e = e1 - 1; e >= n0; --e) {
-      if (!uniform) ec = elem_coef<T>(g.q, zs[e + 1] - zs[e]);
-      V wi[6], wj[6];
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) {
-        wi[cc] = W[(e * 6 + cc) * KT + kt];
-        wj[cc] = W[((e + 1) * 6 + cc) * KT + kt];
-      }
-      stepP(P, ec, wi, wj);
-    }
-    SA[ch * KT + kt] = A;
-    SP[ch * KT + kt] = P;
-  }
+  // 3. carries, image field, surface displacement
+  V* u3 = want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr;
+  chunk_carries<T, KT>(X, zs, threadIdx.x, blockDim.x, C, nch, nz, g.q, uniform != 0, hz, false, !special, u3,
+                       (T)1 / ((T)2 * mu));
+  if (want_u3 && ch == 0 && special) *u3 = mk<V>(0, 0);
   __syncthreads();
-
-  // 4. carries: A at node n0 from all chunks above, P at node e1 from all chunks below,
-  //    and the complete + branch at x3 = 0 for the image term.  One exclusive scan per
-  //    branch and mode (thread ch 0: downwards, thread ch 1: upwards), in place over the
-  //    chunk summaries: slot j ends up holding the carry into chunk j.
-  Mom<V>* P0s = SA + (size_t)nch * KT;  // [KT]
-  if (active && !special) {
-    const int pch = nch > 1 ? 1 : 0;
-    if (ch == 0) {
-      Mom<V> run;
-      mom_zero(run);
-      for (int j = 0; j < nch; ++j) {
-        const int a0 = j * C, a1 = min(j * C + C, nz - 1);
-        const Mom<V> sj = SA[j * KT + kt];
-        SA[j * KT + kt] = run;
-        propA(run, g.q * (zs[a1] - zs[a0]));
-        mom_add(run, sj);
-      }
-    }
-    if (ch == pch) {
-      Mom<V> run;
-      mom_zero(run);
-      for (int j = nch - 1; j >= 0; --j) {
-        const int a0 = j * C, a1 = min(j * C + C, nz - 1);
-        const Mom<V> sj = SP[j * KT + kt];
-        SP[j * KT + kt] = run;
-        propP(run, g.q * (zs[a1] - zs[a0]));
-        mom_add(run, sj);
-      }
-      P0s[kt] = run;
-    }
-  }
-  __syncthreads();
-  Mom<V> Ain, Pin, P0;
-  if (active && !special) {
-    Ain = SA[ch * KT + kt];
-    Pin = SP[ch * KT + kt];
-    P0 = P0s[kt];
-  } else {
-    mom_zero(Ain);
-    mom_zero(Pin);
-    mom_zero(P0);
-  }
-  // surface traction of the full-space field (A = 0 at x3 = 0), cancelled by the image
-  V tr[3];
-  if (active && !special) {
-    V w0[6];
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) w0[cc] = W[cc * KT + kt];
-    Mom<V> Z;
-    mom_zero(Z);
-    V e0[6];
-    kelvin_strain<T, V>(Z, P0, w0, g.q, nu, mu, e0);
-    const V trc = cadd(e0[0], e0[2]);
-    tr[0] = csub(cscale(e0[4], (T)2 * mu), w0[4]);
-    tr[1] = csub(cscale(e0[3], (T)2 * mu), w0[3]);
-    tr[2] = csub(caxpy(cscale(trc, lam), (T)2 * mu, e0[2]), w0[2]);
-    if (want_u3 && ch == 0) {
-      // u3(0) = N_inf[w].e3 + B^T(q, 0) t . e3 (rotated frame)
-      const T K = (T)1 / ((T)8 * mu * (nu - (T)1));
-      V u = caxpy(cmuli(P0.m[3]), (T)1, P0.m[1]);        // P_33 + i P_q3
-      u = cadd(cscale(u, (T)2 - (T)4 * nu), P0.n);
-      u = cscale(u, K);
-      V ub = cscale(cmuli(tr[0]), (T)0.5 * ((T)2 * nu - (T)1));
-      ub = caxpy(ub, -(nu - (T)1), tr[2]);
-      u = caxpy(u, (T)1 / (g.q * mu), ub);
-      surf[(size_t)k2 * h1 + k1] = u;
-    }
-  }
-  if (want_u3 && ch == 0 && special) surf[(size_t)k2 * h1 + k1] = mk<V>(0, 0);
-  __syncthreads();  // summaries are dead from here on; Pst is reused for P(i)
-
   if (!active) return;
+
+  // 4. complete moments, output
+  V* out = spec + (size_t)n0 * 6 * plane + (size_t)k2 * h1 + k1;
   if (special) {
-    for (int i = n0; i < nend; ++i) {
+    for (int i = n0; i < nend; ++i, out += 6 * plane) {
       V w[6], o[6];
 #pragma unroll
-      for (int cc = 0; cc < 6; ++cc) w[cc] = W[(i * 6 + cc) * KT + kt];
-      if (g.nyq) {
+      for (int cc = 0; cc < 6; ++cc) w[cc] = W[((size_t)i * SL + cc) * KT + kt];
+      if (ein) hooke_mode(w, lam, mu);
+      node_special(o, w, g.nyq, lam, mu, stress);
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = out_kind == FVIM_STRAIN ? mk<V>(0, 0) : cscale(w[cc], (T)-1);
-      } else {
-        // laminate: eps_33 = w_33/(lam+2mu), eps_a3 = w_a3/(2mu), eps_ab = 0
-        V e[6];
-        e[0] = e[1] = e[5] = mk<V>(0, 0);
-        e[2] = cscale(w[2], (T)1 / (lam + (T)2 * mu));
-        e[3] = cscale(w[3], (T)1 / ((T)2 * mu));
-        e[4] = cscale(w[4], (T)1 / ((T)2 * mu));
-        if (out_kind == FVIM_STRAIN) {
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
-        } else {
-          const V trc = e[2];
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
-          o[0] = caxpy(o[0], lam, trc);
-          o[1] = caxpy(o[1], lam, trc);
-          o[2] = caxpy(o[2], lam, trc);
-        }
-      }
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) spec[(size_t)(i * 6 + cc) * plane + (size_t)k2 * h1 + k1] = o[cc];
+      for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
     }
     return;
   }
-
-  // 5. exact + branch at the chunk nodes (backward from the carry), kept in Pst
-  Mom<V>* Pn = reinterpret_cast<Mom<V>*>(Pst);  // [node][KT]
+  Br<V> cA = br_get<V, KT>(X.A + (size_t)ch * 3 * KT + kt);
+  const Br<V> cP = br_get<V, KT>(X.P + (size_t)ch * 3 * KT + kt);
   {
-    Mom<V> P = Pin;
-    if (e1 < nend) Pn[e1 * KT + kt] = P;   // last chunk: node nz-1 has no element below
-    for (int e = e1 - 1; e >= n0; --e) {
-      if (!uniform) ec = elem_coef<T>(g.q, zs[e + 1] - zs[e]);
-      V wi[6], wj[6];
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) {
-        wi[cc] = W[(e * 6 + cc) * KT + kt];
-        wj[cc] = W[((e + 1) * 6 + cc) * KT + kt];
-      }
-      stepP(P, ec, wi, wj);
-      Pn[e * KT + kt] = P;
-    }
+    const T x = g.q * zs[n0], E = dexp<T>(-x);
+    br_add_prop(cA, br_get<V, KT>(X.I + kt), E, x * E);
   }
-  // 6. forward: - branch, combine, image, epilogue, rotate back, store
-  {
-    Mom<V> A = Ain;
-    const T imu = (T)1 / mu;
-    // exp(-q z_i): one exponential per chunk, then the element factor e^{-qh} per node
-    // on uniform grids
-    T ex = dexp<T>(-g.q * zs[n0]);
+  const OutC<T> oc(rot, g.q, mu, nu, stress);
+  const int last = n0 + C - 1;  // node the P carry arrives at (a ragged last chunk has none: zero)
+  T EA = 1;
+  auto fin = [&](int i, const V* Li) {
+    V* w = W + (size_t)i * SL * KT + kt;
+    Br<V> A = br_get<V, KT>(w), P = br_get<V, KT>(w + 3 * KT);
+    T xA, xP, EP;
+    if (uniform) {
+      xA = ec.a * (T)(i - n0);
+      xP = ec.a * (T)(last - i);
+      EA = pr[(i - n0) * KT + kt];
+      EP = pr[(last - i) * KT + kt];
+    } else {
+      xA = g.q * (zs[i] - zs[n0]);
+      xP = g.q * (zs[nend - 1] - zs[i]);
+      if (i > n0) EA *= el[((size_t)(i - 1) * EL_N) * KT + kt];
+      EP = pr[i * KT + kt];
+    }
+    br_add_prop(A, cA, EA, xA * EA);
+    br_add_prop(P, cP, EP, xP * EP);
+    V o[6];
+    node_out(o, A, P, Li, oc, stress);
+#pragma unroll
+    for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
+    out += 6 * plane;
+  };
+  if constexpr (LS) {
+#pragma unroll
+    for (int l = 0; l < CM; ++l)
+      if (l < nend - n0) fin(n0 + l, L[l]);
+  } else {
     for (int i = n0; i < nend; ++i) {
-      V w[6];
 #pragma unroll
-      for (int cc = 0; cc < 6; ++cc) w[cc] = W[(i * 6 + cc) * KT + kt];
-      const Mom<V> P = Pn[i * KT + kt];
-      V e[6];
-      kelvin_strain<T, V>(A, P, w, g.q, nu, mu, e);
-      if (!uniform && i > n0) ex = dexp<T>(-g.q * zs[i]);
-      bous_strain_add<T, V>(tr, g.q * zs[i], ex, nu, imu, e);
-      if (uniform) ex *= ec.E;
-      V o[6];
-      if (out_kind == FVIM_STRAIN) {
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
-      } else {
-        const V trc = cadd(e[0], e[2]);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
-        o[0] = caxpy(o[0], lam, trc);
-        o[1] = caxpy(o[1], lam, trc);
-        o[2] = caxpy(o[2], lam, trc);
-      }
-      rotate_out(o, g.c, g.s);
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) spec[(size_t)(i * 6 + cc) * plane + (size_t)k2 * h1 + k1] = o[cc];
-      if (i < e1) {
-        if (!uniform) ec = elem_coef<T>(g.q, zs[i + 1] - zs[i]);
-        V wj[6];
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) wj[cc] = W[((i + 1) * 6 + cc) * KT + kt];
-        stepA(A, ec, w, wj);
-      }
+      for (int j = 0; j < 3; ++j) L[0][j] = W[((size_t)i * SL + 6 + j) * KT + kt];
+      fin(i, L[0]);
     }
   }
 }
 
 // ----------------------------------------------------------------------------------
-// Mindlin depth kernel, register variant (C <= 8 nodes per chunk, compile time).  The
-// summary pass keeps the + branch of the chunk's own elements per node in registers, so
-// the final pass adds the propagated carry (one propagation per node) instead of running
-// the + recursion again, and every pass reads each node of the tile once (the other node
-// of an element is carried in registers).
-// smem: W[nz][6][KT] + SA[nch][KT] + SP[nch][KT] (moments) + TR[KT][3] + zs[nz]
+// Mindlin depth kernel, register variant (FP32, C <= 8 nodes per chunk, compile time): the
+// chunk's own moments at its nodes stay in registers, the tile is read twice (sources, local
+// terms) and never written.
+// smem: W[nz][6][KT] (the tile), exchange area, element coefficients, zs[nz]
 // ----------------------------------------------------------------------------------
 template <typename V> __device__ __forceinline__ void ld6(V (&w)[6], const V* W, int node, int KT, int kt) {
 #pragma unroll
   for (int cc = 0; cc < 6; ++cc) w[cc] = W[(node * 6 + cc) * KT + kt];
 }
 
-// Per-column quantities that do not depend on the tile, computed while its copy is in flight:
-// the mode geometry (every thread) and, on a uniform grid, the element integrals (one thread
-// per column, written to the traction area TR as [6][KT] values of T for the body to read
-// after its first barrier).
+// Quantities that do not depend on the tile's values, computed while its copy is in flight: the
+// mode geometry (every thread) and the element coefficients, once per column on a uniform grid,
+// else those of each chunk's own elements (element e below node e; zero below the last node),
+// in el for the body to read after its first barrier.
 template <typename T, int KT>
-__device__ __forceinline__ ModeGeom<T> depth_prep(typename Cx<T>::t* TR, int tid, int kblk, int k2, bool ghost,
-                                                  int n1, int n2, int hs, T w1, T w2, int uniform, T hz) {
+__device__ __forceinline__ ModeGeom<T> depth_prep(T* el, const T* __restrict__ zn, int tid, int kblk, int k2, bool ghost,
+                                                  int nz, int C, int n1, int n2, int hs, T w1, T w2, int uniform, T hz) {
   const int kt = tid & (KT - 1);
   const ModeGeom<T> g = mode_geom<T>(kblk * KT + kt, k2, n1, n2, hs, w1, w2);
-  if (uniform && tid < KT && !ghost) {
-    T* ecs = reinterpret_cast<T*>(TR);
-    const Elem<T> e = elem_coef<T>(g.q, hz);
-    ecs[0 * KT + kt] = e.E;
-    ecs[1 * KT + kt] = e.a;
-    ecs[2 * KT + kt] = e.hI0mI1;
-    ecs[3 * KT + kt] = e.hI1;
-    ecs[4 * KT + kt] = e.ahI1mI2;
-    ecs[5 * KT + kt] = e.ahI2;
+  if (ghost) return g;
+  if (uniform) {
+    if (tid < KT) el_put<T, KT>(el + kt, elem_coef<T>(g.q, hz));
+  } else {
+    const int n0 = (tid / KT) * C, nend = min(n0 + C, nz);
+    for (int e = n0; e < nend; ++e) {
+      El<T> c = {0, 0, 0, 0, 0, 0};
+      if (e + 1 < nz) c = elem_coef<T>(g.q, zn[e + 1] - zn[e]);
+      el_put<T, KT>(el + e * EL_N * KT + kt, c);
+    }
   }
   return g;
 }
 
-// Steps 2-5 of the register depth kernel on a tile already in shared memory: W[nz][6][KT]
-// (the tile), SA / SP [>= nch][KT] (chunk moments), TR[KT][3], zs[nz].  tid = ch * KT + kt is
-// the thread's place in the tile, kblk the tile's block of KT k1 columns.  A ghost tile (a
-// CTA slot without a tile) takes part in the barriers only.
-template <typename T, int KT, int C, bool EIN>
-__device__ __forceinline__ void depth_r_body(typename Cx<T>::t* W, Mom<typename Cx<T>::t>* SA,
-                                             Mom<typename Cx<T>::t>* SP, typename Cx<T>::t* TR, const T* zs, int tid,
-                                             int kblk, int k2, bool ghost, typename Cx<T>::t* __restrict__ spec,
-                                             typename Cx<T>::t* __restrict__ surf, int nz, int n1, int n2, int hs,
-                                             int h1, int nch, T w1, T w2, T lam, T mu, T nu, int out_kind,
-                                             int want_u3, int uniform, T hz, T cut, const ModeGeom<T> g) {
+// Steps 2-4 of the register depth kernel on a tile already in shared memory (W, with its exchange
+// area X, element coefficients el and nodes zs).  tid = ch * KT + kt is the thread's place among
+// the tile's tt threads, kblk the tile's block of KT k1 columns.  A ghost tile (a CTA slot
+// without a tile) takes part in the barriers only.
+template <typename T, int KT, int C, bool EIN, bool UNI>
+__device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const Xch<typename Cx<T>::t, KT>& X, const T* el,
+                                             const T* zs, int tid, int tt, int kblk, int k2, bool ghost,
+                                             typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
+                                             int nz, int n2, int h1, int nch, T lam, T mu, T nu, int out_kind,
+                                             int want_u3, T hz, T cut, const ModeGeom<T> g) {
   typedef typename Cx<T>::t V;
   const int kt = tid & (KT - 1);
   const int ch = tid / KT;
   const int k1 = kblk * KT + kt;
   const size_t plane = (size_t)n2 * h1;
   const bool special = g.zero || g.nyq;
+  const bool stress = out_kind == FVIM_STRESS;
   const int n0 = ch * C;
-  const int nend = min(n0 + C, nz);
-  const int e1 = min(n0 + C, nz - 1);  // elements [n0, e1)
   const bool active = !ghost && n0 < nz;
   const bool work = active && !special;
+  const Rot<T> rot(g.c, g.s);
 
-  // 2. (eps_p input: w = C:eps_p per mode) rotate own nodes into the (q, p, 3) frame
-  if (active) {
+  // 2. own moments of the chunk at its nodes, both branches from zero, and the carries handed on.
+  //    Nodes past the last one count as sources of zero, which changes nothing above them.
+  Br<V> A[C], P[C];
+  if (work) {
+    Src<V> o[C];
+    const T ms = (T)2 * nu - (T)1;
 #pragma unroll
     for (int l = 0; l < C; ++l) {
-      const int i = n0 + l;
-      if (i >= nend) break;
-      V x[6];
-      ld6(x, W, i, KT, kt);
-      if (EIN) {
-        const V tr = cadd(cadd(x[0], x[1]), x[2]);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) x[cc] = cscale(x[cc], (T)2 * mu);
-#pragma unroll
-        for (int cc = 0; cc < 3; ++cc) x[cc] = caxpy(x[cc], lam, tr);
-      }
-      if (!special) rotate_in(x, g.c, g.s);
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) W[(i * 6 + cc) * KT + kt] = x[cc];
-    }
-  }
-  // element coefficients of a uniform grid: the chunk threads of a column share q and h, so
-  // one thread per column evaluated them (depth_prep, before this barrier) and the others read
-  // them here.  They pass through the traction area TR ([6][KT] values of T), which is written
-  // again only after later barriers, when every thread holds them in registers.
-  const T* ecs = reinterpret_cast<const T*>(TR);
-  __syncthreads();
-
-  Elem<T> ec;
-  if (uniform) {
-    ec.E = ecs[0 * KT + kt];
-    ec.a = ecs[1 * KT + kt];
-    ec.h = hz;
-    ec.hI0mI1 = ecs[2 * KT + kt];
-    ec.hI1 = ecs[3 * KT + kt];
-    ec.ahI1mI2 = ecs[4 * KT + kt];
-    ec.ahI2 = ecs[5 * KT + kt];
-  }
-
-  // 3. chunk summaries from zero (- branch at the chunk's last node e1, + branch at its
-  //    first node n0); the + branch of every own node stays in registers
-  Mom<V> Ploc[C];
-  Mom<V> Ta, Up;
-  mom_zero(Ta);
-  mom_zero(Up);
-  if (work && uniform) {
-    // the two recursions are independent chains: advance them together (same steps in the
-    // same order per chain as below, so the same values)
-    V wa[6], wb[6];
-    ld6(wa, W, n0, KT, kt);
-    ld6(wb, W, e1, KT, kt);
-#pragma unroll
-    for (int st = 0; st < C; ++st) {
-      const int la = st, lp = C - 1 - st;
-      if (n0 + la < e1) {
-        V wn[6];
-        ld6(wn, W, n0 + la + 1, KT, kt);
-        stepA(Ta, ec, wa, wn);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) wa[cc] = wn[cc];
-      }
-      if (n0 + lp < e1) {
-        V wc[6];
-        ld6(wc, W, n0 + lp, KT, kt);
-        stepP(Up, ec, wc, wb);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) wb[cc] = wc[cc];
-        Ploc[lp] = Up;
+      if (n0 + l < nz) {
+        V x[6];
+        ld6(x, W, n0 + l, KT, kt);
+        if (EIN) hooke_mode(x, lam, mu);
+        o[l] = node_source(x, rot, ms);
       } else {
-        mom_zero(Ploc[lp]);
+        o[l].nA = o[l].nP = o[l].m = o[l].aA = o[l].aP = mk<V>(0, 0);
       }
     }
-  } else if (work) {
-    V wa[6];
-    ld6(wa, W, n0, KT, kt);
+    El<T> ec;
+    if (UNI) ec = el_get<T, KT>(el + kt);
+    // on a refined grid: element above node n0 + l, zero above node 0 and below the last node
+    auto elem = [&](int e) {
+      El<T> c = {0, 0, 0, 0, 0, 0};
+      if (e >= 0 && e < nz) c = el_get<T, KT>(el + e * EL_N * KT + kt);
+      return c;
+    };
+    Br<V> s = br_zero<V>();
+    if (!UNI) ec = elem(n0 - 1);
 #pragma unroll
     for (int l = 0; l < C; ++l) {
-      const int e = n0 + l;
-      if (e < e1) {
-        if (!uniform) ec = elem_coef<T>(g.q, zs[e + 1] - zs[e]);
-        V wb[6];
-        ld6(wb, W, e + 1, KT, kt);
-        stepA(Ta, ec, wa, wb);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) wa[cc] = wb[cc];
-      }
+      if (!UNI || n0 + l > 0) br_arrive(s, ec, o[l].nA, o[l].m, o[l].aA);
+      A[l] = s;
+      if (!UNI) ec = elem(n0 + l);
+      br_leave(s, ec, o[l].nA, o[l].m, o[l].aA);
     }
-    V wb[6];
-    ld6(wb, W, e1, KT, kt);
+    br_put<V, KT>(X.A + ch * 3 * KT + kt, s);
+    s = br_zero<V>();
 #pragma unroll
     for (int l = C - 1; l >= 0; --l) {
-      const int e = n0 + l;
-      if (e < e1) {
-        if (!uniform) ec = elem_coef<T>(g.q, zs[e + 1] - zs[e]);
-        V wc[6];
-        ld6(wc, W, e, KT, kt);
-        stepP(Up, ec, wc, wb);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) wb[cc] = wc[cc];
-        Ploc[l] = Up;
-      } else {
-        mom_zero(Ploc[l]);
-      }
+      if (!UNI || n0 + l + 1 < nz) br_arrive(s, ec, o[l].nP, o[l].m, o[l].aP);
+      P[l] = s;
+      if (!UNI) ec = elem(n0 + l - 1);
+      br_leave(s, ec, o[l].nP, o[l].m, o[l].aP);
     }
+    br_put<V, KT>(X.P + ch * 3 * KT + kt, s);
+    if (ch == 0) br_put<V, KT>(X.R + kt, P[0]);
+  } else if (active) {
+    br_put<V, KT>(X.A + ch * 3 * KT + kt, br_zero<V>());
+    br_put<V, KT>(X.P + ch * 3 * KT + kt, br_zero<V>());
+    if (ch == 0) br_put<V, KT>(X.R + kt, br_zero<V>());
   }
 
-  // 4. inclusive scans over the chunks, log2(nch) rounds with every chunk thread working:
-  //    - branch downwards, Ta_j = sum_{i<=j} propA(S_i, q (z[e1_j] - z[e1_i]));
-  //    + branch upwards,  Up_j = sum_{i>=j} propP(S_i, q (z[n0_i] - z[n0_j])).
-  //    Propagations compose (prop(prop(M, a), b) = prop(M, a + b)), so the rounds are exact.
-  // Cutoff (Sec. 3.2, eps_co, restated for the recursion): when every chunk span of the tile
-  // damps by e^{-q span} < e^{-cut}, a chunk's carry is its neighbour's own summary to the
-  // rounding of the path (e^{-18} < 2^-24 in FP32): the chunks beyond the neighbour contribute
-  // below it, so the scan rounds are skipped (one block-wide vote keeps the branch uniform)
-  const T span = (work && ch + 1 < nch) ? zs[e1] - zs[n0] : (T)0;
+  // 3. carries.  Cutoff (Sec. 3.2, eps_co, restated for the recursion): when every chunk span of
+  //    the tile damps by e^{-q span} < e^{-cut}, a chunk's carry is its neighbour's own one to
+  //    the rounding of the path (e^{-18} < 2^-24 in FP32).  The vote is block-wide.
+  const T span = (work && ch + 1 < nch) ? zs[min(n0 + C, nz - 1)] - zs[n0] : (T)0;
   const bool far = !work || ch + 1 >= nch || g.q * span > cut;
   const bool local = __syncthreads_and(cut > (T)0 && far) != 0;
-  const int e1c = e1;
-  for (int d = 1; d < nch && !local; d <<= 1) {
-    SA[ch * KT + kt] = Ta;
-    SP[ch * KT + kt] = Up;
-    __syncthreads();
-    if (work && ch >= d) {
-      Mom<V> o = SA[(ch - d) * KT + kt];
-      const int e1o = min((ch - d) * C + C, nz - 1);
-      propA(o, g.q * (zs[e1c] - zs[e1o]));
-      mom_add(Ta, o);
-    }
-    if (work && ch + d < nch) {
-      Mom<V> o = SP[(ch + d) * KT + kt];
-      propP(o, g.q * (zs[(ch + d) * C] - zs[n0]));
-      mom_add(Up, o);
-    }
-    __syncthreads();
-  }
-  SA[ch * KT + kt] = Ta;
-  SP[ch * KT + kt] = Up;
+  if (!ghost)
+    chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, local, !special,
+                         want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr, (T)1 / ((T)2 * mu));
+  if (want_u3 && !ghost && ch == 0 && special) surf[(size_t)k2 * h1 + k1] = mk<V>(0, 0);
   __syncthreads();
-
-  // surface traction of the full-space field (A = 0 at x3 = 0, + branch complete: the
-  // scan value of chunk 0), cancelled by the image; one thread per column, the last chunk's
-  // (it has no carry from below to fold, so it works while the other chunks fold theirs)
-  const int tch = nch - 1;
-  if (ch == tch && work) {
-    V w0[6];
-    ld6(w0, W, 0, KT, kt);
-    const Mom<V> U0 = SP[kt];
-    Mom<V> Z;
-    mom_zero(Z);
-    V e0[6];
-    kelvin_strain<T, V>(Z, U0, w0, g.q, nu, mu, e0);
-    const V trc = cadd(e0[0], e0[2]);
-    const V t0 = csub(cscale(e0[4], (T)2 * mu), w0[4]);
-    const V t1 = csub(cscale(e0[3], (T)2 * mu), w0[3]);
-    const V t2 = csub(caxpy(cscale(trc, lam), (T)2 * mu, e0[2]), w0[2]);
-    TR[3 * kt] = t0;
-    TR[3 * kt + 1] = t1;
-    TR[3 * kt + 2] = t2;
-    if (want_u3) {
-      // u3(0) = N_inf[w].e3 + B^T(q, 0) t . e3 (rotated frame)
-      const T K = (T)1 / ((T)8 * mu * (nu - (T)1));
-      V u = caxpy(cmuli(U0.m[3]), (T)1, U0.m[1]);  // P_33 + i P_q3
-      u = cadd(cscale(u, (T)2 - (T)4 * nu), U0.n);
-      u = cscale(u, K);
-      V ub = cscale(cmuli(t0), (T)0.5 * ((T)2 * nu - (T)1));
-      ub = caxpy(ub, -(nu - (T)1), t2);
-      u = caxpy(u, (T)1 / (g.q * mu), ub);
-      surf[(size_t)k2 * h1 + k1] = u;
-    }
-  }
-  if (want_u3 && ch == tch && special) surf[(size_t)k2 * h1 + k1] = mk<V>(0, 0);
-  // the carry from below folded into the per-node + branch (so that it is not live during
-  // the output loop)
-  if (work && ch + 1 < nch) {
-    const Mom<V> Pin = SP[(ch + 1) * KT + kt];
-    if (uniform) {
-      // a chunk above the last one is whole (e1 = n0 + C): node n0 + l lies C - l elements
-      // above e1, so its propagator is E^(C - l), built by products
-      T Ek = ec.E;
-#pragma unroll
-      for (int l = C - 1; l >= 0; --l) {
-        Mom<V> P = Pin;
-        propP_E(P, g.q * hz * (T)(C - l), Ek);
-        mom_add(Ploc[l], P);
-        Ek *= ec.E;
-      }
-    } else {
-#pragma unroll
-      for (int l = 0; l < C; ++l) {
-        if (n0 + l < nend) {
-          Mom<V> P = Pin;
-          propP(P, g.q * (zs[e1] - zs[n0 + l]));
-          mom_add(Ploc[l], P);
-        }
-      }
-    }
-  }
-  __syncthreads();
-
   if (!active) return;
+
+  // 4. complete moments, output
+  V* out = spec + (size_t)n0 * 6 * plane + (size_t)k2 * h1 + k1;
   if (special) {
-    for (int i = n0; i < nend; ++i) {
+    const int nend = min(n0 + C, nz);
+    for (int i = n0; i < nend; ++i, out += 6 * plane) {
       V w[6], o[6];
       ld6(w, W, i, KT, kt);
-      if (g.nyq) {
+      if (EIN) hooke_mode(w, lam, mu);
+      node_special(o, w, g.nyq, lam, mu, stress);
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = out_kind == FVIM_STRAIN ? mk<V>(0, 0) : cscale(w[cc], (T)-1);
-      } else {
-        // laminate: eps_33 = w_33/(lam+2mu), eps_a3 = w_a3/(2mu), eps_ab = 0
-        V e[6];
-        e[0] = e[1] = e[5] = mk<V>(0, 0);
-        e[2] = cscale(w[2], (T)1 / (lam + (T)2 * mu));
-        e[3] = cscale(w[3], (T)1 / ((T)2 * mu));
-        e[4] = cscale(w[4], (T)1 / ((T)2 * mu));
-        if (out_kind == FVIM_STRAIN) {
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
-        } else {
-          const V trc = e[2];
-#pragma unroll
-          for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
-          o[0] = caxpy(o[0], lam, trc);
-          o[1] = caxpy(o[1], lam, trc);
-          o[2] = caxpy(o[2], lam, trc);
-        }
-      }
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) spec[(size_t)(i * 6 + cc) * plane + (size_t)k2 * h1 + k1] = o[cc];
+      for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
     }
     return;
   }
-
-  // 5. forward over the chunk: - branch from its carry (scan value of the chunk above),
-  //    + branch = own part + carry from below (folded above), image term, epilogue, rotate
-  //    back, store
-  Mom<V> A;
-  if (ch > 0) A = SA[(ch - 1) * KT + kt];
-  else mom_zero(A);
-  V tr[3];
+  Br<V> cA = br_get<V, KT>(X.A + ch * 3 * KT + kt);
+  const Br<V> cP = br_get<V, KT>(X.P + ch * 3 * KT + kt);
+  {
+    const T x = g.q * zs[n0], E = dexp<T>(-x);
+    br_add_prop(cA, br_get<V, KT>(X.I + kt), E, x * E);
+  }
+  // propagators from the chunk's first node (A) and to its last one (P) and q times the distances
+  T EA[C], EP[C], xA[C], xP[C];
+  EA[0] = EP[C - 1] = (T)1;
+  xA[0] = xP[C - 1] = (T)0;
+  if (UNI) {
+    const T E = el[kt], a = el[KT + kt];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) tr[j] = TR[3 * kt + j];
-  const T imu = (T)1 / mu;
-  T ex = dexp<T>(-g.q * zs[n0]);
-  V w[6];
-  ld6(w, W, n0, KT, kt);
+    for (int l = 1; l < C; ++l) {
+      EA[l] = EP[C - 1 - l] = EA[l - 1] * E;
+      xA[l] = xP[C - 1 - l] = a * (T)l;
+    }
+  } else {
+    T Ee[C], ae[C];
+#pragma unroll
+    for (int l = 0; l < C; ++l) {
+      const bool in = n0 + l < nz;
+      Ee[l] = in ? el[(n0 + l) * EL_N * KT + kt] : (T)0;
+      ae[l] = in ? el[((n0 + l) * EL_N + 1) * KT + kt] : (T)0;
+    }
+#pragma unroll
+    for (int l = 1; l < C; ++l) {
+      EA[l] = EA[l - 1] * Ee[l - 1];
+      xA[l] = xA[l - 1] + ae[l - 1];
+      EP[C - 1 - l] = EP[C - l] * Ee[C - 1 - l];
+      xP[C - 1 - l] = xP[C - l] + ae[C - 1 - l];
+    }
+  }
+  const OutC<T> oc(rot, g.q, mu, nu, stress);
+  const LocC<T> lc(lam, mu, nu, stress);
 #pragma unroll
   for (int l = 0; l < C; ++l) {
-    const int i = n0 + l;
-    if (i < nend) {
-      const Mom<V>& P = Ploc[l];
-      V e[6];
-      kelvin_strain<T, V>(A, P, w, g.q, nu, mu, e);
-      if (!uniform && l > 0) ex = dexp<T>(-g.q * zs[i]);
-      bous_strain_add<T, V>(tr, g.q * zs[i], ex, nu, imu, e);
-      if (uniform) ex *= ec.E;
-      V o[6];
-      if (out_kind == FVIM_STRAIN) {
+    if (n0 + l < nz) {
+      br_add_prop(A[l], cA, EA[l], xA[l] * EA[l]);
+      br_add_prop(P[l], cP, EP[l], xP[l] * EP[l]);
+      V x[6], L[3], o[6];
+      ld6(x, W, n0 + l, KT, kt);
+      if (EIN) hooke_mode(x, lam, mu);
+      node_local(L, x, lc, stress);
+      node_out(o, A[l], P[l], L, oc, stress);
 #pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
-      } else {
-        const V trc = cadd(e[0], e[2]);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
-        o[0] = caxpy(o[0], lam, trc);
-        o[1] = caxpy(o[1], lam, trc);
-        o[2] = caxpy(o[2], lam, trc);
-      }
-      rotate_out(o, g.c, g.s);
-#pragma unroll
-      for (int cc = 0; cc < 6; ++cc) spec[(size_t)(i * 6 + cc) * plane + (size_t)k2 * h1 + k1] = o[cc];
-      if (i < e1) {
-        if (!uniform) ec = elem_coef<T>(g.q, zs[i + 1] - zs[i]);
-        V wj[6];
-        ld6(wj, W, i + 1, KT, kt);
-        stepA(A, ec, w, wj);
-#pragma unroll
-        for (int cc = 0; cc < 6; ++cc) w[cc] = wj[cc];
-      }
+      for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
+      out += 6 * plane;
     }
   }
 }
 
-template <typename T, int KT, int C, bool EIN, int MB>
+// shared memory of a register-variant tile
+template <typename T, int KT> struct RegSmem {
+  typedef typename Cx<T>::t V;
+  static __host__ __device__ size_t el_count(int nz, int uniform) { return (size_t)(uniform ? 1 : nz) * EL_N * KT; }
+  static __host__ __device__ size_t bytes(int nz, int nch, int uniform) {
+    return ((size_t)nz * 6 * KT + Xch<V, KT>::count(nch)) * sizeof(V) + el_count(nz, uniform) * sizeof(T) +
+           (((size_t)nz * sizeof(T) + 15) & ~(size_t)15);
+  }
+};
+
+template <typename T, int KT, int C, bool EIN, bool UNI, int MB>
 __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* __restrict__ spec,
                                                             typename Cx<T>::t* __restrict__ surf,
                                                             const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int nch,
                                                             T w1, T w2, T lam, T mu, T nu, int out_kind, int want_u3,
-                                                            int uniform, T hz, const int* __restrict__ zr, T cut,
+                                                            T hz, const int* __restrict__ zr, T cut,
                                                             const __grid_constant__ CUtensorMap tmap, int tma_rows,
                                                             int tx_extra, int* __restrict__ status) {
   typedef typename Cx<T>::t V;
   static_assert(sizeof(V) == 8 && KT % 2 == 0, "FP32 tiles of an even width");
   extern __shared__ __align__(128) unsigned char smraw[];  // tensor-copy boxes land at 128-byte offsets
   V* W = reinterpret_cast<V*>(smraw);                               // [nz][6][KT]
-  Mom<V>* SA = reinterpret_cast<Mom<V>*>(W + (size_t)nz * 6 * KT);  // [nch][KT]
-  Mom<V>* SP = SA + (size_t)nch * KT;                               // [nch][KT]
-  V* TR = reinterpret_cast<V*>(SP + (size_t)nch * KT);              // [KT][3] image traction
-  T* zs = reinterpret_cast<T*>(TR + 3 * KT);                        // [nz]
-  // mbarrier of the tensor copies, 8-byte aligned after the depth nodes
-  unsigned long long* tbar = reinterpret_cast<unsigned long long*>(
-      reinterpret_cast<unsigned char*>(zs) + (((size_t)nz * sizeof(T) + 7) & ~(size_t)7));
+  V* xbase = W + (size_t)nz * 6 * KT;
+  const Xch<V, KT> X(xbase, nch);
+  T* el = reinterpret_cast<T*>(xbase + Xch<V, KT>::count(nch));
+  T* zs = el + RegSmem<T, KT>::el_count(nz, UNI);                   // [nz]
+  // mbarrier of the tensor copies, after the depth nodes
+  unsigned long long* tbar = reinterpret_cast<unsigned long long*>(smraw + RegSmem<T, KT>::bytes(nz, nch, UNI));
   const int k2 = blockIdx.y;
   const size_t plane = (size_t)n2 * h1;
   const size_t colofs = (size_t)k2 * h1 + blockIdx.x * KT;
@@ -965,7 +838,7 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
       }
     }
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-    g = depth_prep<T, KT>(TR, threadIdx.x, blockIdx.x, k2, false, n1, n2, hs, w1, w2, uniform, hz);
+    g = depth_prep<T, KT>(el, zn, threadIdx.x, blockIdx.x, k2, false, nz, C, n1, n2, hs, w1, w2, UNI, hz);
     bool done = mbar_wait_bounded(bar, 1000000000ull);   // 1 s
     if (__syncthreads_or(!done)) {
       if (threadIdx.x == 0 && status) atomicOr(status, 1);
@@ -978,15 +851,10 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
         const int zl = idx / (6 * KT);
         if (zl < zlo || zl >= zhi) W[idx] = mk<V>(0, 0);
       }
-    }
-    __syncthreads();
-  } else if (!zr) {
-    for (int idx = threadIdx.x; idx < nz * 6 * (KT / 2); idx += blockDim.x) {
-      const int zc = idx / (KT / 2), j = 2 * (idx % (KT / 2));
-      cp_async_16(W + zc * KT + j, spec + (size_t)zc * plane + colofs + j);
+      __syncthreads();
     }
   } else {
-    const int zlo = zr[0], zhi = zr[1];
+    const int zlo = zr ? zr[0] : 0, zhi = zr ? zr[1] : nz;
     for (int idx = threadIdx.x; idx < nz * 6 * (KT / 2); idx += blockDim.x) {
       const int zc = idx / (KT / 2), j = 2 * (idx % (KT / 2));
       const int zl = zc / 6;
@@ -997,16 +865,14 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
         W[zc * KT + j + 1] = mk<V>(0, 0);
       }
     }
-  }
-  if (tma_rows <= 0) {
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-    g = depth_prep<T, KT>(TR, threadIdx.x, blockIdx.x, k2, false, n1, n2, hs, w1, w2, uniform, hz);
+    g = depth_prep<T, KT>(el, zn, threadIdx.x, blockIdx.x, k2, false, nz, C, n1, n2, hs, w1, w2, UNI, hz);
     cp_async_wait_all();
     __syncthreads();
   }
 
-  depth_r_body<T, KT, C, EIN>(W, SA, SP, TR, zs, threadIdx.x, blockIdx.x, k2, false, spec, surf, nz, n1, n2, hs, h1,
-                              nch, w1, w2, lam, mu, nu, out_kind, want_u3, uniform, hz, cut, g);
+  depth_r_body<T, KT, C, EIN, UNI>(W, X, el, zs, threadIdx.x, blockDim.x, blockIdx.x, k2, false, spec, surf, nz, n2, h1,
+                                   nch, lam, mu, nu, out_kind, want_u3, hz, cut, g);
 }
 
 // ----------------------------------------------------------------------------------
@@ -1016,9 +882,8 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
 // with its own shared-memory slot, loaded with 16-byte cp.async copies.  The cutoff vote is
 // taken over the CTA's tiles together.
 // ----------------------------------------------------------------------------------
-__host__ __device__ constexpr size_t grp_depth_slot(int nz, int nchp) {
-  return (size_t)nz * 6 * 16 * sizeof(float2) + (size_t)2 * nchp * 16 * sizeof(Mom<float2>) +
-         (size_t)3 * 16 * sizeof(float2) + (((size_t)nz * sizeof(float) + 15) & ~(size_t)15);
+inline __host__ __device__ size_t grp_depth_slot(int nz, int nchp, int uniform) {
+  return RegSmem<float, 16>::bytes(nz, nchp, uniform);
 }
 
 __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ GrpTable tab) {
@@ -1033,12 +898,12 @@ __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ Gr
   const int tile = ((int)blockIdx.x - tab.start[pi]) * tpc + j;
   const bool ghost = tile >= tiles;
   const int kblk = ghost ? 0 : tile % ncb, k2 = ghost ? 0 : tile / ncb;
-  unsigned char* base = smraw + (size_t)j * grp_depth_slot(nz, nchp);
+  unsigned char* base = smraw + (size_t)j * grp_depth_slot(nz, nchp, P.uniform);
   V* W = reinterpret_cast<V*>(base);                                // [nz][6][KT]
-  Mom<V>* SA = reinterpret_cast<Mom<V>*>(W + (size_t)nz * 6 * KT);  // [nchp][KT]
-  Mom<V>* SP = SA + (size_t)nchp * KT;                              // [nchp][KT]
-  V* TR = reinterpret_cast<V*>(SP + (size_t)nchp * KT);             // [KT][3]
-  float* zs = reinterpret_cast<float*>(TR + 3 * KT);                // [nz]
+  V* xbase = W + (size_t)nz * 6 * KT;
+  const Xch<V, KT> X(xbase, nchp);
+  float* el = reinterpret_cast<float*>(xbase + Xch<V, KT>::count(nchp));
+  float* zs = el + RegSmem<float, KT>::el_count(nz, P.uniform);     // [nz]
   if (!ghost) {
     const size_t plane = (size_t)P.n2 * P.h1;
     const size_t colofs = (size_t)k2 * P.h1 + (size_t)kblk * KT;
@@ -1049,12 +914,50 @@ __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ Gr
     for (int i = tid; i < nz; i += tt) zs[i] = P.zn[i];
   }
   const ModeGeom<float> g =
-      depth_prep<float, KT>(TR, tid, kblk, k2, ghost, P.n1, P.n2, P.hs, P.w1, P.w2, P.uniform, P.hz);
+      depth_prep<float, KT>(el, P.zn, tid, kblk, k2, ghost, nz, C, P.n1, P.n2, P.hs, P.w1, P.w2, P.uniform, P.hz);
   cp_async_wait_all();
   __syncthreads();
-  depth_r_body<float, KT, C, false>(W, SA, SP, TR, zs, tid, kblk, k2, ghost, P.spec, nullptr, nz, P.n1, P.n2, P.hs,
-                                    P.h1, P.nch, P.w1, P.w2, P.lam, P.mu, P.nu, P.out_kind, 0, P.uniform, P.hz,
-                                    P.cut, g);
+  // one body per grid kind: a CTA's tiles belong to one problem
+  if (P.uniform)
+    depth_r_body<float, KT, C, false, true>(W, X, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2, P.h1,
+                                            P.nch, P.lam, P.mu, P.nu, P.out_kind, 0, P.hz, P.cut, g);
+  else
+    depth_r_body<float, KT, C, false, false>(W, X, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2, P.h1,
+                                             P.nch, P.lam, P.mu, P.nu, P.out_kind, 0, P.hz, P.cut, g);
+}
+
+// strain of the Boussinesq-Cerruti field of a surface traction t (rotated frame, force on
+// the body per unit area, Eq. B:fourier with its gradient recurrence) at zeta = q z
+template <typename T, typename V>
+__device__ __forceinline__ void bous_strain_add(const V* tr, T zeta, T ex, T nu, T imu, V* e) {
+  // ex = exp(-zeta), imu = 1 / mu
+  const T c1 = ex * imu, c2 = (T)0.5 * ex * imu;
+  const V t0 = tr[0], t1 = tr[1], t2 = tr[2];
+  // qq: ((1-nu) i t0 + (nu - 1/2) t2 + zeta(-i t0/2 + t2/2)) / mu
+  //   = ((1 - nu) - zeta/2) i t0 + ((nu - 1/2) + zeta/2) t2
+  V v = caxpy_i(cscale(t2, nu - (T)0.5 + (T)0.5 * zeta), (T)1 - nu - (T)0.5 * zeta, t0);
+  e[0] = caxpy(e[0], c1, v);
+  // 33: (-2 i nu t0 + (2nu-1) t2 + zeta (i t0 - t2)) / (2 mu)
+  //   = (zeta - 2 nu) i t0 + ((2 nu - 1) - zeta) t2
+  v = caxpy_i(cscale(t2, (T)2 * nu - (T)1 - zeta), zeta - (T)2 * nu, t0);
+  e[2] = caxpy(e[2], c2, v);
+  // p3: -t1 / (2 mu) ; qp: i t1 / (2 mu)
+  e[3] = caxpy(e[3], -c2, t1);
+  e[5] = caxpy_i(e[5], c2, t1);
+  // q3: (-t0 + zeta (t0 + i t2)) / (2 mu) = (zeta - 1) t0 + zeta i t2
+  v = caxpy_i(cscale(t0, zeta - (T)1), zeta, t2);
+  e[4] = caxpy(e[4], c2, v);
+}
+
+template <typename T, typename V>
+__device__ __forceinline__ void rotate_out(V* y, T c, T s) {
+  const V qq = y[0], pp = y[1], p3 = y[3], q3 = y[4], qp = y[5];
+  const T cc = c * c, ss = s * s, cs = c * s;
+  y[0] = caxpy(caxpy(cscale(qq, cc), ss, pp), (T)-2 * cs, qp);
+  y[1] = caxpy(caxpy(cscale(qq, ss), cc, pp), (T)2 * cs, qp);
+  y[3] = caxpy(cscale(q3, s), c, p3);
+  y[4] = caxpy(cscale(q3, c), -s, p3);
+  y[5] = caxpy(caxpy(cscale(qq, cs), -cs, pp), cc - ss, qp);
 }
 
 // ----------------------------------------------------------------------------------
@@ -1142,18 +1045,22 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   const int nz = c->nz, h1 = c->h1;
   d.ok = false;
   if (C < 2 || C > nz) return d;
+  // the launch limits of a plan: 16-column tiles of [Nz][6] values and 12 values per chunk (register
+  // variant) or per node (shared-memory variant), which every layout below stays within
+  constexpr size_t kMom = 6 * sizeof(V);
   if constexpr (sizeof(T) == 4) {
     // FP32, 16-column tiles, at most 8 nodes per chunk: the register variant (C rounded up
     // to an instantiated chunk length)
     if (h1 >= KT_MAX && C <= 8) {
       const int CR = C <= 2 ? 2 : (C <= 3 ? 3 : (C <= 4 ? 4 : (C <= 6 ? 6 : 8)));
       const int nchr = (nz + CR - 1) / CR;
-      const size_t smr = (size_t)nz * 6 * 16 * sizeof(V) + (size_t)(2 * nchr) * 16 * sizeof(Mom<V>) +
+      const size_t lim = (size_t)nz * 6 * 16 * sizeof(V) + (size_t)(2 * nchr) * 16 * kMom +
                          (size_t)3 * 16 * sizeof(V) + (((size_t)nz * sizeof(T) + 7) & ~(size_t)7) + 16;
-      if (smr <= 227 * 1024 && 16 * nchr <= 256) {
+      if (lim <= 227 * 1024 && 16 * nchr <= 256) {
         // three CTAs per SM (85 registers): chunk lengths 4..8 whose tile fits three times
-        if (ctas == 3 && !(CR >= 4 && 3 * (smr + 1024) <= 228 * 1024)) return d;
-        d = DepthCfg<T>{true, true, CR, nchr, 16, 16 * nchr, smr, ctas == 3 ? 3 : 2};
+        if (ctas == 3 && !(CR >= 4 && 3 * (lim + 1024) <= 228 * 1024)) return d;
+        d = DepthCfg<T>{true, true, CR, nchr, 16, 16 * nchr, RegSmem<T, 16>::bytes(nz, nchr, c->uniform) + 16,
+                        ctas == 3 ? 3 : 2};
         return d;
       }
     }
@@ -1161,20 +1068,26 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   if (ctas == 3) return d;  // the shared-memory variant has one launch shape per chunk length
   const int nch = (nz + C - 1) / C;
   const int prow = nz > 2 * nch + 1 ? nz : 2 * nch + 1;
-  // tile width: 16 k1 columns (128-byte rows in FP32), narrower where the depth column of
-  // the tile does not fit in shared memory (deep grids, FP64)
-  int KT = h1 < KT_MAX ? h1 : KT_MAX;  // h1 is a power of two
-  auto smem_of = [&](int kt) {
-    return (size_t)nz * 6 * kt * sizeof(V) + (size_t)prow * kt * sizeof(Mom<V>) + (size_t)nz * sizeof(T);
+  auto lim_of = [&](int kt) {
+    return (size_t)nz * 6 * kt * sizeof(V) + (size_t)prow * kt * kMom + (size_t)nz * sizeof(T);
   };
-  while (KT > 2 && smem_of(KT) > 227 * 1024) KT >>= 1;
+  int KT = h1 < KT_MAX ? h1 : KT_MAX;  // h1 is a power of two or a multiple of 16
+  while (KT > 2 && lim_of(KT) > 227 * 1024) KT >>= 1;
+  d.ok = lim_of(KT) <= 227 * 1024 && KT * nch <= 256;
+  // tile width of the launch: as wide as fits twice on an SM, and at least one 32-byte sector
+  auto smem_of = [&](int kt) {
+    const size_t vals = (size_t)nz * (C <= 8 ? 6 : 9) * kt + 6 * (size_t)(nch + 1) * kt;
+    const size_t reals = (size_t)(c->uniform ? 1 : nz) * EL_N * kt + (size_t)(c->uniform ? C : nz) * kt + nz;
+    return vals * sizeof(V) + reals * sizeof(T);
+  };
+  const int kmin = 32 / (int)sizeof(V);
+  while (KT > 2 && (smem_of(KT) > 227 * 1024 || (KT > kmin && smem_of(KT) > 113 * 1024))) KT >>= 1;
   d.C = C;
   d.nch = nch;
   d.KT = KT;
   d.threads = KT * nch;
   d.smem = smem_of(KT);
   d.reg = false;
-  d.ok = d.smem <= 227 * 1024 && d.threads <= 256;
   return d;
 }
 
@@ -1196,7 +1109,6 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
   const DepthCfg<T> d = depth_cfg<T>(c, c->depth_chunk > 0 ? c->depth_chunk : depth_chunk_default(nz), c->depth_ctas);
   if (!d.ok) return FVIM_ERR_UNSUPPORTED;
   const int KT = d.KT, C = d.C, nch = d.nch;
-  const int prow = nz > 2 * nch + 1 ? nz : 2 * nch + 1;
   dim3 grid(h1 / KT, n2);
   const T w1 = (T)(kTwoPi / c->L1), w2 = (T)(kTwoPi / c->L2);
   if constexpr (sizeof(T) == 4) if (d.reg) {
@@ -1209,33 +1121,32 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
     } else {
       memset(&tm, 0, sizeof(tm));
     }
-#define DEPTHR(CV, EI, MBV)                                                                                     \
-  if (C == CV && eps_in == EI && d.mb == MBV) {                                                                 \
-    smem_cap(k_mindlin_depth_r<T, 16, CV, EI, MBV>);                                                            \
-    k_mindlin_depth_r<T, 16, CV, EI, MBV><<<grid, d.threads, d.smem, c->stream>>>(                              \
+#define DEPTHR(CV, EI, UN, MBV)                                                                                 \
+  if (C == CV && eps_in == EI && (c->uniform != 0) == UN && d.mb == MBV) {                                      \
+    smem_cap(k_mindlin_depth_r<T, 16, CV, EI, UN, MBV>);                                                        \
+    k_mindlin_depth_r<T, 16, CV, EI, UN, MBV><<<grid, d.threads, d.smem, c->stream>>>(                          \
         (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, nch, w1, w2, (T)c->lam, (T)c->mu, \
-        (T)c->nu,                                                                                              \
-        out_kind, want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,  \
+        (T)c->nu, out_kind, want_u3 ? 1 : 0, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,    \
         c->dev_status);                                                                                          \
   }
-    DEPTHR(2, false, 2) DEPTHR(3, false, 2) DEPTHR(4, false, 2) DEPTHR(6, false, 2) DEPTHR(8, false, 2)
-    DEPTHR(2, true, 2) DEPTHR(3, true, 2) DEPTHR(4, true, 2) DEPTHR(6, true, 2) DEPTHR(8, true, 2)
-    DEPTHR(4, false, 3) DEPTHR(6, false, 3) DEPTHR(8, false, 3)
-    DEPTHR(4, true, 3) DEPTHR(6, true, 3) DEPTHR(8, true, 3)
+#define DEPTHR2(CV, MBV) \
+  DEPTHR(CV, false, true, MBV) DEPTHR(CV, false, false, MBV) DEPTHR(CV, true, true, MBV) DEPTHR(CV, true, false, MBV)
+    DEPTHR2(2, 2) DEPTHR2(3, 2) DEPTHR2(4, 2) DEPTHR2(6, 2) DEPTHR2(8, 2)
+    DEPTHR2(4, 3) DEPTHR2(6, 3) DEPTHR2(8, 3)
+#undef DEPTHR2
 #undef DEPTHR
     FVIM_CUDA_CHECK_LAUNCH();
     return FVIM_OK;
   }
-#define DEPTH(KTV, EI)                                                                                         \
-  if (KT == KTV && eps_in == EI) {                                                                             \
-    smem_cap(k_mindlin_depth<T, KTV, EI>);                                                                     \
-    k_mindlin_depth<T, KTV, EI><<<grid, d.threads, d.smem, c->stream>>>(                                       \
-        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, prow, w1, w2, (T)c->lam,  \
-        (T)c->mu,                                                                                              \
-        (T)c->nu, out_kind, want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr);                                       \
+#define DEPTH(KTV, LSV)                                                                                        \
+  if (KT == KTV && (C <= 8) == LSV) {                                                                          \
+    smem_cap(k_mindlin_depth<T, KTV, LSV>);                                                                    \
+    k_mindlin_depth<T, KTV, LSV><<<grid, d.threads, d.smem, c->stream>>>(                                      \
+        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, w1, w2, (T)c->lam,      \
+        (T)c->mu, (T)c->nu, out_kind, want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, eps_in ? 1 : 0);              \
   }
-  DEPTH(16, false) DEPTH(8, false) DEPTH(4, false) DEPTH(2, false)
   DEPTH(16, true) DEPTH(8, true) DEPTH(4, true) DEPTH(2, true)
+  DEPTH(16, false) DEPTH(8, false) DEPTH(4, false) DEPTH(2, false)
 #undef DEPTH
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -1266,7 +1177,7 @@ int launch_grp_depth(GrpTable& t, cudaStream_t s) {
     const int tpc = 16 / P.nchp, tiles = (P.h1 / 16) * P.n2;
     t.start[i] = b;
     b += (tiles + tpc - 1) / tpc;
-    smem = std::max(smem, (size_t)tpc * grp_depth_slot(P.nz, P.nchp));
+    smem = std::max(smem, (size_t)tpc * grp_depth_slot(P.nz, P.nchp, P.uniform));
   }
   t.start[t.n] = b;
   if (b == 0) return FVIM_OK;
