@@ -615,13 +615,12 @@ int fvim_apply_mindlin_group(fvim_ctx* const* ctx, int n, const void* const* eps
     P.nchp = 1;
     while (P.nchp < P.nch) P.nchp <<= 1;
     P.uniform = c->uniform;
-    P.out_kind = out_kind;
     const double two_pi = 6.283185307179586476925;
     P.w1 = (float)(two_pi / c->L1);
     P.w2 = (float)(two_pi / c->L2);
     P.lam = (float)c->lam;
     P.mu = (float)c->mu;
-    P.nu = (float)c->nu;
+    P.dm = depth_mat<float>(c->lam, c->mu, c->nu, out_kind);
     P.hz = (float)c->hz;
     P.cut = c->depth_cut;
     // the k1 = N1/2 column never goes through the column transforms, so it carries the

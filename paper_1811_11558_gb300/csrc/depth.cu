@@ -16,9 +16,9 @@
 //     n = int g0 n,   a = int g0 a,   v = int g0 m -+ int g1 n.
 //   (The generic form carries five rotated components and one contraction per branch, and
 //   evaluates the image field per node: 457 warp instructions per warp of nodes, measured on
-//   512 x 512 x 64 FP32.  Depth kernel, ms, generic form -> this one: 512 x 512 x 64 FP32 0.204
-//   -> 0.146, 1024 x 1024 x 32 (C = 2) 0.642 -> 0.465, 256 x 128 x 57 refined 0.043 -> 0.027,
-//   128 x 128 x 126 FP64 1.163 -> 0.385.)
+//   512 x 512 x 64 FP32, against 236 here.  Depth kernel, ms, generic form -> this one: 512 x
+//   512 x 64 FP32 0.204 -> 0.146, 1024 x 1024 x 32 (C = 2) 0.642 -> 0.339, 256 x 128 x 57
+//   refined 0.043 -> 0.028, 128 x 128 x 126 FP64 1.163 -> 0.355.)
 // * Depth integral: the g0/g1 kernels are exponentials exp(-q|y3 - x3|) times polynomials, so
 //   the moments follow from those of the neighbouring node by exact one-element steps,
 //     v <- e^{-qh}(v - qh n) + ...,  n <- e^{-qh} n + ...,  a <- e^{-qh} a + ...,
@@ -57,8 +57,7 @@ template <> __device__ __forceinline__ double dexp<double>(double x) { return ex
 // global timer and at most 2^24 polls (should the timer not advance); true when the phase
 // completed
 __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned long long limit_ns) {
-  unsigned long long t0;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+  unsigned long long t0 = 0;
   for (int it = 0; it < (1 << 24); ++it) {
     unsigned ok;
     asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], 0;\n selp.u32 %0, 1, 0, p;\n}"
@@ -68,6 +67,7 @@ __device__ __forceinline__ bool mbar_wait_bounded(unsigned bar, unsigned long lo
     if (ok) return true;
     unsigned long long t;
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    if (it == 0) t0 = t;
     if (t - t0 > limit_ns) return false;
   }
   return false;
@@ -159,132 +159,6 @@ __device__ __forceinline__ void br_add_prop(Br<V>& d, const Br<V>& c, T E, T xE)
   d.a = caxpy(d.a, E, c.a);
 }
 
-// Direction cosines and their products for the rotation into the (q, p, 3) frame.
-template <typename T> struct Rot {
-  T c, s, cc, ss, cs, c2;
-  __device__ __forceinline__ Rot(T c_, T s_) : c(c_), s(s_), cc(c_ * c_), ss(s_ * s_), cs(c_ * s_), c2(c_ * c_ - s_ * s_) {}
-};
-// nodal sources of both branches from w (11, 22, 33, 23, 13, 12)
-template <typename V> struct Src {
-  V nA, nP, m, aA, aP;
-};
-template <typename T, typename V>
-__device__ __forceinline__ Src<V> node_source(const V* x, const Rot<T>& r, T m_scale) {
-  const V qq = caxpy(caxpy(cscale(x[0], r.cc), r.ss, x[1]), (T)2 * r.cs, x[5]);
-  const V qp = caxpy(cscale(csub(x[1], x[0]), r.cs), r.c2, x[5]);
-  const V q3 = caxpy(cscale(x[4], r.c), r.s, x[3]);
-  const V p3 = caxpy(cscale(x[3], r.c), -r.s, x[4]);
-  const V d = csub(x[2], qq);
-  Src<V> o;
-  o.nA = caxpy_i(d, (T)-2, q3);
-  o.nP = caxpy_i(d, (T)2, q3);
-  o.m = cscale(cadd(x[2], qq), m_scale);
-  o.aA = caxpy_i(qp, (T)1, p3);
-  o.aP = caxpy_i(qp, (T)-1, p3);
-  return o;
-}
-template <typename T, typename V> __device__ __forceinline__ void hooke_mode(V* x, T lam, T mu) {
-  const V tr = cadd(cadd(x[0], x[1]), x[2]);
-#pragma unroll
-  for (int cc = 0; cc < 6; ++cc) x[cc] = cscale(x[cc], (T)2 * mu);
-#pragma unroll
-  for (int cc = 0; cc < 3; ++cc) x[cc] = caxpy(x[cc], lam, tr);
-}
-
-// Output of a node from the complete moments of both branches: with kappa = q / (4 (1 - nu)),
-//   sigma_33 = kappa (v_A + v_P),             sigma_q3 = -i kappa (v_A - v_P + n_A - n_P),
-//   sigma_qq = -kappa (v_A + v_P + 2 (n_A + n_P)),   sigma_pp = -2 nu kappa (n_A + n_P),
-//   sigma_p3 = i q/2 (a_A - a_P),             sigma_qp = q/2 (a_A + a_P)
-// plus the local terms; the strain is the same with 2 - 2 nu for the factor 2 of qq, 2 nu (n_A
-// + n_P) added to 33, no pp component, all over 2 mu.  The constants of the rotation back are
-// folded into the combinations.
-template <typename T> struct OutC {
-  T w, t, k11w, k22w, k12w, k11n, k22n, k12n, k11a, k12a, k33, cy, sy, cz, sz;
-  __device__ __forceinline__ OutC(const Rot<T>& r, T q, T mu, T nu, bool stress) {
-    const T sc = stress ? (T)1 : (T)1 / ((T)2 * mu);
-    const T kap = sc * q / ((T)4 * ((T)1 - nu)), q2 = sc * (T)0.5 * q;
-    const T p = stress ? (T)-2 * nu * kap : (T)0;
-    w = stress ? (T)2 : (T)2 - (T)2 * nu;
-    t = stress ? (T)0 : (T)2 * nu;
-    k11w = -kap * r.cc; k22w = -kap * r.ss; k12w = -kap * r.cs;
-    k11n = p * r.ss; k22n = p * r.cc; k12n = -p * r.cs;
-    k11a = (T)-2 * q2 * r.cs; k12a = q2 * r.c2;
-    k33 = kap;
-    cy = kap * r.c; sy = kap * r.s; cz = q2 * r.c; sz = q2 * r.s;
-  }
-};
-// L: local terms (stress: 11, 22, 12; strain: 33, 23, 13)
-template <typename T, typename V>
-__device__ __forceinline__ void node_out(V* o, const Br<V>& A, const Br<V>& P, const V* L, const OutC<T>& k,
-                                         bool stress) {
-  const V N = cadd(A.n, P.n), Vv = cadd(A.v, P.v), z = csub(A.a, P.a), sa = cadd(A.a, P.a);
-  const V y = cadd(csub(A.v, P.v), csub(A.n, P.n));
-  const V W = caxpy(Vv, k.w, N);
-  const V g = caxpy(cscale(y, k.cy), k.sz, z);   // 13 = -i g
-  const V h = caxpy(cscale(z, k.cz), -k.sy, y);  // 23 = i h
-  if (stress) {
-    o[0] = caxpy(caxpy(caxpy(L[0], k.k11w, W), k.k11n, N), k.k11a, sa);
-    o[1] = caxpy(caxpy(caxpy(L[1], k.k22w, W), k.k22n, N), -k.k11a, sa);
-    o[2] = cscale(Vv, k.k33);
-    o[3] = mk<V>(-h.y, h.x);
-    o[4] = mk<V>(g.y, -g.x);
-    o[5] = caxpy(caxpy(caxpy(L[2], k.k12w, W), k.k12n, N), k.k12a, sa);
-  } else {
-    o[0] = caxpy(cscale(W, k.k11w), k.k11a, sa);
-    o[1] = caxpy(cscale(W, k.k22w), -k.k11a, sa);
-    o[2] = caxpy(L[0], k.k33, caxpy(Vv, k.t, N));
-    o[3] = mk<V>(L[1].x - h.y, L[1].y + h.x);
-    o[4] = mk<V>(L[2].x + g.y, L[2].y - g.x);
-    o[5] = caxpy(cscale(W, k.k12w), k.k12a, sa);
-  }
-}
-// local terms of a node from w: stress nu / (1 - nu) w_33 - w_11, .. - w_22, -w_12 (the others
-// cancel); strain w_33 / (lam + 2 mu), w_23 / (2 mu), w_13 / (2 mu)
-template <typename T> struct LocC {
-  T a, b;
-  __device__ __forceinline__ LocC(T lam, T mu, T nu, bool stress)
-      : a(stress ? nu / ((T)1 - nu) : (T)1 / (lam + (T)2 * mu)), b((T)1 / ((T)2 * mu)) {}
-};
-template <typename T, typename V>
-__device__ __forceinline__ void node_local(V* L, const V* x, const LocC<T>& k, bool stress) {
-  if (stress) {
-    const V t = cscale(x[2], k.a);
-    L[0] = csub(t, x[0]);
-    L[1] = csub(t, x[1]);
-    L[2] = mk<V>(-x[5].x, -x[5].y);
-  } else {
-    L[0] = cscale(x[2], k.a);
-    L[1] = cscale(x[3], k.b);
-    L[2] = cscale(x[4], k.b);
-  }
-}
-// output of a node of a mode without depth recursion: k = 0 (laminate) or outside Z^2_N (nyq)
-template <typename T, typename V>
-__device__ __forceinline__ void node_special(V* o, const V* w, bool nyq, T lam, T mu, bool stress) {
-  if (nyq) {
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) o[cc] = stress ? cscale(w[cc], (T)-1) : mk<V>(0, 0);
-    return;
-  }
-  // laminate: eps_33 = w_33/(lam+2mu), eps_a3 = w_a3/(2mu), eps_ab = 0
-  V e[6];
-  e[0] = e[1] = e[5] = mk<V>(0, 0);
-  e[2] = cscale(w[2], (T)1 / (lam + (T)2 * mu));
-  e[3] = cscale(w[3], (T)1 / ((T)2 * mu));
-  e[4] = cscale(w[4], (T)1 / ((T)2 * mu));
-  if (!stress) {
-#pragma unroll
-    for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
-    return;
-  }
-  const V trc = e[2];
-#pragma unroll
-  for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * mu), w[cc]);
-  o[0] = caxpy(o[0], lam, trc);
-  o[1] = caxpy(o[1], lam, trc);
-  o[2] = caxpy(o[2], lam, trc);
-}
-
 template <typename T> struct ModeGeom {
   T q, c, s;
   bool zero, nyq;
@@ -309,6 +183,156 @@ __device__ __forceinline__ ModeGeom<T> mode_geom(int k1, int k2, int n1, int n2,
   return g;
 }
 
+// Constants of a column (one mode), evaluated once per column while the tile is in flight and read
+// from shared memory by the column's chunk threads: evaluated by every thread they were half of
+// the instructions at two nodes per thread.  The trailing pad spreads the columns' 16-byte reads
+// over the banks.  (With this and the four-chunk read-ahead of the carries: C = 2 at 1024 x 1024 x
+// 32 0.465 -> 0.339 ms, FP64 128 x 128 x 126 0.385 -> 0.355.)
+template <typename T> struct __align__(16) ColIn {
+  T E, a, b0, b1, d0, d1;        // element coefficients of a uniform grid
+  T c, s, cc, ss, cs2, cs, c2;   // rotation: cos, sin, cos^2, sin^2, 2 cos sin, cos sin, cos^2 - sin^2
+  T q, kind, pad;                // wavenumber; 0 recursion, 1 laminate (k = 0), 2 outside Z^2_N
+  __device__ __forceinline__ El<T> el() const {
+    El<T> e;
+    e.E = E; e.a = a; e.b0 = b0; e.b1 = b1; e.d0 = d0; e.d1 = d1;
+    return e;
+  }
+};
+// Output of a node from the complete moments of both branches: with kappa = q / (4 (1 - nu)),
+//   sigma_33 = kappa (v_A + v_P),             sigma_q3 = -i kappa (v_A - v_P + n_A - n_P),
+//   sigma_qq = -kappa (v_A + v_P + 2 (n_A + n_P)),   sigma_pp = -2 nu kappa (n_A + n_P),
+//   sigma_p3 = i q/2 (a_A - a_P),             sigma_qp = q/2 (a_A + a_P)
+// plus the local terms; the strain is the same with 2 - 2 nu for the factor 2 of qq, 2 nu (n_A
+// + n_P) added to 33, no pp component, all over 2 mu.  The constants of the rotation back are
+// folded into the combinations.
+template <typename T> struct __align__(16) ColOut {
+  T k11w, k22w, k12w, k11n, k22n, k12n, k11a, k12a, k33, cy, sy, cz, sz, pad[3];
+};
+template <typename T> struct __align__(16) Col {
+  ColIn<T> in;
+  ColOut<T> out;
+  T pad[4];
+};
+
+// constants of column k1 of row k2 (uniform: with the element coefficients of spacing hz)
+template <typename T>
+__device__ __forceinline__ void col_put(Col<T>* p, int k1, int k2, int n1, int n2, int hs, T w1, T w2, const DepthMat<T>& m,
+                                        bool uniform, T hz) {
+  const ModeGeom<T> g = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2);
+  ColIn<T> i;
+  El<T> e = {0, 0, 0, 0, 0, 0};
+  if (uniform) e = elem_coef<T>(g.q, hz);
+  i.E = e.E; i.a = e.a; i.b0 = e.b0; i.b1 = e.b1; i.d0 = e.d0; i.d1 = e.d1;
+  i.c = g.c; i.s = g.s; i.cc = g.c * g.c; i.ss = g.s * g.s; i.cs = g.c * g.s; i.cs2 = (T)2 * i.cs; i.c2 = i.cc - i.ss;
+  i.q = g.q;
+  i.kind = g.nyq ? (T)2 : (g.zero ? (T)1 : (T)0);
+  i.pad = 0;
+  p->in = i;
+  const T kap = m.kap * g.q, q2 = m.hq * g.q, pp = m.p * kap;
+  ColOut<T> o;
+  o.k11w = -kap * i.cc; o.k22w = -kap * i.ss; o.k12w = -kap * i.cs;
+  o.k11n = pp * i.ss; o.k22n = pp * i.cc; o.k12n = -pp * i.cs;
+  o.k11a = -q2 * i.cs2; o.k12a = q2 * i.c2;
+  o.k33 = kap;
+  o.cy = kap * g.c; o.sy = kap * g.s; o.cz = q2 * g.c; o.sz = q2 * g.s;
+  o.pad[0] = o.pad[1] = o.pad[2] = 0;
+  p->out = o;
+}
+
+// nodal sources of both branches from w (11, 22, 33, 23, 13, 12)
+template <typename V> struct Src {
+  V nA, nP, m, aA, aP;
+};
+template <typename T, typename V>
+__device__ __forceinline__ Src<V> node_source(const V* x, const ColIn<T>& r, T m_scale) {
+  const V qq = caxpy(caxpy(cscale(x[0], r.cc), r.ss, x[1]), r.cs2, x[5]);
+  const V qp = caxpy(cscale(csub(x[1], x[0]), r.cs), r.c2, x[5]);
+  const V q3 = caxpy(cscale(x[4], r.c), r.s, x[3]);
+  const V p3 = caxpy(cscale(x[3], r.c), -r.s, x[4]);
+  const V d = csub(x[2], qq);
+  Src<V> o;
+  o.nA = caxpy_i(d, (T)-2, q3);
+  o.nP = caxpy_i(d, (T)2, q3);
+  o.m = cscale(cadd(x[2], qq), m_scale);
+  o.aA = caxpy_i(qp, (T)1, p3);
+  o.aP = caxpy_i(qp, (T)-1, p3);
+  return o;
+}
+template <typename T, typename V> __device__ __forceinline__ void hooke_mode(V* x, T lam, T mu) {
+  const V tr = cadd(cadd(x[0], x[1]), x[2]);
+#pragma unroll
+  for (int cc = 0; cc < 6; ++cc) x[cc] = cscale(x[cc], (T)2 * mu);
+#pragma unroll
+  for (int cc = 0; cc < 3; ++cc) x[cc] = caxpy(x[cc], lam, tr);
+}
+
+// L: local terms (stress: 11, 22, 12; strain: 33, 23, 13)
+template <typename T, typename V>
+__device__ __forceinline__ void node_out(V* o, const Br<V>& A, const Br<V>& P, const V* L, const ColOut<T>& k,
+                                         const DepthMat<T>& m) {
+  const V N = cadd(A.n, P.n), Vv = cadd(A.v, P.v), z = csub(A.a, P.a), sa = cadd(A.a, P.a);
+  const V y = cadd(csub(A.v, P.v), csub(A.n, P.n));
+  const V W = caxpy(Vv, m.w, N);
+  const V g = caxpy(cscale(y, k.cy), k.sz, z);   // 13 = -i g
+  const V h = caxpy(cscale(z, k.cz), -k.sy, y);  // 23 = i h
+  if (m.stress) {
+    o[0] = caxpy(caxpy(caxpy(L[0], k.k11w, W), k.k11n, N), k.k11a, sa);
+    o[1] = caxpy(caxpy(caxpy(L[1], k.k22w, W), k.k22n, N), -k.k11a, sa);
+    o[2] = cscale(Vv, k.k33);
+    o[3] = mk<V>(-h.y, h.x);
+    o[4] = mk<V>(g.y, -g.x);
+    o[5] = caxpy(caxpy(caxpy(L[2], k.k12w, W), k.k12n, N), k.k12a, sa);
+  } else {
+    o[0] = caxpy(cscale(W, k.k11w), k.k11a, sa);
+    o[1] = caxpy(cscale(W, k.k22w), -k.k11a, sa);
+    o[2] = caxpy(L[0], k.k33, caxpy(Vv, m.t, N));
+    o[3] = mk<V>(L[1].x - h.y, L[1].y + h.x);
+    o[4] = mk<V>(L[2].x + g.y, L[2].y - g.x);
+    o[5] = caxpy(cscale(W, k.k12w), k.k12a, sa);
+  }
+}
+// local terms of a node from w: stress nu / (1 - nu) w_33 - w_11, .. - w_22, -w_12 (the others
+// cancel); strain w_33 / (lam + 2 mu), w_23 / (2 mu), w_13 / (2 mu)
+template <typename T, typename V>
+__device__ __forceinline__ void node_local(V* L, const V* x, const DepthMat<T>& m) {
+  if (m.stress) {
+    const V t = cscale(x[2], m.la);
+    L[0] = csub(t, x[0]);
+    L[1] = csub(t, x[1]);
+    L[2] = mk<V>(-x[5].x, -x[5].y);
+  } else {
+    L[0] = cscale(x[2], m.la);
+    L[1] = cscale(x[3], m.iu);
+    L[2] = cscale(x[4], m.iu);
+  }
+}
+// output of a node of a mode without depth recursion: k = 0 (laminate) or outside Z^2_N (nyq)
+template <typename T, typename V>
+__device__ __forceinline__ void node_special(V* o, const V* w, bool nyq, const DepthMat<T>& m) {
+  if (nyq) {
+#pragma unroll
+    for (int cc = 0; cc < 6; ++cc) o[cc] = m.stress ? cscale(w[cc], (T)-1) : mk<V>(0, 0);
+    return;
+  }
+  // laminate: eps_33 = w_33/(lam+2mu), eps_a3 = w_a3/(2mu), eps_ab = 0
+  V e[6];
+  e[0] = e[1] = e[5] = mk<V>(0, 0);
+  e[2] = cscale(w[2], (T)1 / (m.lam + (T)2 * m.mu));
+  e[3] = cscale(w[3], m.iu);
+  e[4] = cscale(w[4], m.iu);
+  if (!m.stress) {
+#pragma unroll
+    for (int cc = 0; cc < 6; ++cc) o[cc] = e[cc];
+    return;
+  }
+  const V trc = e[2];
+#pragma unroll
+  for (int cc = 0; cc < 6; ++cc) o[cc] = csub(cscale(e[cc], (T)2 * m.mu), w[cc]);
+  o[0] = caxpy(o[0], m.lam, trc);
+  o[1] = caxpy(o[1], m.lam, trc);
+  o[2] = caxpy(o[2], m.lam, trc);
+}
+
 // Chunk exchange area of a tile (values per column): the carries S of the A branch and T of the
 // P branch, [nch][3] each; slot R: the P moments of node 0 without their carry; slot I: the
 // image field at the surface.
@@ -330,11 +354,11 @@ template <typename V, int KT> __device__ __forceinline__ Br<V> br_get(const V* p
 // Carries into every chunk, in place over the chunks' own ones (A: arriving at the chunk's first
 // node, P: at its last), then the complete P moments of node 0, the image field and the surface
 // displacement.  Work item t = role KT + column, roles 0: P (n, v), 1: A (n, v), 2: P a, 3: A a.
-// The column of item t is that of the calling thread (KT divides both thread counts).  local: a
-// chunk's carry is its neighbour's own one (cutoff).
+// The column of item t is that of the calling thread (KT divides both thread counts).  Four chunks
+// are read ahead of the recurrence, whose chain is then one multiply-add per chunk.
 template <typename T, int KT>
 __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& X, const T* zs, int tid, int nthr, int C,
-                                              int nch, int nz, T q, bool uniform, T hz, bool local, bool live,
+                                              int nch, int nz, T q, bool uniform, T hz, bool live,
                                               typename Cx<T>::t* u3, T u3_scale) {
   typedef typename Cx<T>::t V;
   const int col = tid & (KT - 1);
@@ -346,32 +370,40 @@ __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& 
   for (int t = tid; t < 4 * KT; t += nthr) {
     const bool isA = (t / KT) & 1, isa = t / KT >= 2;
     const int step = isA ? 3 * KT : -3 * KT;
+    // components: slot 0 (n) and slot 1 (v), or slot 2 (a) alone
     V* p = (isA ? X.A : X.P + (size_t)(nch - 1) * 3 * KT) + col + (isa ? 2 * KT : 0);
     V rn = mk<V>(0, 0), rv = mk<V>(0, 0);
-    V sn = p[0], sv = isa ? rv : p[KT];
-    for (int jj = 0; jj < nch; ++jj) {
-      V* pn = p + step;
-      V nn = rn, nv = rv;
-      if (jj + 1 < nch) {   // the next chunk's own carry, ahead of the recurrence
-        nn = pn[0];
-        if (!isa) nv = pn[KT];
+    for (int j0 = 0; j0 < nch; j0 += 4) {
+      V sn[4], sv[4];
+      T E[4], xE[4];
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        sn[k] = sv[k] = mk<V>(0, 0);
+        E[k] = Eu;
+        xE[k] = xu * Eu;
+        if (j0 + k < nch) {
+          sn[k] = p[k * step];
+          if (!isa) sv[k] = p[k * step + KT];
+          if (!uniform) {
+            const int n0 = (isA ? j0 + k : nch - 1 - j0 - k) * C;
+            const int lo = isA ? n0 : max(n0 - 1, 0);
+            const int hi = min(isA ? n0 + C : n0 + C - 1, nz - 1);
+            const T x = q * (zs[hi] - zs[lo]);
+            E[k] = dexp<T>(-x);
+            xE[k] = x * E[k];
+          }
+        }
       }
-      p[0] = rn;
-      if (!isa) p[KT] = rv;
-      T E = Eu, x = xu;
-      if (!uniform) {
-        const int n0 = (isA ? jj : nch - 1 - jj) * C;
-        const int lo = isA ? n0 : max(n0 - 1, 0);
-        const int hi = min(isA ? n0 + C : n0 + C - 1, nz - 1);
-        x = q * (zs[hi] - zs[lo]);
-        E = dexp<T>(-x);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (j0 + k < nch) {
+          p[k * step] = rn;
+          if (!isa) p[k * step + KT] = rv;
+          rv = caxpy(caxpy(sv[k], -xE[k], rn), E[k], rv);
+          rn = caxpy(sn[k], E[k], rn);
+        }
       }
-      if (local) E = (T)0;
-      rv = caxpy(sv, E, caxpy(rv, -x, rn));
-      rn = caxpy(sn, E, rn);
-      sn = nn;
-      sv = nv;
-      p = pn;
+      p += 4 * step;
     }
     if (!isA && live) {
       const T x = q * (zs[min(C - 1, nz - 1)] - zs[0]);
@@ -381,7 +413,7 @@ __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& 
       } else {
         const V dn = X.P[col], dv = X.P[KT + col];
         const V n = caxpy(X.R[col], E, dn);
-        const V v = caxpy(X.R[KT + col], E, caxpy(dv, -x, dn));
+        const V v = caxpy(caxpy(X.R[KT + col], E, dv), -x * E, dn);
         X.I[col] = caxpy(n, (T)2, v);
         X.I[KT + col] = mk<V>(-v.x, -v.y);
         if (u3) *u3 = cscale(v, u3_scale);
@@ -396,13 +428,13 @@ __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& 
 // smem: W[nz][6][KT] (input, then the chunk's own moments in place; LS false: [nz][9][KT] with the
 // local terms), exchange area, element coefficients, depth nodes.
 // LS: at most 8 nodes per chunk, their local terms in registers.
-// Bound by the FP64 pipe in FP64 (two multiply-adds per clock and SM): 1163 -> 385 us at
+// Bound by the FP64 pipe in FP64 (two multiply-adds per clock and SM): 1163 -> 355 us at
 // 128 x 128 x 126 when the moments went from six to three per branch.
 // ----------------------------------------------------------------------------------
 template <typename T, int KT, bool LS>
 __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
                                 const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int C, int nch, T w1,
-                                T w2, T lam, T mu, T nu, int out_kind, int want_u3, int uniform, T hz,
+                                T w2, const DepthMat<T> m, int want_u3, int uniform, T hz,
                                 const int* __restrict__ zr, int ein) {
   typedef typename Cx<T>::t V;
   constexpr int SL = LS ? 6 : 9, CM = LS ? 8 : 1;
@@ -410,8 +442,9 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   V* W = reinterpret_cast<V*>(smraw);                      // [nz][SL][KT]
   V* xbase = W + (size_t)nz * SL * KT;
   const Xch<V, KT> X(xbase, nch);
-  T* el = reinterpret_cast<T*>(xbase + Xch<V, KT>::count(nch));  // [uniform ? 1 : nz][6][KT]
-  T* pr = el + (size_t)(uniform ? 1 : nz) * EL_N * KT;     // [uniform ? C : nz][KT] propagators
+  Col<T>* cols = reinterpret_cast<Col<T>*>(xbase + Xch<V, KT>::count(nch));  // [KT]
+  T* el = reinterpret_cast<T*>(cols + KT);                 // [uniform ? 0 : nz][6][KT]
+  T* pr = el + (size_t)(uniform ? 0 : nz) * EL_N * KT;     // [uniform ? C : nz][KT] propagators
   T* zs = pr + (size_t)(uniform ? C : nz) * KT;            // [nz] depth nodes
   const int kt = threadIdx.x & (KT - 1);
   const int ch = threadIdx.x / KT;
@@ -432,38 +465,35 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     else *dst = mk<V>(0, 0);
   }
   for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-  const ModeGeom<T> g = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2);
-  const bool special = g.zero || g.nyq;
-  const bool stress = out_kind == FVIM_STRESS;
   const int n0 = ch * C;
   const int nend = min(n0 + C, nz);
   const bool active = n0 < nz;
-  const bool work = active && !special;
-  // element coefficients while the tile is in flight: element e below node e; none below the
-  // last node (zero)
-  if (uniform) {
-    // and the powers E^0 .. E^(C-1) of a uniform grid's propagator
-    if (threadIdx.x < KT) {
-      const El<T> c = elem_coef<T>(g.q, hz);
-      el_put<T, KT>(el + kt, c);
+  // column constants while the tile is in flight, and the powers E^0 .. E^(C-1) of a uniform
+  // grid's propagator; on a refined grid the coefficients of element e below node e (none, zero,
+  // below the last node)
+  if (threadIdx.x < KT) {
+    col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, uniform != 0, hz);
+    if (uniform) {
       T p = 1;
-      for (int k = 0; k < C; ++k, p *= c.E) pr[k * KT + kt] = p;
+      const T E = cols[kt].in.E;
+      for (int k = 0; k < C; ++k, p *= E) pr[k * KT + kt] = p;
     }
-  } else {
+  }
+  if (!uniform) {
+    const T q = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2).q;
     for (int e = n0; e < nend; ++e) {
       El<T> c = {0, 0, 0, 0, 0, 0};
-      if (e + 1 < nz) c = elem_coef<T>(g.q, zn[e + 1] - zn[e]);
+      if (e + 1 < nz) c = elem_coef<T>(q, zn[e + 1] - zn[e]);
       el_put<T, KT>(el + (size_t)e * EL_N * KT + kt, c);
     }
   }
   cp_async_wait_all();
   __syncthreads();
 
-  const Rot<T> rot(g.c, g.s);
-  El<T> ec = {0, 0, 0, 0, 0, 0};
-  if (uniform) ec = el_get<T, KT>(el + kt);
-  const LocC<T> lc(lam, mu, nu, stress);
-  const T ms = (T)2 * nu - (T)1;
+  const ColIn<T> g = cols[kt].in;
+  const bool special = g.kind != (T)0;
+  const bool work = active && !special;
+  El<T> ec = g.el();
   V L[CM][3];
   // 2. own moments of the chunk: A forward (slots 0..2), the P sources kept in slots 3..5 and
   //    then replaced by the P moments, backward
@@ -474,9 +504,9 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
       V x[6];
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) x[cc] = w[cc * KT];
-      if (ein) hooke_mode(x, lam, mu);
-      const Src<V> o = node_source(x, rot, ms);
-      node_local(Li, x, lc, stress);
+      if (ein) hooke_mode(x, m.lam, m.mu);
+      const Src<V> o = node_source(x, g, m.ms);
+      node_local(Li, x, m);
       if (uniform) {
         if (i > 0) br_arrive(s, ec, o.nA, o.m, o.aA);
         br_put<V, KT>(w, s);
@@ -506,17 +536,17 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     T ep = 1;  // propagator from node i to the chunk's last node
     for (int i = nend - 1; i >= n0; --i) {
       V* w = W + (size_t)i * SL * KT + kt;
-      const V n = w[3 * KT], m = w[4 * KT], a = w[5 * KT];
+      const V sn = w[3 * KT], sm = w[4 * KT], sa = w[5 * KT];
       if (!uniform) {
         ec = el_get<T, KT>(el + (size_t)i * EL_N * KT + kt);
         if (i + 1 < nend) ep *= ec.E;
         pr[i * KT + kt] = ep;
       }
-      if (i + 1 < nz) br_arrive(s, ec, n, m, a);
+      if (i + 1 < nz) br_arrive(s, ec, sn, sm, sa);
       br_put<V, KT>(w + 3 * KT, s);
       if (i == 0) br_put<V, KT>(X.R + kt, s);
       if (!uniform) ec = el_get<T, KT>(el + (size_t)max(i - 1, 0) * EL_N * KT + kt);
-      br_leave(s, ec, n, m, a);
+      br_leave(s, ec, sn, sm, sa);
     }
     br_put<V, KT>(X.P + (size_t)ch * 3 * KT + kt, s);
   } else if (active) {
@@ -527,8 +557,8 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
 
   // 3. carries, image field, surface displacement
   V* u3 = want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr;
-  chunk_carries<T, KT>(X, zs, threadIdx.x, blockDim.x, C, nch, nz, g.q, uniform != 0, hz, false, !special, u3,
-                       (T)1 / ((T)2 * mu));
+  chunk_carries<T, KT>(X, zs, threadIdx.x, blockDim.x, C, nch, nz, g.q, uniform != 0, hz, !special, u3,
+                       m.iu);
   if (want_u3 && ch == 0 && special) *u3 = mk<V>(0, 0);
   __syncthreads();
   if (!active) return;
@@ -540,8 +570,8 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
       V w[6], o[6];
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) w[cc] = W[((size_t)i * SL + cc) * KT + kt];
-      if (ein) hooke_mode(w, lam, mu);
-      node_special(o, w, g.nyq, lam, mu, stress);
+      if (ein) hooke_mode(w, m.lam, m.mu);
+      node_special(o, w, g.kind == (T)2, m);
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
     }
@@ -553,7 +583,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     const T x = g.q * zs[n0], E = dexp<T>(-x);
     br_add_prop(cA, br_get<V, KT>(X.I + kt), E, x * E);
   }
-  const OutC<T> oc(rot, g.q, mu, nu, stress);
+  const ColOut<T> oc = cols[kt].out;
   const int last = n0 + C - 1;  // node the P carry arrives at (a ragged last chunk has none: zero)
   T EA = 1;
   auto fin = [&](int i, const V* Li) {
@@ -574,7 +604,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     br_add_prop(A, cA, EA, xA * EA);
     br_add_prop(P, cP, EP, xP * EP);
     V o[6];
-    node_out(o, A, P, Li, oc, stress);
+    node_out(o, A, P, Li, oc, m);
 #pragma unroll
     for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
     out += 6 * plane;
@@ -604,69 +634,62 @@ template <typename V> __device__ __forceinline__ void ld6(V (&w)[6], const V* W,
 }
 
 // Quantities that do not depend on the tile's values, computed while its copy is in flight: the
-// mode geometry (every thread) and the element coefficients, once per column on a uniform grid,
-// else those of each chunk's own elements (element e below node e; zero below the last node),
-// in el for the body to read after its first barrier.
-template <typename T, int KT>
-__device__ __forceinline__ ModeGeom<T> depth_prep(T* el, const T* __restrict__ zn, int tid, int kblk, int k2, bool ghost,
-                                                  int nz, int C, int n1, int n2, int hs, T w1, T w2, int uniform, T hz) {
-  const int kt = tid & (KT - 1);
-  const ModeGeom<T> g = mode_geom<T>(kblk * KT + kt, k2, n1, n2, hs, w1, w2);
-  if (ghost) return g;
-  if (uniform) {
-    if (tid < KT) el_put<T, KT>(el + kt, elem_coef<T>(g.q, hz));
-  } else {
+// column constants, and on a refined grid the coefficients of each chunk's own elements (element
+// e below node e; zero below the last node).
+template <typename T, int KT, bool UNI>
+__device__ __forceinline__ void depth_prep(Col<T>* cols, T* el, const T* __restrict__ zn, int tid, int kblk, int k2, int nz,
+                                           int C, int n1, int n2, int hs, T w1, T w2, const DepthMat<T>& m, T hz) {
+  const int kt = tid & (KT - 1), k1 = kblk * KT + kt;
+  if (tid < KT) col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, UNI, hz);
+  if (!UNI) {
+    const T q = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2).q;
     const int n0 = (tid / KT) * C, nend = min(n0 + C, nz);
     for (int e = n0; e < nend; ++e) {
       El<T> c = {0, 0, 0, 0, 0, 0};
-      if (e + 1 < nz) c = elem_coef<T>(g.q, zn[e + 1] - zn[e]);
+      if (e + 1 < nz) c = elem_coef<T>(q, zn[e + 1] - zn[e]);
       el_put<T, KT>(el + e * EL_N * KT + kt, c);
     }
   }
-  return g;
 }
 
 // Steps 2-4 of the register depth kernel on a tile already in shared memory (W, with its exchange
 // area X, element coefficients el and nodes zs).  tid = ch * KT + kt is the thread's place among
 // the tile's tt threads, kblk the tile's block of KT k1 columns.  A ghost tile (a CTA slot
 // without a tile) takes part in the barriers only.
-template <typename T, int KT, int C, bool EIN, bool UNI>
-__device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const Xch<typename Cx<T>::t, KT>& X, const T* el,
-                                             const T* zs, int tid, int tt, int kblk, int k2, bool ghost,
+template <typename T, int KT, int C, bool UNI>
+__device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const Xch<typename Cx<T>::t, KT>& X,
+                                             const Col<T>* cols, const T* el, const T* zs, int tid, int tt, int kblk, int k2, bool ghost,
                                              typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
-                                             int nz, int n2, int h1, int nch, T lam, T mu, T nu, int out_kind,
-                                             int want_u3, T hz, T cut, const ModeGeom<T> g) {
+                                             int nz, int n2, int h1, int nch, const DepthMat<T>& m,
+                                             bool ein, int want_u3, T hz, T cut) {
   typedef typename Cx<T>::t V;
   const int kt = tid & (KT - 1);
   const int ch = tid / KT;
   const int k1 = kblk * KT + kt;
   const size_t plane = (size_t)n2 * h1;
-  const bool special = g.zero || g.nyq;
-  const bool stress = out_kind == FVIM_STRESS;
+  const ColIn<T> g = cols[kt].in;
+  const bool special = g.kind != (T)0;
   const int n0 = ch * C;
   const bool active = !ghost && n0 < nz;
   const bool work = active && !special;
-  const Rot<T> rot(g.c, g.s);
 
   // 2. own moments of the chunk at its nodes, both branches from zero, and the carries handed on.
   //    Nodes past the last one count as sources of zero, which changes nothing above them.
   Br<V> A[C], P[C];
   if (work) {
     Src<V> o[C];
-    const T ms = (T)2 * nu - (T)1;
 #pragma unroll
     for (int l = 0; l < C; ++l) {
       if (n0 + l < nz) {
         V x[6];
         ld6(x, W, n0 + l, KT, kt);
-        if (EIN) hooke_mode(x, lam, mu);
-        o[l] = node_source(x, rot, ms);
+        if (ein) hooke_mode(x, m.lam, m.mu);
+        o[l] = node_source(x, g, m.ms);
       } else {
         o[l].nA = o[l].nP = o[l].m = o[l].aA = o[l].aP = mk<V>(0, 0);
       }
     }
-    El<T> ec;
-    if (UNI) ec = el_get<T, KT>(el + kt);
+    El<T> ec = g.el();
     // on a refined grid: element above node n0 + l, zero above node 0 and below the last node
     auto elem = [&](int e) {
       El<T> c = {0, 0, 0, 0, 0, 0};
@@ -705,12 +728,33 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
   const T span = (work && ch + 1 < nch) ? zs[min(n0 + C, nz - 1)] - zs[n0] : (T)0;
   const bool far = !work || ch + 1 >= nch || g.q * span > cut;
   const bool local = __syncthreads_and(cut > (T)0 && far) != 0;
-  if (!ghost)
-    chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, local, !special,
-                         want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr, (T)1 / ((T)2 * mu));
-  if (want_u3 && !ghost && ch == 0 && special) surf[(size_t)k2 * h1 + k1] = mk<V>(0, 0);
-  __syncthreads();
-  if (!active) return;
+  const int last = min(C - 1, nz - 1);  // last node of chunk 0
+  Br<V> cA = br_zero<V>(), cP = br_zero<V>(), im;
+  if (!local) {
+    if (!ghost)
+      chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, !special,
+                           want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr, m.iu);
+    __syncthreads();
+    if (!active) return;
+    cA = br_get<V, KT>(X.A + ch * 3 * KT + kt);
+    cP = br_get<V, KT>(X.P + ch * 3 * KT + kt);
+    im = br_get<V, KT>(X.I + kt);
+  } else {
+    if (!active) return;
+    if (ch > 0) cA = br_get<V, KT>(X.A + (ch - 1) * 3 * KT + kt);
+    if (ch + 1 < nch) cP = br_get<V, KT>(X.P + (ch + 1) * 3 * KT + kt);
+    // complete P moments of node 0 and the image field, by every thread (no second barrier)
+    Br<V> p0 = br_get<V, KT>(X.R + kt);
+    if (nch > 1) {
+      const T x = g.q * (zs[last] - zs[0]), E = dexp<T>(-x);
+      br_add_prop(p0, br_get<V, KT>(X.P + 3 * KT + kt), E, x * E);
+    }
+    im.n = caxpy(p0.n, (T)2, p0.v);
+    im.v = mk<V>(-p0.v.x, -p0.v.y);
+    im.a = p0.a;
+    if (want_u3 && ch == 0 && !special) surf[(size_t)k2 * h1 + k1] = cscale(p0.v, m.iu);
+  }
+  if (want_u3 && ch == 0 && special) surf[(size_t)k2 * h1 + k1] = mk<V>(0, 0);
 
   // 4. complete moments, output
   V* out = spec + (size_t)n0 * 6 * plane + (size_t)k2 * h1 + k1;
@@ -719,25 +763,23 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
     for (int i = n0; i < nend; ++i, out += 6 * plane) {
       V w[6], o[6];
       ld6(w, W, i, KT, kt);
-      if (EIN) hooke_mode(w, lam, mu);
-      node_special(o, w, g.nyq, lam, mu, stress);
+      if (ein) hooke_mode(w, m.lam, m.mu);
+      node_special(o, w, g.kind == (T)2, m);
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
     }
     return;
   }
-  Br<V> cA = br_get<V, KT>(X.A + ch * 3 * KT + kt);
-  const Br<V> cP = br_get<V, KT>(X.P + ch * 3 * KT + kt);
   {
     const T x = g.q * zs[n0], E = dexp<T>(-x);
-    br_add_prop(cA, br_get<V, KT>(X.I + kt), E, x * E);
+    br_add_prop(cA, im, E, x * E);
   }
   // propagators from the chunk's first node (A) and to its last one (P) and q times the distances
   T EA[C], EP[C], xA[C], xP[C];
   EA[0] = EP[C - 1] = (T)1;
   xA[0] = xP[C - 1] = (T)0;
   if (UNI) {
-    const T E = el[kt], a = el[KT + kt];
+    const T E = g.E, a = g.a;
 #pragma unroll
     for (int l = 1; l < C; ++l) {
       EA[l] = EP[C - 1 - l] = EA[l - 1] * E;
@@ -759,8 +801,7 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
       xP[C - 1 - l] = xP[C - l] + ae[C - 1 - l];
     }
   }
-  const OutC<T> oc(rot, g.q, mu, nu, stress);
-  const LocC<T> lc(lam, mu, nu, stress);
+  const ColOut<T> oc = cols[kt].out;
 #pragma unroll
   for (int l = 0; l < C; ++l) {
     if (n0 + l < nz) {
@@ -768,9 +809,9 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
       br_add_prop(P[l], cP, EP[l], xP[l] * EP[l]);
       V x[6], L[3], o[6];
       ld6(x, W, n0 + l, KT, kt);
-      if (EIN) hooke_mode(x, lam, mu);
-      node_local(L, x, lc, stress);
-      node_out(o, A[l], P[l], L, oc, stress);
+      if (ein) hooke_mode(x, m.lam, m.mu);
+      node_local(L, x, m);
+      node_out(o, A[l], P[l], L, oc, m);
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) out[cc * plane] = o[cc];
       out += 6 * plane;
@@ -781,18 +822,18 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
 // shared memory of a register-variant tile
 template <typename T, int KT> struct RegSmem {
   typedef typename Cx<T>::t V;
-  static __host__ __device__ size_t el_count(int nz, int uniform) { return (size_t)(uniform ? 1 : nz) * EL_N * KT; }
+  static __host__ __device__ size_t el_count(int nz, int uniform) { return (size_t)(uniform ? 0 : nz) * EL_N * KT; }
   static __host__ __device__ size_t bytes(int nz, int nch, int uniform) {
-    return ((size_t)nz * 6 * KT + Xch<V, KT>::count(nch)) * sizeof(V) + el_count(nz, uniform) * sizeof(T) +
+    return ((size_t)nz * 6 * KT + Xch<V, KT>::count(nch)) * sizeof(V) + KT * sizeof(Col<T>) + el_count(nz, uniform) * sizeof(T) +
            (((size_t)nz * sizeof(T) + 15) & ~(size_t)15);
   }
 };
 
-template <typename T, int KT, int C, bool EIN, bool UNI, int MB>
+template <typename T, int KT, int C, bool UNI, int MB>
 __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* __restrict__ spec,
                                                             typename Cx<T>::t* __restrict__ surf,
                                                             const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int nch,
-                                                            T w1, T w2, T lam, T mu, T nu, int out_kind, int want_u3,
+                                                            T w1, T w2, const DepthMat<T> m, int ein, int want_u3,
                                                             T hz, const int* __restrict__ zr, T cut,
                                                             const __grid_constant__ CUtensorMap tmap, int tma_rows,
                                                             int tx_extra, int* __restrict__ status) {
@@ -802,14 +843,14 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
   V* W = reinterpret_cast<V*>(smraw);                               // [nz][6][KT]
   V* xbase = W + (size_t)nz * 6 * KT;
   const Xch<V, KT> X(xbase, nch);
-  T* el = reinterpret_cast<T*>(xbase + Xch<V, KT>::count(nch));
+  Col<T>* cols = reinterpret_cast<Col<T>*>(xbase + Xch<V, KT>::count(nch));  // [KT]
+  T* el = reinterpret_cast<T*>(cols + KT);
   T* zs = el + RegSmem<T, KT>::el_count(nz, UNI);                   // [nz]
   // mbarrier of the tensor copies, after the depth nodes
   unsigned long long* tbar = reinterpret_cast<unsigned long long*>(smraw + RegSmem<T, KT>::bytes(nz, nch, UNI));
   const int k2 = blockIdx.y;
   const size_t plane = (size_t)n2 * h1;
   const size_t colofs = (size_t)k2 * h1 + blockIdx.x * KT;
-  ModeGeom<T> g;
 
   // 1. load the tile and the depth nodes (layers outside zr hold no input: their spectrum was
   //    not computed and reads as zero).  With a tensor map (tma_rows > 0): one thread issues
@@ -838,7 +879,7 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
       }
     }
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-    g = depth_prep<T, KT>(el, zn, threadIdx.x, blockIdx.x, k2, false, nz, C, n1, n2, hs, w1, w2, UNI, hz);
+    depth_prep<T, KT, UNI>(cols, el, zn, threadIdx.x, blockIdx.x, k2, nz, C, n1, n2, hs, w1, w2, m, hz);
     bool done = mbar_wait_bounded(bar, 1000000000ull);   // 1 s
     if (__syncthreads_or(!done)) {
       if (threadIdx.x == 0 && status) atomicOr(status, 1);
@@ -866,13 +907,13 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
       }
     }
     for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-    g = depth_prep<T, KT>(el, zn, threadIdx.x, blockIdx.x, k2, false, nz, C, n1, n2, hs, w1, w2, UNI, hz);
+    depth_prep<T, KT, UNI>(cols, el, zn, threadIdx.x, blockIdx.x, k2, nz, C, n1, n2, hs, w1, w2, m, hz);
     cp_async_wait_all();
     __syncthreads();
   }
 
-  depth_r_body<T, KT, C, EIN, UNI>(W, X, el, zs, threadIdx.x, blockDim.x, blockIdx.x, k2, false, spec, surf, nz, n2, h1,
-                                   nch, lam, mu, nu, out_kind, want_u3, hz, cut, g);
+  depth_r_body<T, KT, C, UNI>(W, X, cols, el, zs, threadIdx.x, blockDim.x, blockIdx.x, k2, false, spec, surf, nz, n2,
+                                   h1, nch, m, ein != 0, want_u3, hz, cut);
 }
 
 // ----------------------------------------------------------------------------------
@@ -902,7 +943,8 @@ __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ Gr
   V* W = reinterpret_cast<V*>(base);                                // [nz][6][KT]
   V* xbase = W + (size_t)nz * 6 * KT;
   const Xch<V, KT> X(xbase, nchp);
-  float* el = reinterpret_cast<float*>(xbase + Xch<V, KT>::count(nchp));
+  Col<float>* cols = reinterpret_cast<Col<float>*>(xbase + Xch<V, KT>::count(nchp));  // [KT]
+  float* el = reinterpret_cast<float*>(cols + KT);
   float* zs = el + RegSmem<float, KT>::el_count(nz, P.uniform);     // [nz]
   if (!ghost) {
     const size_t plane = (size_t)P.n2 * P.h1;
@@ -913,17 +955,21 @@ __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ Gr
     }
     for (int i = tid; i < nz; i += tt) zs[i] = P.zn[i];
   }
-  const ModeGeom<float> g =
-      depth_prep<float, KT>(el, P.zn, tid, kblk, k2, ghost, nz, C, P.n1, P.n2, P.hs, P.w1, P.w2, P.uniform, P.hz);
+  if (!ghost) {
+    if (P.uniform)
+      depth_prep<float, KT, true>(cols, el, P.zn, tid, kblk, k2, nz, C, P.n1, P.n2, P.hs, P.w1, P.w2, P.dm, P.hz);
+    else
+      depth_prep<float, KT, false>(cols, el, P.zn, tid, kblk, k2, nz, C, P.n1, P.n2, P.hs, P.w1, P.w2, P.dm, P.hz);
+  }
   cp_async_wait_all();
   __syncthreads();
   // one body per grid kind: a CTA's tiles belong to one problem
   if (P.uniform)
-    depth_r_body<float, KT, C, false, true>(W, X, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2, P.h1,
-                                            P.nch, P.lam, P.mu, P.nu, P.out_kind, 0, P.hz, P.cut, g);
+    depth_r_body<float, KT, C, true>(W, X, cols, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2,
+                                            P.h1, P.nch, P.dm, false, 0, P.hz, P.cut);
   else
-    depth_r_body<float, KT, C, false, false>(W, X, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2, P.h1,
-                                             P.nch, P.lam, P.mu, P.nu, P.out_kind, 0, P.hz, P.cut, g);
+    depth_r_body<float, KT, C, false>(W, X, cols, el, zs, tid, tt, kblk, k2, ghost, P.spec, nullptr, nz, P.n2,
+                                             P.h1, P.nch, P.dm, false, 0, P.hz, P.cut);
 }
 
 // strain of the Boussinesq-Cerruti field of a surface traction t (rotated frame, force on
@@ -1077,8 +1123,8 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   // tile width of the launch: as wide as fits twice on an SM, and at least one 32-byte sector
   auto smem_of = [&](int kt) {
     const size_t vals = (size_t)nz * (C <= 8 ? 6 : 9) * kt + 6 * (size_t)(nch + 1) * kt;
-    const size_t reals = (size_t)(c->uniform ? 1 : nz) * EL_N * kt + (size_t)(c->uniform ? C : nz) * kt + nz;
-    return vals * sizeof(V) + reals * sizeof(T);
+    const size_t reals = (size_t)(c->uniform ? 0 : nz) * EL_N * kt + (size_t)(c->uniform ? C : nz) * kt + nz;
+    return vals * sizeof(V) + kt * sizeof(Col<T>) + reals * sizeof(T);
   };
   const int kmin = 32 / (int)sizeof(V);
   while (KT > 2 && (smem_of(KT) > 227 * 1024 || (KT > kmin && smem_of(KT) > 113 * 1024))) KT >>= 1;
@@ -1111,6 +1157,7 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
   const int KT = d.KT, C = d.C, nch = d.nch;
   dim3 grid(h1 / KT, n2);
   const T w1 = (T)(kTwoPi / c->L1), w2 = (T)(kTwoPi / c->L2);
+  const DepthMat<T> dm = depth_mat<T>(c->lam, c->mu, c->nu, out_kind);
   if constexpr (sizeof(T) == 4) if (d.reg) {
     // tensor-map copies of the tile where the context has its map (rows per box divide 6 Nz)
     CUtensorMap tm;
@@ -1121,18 +1168,17 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
     } else {
       memset(&tm, 0, sizeof(tm));
     }
-#define DEPTHR(CV, EI, UN, MBV)                                                                                 \
-  if (C == CV && eps_in == EI && (c->uniform != 0) == UN && d.mb == MBV) {                                      \
-    smem_cap(k_mindlin_depth_r<T, 16, CV, EI, UN, MBV>);                                                        \
-    k_mindlin_depth_r<T, 16, CV, EI, UN, MBV><<<grid, d.threads, d.smem, c->stream>>>(                          \
-        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, nch, w1, w2, (T)c->lam, (T)c->mu, \
-        (T)c->nu, out_kind, want_u3 ? 1 : 0, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,    \
+#define DEPTHR(CV, UN, MBV, MBK)                                                                                \
+  if (C == CV && (c->uniform != 0) == UN && d.mb == MBV) {                                                      \
+    smem_cap(k_mindlin_depth_r<T, 16, CV, UN, MBK>);                                                            \
+    k_mindlin_depth_r<T, 16, CV, UN, MBK><<<grid, d.threads, d.smem, c->stream>>>(                              \
+        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, nch, w1, w2, dm, eps_in ? 1 : 0, \
+        want_u3 ? 1 : 0, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,    \
         c->dev_status);                                                                                          \
   }
-#define DEPTHR2(CV, MBV) \
-  DEPTHR(CV, false, true, MBV) DEPTHR(CV, false, false, MBV) DEPTHR(CV, true, true, MBV) DEPTHR(CV, true, false, MBV)
-    DEPTHR2(2, 2) DEPTHR2(3, 2) DEPTHR2(4, 2) DEPTHR2(6, 2) DEPTHR2(8, 2)
-    DEPTHR2(4, 3) DEPTHR2(6, 3) DEPTHR2(8, 3)
+#define DEPTHR2(CV, MBV, MBK) DEPTHR(CV, true, MBV, MBK) DEPTHR(CV, false, MBV, MBK)
+    DEPTHR2(2, 2, 4) DEPTHR2(3, 2, 3) DEPTHR2(4, 2, 2) DEPTHR2(6, 2, 2) DEPTHR2(8, 2, 2)
+    DEPTHR2(4, 3, 3) DEPTHR2(6, 3, 3) DEPTHR2(8, 3, 3)
 #undef DEPTHR2
 #undef DEPTHR
     FVIM_CUDA_CHECK_LAUNCH();
@@ -1142,8 +1188,8 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
   if (KT == KTV && (C <= 8) == LSV) {                                                                          \
     smem_cap(k_mindlin_depth<T, KTV, LSV>);                                                                    \
     k_mindlin_depth<T, KTV, LSV><<<grid, d.threads, d.smem, c->stream>>>(                                      \
-        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, w1, w2, (T)c->lam,      \
-        (T)c->mu, (T)c->nu, out_kind, want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, eps_in ? 1 : 0);              \
+        (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, w1, w2, dm,      \
+        want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, eps_in ? 1 : 0);              \
   }
   DEPTH(16, true) DEPTH(8, true) DEPTH(4, true) DEPTH(2, true)
   DEPTH(16, false) DEPTH(8, false) DEPTH(4, false) DEPTH(2, false)

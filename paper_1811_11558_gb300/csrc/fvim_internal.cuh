@@ -484,6 +484,31 @@ int plan_lookup_ctas(const fvim_ctx* c);
 // whether an in-plane FFT path is built for the context's grid and precision (capi.cu)
 bool fft_path_available(const fvim_ctx* c, int path);
 
+// material constants of the depth operator for one kind of output, evaluated on the host in FP64
+template <typename T> struct DepthMat {
+  T lam, mu, iu;      // iu = 1 / (2 mu)
+  T ms, la;           // 2 nu - 1; factor of w_33 in the local terms
+  T kap, hq, p, w, t; // factors of the moments in the output (depth.cu, node_out)
+  int stress;
+};
+template <typename T> inline DepthMat<T> depth_mat(double lam, double mu, double nu, int out_kind) {
+  const bool st = out_kind == FVIM_STRESS;
+  const double sc = st ? 1.0 : 1.0 / (2.0 * mu);
+  DepthMat<T> m;
+  m.lam = (T)lam;
+  m.mu = (T)mu;
+  m.iu = (T)(1.0 / (2.0 * mu));
+  m.ms = (T)(2.0 * nu - 1.0);
+  m.la = (T)(st ? nu / (1.0 - nu) : 1.0 / (lam + 2.0 * mu));
+  m.kap = (T)(sc / (4.0 * (1.0 - nu)));
+  m.hq = (T)(0.5 * sc);
+  m.p = (T)(st ? -2.0 * nu : 0.0);
+  m.w = (T)(st ? 2.0 : 2.0 - 2.0 * nu);
+  m.t = (T)(st ? 0.0 : 2.0 * nu);
+  m.stress = st ? 1 : 0;
+  return m;
+}
+
 // kernel kinds for fvim_profile_read
 enum ProfSlot {
   PROF_ROWS_FWD6 = 0, PROF_COLS_FWD, PROF_MINDLIN_DEPTH, PROF_COLS_INV, PROF_ROWS_INV6,
@@ -599,8 +624,9 @@ struct GrpProb {
   const float* zn;       // depth nodes [nz]
   int n1, n2, nz, h1, hs;
   int nch, nchp;         // depth chunks of 4 nodes, and that count rounded up to a power of two
-  int uniform, out_kind;
-  float w1, w2, lam, mu, nu, hz, cut;
+  int uniform;
+  float w1, w2, lam, mu, hz, cut;
+  DepthMat<float> dm;
   float nq_scale, scale; // inverse rows: Nyquist factor and 1 / (N1 N2)
 };
 struct GrpTable {
