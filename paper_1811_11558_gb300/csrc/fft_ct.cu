@@ -259,11 +259,14 @@ __global__ void __launch_bounds__(256) k_rows_inv6_ct(const typename Cx<T>::t* _
                        reinterpret_cast<V*>(smraw) + (size_t)r * 3 * LD, nq_scale, scale);
 }
 
-// FP32 forward row pass with 16-byte global accesses: the CTA's six eps_p rows are staged in
-// shared memory with 16-byte cp.async copies and read from there in the FFT's strided order;
-// the staging area then serves as the FFT exchange area, and the half spectrum leaves as
-// float4 pairs of entries.  (Staging the inverse pass the same way made it slower: 0.254
-// against 0.183 ms at 512 x 512 x 64, from the extra shared-memory traffic and registers.)
+// FP32 forward row pass: the CTA's six eps_p rows are staged in shared memory with 16-byte
+// cp.async copies (two per thread and component) and read from there in the FFT's strided order;
+// the staging area then serves as the FFT exchange area.  The two real rows of a transform are
+// separated in registers: thread t holds Z(t + m N/8), m < 8, and fetches only the mirrored
+// Z(N - k) of its four k < N/2 through the exchange area.  Bound by instruction issue: index
+// arithmetic and the round trip of the whole spectrum through shared memory before the
+// separation were a third of the instructions.  512 x 512 x 64: 171 -> 135 us (1024 x 1024 x
+// 32: 367 -> 305).
 // row stride (floats) of the forward rows' staging area: rows of 64 or 128 points put two or
 // four rows in one warp, which would read the same banks; N / 8 extra floats shift each row
 // by a warp's span of one row
@@ -282,15 +285,18 @@ __device__ __forceinline__ void rows_fwd6_v_body(const float* __restrict__ eps_p
   const int r = threadIdx.x / T8, t = threadIdx.x % T8;
   const int x2 = x2b + r;
   float* stg = reinterpret_cast<float*>(smraw);  // [6][rb][SLD]
-  const int per_c = rb * N / 4;
-  for (int i = threadIdx.x; i < 6 * per_c; i += blockDim.x) {
-    const int c = i / per_c, j = i - c * per_c;
-    float* dst = stg + (size_t)c * rb * SLD + 4 * j;
-    if constexpr (SLD != N) {
-      const int row = (4 * j) / N;
-      dst += row * (SLD - N);
+  {
+    // the rb rows of a component are contiguous: rb N / 4 = 2 blockDim float4
+    const int j = 4 * threadIdx.x, half = 4 * blockDim.x;
+    const float* src = eps_p + ((size_t)z * 6 * n2 + x2b) * N + j;
+    float* d0 = stg + j + (j / N) * (SLD - N);
+    float* d1 = stg + (j + half) + ((j + half) / N) * (SLD - N);
+    const size_t cs = (size_t)n2 * N;
+#pragma unroll
+    for (int c = 0; c < 6; ++c) {
+      cp_async_16(d0 + c * rb * SLD, src + c * cs);
+      cp_async_16(d1 + c * rb * SLD, src + c * cs + half);
     }
-    cp_async_16(dst, eps_p + (((size_t)z * 6 + c) * n2 + x2b) * N + 4 * j);
   }
   cp_async_wait_all();
   __syncthreads();
@@ -309,26 +315,34 @@ __device__ __forceinline__ void rows_fwd6_v_body(const float* __restrict__ eps_p
   __syncthreads();  // staging is dead: the exchange area takes its place
   RowSm<float2, N> sm{reinterpret_cast<float2*>(smraw) + (size_t)r * 3 * LD};
   fft_ct<float2, false, N, 3, 1>(v, t, sm, tw);
+  // mirrored halves: Z(N - k) of k = t + m N/8, m < 4, is in the upper half, slots 4..7 of another
+  // thread (Z(0) is its own mirror)
 #pragma unroll
   for (int g = 0; g < 3; ++g)
 #pragma unroll
-    for (int m = 0; m < 8; ++m) sm.put(g, t + m * T8, v[g][m]);
+    for (int m = 4; m < 8; ++m) sm.put(g, t + m * T8, v[g][m]);
   __syncthreads();
-  for (int idx = t; idx < 3 * (H1 / 2); idx += T8) {
-    const int g = idx / (H1 / 2), k = 2 * (idx - g * (H1 / 2));
-    float2 A0, B0, A1, B1;
-    split_pair_ct(sm.get(g, k), sm.get(g, (N - k) & (N - 1)), A0, B0);
-    split_pair_ct(sm.get(g, k + 1), sm.get(g, N - k - 1), A1, B1);
-    float4* ra = reinterpret_cast<float4*>(spec + (((size_t)z * 6 + 2 * g) * n2 + x2) * H1 + k);
-    float4* rbp = reinterpret_cast<float4*>(spec + (((size_t)z * 6 + 2 * g + 1) * n2 + x2) * H1 + k);
-    *ra = make_float4(A0.x, A0.y, A1.x, A1.y);
-    *rbp = make_float4(B0.x, B0.y, B1.x, B1.y);
-  }
-  if (t < 3) {
-    float2 A, B;
-    split_pair_ct(sm.get(t, H1), sm.get(t, H1), A, B);
-    nq[((size_t)z * 6 + 2 * t) * n2 + x2] = A.x;
-    nq[((size_t)z * 6 + 2 * t + 1) * n2 + x2] = B.x;
+  float2* o = spec + ((size_t)z * 6 * n2 + x2) * H1 + t;
+  const size_t cs = (size_t)n2 * H1;
+#pragma unroll
+  for (int g = 0; g < 3; ++g)
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      float2 zm = sm.get(g, (N - t - m * T8) & (N - 1));
+      if (m == 0 && t == 0) zm = v[g][0];
+      float2 A, B;
+      split_pair_ct(v[g][m], zm, A, B);
+      o[2 * g * cs + m * T8] = A;
+      o[(2 * g + 1) * cs + m * T8] = B;
+    }
+  if (t == 0) {
+    // k1 = N1/2: Z there is A + i B with real A, B
+    float* q = nq + (size_t)z * 6 * n2 + x2;
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      q[(size_t)(2 * g) * n2] = v[g][4].x;
+      q[(size_t)(2 * g + 1) * n2] = v[g][4].y;
+    }
   }
 }
 
