@@ -74,9 +74,17 @@ template <int CW> struct ColPairSm {
   __device__ __forceinline__ float2 get(int g, int p) const { return buf[p * CW + 2 * f2 + g]; }
 };
 
+// 16-byte load that asks L2 for the whole 128-byte line: the other half of a 64-byte row segment is
+// the neighbouring CTA's
+__device__ __forceinline__ float4 ld_line(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.L2::128B.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+  return v;
+}
+
 template <int N, int CW> struct ColsV {
   static constexpr int threads = N / 16 * CW;
-  static constexpr int min_blocks = CW == 16 ? 1024 / threads : 1;  // CW = 16: 64 registers
+  static constexpr int min_blocks = CW == 16 ? 1024 / threads : (N >= 1024 ? 2 : 1);  // 64 registers
 };
 
 // one CW-column block of one plane: tid in [0, N / 16 * CW), sm the block's [N][CW] exchange
@@ -91,7 +99,8 @@ __device__ __forceinline__ void cols_v_body(float2* __restrict__ planes, const f
   float2 v[2][8];
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    const float4 a = live ? col[(size_t)(t + m * T8) * rs] : make_float4(0.f, 0.f, 0.f, 0.f);
+    const float4* src = col + (size_t)(t + m * T8) * rs;
+    const float4 a = live ? (CW < 16 ? ld_line(src) : *src) : make_float4(0.f, 0.f, 0.f, 0.f);
     v[0][m] = make_float2(a.x, a.y);
     v[1][m] = make_float2(a.z, a.w);
   }
@@ -384,8 +393,10 @@ template <int N, int CW> void cols_v_launch(const fvim_ctx* c, bool inverse, voi
 template <typename T, int N> void cols_n(const fvim_ctx* c, bool inverse, void* planes, int nplanes, const int* zr) {
   typedef typename Cx<T>::t V;
   if constexpr (sizeof(T) == 4 && N >= 64) {
-    // 16 columns per CTA (whole 128-byte rows): N threads, 1024 at N = 1024 (one CTA per SM)
-    if (c->h1 % 16 == 0) {
+    // 16 columns per CTA (whole 128-byte rows, N threads); at N = 1024 that is one CTA per SM, whose
+    // load, transform and store phases do not overlap: 8 columns, two CTAs
+    // (1024 x 1024 x 32: 420 -> 361 us per direction).
+    if (c->h1 % 16 == 0 && N <= 512) {
       cols_v_launch<N, 16>(c, inverse, planes, nplanes, zr);
       return;
     }
