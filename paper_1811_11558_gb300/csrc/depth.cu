@@ -101,17 +101,21 @@ template <typename T> __device__ __forceinline__ El<T> elem_coef(T q, T h) {
   T I0, I1, I2;
   const T thr = sizeof(T) == 4 ? (T)1.0 : (T)0.5;
   if (a < thr) {
-    // I_n(a) = sum_m (-a)^m / (m! (n + m + 1)); the reciprocals are compile-time constants
+    // I_2(a) = sum_m (-a)^m / (m! (m + 3)) by Horner's rule (constant coefficients), then upwards by
+    // parts, I_{n-1} = (a I_n + E) / n, which loses nothing
     constexpr int M = sizeof(T) == 4 ? 12 : 18;
-    T term = 1, s0 = 0, s1 = 0, s2 = 0;
+    double f = 1;  // 1 / m!, folded at compile time
+    T cm[M];
 #pragma unroll
     for (int m = 0; m < M; ++m) {
-      s0 += term * (T)(1.0 / (m + 1));
-      s1 += term * (T)(1.0 / (m + 2));
-      s2 += term * (T)(1.0 / (m + 3));
-      term *= -a * (T)(1.0 / (m + 1));
+      cm[m] = (T)(f / (m + 3));
+      f /= m + 1;
     }
-    I0 = s0; I1 = s1; I2 = s2;
+    I2 = cm[M - 1];
+#pragma unroll
+    for (int m = M - 2; m >= 0; --m) I2 = fma(-a, I2, cm[m]);
+    I1 = (T)0.5 * fma(a, I2, E);
+    I0 = fma(a, I1, E);
   } else {
     const T ia = (T)1 / a;
     I0 = ((T)1 - E) * ia;
@@ -355,17 +359,18 @@ template <typename V, int KT> __device__ __forceinline__ Br<V> br_get(const V* p
 // node, P: at its last), then the complete P moments of node 0, the image field and the surface
 // displacement.  Work item t = role KT + column, roles 0: P (n, v), 1: A (n, v), 2: P a, 3: A a.
 // The column of item t is that of the calling thread (KT divides both thread counts).  Four chunks
-// are read ahead of the recurrence, whose chain is then one multiply-add per chunk.
+// are read ahead of the recurrence, whose chain is then one multiply-add per chunk.  EC, EC1: on a
+// uniform grid the propagators over C elements and over the first chunk's nodes.
 template <typename T, int KT>
 __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& X, const T* zs, int tid, int nthr, int C,
-                                              int nch, int nz, T q, bool uniform, T hz, bool live,
+                                              int nch, int nz, T q, bool uniform, T hz, T EC, T EC1, bool live,
                                               typename Cx<T>::t* u3, T u3_scale) {
   typedef typename Cx<T>::t V;
   const int col = tid & (KT - 1);
   T Eu = 0, xu = 0;
   if (uniform) {
     xu = q * hz * (T)C;
-    Eu = dexp<T>(-xu);
+    Eu = EC;
   }
   for (int t = tid; t < 4 * KT; t += nthr) {
     const bool isA = (t / KT) & 1, isa = t / KT >= 2;
@@ -407,7 +412,7 @@ __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& 
     }
     if (!isA && live) {
       const T x = q * (zs[min(C - 1, nz - 1)] - zs[0]);
-      const T E = dexp<T>(-x);
+      const T E = uniform ? EC1 : dexp<T>(-x);
       if (isa) {
         X.I[2 * KT + col] = caxpy(X.R[2 * KT + col], E, X.P[2 * KT + col]);
       } else {
@@ -444,8 +449,8 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   const Xch<V, KT> X(xbase, nch);
   Col<T>* cols = reinterpret_cast<Col<T>*>(xbase + Xch<V, KT>::count(nch));  // [KT]
   T* el = reinterpret_cast<T*>(cols + KT);                 // [uniform ? 0 : nz][6][KT]
-  T* pr = el + (size_t)(uniform ? 0 : nz) * EL_N * KT;     // [uniform ? C : nz][KT] propagators
-  T* zs = pr + (size_t)(uniform ? C : nz) * KT;            // [nz] depth nodes
+  T* pr = el + (size_t)(uniform ? 0 : nz) * EL_N * KT;     // [uniform ? C + nch + 1 : nz][KT] propagators
+  T* zs = pr + (size_t)(uniform ? C + nch + 1 : nz) * KT;  // [nz] depth nodes
   const int kt = threadIdx.x & (KT - 1);
   const int ch = threadIdx.x / KT;
   const int k1 = blockIdx.x * KT + kt;
@@ -468,8 +473,9 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   const int n0 = ch * C;
   const int nend = min(n0 + C, nz);
   const bool active = n0 < nz;
-  // column constants while the tile is in flight, and the powers E^0 .. E^(C-1) of a uniform
-  // grid's propagator; on a refined grid the coefficients of element e below node e (none, zero,
+  // column constants while the tile is in flight, and on a uniform grid the powers of its
+  // propagator (an FP64 exponential costs as much as eighteen multiplications): E^0 .. E^(C-1), then
+  // E^0, E^C, .. E^(nch C); on a refined grid the coefficients of element e below node e (none, zero,
   // below the last node)
   if (threadIdx.x < KT) {
     col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, uniform != 0, hz);
@@ -477,6 +483,8 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
       T p = 1;
       const T E = cols[kt].in.E;
       for (int k = 0; k < C; ++k, p *= E) pr[k * KT + kt] = p;
+      T pc = 1;
+      for (int k = 0; k <= nch; ++k, pc *= p) pr[(C + k) * KT + kt] = pc;
     }
   }
   if (!uniform) {
@@ -557,7 +565,8 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
 
   // 3. carries, image field, surface displacement
   V* u3 = want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr;
-  chunk_carries<T, KT>(X, zs, threadIdx.x, blockDim.x, C, nch, nz, g.q, uniform != 0, hz, !special, u3,
+  chunk_carries<T, KT>(X, zs, threadIdx.x, blockDim.x, C, nch, nz, g.q, uniform != 0, hz,
+                       uniform ? pr[(C + 1) * KT + kt] : (T)0, uniform ? pr[min(C - 1, nz - 1) * KT + kt] : (T)0, !special, u3,
                        m.iu);
   if (want_u3 && ch == 0 && special) *u3 = mk<V>(0, 0);
   __syncthreads();
@@ -580,7 +589,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   Br<V> cA = br_get<V, KT>(X.A + (size_t)ch * 3 * KT + kt);
   const Br<V> cP = br_get<V, KT>(X.P + (size_t)ch * 3 * KT + kt);
   {
-    const T x = g.q * zs[n0], E = dexp<T>(-x);
+    const T x = g.q * zs[n0], E = uniform ? pr[(C + ch) * KT + kt] : dexp<T>(-x);
     br_add_prop(cA, br_get<V, KT>(X.I + kt), E, x * E);
   }
   const ColOut<T> oc = cols[kt].out;
@@ -732,7 +741,8 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
   Br<V> cA = br_zero<V>(), cP = br_zero<V>(), im;
   if (!local) {
     if (!ghost)
-      chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, !special,
+      chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, UNI ? dexp<T>(-g.q * hz * (T)C) : (T)0,
+                           UNI ? dexp<T>(-g.q * (zs[last] - zs[0])) : (T)0, !special,
                            want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr, m.iu);
     __syncthreads();
     if (!active) return;
@@ -1123,7 +1133,7 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   // tile width of the launch: as wide as fits twice on an SM, and at least one 32-byte sector
   auto smem_of = [&](int kt) {
     const size_t vals = (size_t)nz * (C <= 8 ? 6 : 9) * kt + 6 * (size_t)(nch + 1) * kt;
-    const size_t reals = (size_t)(c->uniform ? 0 : nz) * EL_N * kt + (size_t)(c->uniform ? C : nz) * kt + nz;
+    const size_t reals = (size_t)(c->uniform ? 0 : nz) * EL_N * kt + (size_t)(c->uniform ? C + nch + 1 : nz) * kt + nz;
     return vals * sizeof(V) + kt * sizeof(Col<T>) + reals * sizeof(T);
   };
   const int kmin = 32 / (int)sizeof(V);

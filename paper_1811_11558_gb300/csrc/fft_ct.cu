@@ -74,6 +74,13 @@ template <int CW> struct ColPairSm {
   __device__ __forceinline__ float2 get(int g, int p) const { return buf[p * CW + 2 * f2 + g]; }
 };
 
+}  // namespace
+// 1024-point columns, 8 per CTA: 361 -> 339 us per direction at 1024 x 1024 x 32
+template <> struct UseBf2<float2, 1024, ColPairSm<8>> {
+  static constexpr bool v = true;
+};
+namespace {
+
 // 16-byte load that asks L2 for the whole 128-byte line: the other half of a 64-byte row segment is
 // the neighbouring CTA's
 __device__ __forceinline__ float4 ld_line(const float4* p) {
@@ -165,10 +172,16 @@ __device__ __forceinline__ void split_pair_ct(V zk, V zmk, V& A, V& B) {
   B = mk<V>((T)0.5 * d.y, (T)-0.5 * d.x);
 }
 
-template <typename T, int N>
+// Forward rows straight from global memory (FP64, and FP32 rows of 16 and 32 points): the Hooke
+// constants come halved (hlam = lam / 2, hmu2 = mu), which is the 1/2 of the separation.  NF = 3:
+// a thread runs the row's three pair transforms; NF = 1: one of them (blockIdx.z), for grids whose
+// rows would leave most of the FP64 pipes idle (an FP64 instruction holds its pipe for 64 cycles
+// however few warps there are).  The mirrored half of a spectrum comes from another thread's upper
+// slots through shared memory.
+template <typename T, int N, int NF>
 __global__ void __launch_bounds__(256) k_rows_fwd6_ct(const T* __restrict__ eps_p, typename Cx<T>::t* __restrict__ spec,
                                                       T* __restrict__ nq, const typename Cx<T>::t* __restrict__ tw,
-                                                      int n2, int rb, int z0, T lam, T mu, const int* __restrict__ zr) {
+                                                      int n2, int rb, int z0, T hlam, T hmu2, const int* __restrict__ zr) {
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8, LD = RowLayout<V, N>::LD, H1 = N / 2;
@@ -176,52 +189,66 @@ __global__ void __launch_bounds__(256) k_rows_fwd6_ct(const T* __restrict__ eps_
   const int z = z0 + blockIdx.y;
   if (zr && (z < zr[0] || z >= zr[1])) return;  // layer without input
   const int x2 = blockIdx.x * rb + r;
-  V v[3][8];
+  const int g0 = NF == 3 ? 0 : blockIdx.z;
+  V v[NF][8];
+  const T* src = eps_p + ((size_t)z * 6 * n2 + x2) * N + t;
+  const size_t cs = (size_t)n2 * N;
 #pragma unroll
   for (int m = 0; m < 8; ++m) {
-    const int x1 = t + m * T8;
-    T e[6], w[6];
-#pragma unroll
-    for (int c = 0; c < 6; ++c) e[c] = eps_p[(((size_t)z * 6 + c) * n2 + x2) * N + x1];
-    hooke6_ct(e, w, lam, mu);
-    v[0][m] = mk<V>(w[0], w[1]);
-    v[1][m] = mk<V>(w[2], w[3]);
-    v[2][m] = mk<V>(w[4], w[5]);
-  }
-  RowSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * 3 * LD};
-  fft_ct<V, false, N, 3, 1>(v, t, sm, tw);
-#pragma unroll
-  for (int g = 0; g < 3; ++g)
-#pragma unroll
-    for (int m = 0; m < 8; ++m) sm.put(g, t + m * T8, v[g][m]);
-  __syncthreads();
-  for (int idx = t; idx < 3 * (H1 + 1); idx += T8) {
-    const int g = idx / (H1 + 1), k = idx - g * (H1 + 1);
-    V A, B;
-    split_pair_ct(sm.get(g, k), sm.get(g, (N - k) & (N - 1)), A, B);
-    const int ca = 2 * g, cb = 2 * g + 1;
-    if (k < H1) {
-      spec[(((size_t)z * 6 + ca) * n2 + x2) * H1 + k] = A;
-      spec[(((size_t)z * 6 + cb) * n2 + x2) * H1 + k] = B;
+    const T* e = src + m * T8;
+    if (NF == 3) {
+      const T e0 = e[0], e1 = e[cs], e2 = e[2 * cs];
+      const T ltr = hlam * (e0 + e1 + e2);
+      v[0][m] = mk<V>(ltr + hmu2 * e0, ltr + hmu2 * e1);
+      v[NF / 3][m] = mk<V>(ltr + hmu2 * e2, hmu2 * e[3 * cs]);
+      v[2 * (NF / 3)][m] = mk<V>(hmu2 * e[4 * cs], hmu2 * e[5 * cs]);
+    } else if (g0 == 2) {
+      v[0][m] = mk<V>(hmu2 * e[4 * cs], hmu2 * e[5 * cs]);
     } else {
-      nq[((size_t)z * 6 + ca) * n2 + x2] = A.x;
-      nq[((size_t)z * 6 + cb) * n2 + x2] = B.x;
+      const T e0 = e[0], e1 = e[cs], e2 = e[2 * cs];
+      const T ltr = hlam * (e0 + e1 + e2);
+      v[0][m] = g0 == 0 ? mk<V>(ltr + hmu2 * e0, ltr + hmu2 * e1) : mk<V>(ltr + hmu2 * e2, hmu2 * e[3 * cs]);
+    }
+  }
+  RowSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * NF * LD};
+  fft_ct<V, false, N, NF, 1>(v, t, sm, tw);
+#pragma unroll
+  for (int g = 0; g < NF; ++g)
+#pragma unroll
+    for (int m = 4; m < 8; ++m) sm.put(g, t + m * T8, v[g][m]);
+  __syncthreads();
+  const size_t ps = (size_t)n2 * H1;
+#pragma unroll
+  for (int g = 0; g < NF; ++g) {
+    V* o = spec + ((size_t)(z * 6 + 2 * (g0 + g)) * n2 + x2) * H1 + t;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      V zm = sm.get(g, (N - t - m * T8) & (N - 1));
+      if (m == 0 && t == 0) zm = v[g][0];
+      // A = Z + conj Zm, B = (Z - conj Zm) / i
+      o[m * T8] = mk<V>(v[g][m].x + zm.x, v[g][m].y - zm.y);
+      o[ps + m * T8] = mk<V>(v[g][m].y + zm.y, zm.x - v[g][m].x);
+    }
+    if (t == 0) {  // k1 = N1/2: Z there is (A + i B) / 2 with real A, B
+      T* q = nq + (size_t)(z * 6 + 2 * (g0 + g)) * n2 + x2;
+      q[0] = (T)2 * v[g][4].x;
+      q[n2] = (T)2 * v[g][4].y;
     }
   }
 }
 
 // inverse row FFTs of row x2 of layer z (thread t of the row's N / 8; sm the row's exchange
-// area [3][LD])
-template <typename T, int N>
+// area [NF][LD]): the pair transforms g0 .. g0 + NF - 1 of the row's three
+template <typename T, int N, int NF = 3>
 __device__ __forceinline__ void rows_inv6_body(const typename Cx<T>::t* __restrict__ spec, const T* __restrict__ nq,
                                                T* __restrict__ out, const typename Cx<T>::t* __restrict__ tw, int n2,
-                                               int z, int x2, int t, typename Cx<T>::t* smrow, T nq_scale, T scale) {
+                                               int z, int x2, int t, typename Cx<T>::t* smrow, T nq_scale, T scale, int g0 = 0) {
   typedef typename Cx<T>::t V;
   constexpr int T8 = N / 8, H1 = N / 2;
-  V v[3][8];
+  V v[NF][8];
 #pragma unroll
-  for (int g = 0; g < 3; ++g) {
-    const int ca = 2 * g, cb = 2 * g + 1;
+  for (int g = 0; g < NF; ++g) {
+    const int ca = 2 * (g0 + g), cb = ca + 1;
     const V* sa = spec + (((size_t)z * 6 + ca) * n2 + x2) * H1;
     const V* sb = spec + (((size_t)z * 6 + cb) * n2 + x2) * H1;
     V ra[8], rbv[8];
@@ -244,18 +271,18 @@ __device__ __forceinline__ void rows_inv6_body(const typename Cx<T>::t* __restri
     }
   }
   RowSm<V, N> sm{smrow};
-  fft_ct<V, true, N, 3, 1>(v, t, sm, tw);
+  fft_ct<V, true, N, NF, 1>(v, t, sm, tw);
 #pragma unroll
-  for (int g = 0; g < 3; ++g)
+  for (int g = 0; g < NF; ++g)
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
       const int x1 = t + m * T8;
-      out[(((size_t)z * 6 + 2 * g) * n2 + x2) * N + x1] = v[g][m].x * scale;
-      out[(((size_t)z * 6 + 2 * g + 1) * n2 + x2) * N + x1] = v[g][m].y * scale;
+      out[(((size_t)z * 6 + 2 * (g0 + g)) * n2 + x2) * N + x1] = v[g][m].x * scale;
+      out[(((size_t)z * 6 + 2 * (g0 + g) + 1) * n2 + x2) * N + x1] = v[g][m].y * scale;
     }
 }
 
-template <typename T, int N>
+template <typename T, int N, int NF>
 __global__ void __launch_bounds__(256) k_rows_inv6_ct(const typename Cx<T>::t* __restrict__ spec,
                                                       const T* __restrict__ nq, T* __restrict__ out,
                                                       const typename Cx<T>::t* __restrict__ tw, int n2, int rb, int z0,
@@ -264,8 +291,8 @@ __global__ void __launch_bounds__(256) k_rows_inv6_ct(const typename Cx<T>::t* _
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8, LD = RowLayout<V, N>::LD;
   const int r = threadIdx.x / T8, t = threadIdx.x % T8;
-  rows_inv6_body<T, N>(spec, nq, out, tw, n2, z0 + blockIdx.y, blockIdx.x * rb + r, t,
-                       reinterpret_cast<V*>(smraw) + (size_t)r * 3 * LD, nq_scale, scale);
+  rows_inv6_body<T, N, NF>(spec, nq, out, tw, n2, z0 + blockIdx.y, blockIdx.x * rb + r, t,
+                           reinterpret_cast<V*>(smraw) + (size_t)r * NF * LD, nq_scale, scale, NF == 3 ? 0 : blockIdx.z);
 }
 
 // FP32 forward row pass: the CTA's six eps_p rows are staged in shared memory with 16-byte
@@ -420,6 +447,13 @@ template <typename T, int N> void cols_n(const fvim_ctx* c, bool inverse, void* 
   }
 }
 
+// The three pair transforms of a row in separate CTAs: FP64 grids with fewer warps than FP64 pipes
+// (four per SM) when one thread runs all three.  With the FP64 stages of
+// stage_bf2 and the halved constants the 32 x 32 x 16 FP64 Hertz solve went from 301 to 266 ms.
+template <typename T, int N> bool rows_apart(const fvim_ctx* c, int nzs) {
+  return sizeof(T) == 8 && (size_t)nzs * c->n2 * (N / 8) / 32 < (size_t)4 * sm_count();
+}
+
 template <typename T, int N> void rows_fwd_n(const fvim_ctx* c, const T* eps_p, int z0, int nzs, const int* zr) {
   typedef typename Cx<T>::t V;
   const int rb = ct_rows(N, c->n2);
@@ -432,11 +466,19 @@ template <typename T, int N> void rows_fwd_n(const fvim_ctx* c, const T* eps_p, 
                                                             (float)c->mu, zr);
     return;
   }
-  const size_t smem = (size_t)rb * 3 * RowLayout<V, N>::LD * sizeof(V);
-  dim3 grid(c->n2 / rb, nzs);
-  smem_attr(k_rows_fwd6_ct<T, N>, smem);
-  k_rows_fwd6_ct<T, N><<<grid, rb * (N / 8), smem, c->stream>>>(eps_p, (V*)c->spec, (T*)c->nq, (const V*)c->tw1,
-                                                              c->n2, rb, z0, (T)c->lam, (T)c->mu, zr);
+  auto go = [&](auto kern, int nf) {
+    const size_t smem = (size_t)rb * nf * RowLayout<V, N>::LD * sizeof(V);
+    smem_attr(kern, smem);
+    kern<<<dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, c->stream>>>(eps_p, (V*)c->spec, (T*)c->nq, (const V*)c->tw1,
+                                                                         c->n2, rb, z0, (T)(0.5 * c->lam), (T)c->mu, zr);
+  };
+  if constexpr (sizeof(T) == 8) {
+    if (rows_apart<T, N>(c, nzs)) {
+      go(k_rows_fwd6_ct<T, N, 1>, 1);
+      return;
+    }
+  }
+  go(k_rows_fwd6_ct<T, N, 3>, 3);
 }
 
 template <typename T, int N> void rows_inv_n(const fvim_ctx* c, T* out, T nq_scale, int z0, int nzs) {
@@ -444,12 +486,20 @@ template <typename T, int N> void rows_inv_n(const fvim_ctx* c, T* out, T nq_sca
   int rb = ct_rows(N, c->n2);
   // smaller CTAs in FP32 (128 threads at N = 512 and 1024): 5 instead of 2 per SM at ~100 registers
   if (sizeof(T) == 4 && (rb >= 4 || N >= 1024)) rb = std::max(1, rb / 2);
-  const size_t smem = (size_t)rb * 3 * RowLayout<V, N>::LD * sizeof(V);
-  dim3 grid(c->n2 / rb, nzs);
   const T scale = (T)(1.0 / ((double)N * (double)c->n2));
-  smem_attr(k_rows_inv6_ct<T, N>, smem);
-  k_rows_inv6_ct<T, N><<<grid, rb * (N / 8), smem, c->stream>>>((const V*)c->spec, (const T*)c->nq, out,
-                                                              (const V*)c->tw1, c->n2, rb, z0, nq_scale, scale);
+  auto go = [&](auto kern, int nf) {
+    const size_t smem = (size_t)rb * nf * RowLayout<V, N>::LD * sizeof(V);
+    smem_attr(kern, smem);
+    kern<<<dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, c->stream>>>((const V*)c->spec, (const T*)c->nq, out,
+                                                                         (const V*)c->tw1, c->n2, rb, z0, nq_scale, scale);
+  };
+  if constexpr (sizeof(T) == 8) {
+    if (rows_apart<T, N>(c, nzs)) {
+      go(k_rows_inv6_ct<T, N, 1>, 1);
+      return;
+    }
+  }
+  go(k_rows_inv6_ct<T, N, 3>, 3);
 }
 
 // ---- grouped launches: every problem of a GrpTable in one launch per pass ---------------

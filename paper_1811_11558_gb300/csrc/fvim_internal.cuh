@@ -125,23 +125,19 @@ __device__ __forceinline__ void dft8(V* v) {
   V o[4] = {v[1], v[3], v[5], v[7]};
   dft4<V, INV>(e);
   dft4<V, INV>(o);
-  // twiddles W8^m, m = 0..3 (forward exp(-i pi m/4)): products by r(1 -/+ i), -/+ i and
-  // r(-1 -/+ i) written out (the zero parts of the twiddles cost nothing)
-  const V o1 = o[1], o2 = o[2], o3 = o[3];
-  if (INV) {
-    o[1] = mk<V>(r * (o1.x - o1.y), r * (o1.x + o1.y));
-    o[2] = mk<V>(-o2.y, o2.x);
-    o[3] = mk<V>(-r * (o3.x + o3.y), r * (o3.x - o3.y));
-  } else {
-    o[1] = mk<V>(r * (o1.x + o1.y), r * (o1.y - o1.x));
-    o[2] = mk<V>(o2.y, -o2.x);
-    o[3] = mk<V>(r * (o3.y - o3.x), -r * (o3.x + o3.y));
-  }
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    v[m] = cadd(e[m], o[m]);
-    v[m + 4] = csub(e[m], o[m]);
-  }
+  // last level v[m] = e[m] + W8^m o[m], v[m + 4] = e[m] - W8^m o[m]: W8 = r (1 -/+ i) and W8^3 =
+  // r (-1 -/+ i) as a sum and a multiply-add per component
+  v[0] = cadd(e[0], o[0]);
+  v[4] = csub(e[0], o[0]);
+  const V x2 = INV ? mk<V>(-o[2].y, o[2].x) : mk<V>(o[2].y, -o[2].x);
+  v[2] = cadd(e[2], x2);
+  v[6] = csub(e[2], x2);
+  const V x1 = INV ? mk<V>(o[1].x - o[1].y, o[1].x + o[1].y) : mk<V>(o[1].x + o[1].y, o[1].y - o[1].x);
+  v[1] = caxpy(e[1], r, x1);
+  v[5] = caxpy(e[1], -r, x1);
+  const V x3 = INV ? mk<V>(-(o[3].x + o[3].y), o[3].x - o[3].y) : mk<V>(o[3].y - o[3].x, -(o[3].x + o[3].y));
+  v[3] = caxpy(e[3], r, x3);
+  v[7] = caxpy(e[3], -r, x3);
 }
 
 template <typename V, bool INV, int R, int MAXI>
@@ -278,7 +274,7 @@ __device__ __forceinline__ void twiddles8(const V* __restrict__ tw, int idx, V (
 }
 
 template <typename V, bool INV, int N, int R, int NS>
-__device__ __forceinline__ void stage_ct(V (&v)[8], int (&pos)[8], int t, const V* __restrict__ tw) {
+__device__ __forceinline__ void stage_prod(V (&v)[8], int (&pos)[8], int t, const V* __restrict__ tw) {
   constexpr int T8 = N / 8;
   if constexpr (R == 8) {
     const int k = t & (NS - 1);
@@ -335,6 +331,114 @@ __device__ __forceinline__ void stage_ct(V (&v)[8], int (&pos)[8], int t, const 
   }
 }
 
+// Radix-2 butterfly with the twiddle inside: t = a + w b, s = a - w b = 2 a - t, six multiply-adds
+// (a separate complex product and two complex sums are eight operations)
+template <typename V> __device__ __forceinline__ void bf2(V& a, V& b, V w) {
+  typedef decltype(V::x) T;
+  V t;
+  t.x = fma(w.x, b.x, fma(-w.y, b.y, a.x));
+  t.y = fma(w.x, b.y, fma(w.y, b.x, a.y));
+  b.x = fma((T)2, a.x, -t.x);
+  b.y = fma((T)2, a.y, -t.y);
+  a = t;
+}
+// w times -i (forward) or i (inverse)
+template <typename V, bool INV> __device__ __forceinline__ V quarter(V w) {
+  return INV ? mk<V>(-w.y, w.x) : mk<V>(w.y, -w.x);
+}
+
+// One stage of a radix-8, 4 or 2 transform on the eight values of a thread, twiddled stages run
+// as radix-2 levels of bf2 (72, 24 and 6 multiply-adds for 8, 4 and 2 values, against 84, 28 and 8
+// with the products apart), from four, two or one table reads: w, w^2, w^4 and w W_8.
+// FP64 is bound by its pipe (one instruction per warp and 64 cycles), so the fewest operations win:
+// 128 x 128 x 126 rows 353 -> 319, columns 261 -> 212, inverse rows 317 -> 278 us.  In FP32 the
+// levels' longer dependency chains cost more than the operations save (512 x 512 x 64 columns 126
+// -> 151 us at 64 registers), so it keeps stage_prod, but for the 8-column CTAs of 1024 points.
+template <typename V, bool INV, int N, int R, int NS>
+__device__ __forceinline__ void stage_bf2(V (&v)[8], int (&pos)[8], int t, const V* __restrict__ tw) {
+  constexpr int T8 = N / 8;
+  if constexpr (R == 8) {
+    const int k = t & (NS - 1);
+    if constexpr (NS > 1) {
+      const int idx = k * (N / (NS * 8));
+      const V w1 = twiddle<V, INV>(tw, idx), w2 = twiddle<V, INV>(tw, 2 * idx), w4 = twiddle<V, INV>(tw, 4 * idx);
+      const V w1e = twiddle<V, INV>(tw, idx + N / 8);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) bf2(v[r], v[r + 4], w4);
+      const V w2q = quarter<V, INV>(w2);
+      bf2(v[0], v[2], w2);
+      bf2(v[1], v[3], w2);
+      bf2(v[4], v[6], w2q);
+      bf2(v[5], v[7], w2q);
+      bf2(v[0], v[1], w1);
+      bf2(v[4], v[5], w1e);
+      bf2(v[2], v[3], quarter<V, INV>(w1));
+      bf2(v[6], v[7], quarter<V, INV>(w1e));
+      // bit-reversed slots hold outputs 0, 4, 2, 6, 1, 5, 3, 7
+      const int base = (t / NS) * NS * 8 + k;
+      constexpr int out[8] = {0, 4, 2, 6, 1, 5, 3, 7};
+      V u[8];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) u[out[r]] = v[r];
+#pragma unroll
+      for (int r = 0; r < 8; ++r) {
+        v[r] = u[r];
+        pos[r] = base + r * NS;
+      }
+    } else {
+      dft8<V, INV>(v);
+      const int base = t * 8;
+#pragma unroll
+      for (int r = 0; r < 8; ++r) pos[r] = base + r;
+    }
+  } else if constexpr (R == 4) {
+    constexpr int step = N / (NS * 4);
+#pragma unroll
+    for (int g = 0; g < 2; ++g) {
+      const int b = t + g * T8;
+      const int k = b & (NS - 1);
+      V u[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) u[r] = v[2 * r + g];
+      if constexpr (NS > 1) {
+        const V w1 = twiddle<V, INV>(tw, k * step), w2 = twiddle<V, INV>(tw, 2 * k * step);
+        bf2(u[0], u[2], w2);
+        bf2(u[1], u[3], w2);
+        bf2(u[0], u[1], w1);
+        bf2(u[2], u[3], quarter<V, INV>(w1));
+        const V x = u[1];  // slots hold outputs 0, 2, 1, 3
+        u[1] = u[2];
+        u[2] = x;
+      } else {
+        dft4<V, INV>(u);
+      }
+      const int base = (b / NS) * NS * 4 + k;
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        v[2 * r + g] = u[r];
+        pos[2 * r + g] = base + r * NS;
+      }
+    }
+  } else {
+    constexpr int step = N / (NS * 2);
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      const int b = t + m * T8;
+      const int k = b & (NS - 1);
+      if constexpr (NS > 1) {
+        bf2(v[m], v[m + 4], twiddle<V, INV>(tw, k * step));
+      } else {
+        const V a = v[m], c = v[m + 4];
+        v[m] = cadd(a, c);
+        v[m + 4] = csub(a, c);
+      }
+      const int base = (b / NS) * NS * 2 + k;
+      pos[m] = base;
+      pos[m + 4] = base + NS;
+    }
+  }
+}
+
 // barrier over the whole CTA (the default exchange synchronisation of fft_ct)
 struct CtaSync {
   __device__ __forceinline__ void operator()() const { __syncthreads(); }
@@ -352,6 +456,11 @@ template <int NG> struct GroupSync {
   }
 };
 
+// whether the stages of a transform run as bf2 levels (stage_bf2) or with the products apart
+template <typename V, int N, class Sm> struct UseBf2 {
+  static constexpr bool v = sizeof(V) == 16;
+};
+
 template <typename V, bool INV, int N, int NF, int NS, class Sm, class Sync = CtaSync>
 __device__ __forceinline__ void fft_ct(V (&v)[NF][8], int t, const Sm& sm, const V* __restrict__ tw,
                                        const Sync& sync = Sync()) {
@@ -359,7 +468,8 @@ __device__ __forceinline__ void fft_ct(V (&v)[NF][8], int t, const Sm& sm, const
   int pos[8];
 #pragma unroll
   for (int f = 0; f < NF; ++f) {
-    stage_ct<V, INV, N, R, NS>(v[f], pos, t, tw);
+    if constexpr (UseBf2<V, N, Sm>::v) stage_bf2<V, INV, N, R, NS>(v[f], pos, t, tw);
+    else stage_prod<V, INV, N, R, NS>(v[f], pos, t, tw);
     if constexpr (NS * R < N) {
 #pragma unroll
       for (int m = 0; m < 8; ++m) sm.put(f, pos[m], v[f][m]);
@@ -410,6 +520,16 @@ inline int smem_optin_max() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&m, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     return m > 0 ? m : 48 * 1024;
+  }();
+  return v;
+}
+// multiprocessors of the current device
+inline int sm_count() {
+  static const int v = [] {
+    int dev = 0, m = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&m, cudaDevAttrMultiProcessorCount, dev);
+    return m > 0 ? m : 1;
   }();
   return v;
 }
@@ -569,6 +689,36 @@ template <typename T> bool launch_cols_ct(const fvim_ctx* c, bool inverse, void*
 template <typename T> bool launch_cols_conv_ct(const fvim_ctx* c);
 template <typename T> bool launch_rows_fwd6_ct(const fvim_ctx* c, const T* eps_p, int z0, int nzs, const int* zr = nullptr);
 template <typename T> bool launch_rows_inv6_ct(const fvim_ctx* c, T* out, T nq_scale, int z0, int nzs);
+
+// ---- fused Polonsky-Keer iteration (contact_cg.cu) ---------------------------------------
+// device state of one contact solve
+struct PkState {
+  double nIc, gbar, G_old, beta, delta, tau, s, err;  // scalars of the iteration
+  double start, unif;                                  // scale of the initial pressure (0: uniform), uniform pressure
+  double W, dA, tol;
+  const void* h;
+  void* p;
+  int done, it, bad, max_it;
+};
+static_assert(sizeof(PkState) <= 256, "pinned copy of the contact state");
+struct PkfArgs {
+  int n1, n2, h1;
+  double L1, L2, nu, mu;
+  cudaStream_t stream;
+  PkState* S;
+  void *u, *g, *t, *pold;  // surface work arrays [n2][n1]
+  void* surf;              // half spectrum [n2][h1]
+  const void *tw1, *tw2;
+  double* part;            // block partials of the sums
+  unsigned* cnt;           // arrival counter, zero between kernels
+  cudaGraphConditionalHandle cond;
+  int use_cond;            // the last kernel of an iteration sets the loop condition
+};
+bool pkf_available(const fvim_ctx* c);
+// state, initial pressure scaled to the load, its displacement and mean gap
+template <typename T> int pkf_begin(const PkfArgs& a, const PkState& init);
+// one iteration; does nothing once the state's done flag is set
+template <typename T> int pkf_iteration(const PkfArgs& a);
 
 // ---- J2 radial return with linear isotropic hardening (Sec. 4.1) at one voxel -----------
 // de: strain increment, sig: stress of the last converged increment, ep: cumulated plastic
