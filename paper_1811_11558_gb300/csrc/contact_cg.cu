@@ -18,8 +18,9 @@
 // do not depend on timing.  Every scalar, the surface and pressure pointers, the load and the
 // tolerance live in the device state (PkState): one captured loop serves every call of a context.
 //
-// Why: each kernel is a few microseconds of launch, latency and one or two dependent global reads,
-// so the iteration's time was its kernel count (62 us at 32^2 FP32, 132 us at 512^2).  PKF_FIGURES
+// Why: each kernel is a few microseconds of launch, latency and dependent global reads, and the
+// surface FFTs ran on a generic runtime-length kernel: 132 -> 75 us per iteration at 512^2 FP32, 206
+// -> 156 at 1024^2.
 #include <algorithm>
 
 #include "fvim_internal.cuh"

@@ -29,11 +29,12 @@ constexpr int RMAXB = 1024;   // blocks of a reduction grid
 constexpr int NVMAX = 3;      // values reduced per pass
 constexpr size_t kScalarBlock = 256;  // bytes of the solver's device scalar block (V_PKS)
 constexpr size_t kDfsBytes = 1024;     // bytes of the device DF-SANE state (V_DFS)
+constexpr size_t kPkfBytes = 512;      // fused contact iteration (V_PKF): PkState, arrival counter at byte 256
 
 // surface buffers [N2][N1]
 enum { S_P = 0, S_POLD, S_T, S_G, S_U, S_R, S_H, S_H0, S_DU, S_DUPREV, S_TPREV, S_DT, S_NSURF };
 // volume buffers [Nz][6][N2][N1] and the scalar field [Nz][N2][N1]
-enum { V_X = S_NSURF, V_F, V_XT, V_FT, V_B, V_DEP, V_TMP, V_DE, V_EP, V_PART, V_WZ, V_PKS, V_DFS, V_END };
+enum { V_X = S_NSURF, V_F, V_XT, V_FT, V_B, V_DEP, V_TMP, V_DE, V_EP, V_PART, V_WZ, V_PKS, V_DFS, V_PKF, V_END };
 static_assert(V_END <= FVIM_NSOLVER_BUFS, "workspace slots");
 
 template <typename T> size_t esz() { return sizeof(T); }
@@ -50,6 +51,8 @@ template <typename T> int ensure_ws(fvim_ctx* c) {
   if (FVIM_CU(cudaMalloc(&c->sv[V_WZ], (size_t)c->nz * sizeof(double)))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_PKS], kScalarBlock))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_DFS], kDfsBytes))) return FVIM_ERR_OOM;
+  if (FVIM_CU(cudaMalloc(&c->sv[V_PKF], kPkfBytes)) || FVIM_CU(cudaMemset(c->sv[V_PKF], 0, kPkfBytes)))
+    return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMallocHost(&c->h_part, (size_t)RMAXB * NVMAX * sizeof(double) + 256 + kDfsBytes))) {
     c->h_part = nullptr;
     return FVIM_ERR_OOM;
@@ -91,6 +94,8 @@ struct SolverRT {
   cudaGraphExec_t dfloop = nullptr;                          // device DF-SANE loop (WHILE node)
   bool dfloop_failed = false;                                // building it failed: host loop
   bool cgw_failed = false;                                   // building a CG loop failed: host loop
+  cudaGraphExec_t cgf = nullptr;                             // fused device CG loop (WHILE node)
+  bool cgf_failed = false;                                   // building it failed: host loop
 };
 constexpr size_t kMaxGraphs = 8;
 
@@ -277,82 +282,6 @@ template <int NV> int finish(fvim_ctx* c, int nblk, double* out) {
 }
 
 // ---- Polonsky-Keer kernels (surface, n = N1 N2) ------------------------------------
-// sum over the contact set of u - h, and its size
-template <typename T>
-__global__ void k_pk_stats(const T* __restrict__ u, const T* __restrict__ h, const T* __restrict__ p, size_t n,
-                           double* part) {
-  double v[2] = {0, 0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-    if (p[i] > 0) { v[0] += (double)u[i] - (double)h[i]; v[1] += 1; }
-  block_reduce<2>(v, part);
-}
-// g = u - h - gbar; sum over the contact set of g^2
-template <typename T>
-__global__ void k_pk_g(const T* __restrict__ u, const T* __restrict__ h, const T* __restrict__ p, T* __restrict__ g,
-                       double gbar, size_t n, double* part) {
-  double v[1] = {0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-    const T gi = (T)((double)u[i] - (double)h[i] - gbar);
-    g[i] = gi;
-    if (p[i] > 0) v[0] += (double)gi * (double)gi;
-  }
-  block_reduce<1>(v, part);
-}
-// conjugate direction t = g + beta t on the contact set, 0 elsewhere
-template <typename T>
-__global__ void k_pk_dir(const T* __restrict__ g, const T* __restrict__ p, T* __restrict__ t, double beta, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-    t[i] = p[i] > 0 ? (T)((double)g[i] + beta * (double)t[i]) : (T)0;
-}
-// sum over the contact set of r
-template <typename T>
-__global__ void k_pk_rsum(const T* __restrict__ r, const T* __restrict__ p, size_t n, double* part) {
-  double v[1] = {0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-    if (p[i] > 0) v[0] += (double)r[i];
-  block_reduce<1>(v, part);
-}
-// <g, t> and <r - rbar, t> over the contact set
-template <typename T>
-__global__ void k_pk_dots(const T* __restrict__ g, const T* __restrict__ t, const T* __restrict__ r,
-                          const T* __restrict__ p, double rbar, size_t n, double* part) {
-  double v[2] = {0, 0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT)
-    if (p[i] > 0) {
-      v[0] += (double)g[i] * (double)t[i];
-      v[1] += ((double)r[i] - rbar) * (double)t[i];
-    }
-  block_reduce<2>(v, part);
-}
-// p <- max(p - tau t, 0); penetrating points with zero pressure get -tau g
-template <typename T>
-__global__ void k_pk_update(T* __restrict__ p, T* __restrict__ pold, const T* __restrict__ t,
-                            const T* __restrict__ g, double tau, size_t n, double* part) {
-  double v[2] = {0, 0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-    const T po = p[i];
-    T pn = (T)fmax((double)po - tau * (double)t[i], 0.0);
-    const bool ol = (pn == (T)0) && (g[i] < (T)0);
-    if (ol) pn = (T)(-tau * (double)g[i]);
-    pold[i] = po;
-    p[i] = pn;
-    v[0] += (double)pn;
-    v[1] += ol ? 1.0 : 0.0;
-  }
-  block_reduce<2>(v, part);
-}
-// p <- s p; sum |p - p_old| and the size of the contact set
-template <typename T>
-__global__ void k_pk_scale(T* __restrict__ p, const T* __restrict__ pold, double s, size_t n, double* part) {
-  double v[2] = {0, 0};
-  for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-    const T pn = (T)(s * (double)p[i]);
-    p[i] = pn;
-    v[0] += fabs((double)pn - (double)pold[i]);
-    v[1] += pn > (T)0 ? 1.0 : 0.0;
-  }
-  block_reduce<2>(v, part);
-}
 template <typename T> __global__ void k_fill(T* __restrict__ a, T v, size_t n) {
   for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) a[i] = v;
 }
@@ -749,8 +678,96 @@ static bool device_cg_enabled() {
   return !(e && e[0] == '0');
 }
 
+// The fused iteration (contact_cg.cu): one WHILE graph per context, whatever the surface, pressure,
+// load and tolerance (all in the device state), one read of the state per solve; with
+// FVIM_DEVICE_CG=0, graphs off or while kernels are timed, batches of iterations with one read each.
+template <typename T>
+int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_opts* o, int* iters, double* err_out) {
+  const size_t n = (size_t)c->n1 * c->n2;
+  PkfArgs a;
+  memset(&a, 0, sizeof(a));
+  a.n1 = c->n1;
+  a.n2 = c->n2;
+  a.h1 = c->h1;
+  a.L1 = c->L1;
+  a.L2 = c->L2;
+  a.nu = c->nu;
+  a.mu = c->mu;
+  a.stream = c->stream;
+  a.S = (PkState*)c->sv[V_PKF];
+  a.u = c->sv[S_U];
+  a.g = c->sv[S_G];
+  a.t = c->sv[S_T];
+  a.pold = c->sv[S_POLD];
+  a.surf = c->surf;
+  a.tw1 = c->tw1;
+  a.tw2 = c->tw2;
+  a.part = (double*)c->sv[V_PART];
+  a.cnt = reinterpret_cast<unsigned*>(static_cast<char*>(c->sv[V_PKF]) + 256);
+  PkState s0;
+  memset(&s0, 0, sizeof(s0));
+  s0.G_old = 1.0;
+  s0.s = 1.0;
+  s0.err = INFINITY;
+  s0.unif = W / (c->L1 * c->L2);
+  s0.W = W;
+  s0.dA = c->L1 * c->L2 / (double)n;
+  s0.tol = o->cg_tol;
+  s0.h = h;
+  s0.p = p;
+  s0.max_it = o->cg_max_iter;
+  PkState* sh = reinterpret_cast<PkState*>(c->h_part + (size_t)RMAXB * NVMAX);  // pinned
+  int rc;
+  if ((rc = pkf_begin<T>(a, s0))) return rc;
+  SolverRT* srt = rt(c);
+  bool ran_device = false;
+  if (srt && !c->prof && graphs_enabled() && device_cg_enabled()) {
+    if (!srt->cgf && !srt->cgf_failed &&
+        build_while_graph(
+            c,
+            [&](cudaGraphConditionalHandle cond) -> int {
+              PkfArgs b = a;
+              b.cond = cond;
+              b.use_cond = 1;
+              return pkf_iteration<T>(b);
+            },
+            &srt->cgf) != FVIM_OK) {
+      srt->cgf_failed = true;  // the batches below take over
+      srt->cgf = nullptr;
+      cudaGetLastError();
+    }
+    if (srt->cgf) {
+      if (FVIM_CU(cudaGraphLaunch(srt->cgf, c->stream)) ||
+          FVIM_CU(cudaMemcpyAsync(sh, a.S, sizeof(PkState), cudaMemcpyDeviceToHost, c->stream)) ||
+          FVIM_CU(cudaStreamSynchronize(c->stream)))
+        return FVIM_ERR_CUDA;
+      ran_device = true;
+    }
+  }
+  const int batch = 4;  // iterations issued between two reads of the stop flag
+  for (int issued = 0; !ran_device && issued < o->cg_max_iter; issued += batch) {
+    auto iterations = [&]() -> int {
+      int r;
+      for (int b = 0; b < batch; ++b)
+        if ((r = pkf_iteration<T>(a))) return r;
+      return FVIM_OK;
+    };
+    const GraphKey key{{nullptr, nullptr, nullptr}, {0.0, 0.0}, 0};
+    if ((rc = srt ? graph_run(c, srt->cg, key, iterations) : iterations())) return rc;
+    if (FVIM_CU(cudaMemcpyAsync(sh, a.S, sizeof(PkState), cudaMemcpyDeviceToHost, c->stream)) ||
+        FVIM_CU(cudaStreamSynchronize(c->stream)))
+      return FVIM_ERR_CUDA;
+    if (sh->done) break;
+  }
+  if (sh->bad) return FVIM_ERR_NONFINITE;
+  if (iters) *iters = sh->it;
+  if (err_out) *err_out = sh->err;
+  return sh->err < o->cg_tol ? FVIM_OK : FVIM_ERR_NOT_CONVERGED;
+}
+
 template <typename T>
 int elastic_contact_t(fvim_ctx* c, const T* h, double W, T* p, const fvim_opts* o, int* iters, double* err_out) {
+  if (pkf_available(c)) return elastic_contact_fused<T>(c, h, W, p, o, iters, err_out);
   const size_t n = (size_t)c->n1 * c->n2;
   const double dA = c->L1 * c->L2 / (double)n;
   double* part = (double*)c->sv[V_PART];
@@ -1368,6 +1385,8 @@ void solver_drop_graphs(fvim_ctx* c) {
   drop(r->cg);
   drop(r->df);
   drop(r->cgw);
+  if (r->cgf) cudaGraphExecDestroy(r->cgf);
+  r->cgf = nullptr;
   if (r->dfloop) cudaGraphExecDestroy(r->dfloop);
   r->dfloop = nullptr;
 }
@@ -1377,6 +1396,8 @@ void solver_release(fvim_ctx* c) {
   if (r) {
     drop(r->cg);
     drop(r->df);
+    drop(r->cgw);
+    if (r->cgf) cudaGraphExecDestroy(r->cgf);
     if (r->dfloop) cudaGraphExecDestroy(r->dfloop);
     if (r->stream) cudaStreamDestroy(r->stream);
     if (r->ev_in) cudaEventDestroy(r->ev_in);
