@@ -1,26 +1,31 @@
 // Fused kernels of the Polonsky-Keer contact iteration (Sec. 5.1) on power-of-two surfaces with
-// both sides from 16 to 1024: seven kernels per iteration instead of fourteen.
+// both sides from 16 to 1024: six kernels per iteration.
 //
-// An iteration is a chain of global sums (mean gap, G, tau, total load, change), each of which the
-// next elementwise step needs, and two surface convolutions u = K*p, r = K*t.  Each elementwise
-// step runs inside the row pass of the convolution next to it:
-//   gap    g = u - h - gbar on the surface; G = sum over the contact of g^2 -> beta
-//   rowsT  t = g + beta t on the contact, 0 elsewhere; forward rows of t
+// An iteration is a chain of global sums (mean gap and G, tau, total load), each of which the next
+// elementwise step needs, and two surface convolutions u = K*p, r = K*t.  Each elementwise step
+// runs inside the row pass of the convolution next to it:
+//   rowsT  g = u - h - gbar; t = g + beta t on the contact, 0 elsewhere; forward rows of t
 //   cols   columns: transform, surface compliance, inverse
 //   rowsR  inverse rows of r = K*t, kept in registers; sums of r, t, g t and r t over the contact
 //          -> tau = <g, t> / (<r, t> - rbar <t, 1>)
 //   rowsP  p <- max(p - tau t, 0), points that would penetrate re-enter; sum p -> load scale s;
 //          forward rows of the unscaled p
 //   cols   as above, times s (the transform is linear)
-//   rowsU  inverse rows of u = K*p; p <- s p, change against the old pressure, mean gap over the
-//          contact -> gbar, stop test
-// The sums are FP64, block partials in block order added by the last block to finish, so results
-// do not depend on timing.  Every scalar, the surface and pressure pointers, the load and the
-// tolerance live in the device state (PkState): one captured loop serves every call of a context.
+//   rowsU  inverse rows of u = K*p; p <- s p, change against the old pressure -> stop test; over
+//          the contact sums of d and d^2, d = u - h - (last gbar) -> gbar, G = sum of g^2 -> beta
+// (d is the gap up to the change of its mean, so G = sum d^2 - (sum d)^2 / n cancels nothing that
+// the iteration does not itself lose; the first G is summed from g.)  The sums are FP64, block
+// partials in block order added by the last block to finish, so results do not depend on timing.
+// Every scalar, the surface and pressure pointers, the load and the tolerance live in the device
+// state (PkState): one captured loop serves every call of a context.
 //
-// Why: each kernel is a few microseconds of launch, latency and dependent global reads, and the
-// surface FFTs ran on a generic runtime-length kernel: 132 -> 75 us per iteration at 512^2 FP32, 206
-// -> 156 at 1024^2.
+// What bounds it: an FP64 instruction holds its pipe for 64 cycles per warp here (a conversion
+// counts as one), so a kernel's time is its FP64 instructions per warp and the dependent chain of
+// its sums.  So: four complex values per thread (more warps with less each); elementwise FP32
+// updates in two-float arithmetic, rounded once as the FP64 expression is; FP64 only in the sums,
+// and there only at points that carry pressure; a warp's sums of several values reduced together.
+// us per iteration, fourteen kernels -> seven with eight values per thread and FP64 updates -> this:
+// 32^2 FP64 100 -> 97 -> 56, 32^2 FP32 62 -> 63 -> 41, 512^2 132 -> 75 -> 56, 1024^2 206 -> 156 -> 112.
 #include <algorithm>
 
 #include "fvim_internal.cuh"
@@ -30,191 +35,303 @@ namespace {
 enum { FWD_INIT = 0, FWD_P, FWD_T };
 enum { INV_U0 = 0, INV_U, INV_R };
 
-// sums of NV doubles over the block (any whole number of warps) into part[blockIdx.x * NV + j]
-template <int NV> __device__ __forceinline__ void block_sum(double (&v)[NV], double* part) {
-  __shared__ double sh[NV][32];
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int j = 0; j < NV; ++j) {
-    double x = v[j];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) sh[j][w] = x;
-  }
-  __syncthreads();
-  if (threadIdx.x < NV) {
-    double s = 0;
-    for (int k = 0; k < nw; ++k) s += sh[threadIdx.x][k];
-    part[blockIdx.x * NV + threadIdx.x] = s;
-  }
+// ---- sums -----------------------------------------------------------------------------
+// Sums of up to four values over a warp, reduced together: six additions instead of five per value.
+// Lane l ends with the sum of value ((l >> 4) & 1) 2 + ((l >> 3) & 1).
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3) {
+  const unsigned all = 0xffffffffu;
+  const bool h16 = threadIdx.x & 16, h8 = threadIdx.x & 8;
+  double a = (h16 ? v2 : v0) + __shfl_xor_sync(all, h16 ? v0 : v2, 16);
+  const double b = (h16 ? v3 : v1) + __shfl_xor_sync(all, h16 ? v1 : v3, 16);
+  a = (h8 ? b : a) + __shfl_xor_sync(all, h8 ? a : b, 8);
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
+  return a;
 }
-// true in the last block of the grid to arrive; its first warp then adds the partials in a fixed
-// order and every lane gets the sums
-template <int NV> __device__ __forceinline__ bool grid_sum(double (&v)[NV], double* part, unsigned* cnt) {
+// over the block's whole warps of per-thread values x of kind j = threadIdx.x & 3 that are already
+// summed over the lanes of equal j: lanes 0..3 of warp 0 end with the sums
+__device__ __forceinline__ double block_sum_kind(double x, double* sh) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (nw == 1) return x;
+  if (l < 4) sh[w * 4 + l] = x;
+  __syncthreads();
+  if (w > 0) return 0;
+  x = 0;
+  for (int k = l >> 2; k < nw; k += 8) x += sh[k * 4 + (l & 3)];
+  for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// sums of v over the grid: true in thread 0 of the last block to arrive, which then holds them
+__device__ __forceinline__ bool grid_sum(double (&v)[4], double* part, unsigned* cnt) {
+  __shared__ double sh[32 * 4];
   __shared__ bool last;
-  block_sum<NV>(v, part);
-  __threadfence();
+  const int l = threadIdx.x & 31;
+  double x = warp_sum4(v[0], v[1], v[2], v[3]);
+  // value j from the lane group that holds it
+  x = __shfl_sync(0xffffffffu, x, ((l & 3) >> 1) * 16 + (l & 1) * 8);
+  x = block_sum_kind(x, sh);
+  if (threadIdx.x < 4) {
+    part[blockIdx.x * 4 + threadIdx.x] = x;
+    __threadfence();
+  }
   __syncthreads();
   if (threadIdx.x == 0) last = atomicAdd(cnt, 1u) == gridDim.x - 1;
   __syncthreads();
-  if (!last || threadIdx.x >= 32) return false;
+  if (!last) return false;
   __threadfence();
-  const int n = gridDim.x;
+  x = 0;
+  for (int b = threadIdx.x >> 2; b < (int)gridDim.x; b += blockDim.x >> 2) x += __ldcg(part + b * 4 + (threadIdx.x & 3));
+  for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  x = block_sum_kind(x, sh);
+  if (threadIdx.x >= 32) return false;
 #pragma unroll
-  for (int j = 0; j < NV; ++j) v[j] = 0;
-  for (int b = threadIdx.x; b < n; b += 32)
-#pragma unroll
-    for (int j = 0; j < NV; ++j) v[j] += __ldcg(part + b * NV + j);
-#pragma unroll
-  for (int j = 0; j < NV; ++j)
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
+  for (int j = 0; j < 4; ++j) v[j] = __shfl_sync(0xffffffffu, x, j);
   if (threadIdx.x == 0) *cnt = 0u;
   return threadIdx.x == 0;
 }
+
+// ---- elementwise updates with FP64 scalars, rounded once to the path's precision ------------
+// FP32: the scalar as a float pair, products and sums as exact pairs (to about 2^-46 of the result
+// before its one rounding)
+__device__ __forceinline__ float2 pair_of(double x) {
+  const float h = (float)x;
+  return make_float2(h, isfinite(h) ? (float)(x - (double)h) : 0.f);
+}
+__device__ __forceinline__ float two_sum_err(float a, float b, float s) {  // a + b - s
+  const float bb = __fsub_rn(s, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// a + k x
+__device__ __forceinline__ float axpy1(float a, double, float2 k, float x) {
+  const float p = __fmul_rn(k.x, x), pl = __fmaf_rn(k.x, x, -p);
+  const float s = __fadd_rn(a, p), e = two_sum_err(a, p, s);
+  return __fadd_rn(s, __fadd_rn(e, __fmaf_rn(k.y, x, pl)));
+}
+__device__ __forceinline__ double axpy1(double a, double k, float2, double x) { return a + k * x; }
+// k x
+__device__ __forceinline__ float mul1(double, float2 k, float x) {
+  const float p = __fmul_rn(k.x, x);
+  return __fadd_rn(p, __fmaf_rn(k.y, x, __fmaf_rn(k.x, x, -p)));
+}
+__device__ __forceinline__ double mul1(double k, float2, double x) { return k * x; }
+// u - h - c
+__device__ __forceinline__ float gap1(float u, float h, double, float2 c) {
+  const float d = __fsub_rn(u, h), e = two_sum_err(u, -h, d);
+  const float s = __fsub_rn(d, c.x), e2 = two_sum_err(d, -c.x, s);
+  return __fadd_rn(s, __fadd_rn(e2, __fsub_rn(e, c.y)));
+}
+__device__ __forceinline__ double gap1(double u, double h, double c, float2) { return u - h - c; }
+
+// ---- transforms of four values per thread -------------------------------------------------
+// Stockham stages of radix 4, the first of radix 2 where log2 N is odd; thread t of N / 4 holds the
+// values t + m N / 4 before and after.  Exchange layout by the caller (Sm), CTA barriers.
+template <int N> struct OddLog2 {
+  static constexpr bool v = (N & 0x55555555) == 0;
+};
+template <typename V, bool INV, int N, int NS, class Sm>
+__device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V* __restrict__ tw) {
+  constexpr int T4 = N / 4, R = (NS == 1 && OddLog2<N>::v) ? 2 : 4;
+  int pos[4];
+  if constexpr (R == 2) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const V a = v[m], c = v[m + 2];
+      v[m] = cadd(a, c);
+      v[m + 2] = csub(a, c);
+      pos[m] = 2 * (t + m * T4);
+      pos[m + 2] = pos[m] + 1;
+    }
+  } else {
+    const int k = t & (NS - 1);
+    if constexpr (NS > 1) {
+      constexpr int step = N / (NS * 4);
+      const V w1 = twiddle<V, INV>(tw, k * step), w2 = twiddle<V, INV>(tw, 2 * k * step);
+      bf2(v[0], v[2], w2);
+      bf2(v[1], v[3], w2);
+      bf2(v[0], v[1], w1);
+      bf2(v[2], v[3], quarter<V, INV>(w1));
+      const V x = v[1];
+      v[1] = v[2];
+      v[2] = x;
+    } else {
+      dft4<V, INV>(v);
+    }
+    const int base = (t / NS) * NS * 4 + k;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) pos[r] = base + r * NS;
+  }
+  if constexpr (NS * R < N) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) sm.put(pos[m], v[m]);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = sm.get(t + m * T4);
+    __syncthreads();
+    fft4_ct<V, INV, N, NS * R>(v, t, sm, tw);
+  }
+}
+// rows: one pad slot every 8 entries
+template <typename V, int N> struct SurfSm {
+  static constexpr int LD = N + N / 8;
+  V* buf;
+  __device__ __forceinline__ void put(int p, V x) const { buf[p + (p >> 3)] = x; }
+  __device__ __forceinline__ V get(int p) const { return buf[p + (p >> 3)]; }
+};
+template <typename V> struct SurfColSm {
+  V* buf;
+  int kc, f;
+  __device__ __forceinline__ void put(int p, V x) const { buf[p * kc + f] = x; }
+  __device__ __forceinline__ V get(int p) const { return buf[p * kc + f]; }
+};
 
 // state of a new solve, with the scale of the initial pressure from its sum (a guess without load
 // is replaced by the uniform pressure)
 template <typename T>
 __global__ void __launch_bounds__(256) k_pkf_begin(PkState* S, const T* __restrict__ p, size_t n, PkState init, double* part,
                                                    unsigned* cnt) {
-  double v[1] = {0};
+  double v[4] = {0, 0, 0, 0};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) v[0] += (double)p[i];
-  if (grid_sum<1>(v, part, cnt)) {
+  if (grid_sum(v, part, cnt)) {
     init.start = v[0] > 0 ? init.W / (init.dA * v[0]) : 0.0;
     *S = init;
   }
 }
+// surface compliance u3_hat / p_hat = (1 - nu) / (mu q) of every mode, 0 for mode 0 and the Nyquist row
+template <typename T>
+__global__ void __launch_bounds__(256) k_pkf_green(T* __restrict__ green, int h1, int n2, T w1, T w2, T nu, T mu) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= h1 * n2) return;
+  const int k2 = i / h1, k1 = i - k2 * h1;
+  const T q1 = w1 * (T)k1;
+  const T q2 = w2 * (T)(k2 < n2 / 2 ? k2 : k2 - n2);
+  const T q = sqrt(q1 * q1 + q2 * q2);
+  green[i] = i == 0 || k2 == n2 / 2 ? (T)0 : ((T)1 - nu) / (mu * q);
+}
 
-// index of entry p of a transform in the exchange area: contiguous rows, swizzled (8-byte entries,
-// 128 points and more) or with a pad slot every 8 entries, conflict-free for the radix-8 stages
-template <typename V, int N> struct SurfSm {
-  static constexpr bool swz = sizeof(V) == 8 && N >= 128;
-  static constexpr int LD = swz ? N : N + N / 8;
-  V* buf;
-  static __device__ __forceinline__ int idx(int p) { return swz ? (p ^ ((p >> 3) & 15)) : p + (p >> 3); }
-  __device__ __forceinline__ void put(int, int p, V x) const { buf[idx(p)] = x; }
-  __device__ __forceinline__ V get(int, int p) const { return buf[idx(p)]; }
-};
-
-// Forward rows of p or t, two rows per transform, N / 8 threads per transform, blockDim.x / (N / 8)
+// Forward rows of p or t, two rows per transform, N / 4 threads per transform, blockDim.x / (N / 4)
 // transforms per CTA; the half spectrum k1 < N/2 goes to surf (the Nyquist column carries no
 // operator term).
 template <typename T, int N, int MODE>
-__global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __restrict__ g, T* __restrict__ t,
-                                                      T* __restrict__ pold, typename Cx<T>::t* __restrict__ surf,
+__global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __restrict__ u, T* __restrict__ g,
+                                                      T* __restrict__ t, T* __restrict__ pold,
+                                                      typename Cx<T>::t* __restrict__ surf,
                                                       const typename Cx<T>::t* __restrict__ tw, int n2, double* part,
                                                       unsigned* cnt) {
   typedef typename Cx<T>::t V;
   if (MODE != FWD_INIT && S->done) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int T8 = N / 8, H1 = N / 2, LD = SurfSm<V, N>::LD;
-  const int r = threadIdx.x / T8, tt = threadIdx.x % T8;
-  const int pair = blockIdx.x * (blockDim.x / T8) + r;
+  constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
+  const int r = threadIdx.x / T4, tt = threadIdx.x % T4;
+  const int pair = blockIdx.x * (blockDim.x / T4) + r;
   const bool live = pair < n2 / 2;
   T* p = static_cast<T*>(S->p);
+  const T* h = static_cast<const T*>(S->h);
   const size_t i0 = (size_t)(live ? 2 * pair : 0) * N + tt;
-  const double beta = S->beta, tau = S->tau, start = S->start, unif = S->unif;
-  V v[1][8];
-  double sum[2] = {0, 0};
+  const double start = S->start, unif = S->unif, tau = S->tau, gbar = S->gbar, beta = S->beta;
+  const float2 tau2 = S->tau2, gbar2 = S->gbar2, beta2 = S->beta2;
+  V v[4];
+  double sum[4] = {0, 0, 0, 0};
+  int nol = 0;
   auto value = [&](size_t i) -> T {
-    if (MODE == FWD_INIT) {
+    if constexpr (MODE == FWD_INIT) {
       const T x = start > 0 ? (T)(start * (double)p[i]) : (T)unif;
       p[i] = x;
       t[i] = (T)0;
       return x;
-    } else if (MODE == FWD_P) {
-      const T po = p[i], gi = g[i];
-      T pn = (T)fmax((double)po - tau * (double)t[i], 0.0);
-      const bool ol = (pn == (T)0) && (gi < (T)0);
-      if (ol) pn = (T)(-tau * (double)gi);
+    } else if constexpr (MODE == FWD_P) {
+      const T po = p[i], ti = t[i], gi = g[i];
+      T pn = (T)0;
+      if (po != (T)0 || ti != (T)0) {
+        const T x = axpy1(po, -tau, make_float2(-tau2.x, -tau2.y), ti);
+        pn = x > (T)0 ? x : (T)0;
+      }
+      if (pn == (T)0 && gi < (T)0) {
+        pn = mul1(-tau, make_float2(-tau2.x, -tau2.y), gi);
+        ++nol;
+      }
       pold[i] = po;
       p[i] = pn;
-      sum[0] += (double)pn;
-      sum[1] += ol ? 1.0 : 0.0;
+      if (pn != (T)0) sum[0] += (double)pn;
       return pn;
     } else {
-      const T x = p[i] > (T)0 ? (T)((double)g[i] + beta * (double)t[i]) : (T)0;
+      const T gi = gap1(u[i], h[i], gbar, gbar2);
+      g[i] = gi;
+      const T x = p[i] > (T)0 ? axpy1(gi, beta, beta2, t[i]) : (T)0;
       t[i] = x;
       return x;
     }
   };
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    v[0][m] = mk<V>(0, 0);
+  for (int m = 0; m < 4; ++m) {
+    v[m] = mk<V>(0, 0);
     if (live) {
-      const size_t i = i0 + m * T8;
-      v[0][m].x = value(i);
-      v[0][m].y = value(i + N);
+      const size_t i = i0 + m * T4;
+      v[m].x = value(i);
+      v[m].y = value(i + N);
     }
   }
   SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
-  fft_ct<V, false, N, 1, 1>(v, tt, sm, tw);
-  // separation of the two rows: Z(N - k) of k = tt + m N/8, m < 4, is in another thread's upper half
-#pragma unroll
-  for (int m = 4; m < 8; ++m) sm.put(0, tt + m * T8, v[0][m]);
+  fft4_ct<V, false, N, 1>(v, tt, sm, tw);
+  // separation of the two rows: Z(N - k) of k = tt + m N/4, m < 2, is in another thread's upper half
+  sm.put(tt + 2 * T4, v[2]);
+  sm.put(tt + 3 * T4, v[3]);
   __syncthreads();
   if (live) {
     V* o = surf + (size_t)2 * pair * H1 + tt;
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      V zm = sm.get(0, (N - tt - m * T8) & (N - 1));
-      if (m == 0 && tt == 0) zm = v[0][0];
-      const V c = cconj(zm), a = cadd(v[0][m], c), d = csub(v[0][m], c);
-      o[m * T8] = cscale(a, (T)0.5);
-      o[H1 + m * T8] = mk<V>((T)0.5 * d.y, (T)-0.5 * d.x);
+    for (int m = 0; m < 2; ++m) {
+      V zm = sm.get((N - tt - m * T4) & (N - 1));
+      if (m == 0 && tt == 0) zm = v[0];
+      const V c = cconj(zm), a = cadd(v[m], c), d = csub(v[m], c);
+      o[m * T4] = cscale(a, (T)0.5);
+      o[H1 + m * T4] = mk<V>((T)0.5 * d.y, (T)-0.5 * d.x);
     }
   }
-  if (MODE == FWD_P && grid_sum<2>(sum, part, cnt)) {
-    S->delta = sum[1] > 0 ? 0.0 : 1.0;
-    if (!(sum[0] > 0) || !isfinite(sum[0])) {
-      S->bad = 1;
-      S->done = 1;
-    } else {
-      S->s = S->W / (S->dA * sum[0]);
+  if (MODE == FWD_P) {
+    sum[1] = (double)nol;
+    if (grid_sum(sum, part, cnt)) {
+      S->delta = sum[1] > 0 ? 0.0 : 1.0;
+      if (!(sum[0] > 0) || !isfinite(sum[0])) {
+        S->bad = 1;
+        S->done = 1;
+      } else {
+        const double x = S->W / (S->dA * sum[0]);
+        S->s = x;
+        S->s2 = pair_of(x);
+      }
     }
   }
 }
 
-// Columns: forward transform of kc k1 columns, surface compliance u3_hat = (1 - nu) / (mu q) p_hat
-// (zero on mode 0 and on the Nyquist row), times the load scale for the pressure, inverse
-// transform.  Few columns per CTA (32-byte row segments): the plane stays in L2, and 512 points
-// in 16-column CTAs would leave most of the chip idle.
+// Columns: forward transform of kc k1 columns, surface compliance, times the load scale for the
+// pressure, inverse transform.  Few columns per CTA (32-byte row segments): the plane stays in L2,
+// and 512 points in 16-column CTAs would leave most of the chip idle.
 template <typename T, int N, bool SCALE>
 __global__ void __launch_bounds__(512) k_pkf_cols(const PkState* S, typename Cx<T>::t* __restrict__ plane,
-                                                  const typename Cx<T>::t* __restrict__ tw, int h1, int kc, T w1, T w2, T nu,
-                                                  T mu) {
+                                                  const T* __restrict__ green, const typename Cx<T>::t* __restrict__ tw,
+                                                  int h1, int kc) {
   typedef typename Cx<T>::t V;
   if (S->done) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int T8 = N / 8;
+  constexpr int T4 = N / 4;
   const int f = threadIdx.x % kc, t = threadIdx.x / kc;
-  const int k1 = blockIdx.x * kc + f;
-  const double s = SCALE ? S->s : 1.0;
-  V* col = plane + k1;
-  V v[1][8];
+  const size_t at = (size_t)blockIdx.x * kc + f;
+  V* col = plane + at;
+  V v[4];
+  const double scl = SCALE ? S->s : 1.0;
+  const float2 scl2 = S->s2;
+  T f0[4];
 #pragma unroll
-  for (int m = 0; m < 8; ++m) v[0][m] = col[(size_t)(t + m * T8) * h1];
-  struct Sm {
-    V* buf;
-    int kc, f;
-    __device__ __forceinline__ void put(int, int p, V x) const { buf[p * kc + f] = x; }
-    __device__ __forceinline__ V get(int, int p) const { return buf[p * kc + f]; }
-  } sm{reinterpret_cast<V*>(smraw), kc, f};
-  fft_ct<V, false, N, 1, 1>(v, t, sm, tw);
-  const T q1 = w1 * (T)k1;
-#pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int k2 = t + m * T8;
-    const T q2 = w2 * (T)(k2 < N / 2 ? k2 : k2 - N);
-    const T q = sqrt(q1 * q1 + q2 * q2);
-    const bool none = (k1 == 0 && k2 == 0) || k2 == N / 2;
-    T f0 = none ? (T)0 : ((T)1 - nu) / (mu * q);
-    if (SCALE) f0 = (T)(s * (double)f0);
-    v[0][m] = cscale(v[0][m], f0);
+  for (int m = 0; m < 4; ++m) {
+    v[m] = col[(size_t)(t + m * T4) * h1];
+    f0[m] = green[(size_t)(t + m * T4) * h1 + at];
   }
-  __syncthreads();  // the exchange area is reused by the inverse transform
-  fft_ct<V, true, N, 1, 1>(v, t, sm, tw);
+  const SurfColSm<V> sm{reinterpret_cast<V*>(smraw), kc, f};
+  fft4_ct<V, false, N, 1>(v, t, sm, tw);
 #pragma unroll
-  for (int m = 0; m < 8; ++m) col[(size_t)(t + m * T8) * h1] = v[0][m];
+  for (int m = 0; m < 4; ++m) v[m] = cscale(v[m], SCALE ? mul1(scl, scl2, f0[m]) : f0[m]);
+  fft4_ct<V, true, N, 1>(v, t, sm, tw);
+#pragma unroll
+  for (int m = 0; m < 4; ++m) col[(size_t)(t + m * T4) * h1] = v[m];
 }
 
 // Inverse rows of u or r (two rows per transform) with the elementwise step and sums that follow.
@@ -230,107 +347,117 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
     return;
   }
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int T8 = N / 8, H1 = N / 2, LD = SurfSm<V, N>::LD;
-  const int r = threadIdx.x / T8, tt = threadIdx.x % T8;
-  const int pair = blockIdx.x * (blockDim.x / T8) + r;
+  constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
+  const int r = threadIdx.x / T4, tt = threadIdx.x % T4;
+  const int pair = blockIdx.x * (blockDim.x / T4) + r;
   const bool live = pair < n2 / 2;
   T* p = static_cast<T*>(S->p);
   const T* h = static_cast<const T*>(S->h);
-  V v[1][8];
+  V v[4];
   const V* sa = surf + (size_t)(live ? 2 * pair : 0) * H1;
 #pragma unroll
-  for (int m = 0; m < 8; ++m) {
-    const int k = tt + m * T8;
+  for (int m = 0; m < 4; ++m) {
+    const int k = tt + m * T4;
     const int kk = k < H1 ? k : (k > H1 ? N - k : 0);
     V A = sa[kk], B = sa[H1 + kk];
     if (k > H1) { A = cconj(A); B = cconj(B); }
     if (k == H1) A = B = mk<V>(0, 0);
-    v[0][m] = cadd(A, cmuli(B));
+    v[m] = cadd(A, cmuli(B));
   }
-  SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
-  fft_ct<V, true, N, 1, 1>(v, tt, sm, tw);
+  const SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
+  fft4_ct<V, true, N, 1>(v, tt, sm, tw);
   const size_t i0 = (size_t)(live ? 2 * pair : 0) * N + tt;
-  if (MODE == INV_R) {
-    double sum[4] = {0, 0, 0, 0};
-    auto add = [&](size_t i, T x) {
+  const double scl = S->s, gbar = S->gbar;
+  const float2 scl2 = S->s2;
+  double sum[4] = {0, 0, 0, 0};
+  int nc = 0;
+  auto add = [&](size_t i, T x) {
+    if constexpr (MODE == INV_R) {
       if (p[i] > (T)0) {
-        const double ti = (double)t[i];
-        sum[0] += (double)x;
+        const double xi = (double)x, ti = (double)t[i];
+        sum[0] += xi;
         sum[1] += ti;
         sum[2] += (double)g[i] * ti;
-        sum[3] += (double)x * ti;
+        sum[3] += xi * ti;
       }
-    };
-    if (live) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        add(i0 + m * T8, v[0][m].x * scale);
-        add(i0 + m * T8 + N, v[0][m].y * scale);
-      }
-    }
-    if (grid_sum<4>(sum, part, cnt)) {
-      const double den = sum[3] - sum[0] / S->nIc * sum[1];
-      S->tau = den != 0 ? sum[2] / den : 0.0;
-    }
-  } else {
-    const double s = S->s;
-    double sum[3] = {0, 0, 0};
-    auto add = [&](size_t i, T x) {
+    } else {
       T pi = p[i];
-      if (MODE == INV_U) {
-        pi = (T)(s * (double)pi);
-        p[i] = pi;
-        sum[2] += fabs((double)pi - (double)pold[i]);
+      if constexpr (MODE == INV_U) {
+        const T po = pold[i];
+        if (pi != (T)0) {
+          pi = mul1(scl, scl2, pi);
+          p[i] = pi;
+        }
+        if (pi != po) sum[2] += fabs((double)pi - (double)po);
       }
       u[i] = x;
       if (pi > (T)0) {
-        sum[0] += (double)x - (double)h[i];
-        sum[1] += 1;
-      }
-    };
-    if (live) {
-#pragma unroll
-      for (int m = 0; m < 8; ++m) {
-        add(i0 + m * T8, v[0][m].x * scale);
-        add(i0 + m * T8 + N, v[0][m].y * scale);
+        const double d = MODE == INV_U ? (double)x - (double)h[i] - gbar : (double)x - (double)h[i];
+        sum[0] += d;
+        if (MODE == INV_U) sum[1] += d * d;
+        ++nc;
       }
     }
-    if (grid_sum<3>(sum, part, cnt)) {
-      int done = 0, bad = 0;
-      if (MODE == INV_U) {
-        S->err = S->dA * sum[2] / S->W;
-        S->it += 1;
-        if (S->err < S->tol || S->it >= S->max_it) done = 1;
-        if (!isfinite(S->err)) bad = 1;
-      }
-      S->nIc = sum[1];
-      if (!done && (!(sum[1] > 0) || !isfinite(sum[0]))) bad = 1;
-      else S->gbar = sum[0] / sum[1];
-      if (bad) S->bad = 1;
-      S->done = done | bad;
-      if (MODE == INV_U && use_cond) cudaGraphSetConditional(cond, (done | bad) ? 0u : 1u);
+  };
+  if (live) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+      add(i0 + m * T4, v[m].x * scale);
+      add(i0 + m * T4 + N, v[m].y * scale);
     }
   }
+  if (MODE != INV_R) sum[3] = (double)nc;
+  if (!grid_sum(sum, part, cnt)) return;
+  if (MODE == INV_R) {
+    // <g, t> / (<r, t> - rbar <t, 1>), rbar = sum r / nIc
+    const double den = sum[3] * S->nIc - sum[0] * sum[1];
+    const double tau = den != 0 ? sum[2] * S->nIc / den : 0.0;
+    S->tau = tau;
+    S->tau2 = pair_of(tau);
+    return;
+  }
+  int done = 0, bad = 0;
+  if (MODE == INV_U) {
+    const double err = sum[2] * S->dA_W;
+    S->err = err;
+    S->it += 1;
+    if (err < S->tol || S->it >= S->max_it) done = 1;
+    if (!isfinite(err)) bad = 1;
+  }
+  S->nIc = sum[3];
+  if (!done && (!(sum[3] > 0) || !isfinite(sum[0]))) {
+    bad = 1;
+  } else {
+    const double mean = sum[0] / sum[3], gb = (MODE == INV_U ? gbar : 0.0) + mean;
+    S->gbar = gb;
+    S->gbar2 = pair_of(gb);
+    if (MODE == INV_U) {
+      const double G = fmax(sum[1] - sum[0] * mean, 0.0), beta = S->delta * (G / S->G_old);
+      S->beta = beta;
+      S->beta2 = pair_of(beta);
+      S->G_old = G;
+    }
+  }
+  if (bad) S->bad = 1;
+  S->done = done | bad;
+  if (MODE == INV_U && use_cond) cudaGraphSetConditional(cond, (done | bad) ? 0u : 1u);
 }
 
-// g = u - h - gbar; sum over the contact of g^2 -> beta
+// G = sum over the contact of g^2, g = u - h - gbar, of the first iteration
 template <typename T>
-__global__ void __launch_bounds__(256) k_pkf_gap(PkState* S, const T* __restrict__ u, T* __restrict__ g, size_t n,
-                                                 double* part, unsigned* cnt) {
+__global__ void __launch_bounds__(256) k_pkf_gap(PkState* S, const T* __restrict__ u, size_t n, double* part, unsigned* cnt) {
   if (S->done) return;
   const double gbar = S->gbar;
   const T* h = static_cast<const T*>(S->h);
   const T* p = static_cast<const T*>(S->p);
-  double v[1] = {0};
+  double v[4] = {0, 0, 0, 0};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const T gi = (T)((double)u[i] - (double)h[i] - gbar);
-    g[i] = gi;
-    if (p[i] > (T)0) v[0] += (double)gi * (double)gi;
+    if (p[i] > (T)0) {
+      const double gi = (double)u[i] - (double)h[i] - gbar;
+      v[0] += gi * gi;
+    }
   }
-  if (grid_sum<1>(v, part, cnt)) {
-    S->beta = S->delta * (v[0] / S->G_old);
-    S->G_old = v[0];
-  }
+  if (grid_sum(v, part, cnt)) S->G_old = v[0];
 }
 
 // CTA of a row pass: about one transform pair per CTA and SM, whole warps
@@ -340,11 +467,11 @@ struct RowCfg {
 };
 template <typename T, int N> RowCfg row_cfg(int n2) {
   typedef typename Cx<T>::t V;
-  const int pairs = n2 / 2, T8 = N / 8;
+  const int pairs = n2 / 2, T4 = N / 4;
   int slots = 1;
-  while (slots * 2 * 128 <= pairs && slots * 2 * T8 <= 512) slots *= 2;
-  const int threads = std::max(32, slots * T8);
-  slots = threads / T8;
+  while (slots * 2 * 128 <= pairs && slots * 2 * T4 <= 512) slots *= 2;
+  const int threads = std::max(32, slots * T4);
+  slots = threads / T4;
   return RowCfg{(pairs + slots - 1) / slots, threads, (size_t)slots * SurfSm<V, N>::LD * sizeof(V)};
 }
 
@@ -358,8 +485,8 @@ template <typename T, int N, int MODE> void rows_fwd(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
   const RowCfg r = row_cfg<T, N>(a.n2);
   row_smem_cap(k_pkf_rows_fwd<T, N, MODE>);
-  k_pkf_rows_fwd<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(a.S, (const T*)a.g, (T*)a.t, (T*)a.pold, (V*)a.surf,
-                                                                   (const V*)a.tw1, a.n2, a.part, a.cnt);
+  k_pkf_rows_fwd<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(a.S, (const T*)a.u, (T*)a.g, (T*)a.t, (T*)a.pold,
+                                                                   (V*)a.surf, (const V*)a.tw1, a.n2, a.part, a.cnt);
 }
 template <typename T, int N, int MODE> void rows_inv(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
@@ -373,10 +500,10 @@ template <typename T, int N, bool SCALE> void cols(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
   int kc = (int)(32 / sizeof(V));
   if (kc > a.h1) kc = a.h1;
-  const double two_pi = 6.283185307179586476925;
+  while (kc * (N / 4) > 512) kc >>= 1;
   smem_cap(k_pkf_cols<T, N, SCALE>);
-  k_pkf_cols<T, N, SCALE><<<a.h1 / kc, kc * (N / 8), (size_t)kc * N * sizeof(V), a.stream>>>(
-      a.S, (V*)a.surf, (const V*)a.tw2, a.h1, kc, (T)(two_pi / a.L1), (T)(two_pi / a.L2), (T)a.nu, (T)a.mu);
+  k_pkf_cols<T, N, SCALE><<<a.h1 / kc, kc * (N / 4), (size_t)kc * N * sizeof(V), a.stream>>>(
+      a.S, (V*)a.surf, (const T*)a.green, (const V*)a.tw2, a.h1, kc);
 }
 
 #define PKF_SIZES(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024)
@@ -395,7 +522,7 @@ template <typename T, bool SCALE> void cols_any(const PkfArgs& a) {
   PKF_SIZES(CASE)
 #undef CASE
 }
-inline int flat_grid(size_t n) { return (int)std::min<size_t>(std::max<size_t>((n + 1023) / 1024, 1), 152); }
+inline int flat_grid(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 256); }
 
 }  // namespace
 
@@ -404,16 +531,18 @@ bool pkf_available(const fvim_ctx* c) { return !c->gen && c->n1 >= 16 && c->n2 >
 template <typename T> int pkf_begin(const PkfArgs& a, const PkState& init) {
   const size_t n = (size_t)a.n1 * a.n2;
   k_pkf_begin<T><<<flat_grid(n), 256, 0, a.stream>>>(a.S, (const T*)init.p, n, init, a.part, a.cnt);
+  const double two_pi = 6.283185307179586476925;
+  k_pkf_green<T><<<(a.h1 * a.n2 + 255) / 256, 256, 0, a.stream>>>((T*)a.green, a.h1, a.n2, (T)(two_pi / a.L1),
+                                                                  (T)(two_pi / a.L2), (T)a.nu, (T)a.mu);
   rows_fwd_any<T, FWD_INIT>(a);
   cols_any<T, false>(a);
   rows_inv_any<T, INV_U0>(a);
+  k_pkf_gap<T><<<flat_grid(n), 256, 0, a.stream>>>(a.S, (const T*)a.u, n, a.part, a.cnt);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
 }
 
 template <typename T> int pkf_iteration(const PkfArgs& a) {
-  const size_t n = (size_t)a.n1 * a.n2;
-  k_pkf_gap<T><<<flat_grid(n), 256, 0, a.stream>>>(a.S, (const T*)a.u, (T*)a.g, n, a.part, a.cnt);
   rows_fwd_any<T, FWD_T>(a);
   cols_any<T, false>(a);
   rows_inv_any<T, INV_R>(a);

@@ -695,7 +695,8 @@ template <typename T> bool launch_rows_inv6_ct(const fvim_ctx* c, T* out, T nq_s
 struct PkState {
   double nIc, gbar, G_old, beta, delta, tau, s, err;  // scalars of the iteration
   double start, unif;                                  // scale of the initial pressure (0: uniform), uniform pressure
-  double W, dA, tol;
+  double W, dA, dA_W, tol;                             // dA_W = dA / W
+  float2 gbar2, beta2, tau2, s2;                       // the scalars of the elementwise steps as float pairs
   const void* h;
   void* p;
   int done, it, bad, max_it;
@@ -707,6 +708,7 @@ struct PkfArgs {
   cudaStream_t stream;
   PkState* S;
   void *u, *g, *t, *pold;  // surface work arrays [n2][n1]
+  void* green;             // surface compliance [n2][h1]
   void* surf;              // half spectrum [n2][h1]
   const void *tw1, *tw2;
   double* part;            // block partials of the sums

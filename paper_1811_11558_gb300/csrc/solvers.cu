@@ -699,6 +699,7 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
   a.g = c->sv[S_G];
   a.t = c->sv[S_T];
   a.pold = c->sv[S_POLD];
+  a.green = c->sv[S_R];
   a.surf = c->surf;
   a.tw1 = c->tw1;
   a.tw2 = c->tw2;
@@ -708,10 +709,12 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
   memset(&s0, 0, sizeof(s0));
   s0.G_old = 1.0;
   s0.s = 1.0;
+  s0.s2 = make_float2(1.f, 0.f);
   s0.err = INFINITY;
   s0.unif = W / (c->L1 * c->L2);
   s0.W = W;
   s0.dA = c->L1 * c->L2 / (double)n;
+  s0.dA_W = s0.dA / W;
   s0.tol = o->cg_tol;
   s0.h = h;
   s0.p = p;
