@@ -10,129 +10,259 @@
 // columns are written as zeros.  There is no side array: every coefficient is in the
 // spectrum.  The full spectrum of a real row follows from X(N1 - k) = conj X(k).
 //
-// These kernels serve grids up to a few hundred points per side, where O(N^2) per line is a
-// small cost next to the depth operator; power-of-two grids take the FFT kernels.
+// Direct evaluation in folded form: with a(n) + a(N - n) and a(n) - a(N - n), n = 1 .. (N-1)/2,
+//   X(k), X(N - k) = a(0) + C(k) -+ i S(k),  C = sum (a(n) + a(N - n)) cos,  S = sum (a(n) - a(N - n)) sin
+// (plus (-1)^k a(N/2) on an even side), and likewise for the inverse rows: half the terms, and two
+// outputs from each column sum.  The inner loops keep one twiddle for several rows or columns per
+// thread (eight rows, four complex columns), read as broadcast vectors: what bounded the plain form
+// was two shared-memory reads per multiply-add.  81 x 81 x 32 FP32, us: rows 39 -> 14, columns 33 ->
+// 18, inverse rows 37 -> 16 (event-bracketed launches); apply 143 -> 64.
 #include "fvim_internal.cuh"
 
 namespace {
 
-constexpr int RB = 4;     // rows per CTA (row kernels)
+constexpr int RB = 32;    // rows per CTA (row kernels)
+constexpr int RT = 8;     // rows per thread
 constexpr int CT = 16;    // columns per CTA (column kernel)
+constexpr int CC = 4;     // columns per thread
+
+// RT consecutive values of T at a 16-byte boundary
+template <typename T> __device__ __forceinline__ void ld_rows(T (&v)[RT], const T* p) {
+  if constexpr (sizeof(T) == 4) {
+#pragma unroll
+    for (int q = 0; q < RT; q += 4) {
+      const float4 a = *reinterpret_cast<const float4*>(p + q);
+      v[q] = a.x; v[q + 1] = a.y; v[q + 2] = a.z; v[q + 3] = a.w;
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < RT; q += 2) {
+      const double2 a = *reinterpret_cast<const double2*>(p + q);
+      v[q] = a.x; v[q + 1] = a.y;
+    }
+  }
+}
+// CC complex columns at a 16-byte boundary
+template <typename V> __device__ __forceinline__ void ld_cols(V (&v)[CC], const V* p) {
+  if constexpr (sizeof(V) == 8) {
+#pragma unroll
+    for (int q = 0; q < CC; q += 2) {
+      const float4 a = *reinterpret_cast<const float4*>(p + q);
+      v[q] = mk<V>(a.x, a.y);
+      v[q + 1] = mk<V>(a.z, a.w);
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < CC; ++q) v[q] = p[q];
+  }
+}
+// row stride of the folded tables: RB values and 16 bytes (the fill walks them along n)
+template <typename T> struct RowLd {
+  static constexpr int v = RB + 16 / (int)sizeof(T);
+};
 
 // forward row DFTs of real rows: src [rows][n1] -> dst [rows][ldh] (k1 < hs, zeros above)
 template <typename T>
-__global__ void __launch_bounds__(128) k_dft_rows_fwd(const T* __restrict__ src, typename Cx<T>::t* __restrict__ dst,
+__global__ void __launch_bounds__(256) k_dft_rows_fwd(const T* __restrict__ src, typename Cx<T>::t* __restrict__ dst,
                                                       const typename Cx<T>::t* __restrict__ tw, int n1, int hs,
                                                       int ldh, size_t rows) {
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  V* w = reinterpret_cast<V*>(smraw);                 // [n1] twiddles
-  T* x = reinterpret_cast<T*>(w + n1);                // [RB][n1]
+  constexpr int LD = RowLd<T>::v;
+  const int H = n1 / 2, J = (n1 - 1) / 2;             // folded terms n = 1 .. J
+  T* P = reinterpret_cast<T*>(smraw);                 // [H + 1][LD] sums; row 0: a(0), row H of an even side: a(N/2)
+  T* Q = P + (size_t)(H + 1) * LD;                    // [H + 1][LD] differences
+  V* w = reinterpret_cast<V*>(Q + (size_t)(H + 1) * LD);  // [n1] twiddles
   const size_t r0 = (size_t)blockIdx.x * RB;
   const int nr = (int)((rows - r0) < (size_t)RB ? rows - r0 : RB);
   for (int i = threadIdx.x; i < n1; i += blockDim.x) w[i] = tw[i];
-  for (int i = threadIdx.x; i < nr * n1; i += blockDim.x) x[i] = src[r0 * n1 + i];
+  for (int i = threadIdx.x; i < RB * (H + 1); i += blockDim.x) {
+    const int r = i / (H + 1), n = i - r * (H + 1);
+    T a = 0, b = 0;
+    if (r < nr) {
+      a = src[(r0 + r) * n1 + n];
+      if (n > 0 && n <= J) b = src[(r0 + r) * n1 + n1 - n];
+    }
+    P[n * LD + r] = a + b;
+    Q[n * LD + r] = a - b;
+  }
   __syncthreads();
-  for (int i = threadIdx.x; i < nr * ldh; i += blockDim.x) {
-    const int r = i / ldh, k = i - r * ldh;
-    V acc = mk<V>(0, 0);
+  for (int i = threadIdx.x; i < (RB / RT) * ldh; i += blockDim.x) {
+    const int g = i / ldh, k = i - g * ldh;
+    T c[RT], s[RT];
+#pragma unroll
+    for (int q = 0; q < RT; ++q) c[q] = s[q] = (T)0;
     if (k < hs) {
-      const T* xr = x + r * n1;
+      ld_rows(c, P + g * RT);
+      const T* pp = P + g * RT + LD;
+      const T* qq = Q + g * RT + LD;
       int j = 0;  // (k n) mod n1
-      for (int n = 0; n < n1; ++n) {
-        acc = caxpy(acc, xr[n], w[j]);
+      for (int n = 1; n <= J; ++n, pp += LD, qq += LD) {
         j += k;
         if (j >= n1) j -= n1;
+        const V e = w[j];
+        T a[RT], b[RT];
+        ld_rows(a, pp);
+        ld_rows(b, qq);
+#pragma unroll
+        for (int q = 0; q < RT; ++q) {
+          c[q] += e.x * a[q];
+          s[q] += e.y * b[q];
+        }
+      }
+      if (J < H) {
+        T a[RT];
+        ld_rows(a, pp);
+#pragma unroll
+        for (int q = 0; q < RT; ++q) c[q] += (k & 1) ? -a[q] : a[q];
       }
     }
-    dst[(r0 + r) * ldh + k] = acc;
+#pragma unroll
+    for (int q = 0; q < RT; ++q)
+      if (g * RT + q < nr) dst[(r0 + g * RT + q) * ldh + k] = mk<V>(c[q], s[q]);
   }
 }
 
-// column DFTs along x2, in place: planes [nplanes][n2][ldh], CT columns per CTA (the tile and
-// its transform both in shared memory)
+// column DFTs along x2, in place: planes [nplanes][n2][ldh], CT columns per CTA
 template <typename T, bool INV>
 __global__ void __launch_bounds__(256) k_dft_cols(typename Cx<T>::t* __restrict__ spec,
                                                   const typename Cx<T>::t* __restrict__ tw, int n2, int ldh) {
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  V* w = reinterpret_cast<V*>(smraw);       // [n2] twiddles
-  V* a = w + n2;                            // [n2][CT] the CTA's columns
-  V* b = a + (size_t)n2 * CT;               // [n2][CT] their transforms
-  V* P = spec + (size_t)blockIdx.y * n2 * ldh + (size_t)blockIdx.x * CT;
+  const int H = n2 / 2, J = (n2 - 1) / 2;
+  V* P = reinterpret_cast<V*>(smraw);       // [H + 1][CT] sums; row 0: a(0), row H of an even side: a(N/2)
+  V* Q = P + (size_t)(H + 1) * CT;          // [H + 1][CT] differences
+  V* w = Q + (size_t)(H + 1) * CT;          // [n2] twiddles
+  V* A = spec + (size_t)blockIdx.y * n2 * ldh + (size_t)blockIdx.x * CT;
   for (int i = threadIdx.x; i < n2; i += blockDim.x) {
     V t = tw[i];
     if (INV) t.y = -t.y;
     w[i] = t;
   }
-  for (int i = threadIdx.x; i < n2 * CT; i += blockDim.x) {
-    const int row = i / CT, c = i - row * CT;
-    a[i] = P[(size_t)row * ldh + c];
+  for (int i = threadIdx.x; i < (H + 1) * CT; i += blockDim.x) {
+    const int n = i / CT, c = i - n * CT;
+    const V a = A[(size_t)n * ldh + c];
+    V b = mk<V>(0, 0);
+    if (n > 0 && n <= J) b = A[(size_t)(n2 - n) * ldh + c];
+    P[i] = cadd(a, b);
+    Q[i] = csub(a, b);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n2 * CT; i += blockDim.x) {
-    const int k = i / CT, c = i - k * CT;
+  for (int i = threadIdx.x; i < (CT / CC) * (H + 1); i += blockDim.x) {
+    const int g = i / (H + 1), k = i - g * (H + 1);
+    V c[CC], s[CC];
+#pragma unroll
+    for (int q = 0; q < CC; ++q) {
+      c[q] = P[g * CC + q];
+      s[q] = mk<V>(0, 0);
+    }
+    const V* pp = P + g * CC + CT;
+    const V* qq = Q + g * CC + CT;
     int j = 0;  // (k n) mod n2
-    V acc = mk<V>(0, 0);
-    for (int n = 0; n < n2; ++n) {
-      acc = cadd(acc, cmul(a[n * CT + c], w[j]));
+    for (int n = 1; n <= J; ++n, pp += CT, qq += CT) {
       j += k;
       if (j >= n2) j -= n2;
+      const V e = w[j];
+      V a[CC], b[CC];
+      ld_cols(a, pp);
+      ld_cols(b, qq);
+#pragma unroll
+      for (int q = 0; q < CC; ++q) {
+        c[q] = caxpy(c[q], e.x, a[q]);
+        s[q] = caxpy(s[q], e.y, b[q]);
+      }
     }
-    b[i] = acc;
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < n2 * CT; i += blockDim.x) {
-    const int row = i / CT, c = i - row * CT;
-    P[(size_t)row * ldh + c] = b[i];
+    if (J < H) {
+#pragma unroll
+      for (int q = 0; q < CC; ++q) c[q] = (k & 1) ? csub(c[q], pp[q]) : cadd(c[q], pp[q]);
+    }
+    V* o = A + (size_t)k * ldh + g * CC;
+    V* om = A + (size_t)(n2 - k) * ldh + g * CC;
+    const bool mirror = k > 0 && 2 * k != n2;
+#pragma unroll
+    for (int q = 0; q < CC; ++q) {
+      o[q] = mk<V>(c[q].x - s[q].y, c[q].y + s[q].x);                 // c + i s, e = cos -+ i sin
+      if (mirror) om[q] = mk<V>(c[q].x + s[q].y, c[q].y - s[q].x);    // c - i s
+    }
   }
 }
 
 // inverse row DFTs to real rows: src [rows][ldh] (k1 < hs) -> dst [rows][n1], times scale;
-// x(n) = X(0) + 2 sum_{0 < k < n1/2} Re(X(k) e^{2 pi i k n / n1}) + (n1 even) X(n1/2) (-1)^n
+// x(n), x(N - n) = X(0) + 2 sum_{0 < k < n1/2} (Re X(k) cos -+ Im X(k) sin) + (n1 even) X(n1/2) (-1)^n
 template <typename T>
-__global__ void __launch_bounds__(128) k_dft_rows_inv(const typename Cx<T>::t* __restrict__ src, T* __restrict__ dst,
+__global__ void __launch_bounds__(256) k_dft_rows_inv(const typename Cx<T>::t* __restrict__ src, T* __restrict__ dst,
                                                       const typename Cx<T>::t* __restrict__ tw, int n1, int hs,
                                                       int ldh, size_t rows, T scale) {
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  V* w = reinterpret_cast<V*>(smraw);   // [n1]
-  V* X = w + n1;                        // [RB][hs]
+  constexpr int LD = RowLd<T>::v;
+  const int H = n1 / 2, J = (n1 - 1) / 2;
+  T* P = reinterpret_cast<T*>(smraw);                 // [H + 1][LD] real parts (H = hs - 1)
+  T* Q = P + (size_t)(H + 1) * LD;                    // [H + 1][LD] imaginary parts
+  V* w = reinterpret_cast<V*>(Q + (size_t)(H + 1) * LD);  // [n1]
   const size_t r0 = (size_t)blockIdx.x * RB;
   const int nr = (int)((rows - r0) < (size_t)RB ? rows - r0 : RB);
   for (int i = threadIdx.x; i < n1; i += blockDim.x) w[i] = tw[i];
-  for (int i = threadIdx.x; i < nr * hs; i += blockDim.x) {
+  for (int i = threadIdx.x; i < RB * hs; i += blockDim.x) {
     const int r = i / hs, k = i - r * hs;
-    X[i] = src[(r0 + r) * ldh + k];
+    V x = mk<V>(0, 0);
+    if (r < nr) x = src[(r0 + r) * ldh + k];
+    P[k * LD + r] = x.x;
+    Q[k * LD + r] = x.y;
   }
   __syncthreads();
-  const bool even = (n1 & 1) == 0;
-  const int kmax = even ? n1 / 2 - 1 : (n1 - 1) / 2;  // last k with a conjugate partner
-  for (int i = threadIdx.x; i < nr * n1; i += blockDim.x) {
-    const int r = i / n1, n = i - r * n1;
-    const V* Xr = X + r * hs;
-    T acc = Xr[0].x;
-    int j = n;  // (k n) mod n1 for k = 1
-    T s = 0;
-    for (int k = 1; k <= kmax; ++k) {
-      // Re(X e^{+i theta}) with tw = e^{-i theta}: X.x tw.x + X.y tw.y
-      s += Xr[k].x * w[j].x + Xr[k].y * w[j].y;
+  for (int i = threadIdx.x; i < (RB / RT) * (H + 1); i += blockDim.x) {
+    const int g = i / (H + 1), n = i - g * (H + 1);
+    T c[RT], s[RT];
+#pragma unroll
+    for (int q = 0; q < RT; ++q) c[q] = s[q] = (T)0;
+    const T* pp = P + g * RT + LD;
+    const T* qq = Q + g * RT + LD;
+    int j = 0;  // (k n) mod n1
+    for (int k = 1; k <= J; ++k, pp += LD, qq += LD) {
       j += n;
       if (j >= n1) j -= n1;
+      const V e = w[j];  // cos - i sin
+      T a[RT], b[RT];
+      ld_rows(a, pp);
+      ld_rows(b, qq);
+#pragma unroll
+      for (int q = 0; q < RT; ++q) {
+        c[q] += e.x * a[q];
+        s[q] += e.y * b[q];
+      }
     }
-    acc += 2 * s;
-    if (even) acc += (n & 1) ? -Xr[n1 / 2].x : Xr[n1 / 2].x;
-    dst[(r0 + r) * n1 + n] = acc * scale;
+    T x0[RT], xn[RT];
+    ld_rows(x0, P + g * RT);
+    if (J < H) {
+      ld_rows(xn, pp);
+#pragma unroll
+      for (int q = 0; q < RT; ++q) x0[q] += (n & 1) ? -xn[q] : xn[q];
+    }
+    const bool mirror = n > 0 && 2 * n != n1;
+#pragma unroll
+    for (int q = 0; q < RT; ++q) {
+      if (g * RT + q >= nr) continue;
+      T* o = dst + (r0 + g * RT + q) * n1;
+      o[n] = (x0[q] + 2 * (c[q] + s[q])) * scale;
+      if (mirror) o[n1 - n] = (x0[q] + 2 * (c[q] - s[q])) * scale;
+    }
   }
+}
+
+// threads of a CTA with `items` work items: whole warps, at most 256, the passes evenly filled
+inline int dft_threads(int items) {
+  const int passes = (items + 255) / 256;
+  return ((items + passes - 1) / passes + 31) / 32 * 32;
 }
 
 }  // namespace
 
 template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, void* dst, size_t rows) {
   typedef typename Cx<T>::t V;
-  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)RB * c->n1 * sizeof(T);
+  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
   smem_cap(k_dft_rows_fwd<T>);
-  k_dft_rows_fwd<T><<<(unsigned)((rows + RB - 1) / RB), 128, smem, c->stream>>>(src, (V*)dst, (const V*)c->tw1, c->n1,
+  k_dft_rows_fwd<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * c->h1), smem, c->stream>>>(src, (V*)dst, (const V*)c->tw1, c->n1,
                                                                                 c->hs, c->h1, rows);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -140,14 +270,15 @@ template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, v
 
 template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void* planes, int nplanes) {
   typedef typename Cx<T>::t V;
-  const size_t smem = (size_t)c->n2 * sizeof(V) + (size_t)2 * c->n2 * CT * sizeof(V);
+  const size_t smem = (size_t)c->n2 * sizeof(V) + (size_t)2 * (c->n2 / 2 + 1) * CT * sizeof(V);
+  const int threads = dft_threads(CT / CC * (c->n2 / 2 + 1));
   dim3 grid(c->h1 / CT, nplanes);
   if (inverse) {
     smem_cap(k_dft_cols<T, true>);
-    k_dft_cols<T, true><<<grid, 256, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
+    k_dft_cols<T, true><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
   } else {
     smem_cap(k_dft_cols<T, false>);
-    k_dft_cols<T, false><<<grid, 256, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
+    k_dft_cols<T, false><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
   }
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -155,9 +286,9 @@ template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void*
 
 template <typename T> int launch_dft_rows_inv(const fvim_ctx* c, const void* src, T* dst, size_t rows, T scale) {
   typedef typename Cx<T>::t V;
-  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)RB * c->hs * sizeof(V);
+  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
   smem_cap(k_dft_rows_inv<T>);
-  k_dft_rows_inv<T><<<(unsigned)((rows + RB - 1) / RB), 128, smem, c->stream>>>((const V*)src, dst, (const V*)c->tw1,
+  k_dft_rows_inv<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * (c->n1 / 2 + 1)), smem, c->stream>>>((const V*)src, dst, (const V*)c->tw1,
                                                                                 c->n1, c->hs, c->h1, rows, scale);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
