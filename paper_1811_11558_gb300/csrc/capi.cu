@@ -389,6 +389,26 @@ template <typename T> int apply_boussinesq_t(fvim_ctx* c, const T* p, T* u3, T* 
   }
   if ((rc = timed(c, PROF_ROWS_FWD1, nk, [&] { return launch_rows_fwd1<T>(c, p); }))) return rc;
   if ((rc = timed(c, PROF_COLS_FWD, nk, [&] { return launch_cols<T>(c, false, c->surf, 1); }))) return rc;
+  if (vol && sizeof(T) == 4 && !use_fft2_fused(c) && !use_fft2_cluster(c)) {
+    // volume field evaluated in the inverse column pass
+    bool fused = false;
+    if ((rc = timed(c, PROF_COLS_INV, nk, [&] {
+           fused = launch_bous_cols(c, kind);
+           FVIM_CUDA_CHECK_LAUNCH();
+           return FVIM_OK;
+         })))
+      return rc;
+    if (fused) {
+      if ((rc = timed(c, PROF_ROWS_INV6, nk, [&] { return launch_rows_inv6<T>(c, vol, (T)0, 0, c->nz); }))) return rc;
+      vol = nullptr;
+      if (!u3) {
+        c->last_kernels = nk;
+        return FVIM_OK;
+      }
+    } else {
+      --nk;
+    }
+  }
   if ((rc = timed(c, PROF_BOUSSINESQ, nk,
                   [&] { return launch_boussinesq<T>(c, kind, vol != nullptr, u3 != nullptr); })))
     return rc;

@@ -121,68 +121,6 @@ __device__ __forceinline__ float gap1(float u, float h, double, float2 c) {
 }
 __device__ __forceinline__ double gap1(double u, double h, double c, float2) { return u - h - c; }
 
-// ---- transforms of four values per thread -------------------------------------------------
-// Stockham stages of radix 4, the first of radix 2 where log2 N is odd; thread t of N / 4 holds the
-// values t + m N / 4 before and after.  Exchange layout by the caller (Sm), CTA barriers.
-template <int N> struct OddLog2 {
-  static constexpr bool v = (N & 0x55555555) == 0;
-};
-template <typename V, bool INV, int N, int NS, class Sm>
-__device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V* __restrict__ tw) {
-  constexpr int T4 = N / 4, R = (NS == 1 && OddLog2<N>::v) ? 2 : 4;
-  int pos[4];
-  if constexpr (R == 2) {
-#pragma unroll
-    for (int m = 0; m < 2; ++m) {
-      const V a = v[m], c = v[m + 2];
-      v[m] = cadd(a, c);
-      v[m + 2] = csub(a, c);
-      pos[m] = 2 * (t + m * T4);
-      pos[m + 2] = pos[m] + 1;
-    }
-  } else {
-    const int k = t & (NS - 1);
-    if constexpr (NS > 1) {
-      constexpr int step = N / (NS * 4);
-      const V w1 = twiddle<V, INV>(tw, k * step), w2 = twiddle<V, INV>(tw, 2 * k * step);
-      bf2(v[0], v[2], w2);
-      bf2(v[1], v[3], w2);
-      bf2(v[0], v[1], w1);
-      bf2(v[2], v[3], quarter<V, INV>(w1));
-      const V x = v[1];
-      v[1] = v[2];
-      v[2] = x;
-    } else {
-      dft4<V, INV>(v);
-    }
-    const int base = (t / NS) * NS * 4 + k;
-#pragma unroll
-    for (int r = 0; r < 4; ++r) pos[r] = base + r * NS;
-  }
-  if constexpr (NS * R < N) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) sm.put(pos[m], v[m]);
-    __syncthreads();
-#pragma unroll
-    for (int m = 0; m < 4; ++m) v[m] = sm.get(t + m * T4);
-    __syncthreads();
-    fft4_ct<V, INV, N, NS * R>(v, t, sm, tw);
-  }
-}
-// rows: one pad slot every 8 entries
-template <typename V, int N> struct SurfSm {
-  static constexpr int LD = N + N / 8;
-  V* buf;
-  __device__ __forceinline__ void put(int p, V x) const { buf[p + (p >> 3)] = x; }
-  __device__ __forceinline__ V get(int p) const { return buf[p + (p >> 3)]; }
-};
-template <typename V> struct SurfColSm {
-  V* buf;
-  int kc, f;
-  __device__ __forceinline__ void put(int p, V x) const { buf[p * kc + f] = x; }
-  __device__ __forceinline__ V get(int p) const { return buf[p * kc + f]; }
-};
-
 // state of a new solve, with the scale of the initial pressure from its sum (a guess without load
 // is replaced by the uniform pressure)
 template <typename T>
@@ -432,7 +370,8 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
     S->gbar = gb;
     S->gbar2 = pair_of(gb);
     if (MODE == INV_U) {
-      const double G = fmax(sum[1] - sum[0] * mean, 0.0), beta = S->delta * (G / S->G_old);
+      // (a gap that vanishes to the last bit restarts the direction)
+      const double G = fmax(sum[1] - sum[0] * mean, 0.0), beta = S->G_old > 0 ? S->delta * (G / S->G_old) : 0.0;
       S->beta = beta;
       S->beta2 = pair_of(beta);
       S->G_old = G;
@@ -460,38 +399,17 @@ __global__ void __launch_bounds__(256) k_pkf_gap(PkState* S, const T* __restrict
   if (grid_sum(v, part, cnt)) S->G_old = v[0];
 }
 
-// CTA of a row pass: about one transform pair per CTA and SM, whole warps
-struct RowCfg {
-  int grid, threads;
-  size_t smem;
-};
-template <typename T, int N> RowCfg row_cfg(int n2) {
-  typedef typename Cx<T>::t V;
-  const int pairs = n2 / 2, T4 = N / 4;
-  int slots = 1;
-  while (slots * 2 * 128 <= pairs && slots * 2 * T4 <= 512) slots *= 2;
-  const int threads = std::max(32, slots * T4);
-  slots = threads / T4;
-  return RowCfg{(pairs + slots - 1) / slots, threads, (size_t)slots * SurfSm<V, N>::LD * sizeof(V)};
-}
-
-// dynamic shared memory cap of the row kernels (at most four FP64 transforms of 1024 points; they
-// hold static shared memory too, so not the whole opt-in maximum); the same value on every call
-template <typename K> void row_smem_cap(K kern) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-}
-
 template <typename T, int N, int MODE> void rows_fwd(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
-  const RowCfg r = row_cfg<T, N>(a.n2);
-  row_smem_cap(k_pkf_rows_fwd<T, N, MODE>);
+  const SurfRowCfg r = surf_row_cfg<T, N>(a.n2);
+  surf_row_smem_cap(k_pkf_rows_fwd<T, N, MODE>);
   k_pkf_rows_fwd<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(a.S, (const T*)a.u, (T*)a.g, (T*)a.t, (T*)a.pold,
                                                                    (V*)a.surf, (const V*)a.tw1, a.n2, a.part, a.cnt);
 }
 template <typename T, int N, int MODE> void rows_inv(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
-  const RowCfg r = row_cfg<T, N>(a.n2);
-  row_smem_cap(k_pkf_rows_inv<T, N, MODE>);
+  const SurfRowCfg r = surf_row_cfg<T, N>(a.n2);
+  surf_row_smem_cap(k_pkf_rows_inv<T, N, MODE>);
   k_pkf_rows_inv<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(
       a.S, (const T*)a.g, (const T*)a.t, (const T*)a.pold, (T*)a.u, (const V*)a.surf, (const V*)a.tw1, a.n2,
       (T)(1.0 / ((double)N * (double)a.n2)), a.part, a.cnt, a.cond, a.use_cond);

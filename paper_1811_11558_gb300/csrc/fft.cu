@@ -491,6 +491,10 @@ template <typename T> int launch_rows_fwd6(const fvim_ctx* c, const T* eps_p, in
 template <typename T> int launch_rows_fwd1(const fvim_ctx* c, const T* f) {
   typedef typename Cx<T>::t V;
   const int n1 = c->n1, n2 = c->n2;
+  if (launch_surf_rows_fwd<T>(c, f)) {
+    FVIM_CUDA_CHECK_LAUNCH();
+    return FVIM_OK;
+  }
   int maxi, threads;
   if (!fft_shape<T>(1, n1, maxi, threads)) return FVIM_ERR_UNSUPPORTED;
   const size_t smem = (size_t)n1 * sizeof(V);
@@ -505,7 +509,8 @@ template <typename T> int launch_rows_fwd1(const fvim_ctx* c, const T* f) {
 template <typename T> int launch_cols(const fvim_ctx* c, bool inverse, void* planes, int nplanes, const int* zr) {
   typedef typename Cx<T>::t V;
   const int n2 = c->n2, h1 = c->h1;
-  if (launch_cols_ct<T>(c, inverse, planes, nplanes, zr)) {
+  if ((nplanes == 1 && planes == c->surf && launch_surf_cols<T>(c, inverse)) ||
+      launch_cols_ct<T>(c, inverse, planes, nplanes, zr)) {
     FVIM_CUDA_CHECK_LAUNCH();
     return FVIM_OK;
   }
@@ -595,10 +600,14 @@ template <typename T> int launch_rows_inv6(const fvim_ctx* c, T* out, T nq_scale
 template <typename T> int launch_rows_inv1(const fvim_ctx* c, T* f) {
   typedef typename Cx<T>::t V;
   const int n1 = c->n1, n2 = c->n2;
+  const T scale = (T)(1.0 / ((double)n1 * (double)n2));
+  if (launch_surf_rows_inv<T>(c, f, scale)) {
+    FVIM_CUDA_CHECK_LAUNCH();
+    return FVIM_OK;
+  }
   int maxi, threads;
   if (!fft_shape<T>(1, n1, maxi, threads)) return FVIM_ERR_UNSUPPORTED;
   const size_t smem = (size_t)n1 * sizeof(V);
-  const T scale = (T)(1.0 / ((double)n1 * (double)n2));
   if (maxi == 2)
     k_rows_inv1<T, 2><<<n2 / 2, threads, smem, c->stream>>>((const V*)c->surf, (const T*)c->surf_nq, f,
                                                             (const V*)c->tw1, n1, n2, (T)0, scale);

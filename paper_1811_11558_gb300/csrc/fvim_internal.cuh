@@ -487,6 +487,93 @@ __device__ __forceinline__ void fft_ct(V (&v)[NF][8], int t, const Sm& sm, const
 }
 
 // ---------------------------------------------------------------------------
+// Transforms of four values per thread (surface kernels: more threads with less work each)
+// ---------------------------------------------------------------------------
+// Stockham stages of radix 4, the first of radix 2 where log2 N is odd; thread t of N / 4 holds the
+// values t + m N / 4 before and after.  Exchange layout by the caller (Sm), CTA barriers.
+template <int N> struct OddLog2 {
+  static constexpr bool v = (N & 0x55555555) == 0;
+};
+template <typename V, bool INV, int N, int NS, class Sm>
+__device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V* __restrict__ tw) {
+  constexpr int T4 = N / 4, R = (NS == 1 && OddLog2<N>::v) ? 2 : 4;
+  int pos[4];
+  if constexpr (R == 2) {
+#pragma unroll
+    for (int m = 0; m < 2; ++m) {
+      const V a = v[m], c = v[m + 2];
+      v[m] = cadd(a, c);
+      v[m + 2] = csub(a, c);
+      pos[m] = 2 * (t + m * T4);
+      pos[m + 2] = pos[m] + 1;
+    }
+  } else {
+    const int k = t & (NS - 1);
+    if constexpr (NS > 1) {
+      constexpr int step = N / (NS * 4);
+      const V w1 = twiddle<V, INV>(tw, k * step), w2 = twiddle<V, INV>(tw, 2 * k * step);
+      if constexpr (sizeof(V) == 16) {
+        bf2(v[0], v[2], w2);
+        bf2(v[1], v[3], w2);
+        bf2(v[0], v[1], w1);
+        bf2(v[2], v[3], quarter<V, INV>(w1));
+        const V x = v[1];
+        v[1] = v[2];
+        v[2] = x;
+      } else {
+        // products apart: a difference as 2 a - t carries the rounding of t, which shows in FP32
+        v[1] = cmul(v[1], w1);
+        v[2] = cmul(v[2], w2);
+        v[3] = cmul(v[3], twiddle<V, INV>(tw, 3 * k * step));
+        dft4<V, INV>(v);
+      }
+    } else {
+      dft4<V, INV>(v);
+    }
+    const int base = (t / NS) * NS * 4 + k;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) pos[r] = base + r * NS;
+  }
+  if constexpr (NS * R < N) {
+#pragma unroll
+    for (int m = 0; m < 4; ++m) sm.put(pos[m], v[m]);
+    __syncthreads();
+#pragma unroll
+    for (int m = 0; m < 4; ++m) v[m] = sm.get(t + m * T4);
+    __syncthreads();
+    fft4_ct<V, INV, N, NS * R>(v, t, sm, tw);
+  }
+}
+// rows: one pad slot every 8 entries
+template <typename V, int N> struct SurfSm {
+  static constexpr int LD = N + N / 8;
+  V* buf;
+  __device__ __forceinline__ void put(int p, V x) const { buf[p + (p >> 3)] = x; }
+  __device__ __forceinline__ V get(int p) const { return buf[p + (p >> 3)]; }
+};
+template <typename V> struct SurfColSm {
+  V* buf;
+  int kc, f;
+  __device__ __forceinline__ void put(int p, V x) const { buf[p * kc + f] = x; }
+  __device__ __forceinline__ V get(int p) const { return buf[p * kc + f]; }
+};
+
+// CTA of a row pass: about one transform pair per CTA and SM, whole warps
+struct SurfRowCfg {
+  int grid, threads;
+  size_t smem;
+};
+template <typename T, int N> inline SurfRowCfg surf_row_cfg(int n2) {
+  typedef typename Cx<T>::t V;
+  const int pairs = n2 / 2, T4 = N / 4;
+  int slots = 1;
+  while (slots * 2 * 128 <= pairs && slots * 2 * T4 <= 512) slots *= 2;
+  const int threads = slots * T4 > 32 ? slots * T4 : 32;
+  slots = threads / T4;
+  return SurfRowCfg{(pairs + slots - 1) / slots, threads, (size_t)slots * SurfSm<V, N>::LD * sizeof(V)};
+}
+
+// ---------------------------------------------------------------------------
 // asynchronous global -> shared copies (cp.async), all in flight before one wait
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async_8(void* smem, const void* gmem) {
@@ -523,6 +610,12 @@ inline int smem_optin_max() {
   }();
   return v;
 }
+// dynamic shared memory cap of the row kernels (at most four FP64 transforms of 1024 points; they
+// hold static shared memory too, so not the whole opt-in maximum); the same value on every call
+template <typename K> inline void surf_row_smem_cap(K kern) {
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
+}
+
 // multiprocessors of the current device
 inline int sm_count() {
   static const int v = [] {
@@ -655,7 +748,14 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
 template <typename T> int launch_boussinesq(const fvim_ctx* c, int out_kind, bool want_vol, bool want_u3);
 template <typename T> int launch_return_map(const fvim_ctx* c, const T* d_eps, T* d_eps_p, T* d_ep);
 template <typename T> int launch_commit(const fvim_ctx* c, const T* d_eps, const T* d_eps_p, const T* d_ep);
-template <typename T> int launch_zero_nq(const fvim_ctx* c);
+// surface transforms with compile-time sides of 16 to 1024 (surface.cu); false when a side has no
+// variant: rows of a real field to and from c->surf, columns of c->surf in place
+template <typename T> bool launch_surf_rows_fwd(const fvim_ctx* c, const T* f);
+template <typename T> bool launch_surf_rows_inv(const fvim_ctx* c, T* f, T scale);
+template <typename T> bool launch_surf_cols(const fvim_ctx* c, bool inverse);
+// strain or stress of the Boussinesq field evaluated in the inverse column pass (FP32): c->surf
+// (p_hat) to the half row spectra in c->spec; false when the grid has no variant
+bool launch_bous_cols(const fvim_ctx* c, int out_kind);
 
 // solver runtime (solvers.cu): release, and drop captured graphs after a material change
 void solver_release(fvim_ctx* c);
