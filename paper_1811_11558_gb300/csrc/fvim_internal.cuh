@@ -574,6 +574,74 @@ template <typename T, int N> inline SurfRowCfg surf_row_cfg(int n2) {
 }
 
 // ---------------------------------------------------------------------------
+// FP64 sums over a grid in a fixed order.  An FP64 instruction holds its pipe for 64 cycles per
+// warp on this chip, so the chain of additions is what they cost.
+// ---------------------------------------------------------------------------
+// Sums of up to four values over a warp, reduced together: six additions instead of five per value.
+// Lane l ends with the sum of value ((l >> 4) & 1) 2 + ((l >> 3) & 1).
+__device__ __forceinline__ double warp_sum4(double v0, double v1, double v2, double v3) {
+  const unsigned all = 0xffffffffu;
+  const bool h16 = threadIdx.x & 16, h8 = threadIdx.x & 8;
+  double a = (h16 ? v2 : v0) + __shfl_xor_sync(all, h16 ? v0 : v2, 16);
+  const double b = (h16 ? v3 : v1) + __shfl_xor_sync(all, h16 ? v1 : v3, 16);
+  a = (h8 ? b : a) + __shfl_xor_sync(all, h8 ? a : b, 8);
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
+  return a;
+}
+// over the block's whole warps of per-thread values x of kind j = threadIdx.x & 3 that are already
+// summed over the lanes of equal j: lanes 0..3 of warp 0 end with the sums
+__device__ __forceinline__ double block_sum_kind(double x, double* sh) {
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (nw == 1) return x;
+  if (l < 4) sh[w * 4 + l] = x;
+  __syncthreads();
+  if (w > 0) return 0;
+  x = 0;
+  for (int k = l >> 2; k < nw; k += 8) x += sh[k * 4 + (l & 3)];
+  for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  return x;
+}
+// sums of v over the grid: true in thread 0 of the last block to arrive, which then holds them
+__device__ __forceinline__ bool grid_sum(double (&v)[4], double* part, unsigned* cnt) {
+  __shared__ double sh[32 * 4];
+  __shared__ bool last;
+  const int l = threadIdx.x & 31;
+  double x = warp_sum4(v[0], v[1], v[2], v[3]);
+  // value j from the lane group that holds it
+  x = __shfl_sync(0xffffffffu, x, ((l & 3) >> 1) * 16 + (l & 1) * 8);
+  x = block_sum_kind(x, sh);
+  if (threadIdx.x < 4) {
+    part[blockIdx.x * 4 + threadIdx.x] = x;
+    __threadfence();
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+  __syncthreads();
+  if (!last) return false;
+  __threadfence();
+  x = 0;
+  for (int b = threadIdx.x >> 2; b < (int)gridDim.x; b += blockDim.x >> 2) x += __ldcg(part + b * 4 + (threadIdx.x & 3));
+  for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  x = block_sum_kind(x, sh);
+  if (threadIdx.x >= 32) return false;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = __shfl_sync(0xffffffffu, x, j);
+  if (threadIdx.x == 0) *cnt = 0u;
+  return threadIdx.x == 0;
+}
+
+__device__ __forceinline__ float two_sum_err(float a, float b, float s) {  // a + b - s
+  const float bb = __fsub_rn(s, a);
+  return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+}
+// running sum of FP32 values as an exact pair
+__device__ __forceinline__ void pair_add(float2& a, float x) {
+  const float s = __fadd_rn(a.x, x);
+  a.y = __fadd_rn(a.y, two_sum_err(a.x, x, s));
+  a.x = s;
+}
+
+// ---------------------------------------------------------------------------
 // asynchronous global -> shared copies (cp.async), all in flight before one wait
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void cp_async_8(void* smem, const void* gmem) {

@@ -27,6 +27,8 @@ namespace {
 constexpr int RT = 256;       // threads of a reduction block
 constexpr int RMAXB = 1024;   // blocks of a reduction grid
 constexpr int NVMAX = 3;      // values reduced per pass
+constexpr int DFS_BLOCKS = 4096;  // blocks of the DF-SANE residual pass (at least one per plane, 3072 planes)
+constexpr size_t kPartBytes = (size_t)DFS_BLOCKS * 4 * sizeof(double);  // block partials, up to four values each
 constexpr size_t kScalarBlock = 256;  // bytes of the solver's device scalar block (V_PKS)
 constexpr size_t kDfsBytes = 1024;     // bytes of the device DF-SANE state (V_DFS)
 constexpr size_t kPkfBytes = 512;      // fused contact iteration (V_PKF): PkState, arrival counter at byte 256
@@ -47,7 +49,7 @@ template <typename T> int ensure_ws(fvim_ctx* c) {
   for (int i = V_X; i <= V_DE; ++i)
     if (FVIM_CU(cudaMalloc(&c->sv[i], nv * 6 * sizeof(T)))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_EP], nv * sizeof(T)))) return FVIM_ERR_OOM;
-  if (FVIM_CU(cudaMalloc(&c->sv[V_PART], (size_t)RMAXB * NVMAX * sizeof(double)))) return FVIM_ERR_OOM;
+  if (FVIM_CU(cudaMalloc(&c->sv[V_PART], kPartBytes))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_WZ], (size_t)c->nz * sizeof(double)))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_PKS], kScalarBlock))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_DFS], kDfsBytes))) return FVIM_ERR_OOM;
@@ -930,10 +932,12 @@ template <typename T> struct DF {
 struct DFS {
   const void* px[2];  // the two point buffers: x = px[cur], trial = px[1 - cur]
   void* pF[2];        // their residuals
-  double f, nF0, fmax, eta, ap, am, fp, fm, ftrial, best_old, tol_abs, tol_rel, gamma, smin, smax, tmin, tmax;
-  double sy[2];
+  double f, nF0, fmax, eta, ap, am, fp, fm, best_old, tol_abs, tol_rel, gamma, smin, smax, tmin, tmax;
   double hist[32];    // ring of the accepted residuals, hist[i & 31] for i < len
   int len, k, bt, phase, done, conv, bad, cur, trials, max_iter, max_trials, evals;
+  double sigma;       // spectral step
+  double coef;        // step of the current trial: -ap sigma (phase 0) or am sigma (phase 1)
+  float coef32;       // the same, rounded once
 };
 static_assert(sizeof(DFS) <= kDfsBytes, "device DF-SANE state");
 constexpr int kDfsM = 10, kDfsStag = 30;
@@ -944,8 +948,7 @@ constexpr int kDfsM = 10, kDfsStag = 30;
 // the increment of cumulated plastic strain, and notes the layer range of the flowing voxels.
 // The loop leaves d_ep out: the solve recomputes the return map of its final point.
 template <typename T>
-__global__ void k_dfd_trial_rmap(const DFS* __restrict__ s, const double* __restrict__ dsig,
-                                 const T* __restrict__ sig_n, const T* __restrict__ ep, T* __restrict__ d_eps_p,
+__global__ void k_dfd_trial_rmap(const DFS* __restrict__ s, const T* __restrict__ sig_n, const T* __restrict__ ep, T* __restrict__ d_eps_p,
                                  T* __restrict__ d_ep, size_t nxy, size_t nvox, T lam, T mu, T sy, T Eh,
                                  int* __restrict__ zr) {
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -954,8 +957,8 @@ __global__ void k_dfd_trial_rmap(const DFS* __restrict__ s, const double* __rest
   const T* a = static_cast<const T*>(s->px[cur]);
   const T* b = static_cast<const T*>(s->pF[cur]);
   T* dst = const_cast<T*>(static_cast<const T*>(s->px[1 - cur]));
-  const double coef = (s->phase == 0 ? -s->ap : s->am) * *dsig;
-  const T cf = (T)coef;
+  const double coef = sizeof(T) == 4 ? 0.0 : s->coef;
+  const float cf = s->coef32;
   const size_t z = v / nxy, xy = v - z * nxy;
   const size_t base = z * 6 * nxy + xy;
   T de[6], sg[6], dp[6];
@@ -974,73 +977,14 @@ __global__ void k_dfd_trial_rmap(const DFS* __restrict__ s, const double* __rest
   if (dEp > 0) flow_range_note(zr, (int)z);
 }
 
-// residual of the trial point into its residual buffer, with ||F||^2 into s->ftrial and <s, s>,
-// <s, y> (s = trial - x, y = F(trial) - F(x)) into s->sy (last block).  The trial point is
-// recomputed from x and F with the expression the trial kernel wrote it with (the same
-// values), so it is not read back.
-template <typename T>
-__global__ void k_dfd_res_sy(DFS* s, const double* __restrict__ dsig, const T* __restrict__ b,
-                             const T* __restrict__ tmp, const double* __restrict__ wz, int lgxy, size_t n,
-                             double* part, unsigned* cnt) {
-  const int cur = s->cur;
-  const T* x = static_cast<const T*>(s->px[cur]);
-  const T* F = static_cast<const T*>(s->pF[cur]);
-  T* Fn = static_cast<T*>(s->pF[1 - cur]);
-  const double coef = (s->phase == 0 ? -s->ap : s->am) * *dsig;
-  double v[3] = {0, 0, 0};
-  if constexpr (sizeof(T) == 4) {
-    const float cf = (float)coef;
-    const size_t n4 = n >> 2;
-    const int lg4 = lgxy - 2;
-    for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n4; i += (size_t)gridDim.x * RT) {
-      const float4 a = reinterpret_cast<const float4*>(x)[i];
-      const float4 g = reinterpret_cast<const float4*>(F)[i];
-      const float4 c = reinterpret_cast<const float4*>(b)[i];
-      const float4 d = reinterpret_cast<const float4*>(tmp)[i];
-      const float4 t = make_float4(fmaf(cf, g.x, a.x), fmaf(cf, g.y, a.y), fmaf(cf, g.z, a.z), fmaf(cf, g.w, a.w));
-      const float4 f = make_float4(t.x - c.x - d.x, t.y - c.y - d.y, t.z - c.z - d.z, t.w - c.w - d.w);
-      reinterpret_cast<float4*>(Fn)[i] = f;
-      const double w = plane_weight(wz, (unsigned)(i >> lg4));
-      const float q = f.x * f.x + f.y * f.y + f.z * f.z + f.w * f.w;
-      v[0] += w * (double)q;
-      const float s0 = t.x - a.x, s1 = t.y - a.y, s2 = t.z - a.z, s3 = t.w - a.w;
-      const float y0 = f.x - g.x, y1 = f.y - g.y, y2 = f.z - g.z, y3 = f.w - g.w;
-      v[1] += w * (double)(s0 * s0 + s1 * s1 + s2 * s2 + s3 * s3);
-      v[2] += w * (double)(s0 * y0 + s1 * y1 + s2 * y2 + s3 * y3);
-    }
-  } else {
-    for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
-      const double w = plane_weight(wz, (unsigned)(i >> lgxy));
-      const double xi = (double)x[i], gi = (double)F[i];
-      const double t = fma(coef, gi, xi);
-      const T f = (T)(t - (double)b[i] - (double)tmp[i]);
-      Fn[i] = f;
-      v[0] += w * (double)f * (double)f;
-      const double a = t - xi;
-      const double y = (double)f - gi;
-      v[1] += w * a * a;
-      v[2] += w * a * y;
-    }
-  }
-  block_reduce<3>(v, part);
-  if (last_block(cnt)) {
-    double r[3];
-    fin_sum<3>(part, gridDim.x, r);
-    if (threadIdx.x == 0) {
-      s->ftrial = r[0];
-      s->sy[0] = r[1];
-      s->sy[1] = r[2];
-    }
-    rearm(cnt);
-  }
-}
-
-// the host loop's decisions after one trial evaluation (one thread)
-__global__ void k_dfd_decide(DFS* s, double* dsig, cudaGraphConditionalHandle cond) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// the host loop's decisions after one trial evaluation: ||F||^2 of the trial, <s, s> and <s, y>
+__device__ void dfd_decide(DFS* s, double ft, double ss, double sy, cudaGraphConditionalHandle cond) {
+  // largest and smallest of non-negative values by their bit patterns (an FP64 comparison costs 64
+  // cycles; the history is up to thirty values long)
+  auto bits = [](double x) { return __double_as_longlong(x); };
   s->trials += 1;
   s->evals += 1;
-  const double ft = s->ftrial;
+  int done = s->done;
   bool acc = false;
   if (s->phase == 0) {
     s->fp = ft;
@@ -1056,16 +1000,16 @@ __global__ void k_dfd_decide(DFS* s, double* dsig, cudaGraphConditionalHandle co
       s->am = fmin(fmax(am * am * f / (s->fm + (2 * am - 1) * f), s->tmin * am), s->tmax * am);
       s->phase = 0;
       s->bt += 1;
-      if (s->bt >= 60) s->done = 1;  // line search failed: stop, not converged
+      if (s->bt >= 60) done = 1;  // line search failed: stop, not converged
     }
   }
   if (acc) {
-    double sigma = s->sy[1] != 0 ? s->sy[0] / s->sy[1] : INFINITY;
+    double sigma = sy != 0 ? ss / sy : INFINITY;
     if (!(fabs(sigma) >= s->smin && fabs(sigma) <= s->smax)) {
       const double nf = sqrt(ft);
       sigma = nf > 1 ? 1.0 : (nf >= 1e-5 ? 1.0 / nf : 1e5);
     }
-    *dsig = sigma;
+    s->sigma = sigma;
     s->cur ^= 1;
     s->f = ft;
     s->hist[s->len & 31] = ft;
@@ -1074,22 +1018,29 @@ __global__ void k_dfd_decide(DFS* s, double* dsig, cudaGraphConditionalHandle co
     // the checks at the top of the next iteration
     if (!isfinite(s->f)) {
       s->bad = 1;
-      s->done = 1;
+      done = 1;
     } else if (sqrt(s->f) <= s->tol_abs + s->tol_rel * s->nF0) {
       s->conv = 1;
-      s->done = 1;
+      done = 1;
     } else {
       if (s->len > kDfsStag) {
-        s->best_old = fmin(s->best_old, s->hist[(s->len - 1 - kDfsStag) & 31]);
-        double best_new = INFINITY;
-        for (int j = s->len - kDfsStag; j < s->len; ++j) best_new = fmin(best_new, s->hist[j & 31]);
-        if (best_new > 0.81 * s->best_old) s->done = 1;
+        const double leaving = s->hist[(s->len - 1 - kDfsStag) & 31];
+        if (bits(leaving) < bits(s->best_old)) s->best_old = leaving;
+        long long best = bits(INFINITY);
+        for (int j = s->len - kDfsStag; j < s->len; ++j) {
+          const long long x = bits(s->hist[j & 31]);
+          if (x < best) best = x;
+        }
+        if (__longlong_as_double(best) > 0.81 * s->best_old) done = 1;
       }
-      if (s->k >= s->max_iter) s->done = 1;
-      if (!s->done) {
-        double fm = 0;
-        for (int j = s->len > kDfsM ? s->len - kDfsM : 0; j < s->len; ++j) fm = fmax(fm, s->hist[j & 31]);
-        s->fmax = fm;
+      if (s->k >= s->max_iter) done = 1;
+      if (!done) {
+        long long fm = 0;
+        for (int j = s->len > kDfsM ? s->len - kDfsM : 0; j < s->len; ++j) {
+          const long long x = bits(s->hist[j & 31]);
+          if (x > fm) fm = x;
+        }
+        s->fmax = __longlong_as_double(fm);
         s->eta = s->nF0 / ((1.0 + s->k) * (1.0 + s->k));
         s->ap = 1;
         s->am = 1;
@@ -1098,8 +1049,94 @@ __global__ void k_dfd_decide(DFS* s, double* dsig, cudaGraphConditionalHandle co
       }
     }
   }
-  if (s->trials >= s->max_trials) s->done = 1;
-  cudaGraphSetConditional(cond, s->done ? 0u : 1u);
+  if (s->trials >= s->max_trials) done = 1;
+  const double coef = (s->phase == 0 ? -s->ap : s->am) * s->sigma;
+  s->coef = coef;
+  s->coef32 = (float)coef;
+  s->done = done;
+  cudaGraphSetConditional(cond, done ? 0u : 1u);
+}
+
+// residual of the trial point into its residual buffer, with ||F||^2, <s, s> and <s, y> (s = trial -
+// x, y = F(trial) - F(x)) and the decisions on them by the last block.  The trial point is
+// recomputed from x and F with the expression the trial kernel wrote it with (the same
+// values), so it is not read back.
+template <typename T>
+__global__ void __launch_bounds__(RT) k_dfd_res_sy(DFS* s, const T* __restrict__ b, const T* __restrict__ tmp,
+                                                   const double* __restrict__ wz, int lgxy, size_t n, int per_plane,
+                                                   double* part, unsigned* cnt, int* zr, cudaGraphConditionalHandle cond) {
+  const int cur = s->cur;
+  const T* x = static_cast<const T*>(s->px[cur]);
+  const T* F = static_cast<const T*>(s->pF[cur]);
+  T* Fn = static_cast<T*>(s->pF[1 - cur]);
+  double v[4] = {0, 0, 0, 0};
+  if constexpr (sizeof(T) == 4) {
+    const float cf = s->coef32;
+    // four values: the residual stored, the three products of the four
+    auto four = [&](size_t i, float& ff, float& ss, float& sy) {
+      const float4 a = reinterpret_cast<const float4*>(x)[i];
+      const float4 g = reinterpret_cast<const float4*>(F)[i];
+      const float4 c = reinterpret_cast<const float4*>(b)[i];
+      const float4 d = reinterpret_cast<const float4*>(tmp)[i];
+      const float4 t = make_float4(fmaf(cf, g.x, a.x), fmaf(cf, g.y, a.y), fmaf(cf, g.z, a.z), fmaf(cf, g.w, a.w));
+      const float4 f = make_float4(t.x - c.x - d.x, t.y - c.y - d.y, t.z - c.z - d.z, t.w - c.w - d.w);
+      reinterpret_cast<float4*>(Fn)[i] = f;
+      ff = f.x * f.x + f.y * f.y + f.z * f.z + f.w * f.w;
+      const float s0 = t.x - a.x, s1 = t.y - a.y, s2 = t.z - a.z, s3 = t.w - a.w;
+      const float y0 = f.x - g.x, y1 = f.y - g.y, y2 = f.z - g.z, y3 = f.w - g.w;
+      ss = s0 * s0 + s1 * s1 + s2 * s2 + s3 * s3;
+      sy = s0 * y0 + s1 * y1 + s2 * y2 + s3 * y3;
+    };
+    if (per_plane > 0) {
+      // per_plane blocks per plane: one weight per block, the thread's sums as exact FP32 pairs (an
+      // FP64 multiply-add per four values held the FP64 pipe as long as the memory traffic took)
+      const unsigned zc = blockIdx.x / per_plane, sub = blockIdx.x - zc * per_plane;
+      const size_t n4 = (size_t)1 << (lgxy - 2), base = (size_t)zc * n4;
+      float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0;
+      for (size_t j = sub * (size_t)RT + threadIdx.x; j < n4; j += (size_t)per_plane * RT) {
+        float ff, ss, sy;
+        four(base + j, ff, ss, sy);
+        pair_add(a0, ff);
+        pair_add(a1, ss);
+        pair_add(a2, sy);
+      }
+      const double w = plane_weight(wz, zc);
+      v[0] = w * ((double)a0.x + (double)a0.y);
+      v[1] = w * ((double)a1.x + (double)a1.y);
+      v[2] = w * ((double)a2.x + (double)a2.y);
+    } else {
+      const size_t n4 = n >> 2;
+      const int lg4 = lgxy - 2;
+      for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n4; i += (size_t)gridDim.x * RT) {
+        float ff, ss, sy;
+        four(i, ff, ss, sy);
+        const double w = plane_weight(wz, (unsigned)(i >> lg4));
+        v[0] += w * (double)ff;
+        v[1] += w * (double)ss;
+        v[2] += w * (double)sy;
+      }
+    }
+  } else {
+    const double coef = s->coef;
+    for (size_t i = blockIdx.x * (size_t)RT + threadIdx.x; i < n; i += (size_t)gridDim.x * RT) {
+      const double w = plane_weight(wz, (unsigned)(i >> lgxy));
+      const double xi = (double)x[i], gi = (double)F[i];
+      const double t = fma(coef, gi, xi);
+      const T f = (T)(t - (double)b[i] - (double)tmp[i]);
+      Fn[i] = f;
+      v[0] += w * (double)f * (double)f;
+      const double a = t - xi;
+      const double y = (double)f - gi;
+      v[1] += w * a * a;
+      v[2] += w * a * y;
+    }
+  }
+  if (grid_sum(v, part, cnt)) {
+    dfd_decide(s, v[0], v[1], v[2], cond);
+    // the flow range of the next trial
+    zr[0] = 0x7f7f7f7f;
+    zr[1] = 0;
+  }
 }
 
 static bool device_dfsane_enabled() {
@@ -1111,7 +1148,6 @@ static bool device_dfsane_enabled() {
 }
 
 inline DFS* dfs_dev(fvim_ctx* c) { return static_cast<DFS*>(c->sv[V_DFS]); }
-inline double* dfs_sigma(fvim_ctx* c) { return reinterpret_cast<double*>(static_cast<char*>(c->sv[V_PKS]) + 128); }
 inline unsigned* dfs_count(fvim_ctx* c) { return reinterpret_cast<unsigned*>(static_cast<char*>(c->sv[V_PKS]) + 196); }
 
 // The WHILE graph of the device DF-SANE loop (built once per context; the material constants
@@ -1122,17 +1158,21 @@ template <typename T> int build_dfloop(fvim_ctx* c, SolverRT* r, size_t n, int g
       c,
       [&](cudaGraphConditionalHandle cond) -> int {
         int e;
-        if ((e = reset_flow_range(c))) return e;
         const size_t nv = n / 6;
         k_dfd_trial_rmap<T><<<(unsigned)((nv + 255) / 256), 256, 0, c->stream>>>(
-            dfs, dfs_sigma(c), (const T*)c->st_sig, (const T*)c->st_ep, S<T>(c, V_DEP), (T*)nullptr,
-            (size_t)c->n1 * c->n2, nv, (T)c->lam, (T)c->mu, (T)c->sigma_y, (T)c->E_h, flow_range(c));
+            dfs, (const T*)c->st_sig, (const T*)c->st_ep, S<T>(c, V_DEP), (T*)nullptr, (size_t)c->n1 * c->n2, nv,
+            (T)c->lam, (T)c->mu, (T)c->sigma_y, (T)c->E_h, flow_range(c));
         FVIM_CUDA_CHECK_LAUNCH();
         if ((e = apply_mindlin_t<T>(c, S<T>(c, V_DEP), S<T>(c, V_TMP), FVIM_STRAIN, nullptr, flow_range(c)))) return e;
-        k_dfd_res_sy<T><<<grd, RT, 0, c->stream>>>(dfs, dfs_sigma(c), S<T>(c, V_B), S<T>(c, V_TMP),
-                                                   (const double*)c->sv[V_WZ], lgxy, n, (double*)c->sv[V_PART],
-                                                   dfs_count(c));
-        k_dfd_decide<<<1, 32, 0, c->stream>>>(dfs, dfs_sigma(c), cond);
+        // FP32 planes of a power of two: whole blocks per plane, about DFS_BLOCKS / 4 in all
+        const size_t nxy = (size_t)c->n1 * c->n2;
+        const bool by_plane = sizeof(T) == 4 && nxy == (size_t)1 << lgxy && lgxy >= 2;
+        const int planes = c->nz * 6;
+        const int per_plane =
+            by_plane ? (int)std::min<size_t>((nxy / 4 + RT - 1) / RT, std::max(1, DFS_BLOCKS / 4 / planes)) : 0;
+        const int g = by_plane ? planes * per_plane : grd;
+        k_dfd_res_sy<T><<<g, RT, 0, c->stream>>>(dfs, S<T>(c, V_B), S<T>(c, V_TMP), (const double*)c->sv[V_WZ], lgxy, n,
+                                                 per_plane, (double*)c->sv[V_PART], dfs_count(c), flow_range(c), cond);
         FVIM_CUDA_CHECK_LAUNCH();
         return FVIM_OK;
       },
@@ -1222,9 +1262,12 @@ int plasticity_t(fvim_ctx* c, const T* dT, T* dE, T* deps_p, T* dep, const fvim_
     hs->len = 1;
     hs->max_iter = o->df_max_iter;
     hs->max_trials = o->df_max_iter * 121 + 1;
+    hs->sigma = 1.0;
+    hs->coef = -1.0;
+    hs->coef32 = -1.f;
     DFS* ds = dfs_dev(c);
     if (FVIM_CU(cudaMemcpyAsync(ds, hs, sizeof(DFS), cudaMemcpyHostToDevice, c->stream)) ||
-        FVIM_CU(cudaMemsetAsync(dfs_count(c), 0, sizeof(unsigned), c->stream)) ||
+        FVIM_CU(cudaMemsetAsync(dfs_count(c), 0, sizeof(unsigned), c->stream)) || reset_flow_range(c) ||
         FVIM_CU(cudaGraphLaunch(srt->dfloop, c->stream)) ||
         FVIM_CU(cudaMemcpyAsync(hs, ds, sizeof(DFS), cudaMemcpyDeviceToHost, c->stream)) ||
         FVIM_CU(cudaStreamSynchronize(c->stream)))
