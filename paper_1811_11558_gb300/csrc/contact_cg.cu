@@ -26,6 +26,8 @@
 // and there only at points that carry pressure; a warp's sums of several values reduced together.
 // us per iteration, fourteen kernels -> seven with eight values per thread and FP64 updates -> this:
 // 32^2 FP64 100 -> 97 -> 56, 32^2 FP32 62 -> 63 -> 41, 512^2 132 -> 75 -> 56, 1024^2 206 -> 156 -> 112.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 
 #include "fvim_internal.cuh"
@@ -366,6 +368,400 @@ template <typename T, int N, bool SCALE> void cols(const PkfArgs& a) {
       a.S, (V*)a.surf, (const T*)a.green, (const V*)a.tw2, a.h1, kc);
 }
 
+// ---- small square surfaces: the whole solve in one cluster of eight CTAs --------------------
+// On 16^2 to 128^2 surfaces an iteration of six kernels is launches and latency (41 us at 32^2
+// FP32, 56 us FP64, whatever the work).  Here eight CTAs keep the surface, the iterate and both
+// spectra in shared memory: CTA r owns rows [r N/8, (r+1) N/8) and columns [r N/16, (r+1) N/16) of
+// the half spectrum, row results go straight to the owners' shared memory (remote stores) and
+// back, and sums are exchanged the same way, each CTA adding the eight partials in rank order (the
+// same value everywhere, so every decision is the same everywhere).  Six cluster barriers per
+// iteration (about 350 cycles each); the loop ends at the stop test or the iteration cap.
+// us per iteration, six kernels -> this: FP64 32^2 56 -> 22, FP32 32^2 41 -> 13, 64^2 42 -> 21, 128^2
+// 47 -> 33 (256^2 does not fit).
+constexpr int CL = 8;
+
+// Stockham stages of radix 2 on two values per thread (FP64: the pipes are idle but for the few
+// warps of a transform, so half the work per thread is half the time)
+template <typename V, bool INV, int N, int NS, class Sm>
+__device__ __forceinline__ void fft2_ct(V (&v)[2], int t, bool on, const Sm& sm, const V* __restrict__ tw) {
+  const int k = t & (NS - 1);
+  if constexpr (NS > 1) {
+    if (on) bf2(v[0], v[1], twiddle<V, INV>(tw, k * (N / (2 * NS))));
+  } else {
+    const V a = v[0], c = v[1];
+    v[0] = cadd(a, c);
+    v[1] = csub(a, c);
+  }
+  if constexpr (2 * NS < N) {
+    const int base = (t / NS) * NS * 2 + k;
+    if (on) {
+      sm.put(base, v[0]);
+      sm.put(base + NS, v[1]);
+    }
+    __syncthreads();
+    if (on) {
+      v[0] = sm.get(t);
+      v[1] = sm.get(t + N / 2);
+    }
+    __syncthreads();
+    fft2_ct<V, INV, N, 2 * NS>(v, t, on, sm, tw);
+  }
+}
+
+template <typename T, int N> struct ClCfg {
+  typedef typename Cx<T>::t V;
+  static constexpr int H1 = N / 2, R = N / CL, K = H1 / CL;   // rows and columns of a CTA
+  static constexpr int E = R * N;                             // points of a CTA
+  static constexpr int BT = E < 64 ? 64 : (E > 512 ? 512 : E);
+  static constexpr int VT = (sizeof(T) == 8 && N <= 64) ? 2 : 4;  // values per transform thread
+  static constexpr int TT = N / VT;                               // threads per transform
+  static constexpr int LD = N + N / 8;
+  static constexpr int NT = R / 2 > K ? R / 2 : K;                // transforms at once (R / 2 == K)
+  static_assert(R / 2 == K && NT * TT <= BT, "transform threads");
+  static constexpr size_t bytes = (size_t)(NT * LD + K * N + R * H1 + N) * sizeof(V) + (size_t)(6 * E + K * N) * sizeof(T);
+};
+
+// transform of NT sequences of the CTA by its first NT TT threads; get(f, i) reads, put(f, i, x) takes
+// the results (natural order)
+template <typename T, int N, bool INV, class G, class P>
+__device__ __forceinline__ void cl_fft(typename Cx<T>::t* xch, const typename Cx<T>::t* tw, G&& get, P&& put) {
+  typedef typename Cx<T>::t V;
+  typedef ClCfg<T, N> C;
+  const int f = threadIdx.x / C::TT, t = threadIdx.x % C::TT;
+  const bool on = f < C::NT;
+  SurfSm<V, N> sm{xch + (size_t)(on ? f : 0) * C::LD};
+  V v[C::VT];
+#pragma unroll
+  for (int m = 0; m < C::VT; ++m) v[m] = on ? get(f, t + m * C::TT) : mk<V>(0, 0);
+  if constexpr (C::VT == 2) {
+    fft2_ct<V, INV, N, 1>(v, t, on, sm, tw);
+  } else {
+    // (threads without a transform take part in the barriers; their exchange area is a spare copy)
+    fft4_on<V, INV, N, 1>(v, t, on, sm, tw);
+  }
+#pragma unroll
+  for (int m = 0; m < C::VT; ++m)
+    if (on) put(f, t + m * C::TT, v[m]);
+}
+
+template <typename T, int N>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
+    k_pkf_cluster(PkState* out, PkState init, const typename Cx<T>::t* __restrict__ tw_g, T w1, T w2, T nu, T mu) {
+  typedef typename Cx<T>::t V;
+  typedef ClCfg<T, N> C;
+  constexpr int H1 = C::H1, R = C::R, K = C::K, E = C::E;
+  namespace cgx = cooperative_groups;
+  cgx::cluster_group cl = cgx::this_cluster();
+  const int rank = (int)cl.block_rank();
+  extern __shared__ __align__(16) unsigned char smraw[];
+  V* xch = reinterpret_cast<V*>(smraw);   // [NT][LD] exchange
+  V* colb = xch + C::NT * C::LD;          // [K][N] columns of this CTA
+  V* rowb = colb + K * N;                 // [R][H1] half spectra of its rows
+  V* tw = rowb + R * H1;                  // [N]
+  T* p = reinterpret_cast<T*>(tw + N);    // [R][N] each
+  T* h = p + E;
+  T* t = h + E;
+  T* g = t + E;
+  T* po = g + E;
+  T* u = po + E;
+  T* green = u + E;                       // [K][N] compliance of its columns
+  __shared__ PkState S;
+  __shared__ double red[4][CL][4];        // partial sums of every CTA: start, tau, load, gap
+  __shared__ double wsum[32 * 4];
+
+  const int tid = threadIdx.x, nth = blockDim.x;
+  T* pg = static_cast<T*>(init.p) + (size_t)rank * E;
+  const T* hg = static_cast<const T*>(init.h) + (size_t)rank * E;
+  if (tid == 0) S = init;
+  for (int i = tid; i < N; i += nth) tw[i] = tw_g[i];
+  for (int i = tid; i < K * N; i += nth) {
+    const int k1 = rank * K + i / N, k2 = i % N;
+    const T q1 = w1 * (T)k1, q2 = w2 * (T)(k2 < N / 2 ? k2 : k2 - N);
+    const T q = sqrt(q1 * q1 + q2 * q2);
+    green[i] = (k1 == 0 && k2 == 0) || k2 == N / 2 ? (T)0 : ((T)1 - nu) / (mu * q);
+  }
+
+  cl.sync();  // every CTA runs before its shared memory is written from outside
+
+  // sums of this CTA to every CTA's slot `which`; totals(which) after the next cluster barrier
+  auto send = [&](int which, double a, double b, double c, double d) {
+    double x = warp_sum4(a, b, c, d);
+    x = __shfl_sync(0xffffffffu, x, ((tid & 3) >> 1) * 16 + (tid & 1) * 8);
+    x = block_sum_kind(x, wsum);
+    // lanes 4 r + j of warp 0: value j to CTA r
+    if (tid < 32) {
+      x = __shfl_sync(0xffffffffu, x, tid & 3);
+      *cl.map_shared_rank(&red[which][rank][tid & 3], tid >> 2) = x;
+    }
+  };
+  // value j of the totals in lanes of equal tid & 3 of warp 0
+  auto total = [&](int which) {
+    double x = red[which][(tid & 31) >> 2][tid & 3];
+    for (int o = 4; o < 32; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+  };
+  auto value = [&](double x, int j) { return __shfl_sync(0xffffffffu, x, j); };
+
+  // rows of `src` forward, half spectra to the column owners
+  auto rows_fwd = [&](const T* src) {
+    cl_fft<T, N, false>(
+        xch, tw, [&](int f, int i) { return mk<V>(src[(2 * f) * N + i], src[(2 * f + 1) * N + i]); },
+        [&](int f, int i, V x) { xch[f * C::LD + i + (i >> 3)] = x; });
+    __syncthreads();
+    for (int i = tid; i < (R / 2) * H1; i += nth) {
+      const int f = i / H1, k = i - f * H1, km = (N - k) & (N - 1);
+      const V zk = xch[f * C::LD + k + (k >> 3)], zm = xch[f * C::LD + km + (km >> 3)];
+      const V c = cconj(zm), a = cadd(zk, c), d = csub(zk, c);
+      V* dst = cl.map_shared_rank(colb, k / K) + (k % K) * N + rank * R + 2 * f;
+      dst[0] = cscale(a, (T)0.5);
+      dst[1] = mk<V>((T)0.5 * d.y, (T)-0.5 * d.x);
+    }
+  };
+  // this CTA's columns: transform, compliance (times the load scale), inverse, rows to their owners
+  auto cols = [&](bool scaled) {
+    const double s = scaled ? S.s : 1.0;
+    const float2 s2 = scaled ? S.s2 : make_float2(1.f, 0.f);
+    cl_fft<T, N, false>(
+        xch, tw, [&](int f, int i) { return colb[f * N + i]; },
+        [&](int f, int i, V x) { colb[f * N + i] = cscale(x, scaled ? mul1(s, s2, green[f * N + i]) : green[f * N + i]); });
+    __syncthreads();
+    cl_fft<T, N, true>(
+        xch, tw, [&](int f, int i) { return colb[f * N + i]; },
+        [&](int f, int i, V x) { cl.map_shared_rank(rowb, i / R)[(i % R) * H1 + rank * K + f] = x; });
+  };
+  const T scale = (T)(1.0 / ((double)N * (double)N));
+  // rows of the result in u
+  auto rows_inv = [&]() {
+    cl_fft<T, N, true>(
+        xch, tw,
+        [&](int f, int k) {
+          const int kk = k < H1 ? k : (k > H1 ? N - k : 0);
+          V A = rowb[(2 * f) * H1 + kk], B = rowb[(2 * f + 1) * H1 + kk];
+          if (k > H1) { A = cconj(A); B = cconj(B); }
+          if (k == H1) A = B = mk<V>(0, 0);
+          return cadd(A, cmuli(B));
+        },
+        [&](int f, int i, V x) {
+          u[(2 * f) * N + i] = x.x * scale;
+          u[(2 * f + 1) * N + i] = x.y * scale;
+        });
+    __syncthreads();
+  };
+
+  // start: pressure scaled to the load (uniform where the guess carries none), its displacement, mean
+  // gap and G
+  {
+    double a = 0;
+    for (int i = tid; i < E; i += nth) {
+      h[i] = hg[i];
+      p[i] = pg[i];
+      t[i] = (T)0;
+      a += (double)p[i];
+    }
+    send(0, a, 0, 0, 0);
+    cl.sync();
+    if (tid < 32) {
+      const double sum = value(total(0), 0);
+      if (tid == 0) S.start = sum > 0 ? S.W / (S.dA * sum) : 0.0;
+    }
+    __syncthreads();
+    const double start = S.start, unif = S.unif;
+    for (int i = tid; i < E; i += nth) p[i] = start > 0 ? (T)(start * (double)p[i]) : (T)unif;
+    __syncthreads();
+    rows_fwd(p);
+    cl.sync();
+    cols(false);
+    cl.sync();
+    rows_inv();
+    double s0 = 0, s1 = 0;
+    for (int i = tid; i < E; i += nth)
+      if (p[i] > (T)0) {
+        s0 += (double)u[i] - (double)h[i];
+        s1 += 1;
+      }
+    send(1, s0, s1, 0, 0);
+    cl.sync();
+    if (tid < 32) {
+      const double x = total(1), sum = value(x, 0), n = value(x, 1);
+      if (tid == 0) {
+        S.nIc = n;
+        if (!(n > 0) || !isfinite(sum)) {
+          S.bad = 1;
+          S.done = 1;
+        } else {
+          S.gbar = sum / n;
+          S.gbar2 = pair_of(S.gbar);
+        }
+      }
+    }
+    __syncthreads();
+    double G = 0;
+    const double gbar = S.gbar;
+    for (int i = tid; i < E; i += nth)
+      if (p[i] > (T)0) {
+        const double gi = (double)u[i] - (double)h[i] - gbar;
+        G += gi * gi;
+      }
+    send(2, G, 0, 0, 0);
+    cl.sync();
+    if (tid < 32) {
+      G = value(total(2), 0);
+      if (tid == 0) S.G_old = G;
+    }
+    __syncthreads();
+  }
+
+  while (!S.done) {  // at most max_it passes; the same decision in every CTA
+    // g, conjugate direction
+    {
+      const double gbar = S.gbar, beta = S.beta;
+      const float2 gbar2 = S.gbar2, beta2 = S.beta2;
+      for (int i = tid; i < E; i += nth) {
+        const T gi = gap1(u[i], h[i], gbar, gbar2);
+        g[i] = gi;
+        t[i] = p[i] > (T)0 ? axpy1(gi, beta, beta2, t[i]) : (T)0;
+      }
+    }
+    __syncthreads();
+    rows_fwd(t);
+    cl.sync();
+    cols(false);
+    cl.sync();
+    rows_inv();
+    // step length
+    {
+      double a = 0, b = 0, c = 0, d = 0;
+      for (int i = tid; i < E; i += nth)
+        if (p[i] > (T)0) {
+          const double xi = (double)u[i], ti = (double)t[i];
+          a += xi;
+          b += ti;
+          c += (double)g[i] * ti;
+          d += xi * ti;
+        }
+      send(1, a, b, c, d);
+    }
+    cl.sync();
+    if (tid < 32) {
+      const double x = total(1), sr = value(x, 0), st = value(x, 1), sgt = value(x, 2), srt = value(x, 3);
+      if (tid == 0) {
+        const double den = srt * S.nIc - sr * st;
+        S.tau = den != 0 ? sgt * S.nIc / den : 0.0;
+        S.tau2 = pair_of(S.tau);
+      }
+    }
+    __syncthreads();
+    // pressure step
+    {
+      const double tau = S.tau;
+      const float2 mt = make_float2(-S.tau2.x, -S.tau2.y);
+      double a = 0;
+      int nol = 0;
+      for (int i = tid; i < E; i += nth) {
+        const T pi = p[i], ti = t[i], gi = g[i];
+        T pn = (T)0;
+        if (pi != (T)0 || ti != (T)0) {
+          const T x = axpy1(pi, -tau, mt, ti);
+          pn = x > (T)0 ? x : (T)0;
+        }
+        if (pn == (T)0 && gi < (T)0) {
+          pn = mul1(-tau, mt, gi);
+          ++nol;
+        }
+        po[i] = pi;
+        p[i] = pn;
+        if (pn != (T)0) a += (double)pn;
+      }
+      send(2, a, (double)nol, 0, 0);
+    }
+    __syncthreads();
+    rows_fwd(p);
+    cl.sync();
+    if (tid < 32) {
+      const double x = total(2), sum = value(x, 0), nol = value(x, 1);
+      if (tid == 0) {
+        S.delta = nol > 0 ? 0.0 : 1.0;
+        if (!(sum > 0) || !isfinite(sum)) {
+          S.bad = 1;
+          S.done = 1;
+        } else {
+          S.s = S.W / (S.dA * sum);
+          S.s2 = pair_of(S.s);
+        }
+      }
+    }
+    __syncthreads();
+    if (S.done) break;  // the same in every CTA
+    cols(true);
+    cl.sync();
+    rows_inv();
+    // load scale, change, mean gap and G
+    {
+      const double s = S.s, gbar = S.gbar;
+      const float2 s2 = S.s2;
+      double a = 0, b = 0, c = 0;
+      int n = 0;
+      for (int i = tid; i < E; i += nth) {
+        T pi = p[i];
+        if (pi != (T)0) {
+          pi = mul1(s, s2, pi);
+          p[i] = pi;
+        }
+        if (pi != po[i]) c += fabs((double)pi - (double)po[i]);
+        if (pi > (T)0) {
+          const double d = (double)u[i] - (double)h[i] - gbar;
+          a += d;
+          b += d * d;
+          ++n;
+        }
+      }
+      send(3, a, b, c, (double)n);
+    }
+    cl.sync();
+    if (tid < 32) {
+      const double x = total(3), sd = value(x, 0), sdd = value(x, 1), ch = value(x, 2), n = value(x, 3);
+      if (tid == 0) {
+        const double err = ch * S.dA_W;
+        int done = 0, bad = 0;
+        S.err = err;
+        S.it += 1;
+        if (err < S.tol || S.it >= S.max_it) done = 1;
+        if (!isfinite(err)) bad = 1;
+        S.nIc = n;
+        if (!done && (!(n > 0) || !isfinite(sd))) {
+          bad = 1;
+        } else {
+          const double mean = sd / n;
+          S.gbar += mean;
+          S.gbar2 = pair_of(S.gbar);
+          const double G = fmax(sdd - sd * mean, 0.0);
+          S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
+          S.beta2 = pair_of(S.beta);
+          S.G_old = G;
+        }
+        if (bad) S.bad = 1;
+        S.done = done | bad;
+      }
+    }
+    __syncthreads();
+  }
+  for (int i = tid; i < E; i += nth) pg[i] = p[i];
+  if (rank == 0 && tid == 0) *out = S;
+  cl.sync();  // no CTA leaves while another may still write to its shared memory
+}
+
+template <typename T, int N> int cluster_solve(const PkfArgs& a, const PkState& init) {
+  const double two_pi = 6.283185307179586476925;
+  // static shared memory besides: a constant cap below the opt-in maximum
+  static_assert(ClCfg<T, N>::bytes <= 200 * 1024, "surface in shared memory");
+  auto kern = k_pkf_cluster<T, N>;
+  if (FVIM_CU(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024))) return FVIM_ERR_CUDA;
+  kern<<<CL, ClCfg<T, N>::BT, ClCfg<T, N>::bytes, a.stream>>>(a.S, init, (const typename Cx<T>::t*)a.tw1,
+                                                            (T)(two_pi / a.L1), (T)(two_pi / a.L2), (T)a.nu, (T)a.mu);
+  FVIM_CUDA_CHECK_LAUNCH();
+  return FVIM_OK;
+}
+
 #define PKF_SIZES(X) X(16) X(32) X(64) X(128) X(256) X(512) X(1024)
 template <typename T, int MODE> void rows_fwd_any(const PkfArgs& a) {
 #define CASE(N) if (a.n1 == N) rows_fwd<T, N, MODE>(a);
@@ -385,6 +781,16 @@ template <typename T, bool SCALE> void cols_any(const PkfArgs& a) {
 inline int flat_grid(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 256); }
 
 }  // namespace
+
+bool pkf_small(const fvim_ctx* c) { return !c->gen && c->n1 == c->n2 && c->n1 >= 16 && c->n1 <= 128; }
+
+template <typename T> int pkf_solve_small(const PkfArgs& a, const PkState& init) {
+  if (a.n1 == 16) return cluster_solve<T, 16>(a, init);
+  if (a.n1 == 32) return cluster_solve<T, 32>(a, init);
+  if (a.n1 == 64) return cluster_solve<T, 64>(a, init);
+  if (a.n1 == 128) return cluster_solve<T, 128>(a, init);
+  return FVIM_ERR_UNSUPPORTED;
+}
 
 bool pkf_available(const fvim_ctx* c) { return !c->gen && c->n1 >= 16 && c->n2 >= 16; }
 
@@ -413,6 +819,8 @@ template <typename T> int pkf_iteration(const PkfArgs& a) {
   return FVIM_OK;
 }
 
+template int pkf_solve_small<float>(const PkfArgs&, const PkState&);
+template int pkf_solve_small<double>(const PkfArgs&, const PkState&);
 template int pkf_begin<float>(const PkfArgs&, const PkState&);
 template int pkf_begin<double>(const PkfArgs&, const PkState&);
 template int pkf_iteration<float>(const PkfArgs&);

@@ -494,8 +494,9 @@ __device__ __forceinline__ void fft_ct(V (&v)[NF][8], int t, const Sm& sm, const
 template <int N> struct OddLog2 {
   static constexpr bool v = (N & 0x55555555) == 0;
 };
+// on: threads without a transform (false) take part in the barriers only.
 template <typename V, bool INV, int N, int NS, class Sm>
-__device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V* __restrict__ tw) {
+__device__ __forceinline__ void fft4_on(V (&v)[4], int t, bool on, const Sm& sm, const V* __restrict__ tw) {
   constexpr int T4 = N / 4, R = (NS == 1 && OddLog2<N>::v) ? 2 : 4;
   int pos[4];
   if constexpr (R == 2) {
@@ -535,14 +536,20 @@ __device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V*
     for (int r = 0; r < 4; ++r) pos[r] = base + r * NS;
   }
   if constexpr (NS * R < N) {
+    if (on) {
 #pragma unroll
-    for (int m = 0; m < 4; ++m) sm.put(pos[m], v[m]);
+      for (int m = 0; m < 4; ++m) sm.put(pos[m], v[m]);
+    }
     __syncthreads();
 #pragma unroll
     for (int m = 0; m < 4; ++m) v[m] = sm.get(t + m * T4);
     __syncthreads();
-    fft4_ct<V, INV, N, NS * R>(v, t, sm, tw);
+    fft4_on<V, INV, N, NS * R>(v, t, on, sm, tw);
   }
+}
+template <typename V, bool INV, int N, int NS, class Sm>
+__device__ __forceinline__ void fft4_ct(V (&v)[4], int t, const Sm& sm, const V* __restrict__ tw) {
+  fft4_on<V, INV, N, NS>(v, t, true, sm, tw);
 }
 // rows: one pad slot every 8 entries
 template <typename V, int N> struct SurfSm {
@@ -885,6 +892,9 @@ struct PkfArgs {
   int use_cond;            // the last kernel of an iteration sets the loop condition
 };
 bool pkf_available(const fvim_ctx* c);
+// whole solve in one kernel (small square surfaces)
+bool pkf_small(const fvim_ctx* c);
+template <typename T> int pkf_solve_small(const PkfArgs& a, const PkState& init);
 // state, initial pressure scaled to the load, its displacement and mean gap
 template <typename T> int pkf_begin(const PkfArgs& a, const PkState& init);
 // one iteration; does nothing once the state's done flag is set

@@ -723,6 +723,16 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
   s0.max_it = o->cg_max_iter;
   PkState* sh = reinterpret_cast<PkState*>(c->h_part + (size_t)RMAXB * NVMAX);  // pinned
   int rc;
+  if (pkf_small(c)) {
+    if ((rc = pkf_solve_small<T>(a, s0))) return rc;
+    if (FVIM_CU(cudaMemcpyAsync(sh, a.S, sizeof(PkState), cudaMemcpyDeviceToHost, c->stream)) ||
+        FVIM_CU(cudaStreamSynchronize(c->stream)))
+      return FVIM_ERR_CUDA;
+    if (sh->bad) return FVIM_ERR_NONFINITE;
+    if (iters) *iters = sh->it;
+    if (err_out) *err_out = sh->err;
+    return sh->err < o->cg_tol ? FVIM_OK : FVIM_ERR_NOT_CONVERGED;
+  }
   if ((rc = pkf_begin<T>(a, s0))) return rc;
   SolverRT* srt = rt(c);
   bool ran_device = false;
