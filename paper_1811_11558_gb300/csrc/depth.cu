@@ -1180,7 +1180,7 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
     }
 #define DEPTHR(CV, UN, MBV, MBK)                                                                                \
   if (C == CV && (c->uniform != 0) == UN && d.mb == MBV) {                                                      \
-    smem_cap(k_mindlin_depth_r<T, 16, CV, UN, MBK>);                                                            \
+    smem_cap(k_mindlin_depth_r<T, 16, CV, UN, MBK>, d.smem);                                                            \
     k_mindlin_depth_r<T, 16, CV, UN, MBK><<<grid, d.threads, d.smem, c->stream>>>(                              \
         (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, nch, w1, w2, dm, eps_in ? 1 : 0, \
         want_u3 ? 1 : 0, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,    \
@@ -1196,7 +1196,7 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
   }
 #define DEPTH(KTV, LSV)                                                                                        \
   if (KT == KTV && (C <= 8) == LSV) {                                                                          \
-    smem_cap(k_mindlin_depth<T, KTV, LSV>);                                                                    \
+    smem_cap(k_mindlin_depth<T, KTV, LSV>, d.smem);                                                                    \
     k_mindlin_depth<T, KTV, LSV><<<grid, d.threads, d.smem, c->stream>>>(                                      \
         (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, w1, w2, dm,      \
         want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, eps_in ? 1 : 0);              \
@@ -1237,7 +1237,7 @@ int launch_grp_depth(GrpTable& t, cudaStream_t s) {
   }
   t.start[t.n] = b;
   if (b == 0) return FVIM_OK;
-  smem_cap(k_grp_depth);
+  smem_cap(k_grp_depth, smem);
   k_grp_depth<<<b, 256, smem, s>>>(t);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;

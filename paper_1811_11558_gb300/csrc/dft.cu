@@ -261,7 +261,7 @@ inline int dft_threads(int items) {
 template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, void* dst, size_t rows) {
   typedef typename Cx<T>::t V;
   const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
-  smem_cap(k_dft_rows_fwd<T>);
+  smem_cap(k_dft_rows_fwd<T>, smem);
   k_dft_rows_fwd<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * c->h1), smem, c->stream>>>(src, (V*)dst, (const V*)c->tw1, c->n1,
                                                                                 c->hs, c->h1, rows);
   FVIM_CUDA_CHECK_LAUNCH();
@@ -274,10 +274,10 @@ template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void*
   const int threads = dft_threads(CT / CC * (c->n2 / 2 + 1));
   dim3 grid(c->h1 / CT, nplanes);
   if (inverse) {
-    smem_cap(k_dft_cols<T, true>);
+    smem_cap(k_dft_cols<T, true>, smem);
     k_dft_cols<T, true><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
   } else {
-    smem_cap(k_dft_cols<T, false>);
+    smem_cap(k_dft_cols<T, false>, smem);
     k_dft_cols<T, false><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
   }
   FVIM_CUDA_CHECK_LAUNCH();
@@ -287,7 +287,7 @@ template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void*
 template <typename T> int launch_dft_rows_inv(const fvim_ctx* c, const void* src, T* dst, size_t rows, T scale) {
   typedef typename Cx<T>::t V;
   const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
-  smem_cap(k_dft_rows_inv<T>);
+  smem_cap(k_dft_rows_inv<T>, smem);
   k_dft_rows_inv<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * (c->n1 / 2 + 1)), smem, c->stream>>>((const V*)src, dst, (const V*)c->tw1,
                                                                                 c->n1, c->hs, c->h1, rows, scale);
   FVIM_CUDA_CHECK_LAUNCH();

@@ -687,7 +687,8 @@ inline int smem_optin_max() {
 }
 // dynamic shared memory cap of the row kernels (at most four FP64 transforms of 1024 points; they
 // hold static shared memory too, so not the whole opt-in maximum); the same value on every call
-template <typename K> inline void surf_row_smem_cap(K kern) {
+template <typename K> inline void surf_row_smem_cap(K kern, size_t smem) {
+  if (smem <= 40 * 1024) return;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
 }
 
@@ -701,7 +702,9 @@ inline int sm_count() {
   }();
   return v;
 }
-template <typename K> inline void smem_cap(K kern) {
+// Launches of at most 48 KB need no cap (a runtime call less on the host path of small grids).
+template <typename K> inline void smem_cap(K kern, size_t smem) {
+  if (smem <= 48 * 1024) return;
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin_max());
 }
 

@@ -180,7 +180,7 @@ template <int N, int CW> void bous_cols(const fvim_ctx* c, int out_kind) {
   const double two_pi = 6.283185307179586476925;
   const bool st = out_kind == FVIM_STRESS;
   const double e33 = -1.0 / (c->lam + 2.0 * c->mu);  // uniform pressure: the strain below it
-  smem_cap(k_bous_cols<N, CW>);
+  smem_cap(k_bous_cols<N, CW>, (size_t)N * CW * sizeof(float2));
   k_bous_cols<N, CW><<<dim3(c->h1 / CW, c->nz * 6), N / 16 * CW, (size_t)N * CW * sizeof(float2), c->stream>>>(
       (const float2*)c->surf, (float2*)c->spec, (const float2*)c->tw2, (const float*)c->z_dev, c->h1,
       (float)(two_pi / c->L1), (float)(two_pi / c->L2), (float)c->nu, st ? 1.f : (float)(0.5 / c->mu),
@@ -197,7 +197,7 @@ template <typename T> bool launch_surf_rows_fwd(const fvim_ctx* c, const T* f) {
 #define CASE(N)                                                                                                 \
   if (c->n1 == N) {                                                                                             \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                             \
-    smem_cap(k_surf_rows_fwd<T, N>);                                                                            \
+    smem_cap(k_surf_rows_fwd<T, N>, r.smem);                                                                            \
     k_surf_rows_fwd<T, N><<<r.grid, r.threads, r.smem, c->stream>>>(f, (V*)c->surf, (const V*)c->tw1, c->n2);   \
     return true;                                                                                                \
   }
@@ -211,7 +211,7 @@ template <typename T> bool launch_surf_rows_inv(const fvim_ctx* c, T* f, T scale
 #define CASE(N)                                                                                                       \
   if (c->n1 == N) {                                                                                                   \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                                   \
-    smem_cap(k_surf_rows_inv<T, N>);                                                                                  \
+    smem_cap(k_surf_rows_inv<T, N>, r.smem);                                                                                  \
     k_surf_rows_inv<T, N><<<r.grid, r.threads, r.smem, c->stream>>>((const V*)c->surf, f, (const V*)c->tw1, c->n2, scale); \
     return true;                                                                                                      \
   }
@@ -230,10 +230,10 @@ template <typename T> bool launch_surf_cols(const fvim_ctx* c, bool inverse) {
 #define CASE(N)                                                                                             \
   if (c->n2 == N) {                                                                                         \
     if (inverse) {                                                                                          \
-      smem_cap(k_surf_cols<T, N, true>);                                                                    \
+      smem_cap(k_surf_cols<T, N, true>, smem);                                                                    \
       k_surf_cols<T, N, true><<<c->h1 / kc, kc * (N / 4), smem, c->stream>>>((V*)c->surf, (const V*)c->tw2, c->h1, kc);  \
     } else {                                                                                                \
-      smem_cap(k_surf_cols<T, N, false>);                                                                   \
+      smem_cap(k_surf_cols<T, N, false>, smem);                                                                   \
       k_surf_cols<T, N, false><<<c->h1 / kc, kc * (N / 4), smem, c->stream>>>((V*)c->surf, (const V*)c->tw2, c->h1, kc); \
     }                                                                                                       \
     return true;                                                                                            \

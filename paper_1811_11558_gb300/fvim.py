@@ -155,19 +155,28 @@ def _check(status, what):
 
 
 def _ptr(t, dtype, shape, name):
-    import torch
-
+    """Device address of a contiguous CUDA tensor of this dtype and shape (None for None)."""
     if t is None:
         return None
+    import torch
+
     if not isinstance(t, torch.Tensor) or not t.is_cuda:
         raise TypeError("%s must be a CUDA tensor" % name)
     if t.dtype != dtype:
         raise TypeError("%s must be %s, got %s" % (name, dtype, t.dtype))
-    if tuple(t.shape) != tuple(shape):
+    if t.shape != shape:
         raise ValueError("%s must have shape %s, got %s" % (name, tuple(shape), tuple(t.shape)))
     if not t.is_contiguous():
         raise ValueError("%s must be contiguous" % name)
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+def _current_stream():
+    """Handle of torch's current stream on the current device (the raw handle: building the
+    Stream object took longer than two kernel launches)."""
+    import torch
+
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 GROUP_MAX = 64
@@ -187,10 +196,9 @@ def apply_mindlin_group(contexts, eps_list, out_list=None, kind="stress"):
     k = FVIM_STRESS if kind == "stress" else FVIM_STRAIN
     arr = ctypes.c_void_p * max(n, 1)
     hs = arr(*[c._h.value for c in contexts])
-    ins = arr(*[_ptr(e, c.dtype, c.vol_shape, "eps_p").value for c, e in zip(contexts, eps_list)])
-    outs = arr(*[_ptr(o, c.dtype, c.vol_shape, "out").value for c, o in zip(contexts, out_list)])
-    stream = ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    _check(lib().fvim_apply_mindlin_group(hs, n, ins, outs, k, stream), "fvim_apply_mindlin_group")
+    ins = arr(*[_ptr(e, c.dtype, c.vol_shape, "eps_p") for c, e in zip(contexts, eps_list)])
+    outs = arr(*[_ptr(o, c.dtype, c.vol_shape, "out") for c, o in zip(contexts, out_list)])
+    _check(lib().fvim_apply_mindlin_group(hs, n, ins, outs, k, _current_stream()), "fvim_apply_mindlin_group")
     return out_list
 
 
@@ -225,10 +233,7 @@ class Context:
 
     # -- plumbing -----------------------------------------------------------------
     def _stream(self):
-        import torch
-
-        _check(lib().fvim_set_stream(self._h, ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)),
-               "fvim_set_stream")
+        _check(lib().fvim_set_stream(self._h, _current_stream()), "fvim_set_stream")
 
     @property
     def vol_shape(self):
@@ -308,9 +313,9 @@ class Context:
         _check(lib().fvim_set_material(self._h, self.E, self.nu, sy, self.E_h), "fvim_set_material")
 
     def apply_mindlin(self, eps_p, out=None, kind="stress", u3=None):
-        import torch
-
         if out is None:
+            import torch
+
             out = torch.empty(self.vol_shape, dtype=self.dtype, device=eps_p.device)
         k = FVIM_STRESS if kind == "stress" else FVIM_STRAIN
         a = _ptr(eps_p, self.dtype, self.vol_shape, "eps_p")
