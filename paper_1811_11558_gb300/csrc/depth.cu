@@ -441,6 +441,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
                                 const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int C, int nch, T w1,
                                 T w2, const DepthMat<T> m, int want_u3, int uniform, T hz,
                                 const int* __restrict__ zr, int ein) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   constexpr int SL = LS ? 6 : 9, CM = LS ? 8 : 1;
   extern __shared__ __align__(128) unsigned char smraw[];  // one alignment for every kernel of this file
@@ -847,6 +848,7 @@ __global__ void __launch_bounds__(256, MB) k_mindlin_depth_r(typename Cx<T>::t* 
                                                             T hz, const int* __restrict__ zr, T cut,
                                                             const __grid_constant__ CUtensorMap tmap, int tma_rows,
                                                             int tx_extra, int* __restrict__ status) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   static_assert(sizeof(V) == 8 && KT % 2 == 0, "FP32 tiles of an even width");
   extern __shared__ __align__(128) unsigned char smraw[];  // tensor-copy boxes land at 128-byte offsets
@@ -938,6 +940,7 @@ inline __host__ __device__ size_t grp_depth_slot(int nz, int nchp, int uniform) 
 }
 
 __global__ void __launch_bounds__(256, 2) k_grp_depth(const __grid_constant__ GrpTable tab) {
+  chain_begin();
   typedef float2 V;
   constexpr int KT = 16, C = 4;
   extern __shared__ __align__(128) unsigned char smraw[];
@@ -1024,6 +1027,7 @@ template <typename T>
 __global__ void k_boussinesq(typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
                              const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, T w1, T w2, T lam,
                              T mu, T nu, int out_kind, int want_vol, int want_u3) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   const int k1 = blockIdx.x * blockDim.x + threadIdx.x;
   const int k2 = blockIdx.y;
@@ -1181,7 +1185,7 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
 #define DEPTHR(CV, UN, MBV, MBK)                                                                                \
   if (C == CV && (c->uniform != 0) == UN && d.mb == MBV) {                                                      \
     smem_cap(k_mindlin_depth_r<T, 16, CV, UN, MBK>, d.smem);                                                            \
-    k_mindlin_depth_r<T, 16, CV, UN, MBK><<<grid, d.threads, d.smem, c->stream>>>(                              \
+    launch_chain(c, k_mindlin_depth_r<T, 16, CV, UN, MBK>, grid, d.threads, d.smem,                               \
         (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, nch, w1, w2, dm, eps_in ? 1 : 0, \
         want_u3 ? 1 : 0, (T)c->hz, zr, (T)c->depth_cut, tm, tma_rows, c->tma_test_extra,    \
         c->dev_status);                                                                                          \
@@ -1197,7 +1201,7 @@ int launch_mindlin_depth(const fvim_ctx* c, int out_kind, bool want_u3, bool eps
 #define DEPTH(KTV, LSV)                                                                                        \
   if (KT == KTV && (C <= 8) == LSV) {                                                                          \
     smem_cap(k_mindlin_depth<T, KTV, LSV>, d.smem);                                                                    \
-    k_mindlin_depth<T, KTV, LSV><<<grid, d.threads, d.smem, c->stream>>>(                                      \
+    launch_chain(c, k_mindlin_depth<T, KTV, LSV>, grid, d.threads, d.smem,                                       \
         (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, nz, c->n1, n2, c->hs, h1, C, nch, w1, w2, dm,      \
         want_u3 ? 1 : 0, c->uniform, (T)c->hz, zr, eps_in ? 1 : 0);              \
   }
@@ -1212,7 +1216,7 @@ template <typename T> int launch_boussinesq(const fvim_ctx* c, int out_kind, boo
   typedef typename Cx<T>::t V;
   const int threads = 128;
   dim3 grid((c->h1 + threads - 1) / threads, c->n2);
-  k_boussinesq<T><<<grid, threads, 0, c->stream>>>((V*)c->spec, (V*)c->surf, (const T*)c->z_dev, c->nz, c->n1, c->n2,
+  launch_chain(c, k_boussinesq<T>, grid, threads, 0, (V*)c->spec, (V*)c->surf, (const T*)c->z_dev, c->nz, c->n1, c->n2,
                                                    c->hs, c->h1,
                                                    (T)(kTwoPi / c->L1), (T)(kTwoPi / c->L2), (T)c->lam, (T)c->mu, (T)c->nu,
                                                    out_kind, want_vol ? 1 : 0, want_u3 ? 1 : 0);
@@ -1238,7 +1242,7 @@ int launch_grp_depth(GrpTable& t, cudaStream_t s) {
   t.start[t.n] = b;
   if (b == 0) return FVIM_OK;
   smem_cap(k_grp_depth, smem);
-  k_grp_depth<<<b, 256, smem, s>>>(t);
+  launch_chain_on(s, true, k_grp_depth, b, 256, smem, t);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
 }

@@ -66,6 +66,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_dft_rows_fwd(const T* __restrict__ src, typename Cx<T>::t* __restrict__ dst,
                                                       const typename Cx<T>::t* __restrict__ tw, int n1, int hs,
                                                       int ldh, size_t rows) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int LD = RowLd<T>::v;
@@ -127,6 +128,7 @@ __global__ void __launch_bounds__(256) k_dft_rows_fwd(const T* __restrict__ src,
 template <typename T, bool INV>
 __global__ void __launch_bounds__(256) k_dft_cols(typename Cx<T>::t* __restrict__ spec,
                                                   const typename Cx<T>::t* __restrict__ tw, int n2, int ldh) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   const int H = n2 / 2, J = (n2 - 1) / 2;
@@ -193,6 +195,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_dft_rows_inv(const typename Cx<T>::t* __restrict__ src, T* __restrict__ dst,
                                                       const typename Cx<T>::t* __restrict__ tw, int n1, int hs,
                                                       int ldh, size_t rows, T scale) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int LD = RowLd<T>::v;
@@ -262,7 +265,7 @@ template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, v
   typedef typename Cx<T>::t V;
   const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
   smem_cap(k_dft_rows_fwd<T>, smem);
-  k_dft_rows_fwd<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * c->h1), smem, c->stream>>>(src, (V*)dst, (const V*)c->tw1, c->n1,
+  launch_chain(c, k_dft_rows_fwd<T>, (unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * c->h1), smem, src, (V*)dst, (const V*)c->tw1, c->n1,
                                                                                 c->hs, c->h1, rows);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -275,10 +278,10 @@ template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void*
   dim3 grid(c->h1 / CT, nplanes);
   if (inverse) {
     smem_cap(k_dft_cols<T, true>, smem);
-    k_dft_cols<T, true><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
+    launch_chain(c, k_dft_cols<T, true>, grid, threads, smem, (V*)planes, (const V*)c->tw2, c->n2, c->h1);
   } else {
     smem_cap(k_dft_cols<T, false>, smem);
-    k_dft_cols<T, false><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->n2, c->h1);
+    launch_chain(c, k_dft_cols<T, false>, grid, threads, smem, (V*)planes, (const V*)c->tw2, c->n2, c->h1);
   }
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -288,7 +291,7 @@ template <typename T> int launch_dft_rows_inv(const fvim_ctx* c, const void* src
   typedef typename Cx<T>::t V;
   const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
   smem_cap(k_dft_rows_inv<T>, smem);
-  k_dft_rows_inv<T><<<(unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * (c->n1 / 2 + 1)), smem, c->stream>>>((const V*)src, dst, (const V*)c->tw1,
+  launch_chain(c, k_dft_rows_inv<T>, (unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * (c->n1 / 2 + 1)), smem, (const V*)src, dst, (const V*)c->tw1,
                                                                                 c->n1, c->hs, c->h1, rows, scale);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;

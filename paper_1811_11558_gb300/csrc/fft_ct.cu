@@ -48,6 +48,7 @@ template <typename T, bool INV, int N>
 __global__ void __launch_bounds__(512) k_cols_ct(typename Cx<T>::t* __restrict__ planes,
                                                  const typename Cx<T>::t* __restrict__ tw, int h1, int kc,
                                                  const int* __restrict__ zr) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   if (zr && ((int)blockIdx.y / 6 < zr[0] || (int)blockIdx.y / 6 >= zr[1])) return;  // layer without input
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -123,6 +124,7 @@ __device__ __forceinline__ void cols_v_body(float2* __restrict__ planes, const f
 template <bool INV, int N, int CW>
 __global__ void __launch_bounds__(ColsV<N, CW>::threads, ColsV<N, CW>::min_blocks)
     k_cols_v(float2* __restrict__ planes, const float2* __restrict__ tw, int h1, const int* __restrict__ zr) {
+  chain_begin();
   if (zr && ((int)blockIdx.y / 6 < zr[0] || (int)blockIdx.y / 6 >= zr[1])) return;  // layer without input
   extern __shared__ __align__(16) unsigned char smraw[];
   cols_v_body<INV, N, CW>(planes, tw, h1, blockIdx.y, blockIdx.x, threadIdx.x, reinterpret_cast<float2*>(smraw), true);
@@ -136,6 +138,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(512) k_cols_conv(typename Cx<T>::t* __restrict__ plane,
                                                    const typename Cx<T>::t* __restrict__ tw, int h1, int kc, T w1,
                                                    T w2, T nu, T mu) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8;
@@ -182,6 +185,7 @@ template <typename T, int N, int NF>
 __global__ void __launch_bounds__(256) k_rows_fwd6_ct(const T* __restrict__ eps_p, typename Cx<T>::t* __restrict__ spec,
                                                       T* __restrict__ nq, const typename Cx<T>::t* __restrict__ tw,
                                                       int n2, int rb, int z0, T hlam, T hmu2, const int* __restrict__ zr) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8, LD = RowLayout<V, N>::LD, H1 = N / 2;
@@ -287,6 +291,7 @@ __global__ void __launch_bounds__(256) k_rows_inv6_ct(const typename Cx<T>::t* _
                                                       const T* __restrict__ nq, T* __restrict__ out,
                                                       const typename Cx<T>::t* __restrict__ tw, int n2, int rb, int z0,
                                                       T nq_scale, T scale) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8, LD = RowLayout<V, N>::LD;
@@ -386,6 +391,7 @@ template <int N>
 __global__ void __launch_bounds__(256) k_rows_fwd6_v(const float* __restrict__ eps_p, float2* __restrict__ spec,
                                                      float* __restrict__ nq, const float2* __restrict__ tw, int n2,
                                                      int rb, int z0, float lam, float mu, const int* __restrict__ zr) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int z = z0 + blockIdx.y;
   if (zr && (z < zr[0] || z >= zr[1])) return;  // layer without input
@@ -408,11 +414,11 @@ template <int N, int CW> void cols_v_launch(const fvim_ctx* c, bool inverse, voi
   const size_t sm = (size_t)N * CW * sizeof(float2);
   if (inverse) {
     smem_attr(k_cols_v<true, N, CW>, sm);
-    k_cols_v<true, N, CW><<<grid, ColsV<N, CW>::threads, sm, c->stream>>>((float2*)planes, (const float2*)c->tw2,
+    launch_chain(c, k_cols_v<true, N, CW>, grid, ColsV<N, CW>::threads, sm, (float2*)planes, (const float2*)c->tw2,
                                                                           c->h1, zr);
   } else {
     smem_attr(k_cols_v<false, N, CW>, sm);
-    k_cols_v<false, N, CW><<<grid, ColsV<N, CW>::threads, sm, c->stream>>>((float2*)planes, (const float2*)c->tw2,
+    launch_chain(c, k_cols_v<false, N, CW>, grid, ColsV<N, CW>::threads, sm, (float2*)planes, (const float2*)c->tw2,
                                                                            c->h1, zr);
   }
 }
@@ -440,10 +446,10 @@ template <typename T, int N> void cols_n(const fvim_ctx* c, bool inverse, void* 
   dim3 grid(c->h1 / kc, nplanes);
   if (inverse) {
     smem_attr(k_cols_ct<T, true, N>, smem);
-    k_cols_ct<T, true, N><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->h1, kc, zr);
+    launch_chain(c, k_cols_ct<T, true, N>, grid, threads, smem, (V*)planes, (const V*)c->tw2, c->h1, kc, zr);
   } else {
     smem_attr(k_cols_ct<T, false, N>, smem);
-    k_cols_ct<T, false, N><<<grid, threads, smem, c->stream>>>((V*)planes, (const V*)c->tw2, c->h1, kc, zr);
+    launch_chain(c, k_cols_ct<T, false, N>, grid, threads, smem, (V*)planes, (const V*)c->tw2, c->h1, kc, zr);
   }
 }
 
@@ -461,7 +467,7 @@ template <typename T, int N> void rows_fwd_n(const fvim_ctx* c, const T* eps_p, 
     const size_t sm = std::max((size_t)rb * 3 * RowLayout<V, N>::LD * sizeof(V), (size_t)6 * rb * StageLd<N>::v * sizeof(T));
     dim3 grid(c->n2 / rb, nzs);
     smem_attr(k_rows_fwd6_v<N>, sm);
-    k_rows_fwd6_v<N><<<grid, rb * (N / 8), sm, c->stream>>>((const float*)eps_p, (float2*)c->spec, (float*)c->nq,
+    launch_chain(c, k_rows_fwd6_v<N>, grid, rb * (N / 8), sm, (const float*)eps_p, (float2*)c->spec, (float*)c->nq,
                                                             (const float2*)c->tw1, c->n2, rb, z0, (float)c->lam,
                                                             (float)c->mu, zr);
     return;
@@ -469,7 +475,7 @@ template <typename T, int N> void rows_fwd_n(const fvim_ctx* c, const T* eps_p, 
   auto go = [&](auto kern, int nf) {
     const size_t smem = (size_t)rb * nf * RowLayout<V, N>::LD * sizeof(V);
     smem_attr(kern, smem);
-    kern<<<dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, c->stream>>>(eps_p, (V*)c->spec, (T*)c->nq, (const V*)c->tw1,
+    launch_chain(c, kern, dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, eps_p, (V*)c->spec, (T*)c->nq, (const V*)c->tw1,
                                                                          c->n2, rb, z0, (T)(0.5 * c->lam), (T)c->mu, zr);
   };
   if constexpr (sizeof(T) == 8) {
@@ -490,7 +496,7 @@ template <typename T, int N> void rows_inv_n(const fvim_ctx* c, T* out, T nq_sca
   auto go = [&](auto kern, int nf) {
     const size_t smem = (size_t)rb * nf * RowLayout<V, N>::LD * sizeof(V);
     smem_attr(kern, smem);
-    kern<<<dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, c->stream>>>((const V*)c->spec, (const T*)c->nq, out,
+    launch_chain(c, kern, dim3(c->n2 / rb, nzs, 3 / nf), rb * (N / 8), smem, (const V*)c->spec, (const T*)c->nq, out,
                                                                          (const V*)c->tw1, c->n2, rb, z0, nq_scale, scale);
   };
   if constexpr (sizeof(T) == 8) {
@@ -519,6 +525,7 @@ template <int N> __device__ __forceinline__ void grp_rows_fwd_case(const GrpProb
 }
 
 __global__ void __launch_bounds__(256) k_grp_rows_fwd(const __grid_constant__ GrpTable tab) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int pi = grp_find(tab, blockIdx.x);
   const GrpProb& P = tab.p[pi];
@@ -542,6 +549,7 @@ template <int N> __device__ __forceinline__ void grp_rows_inv_case(const GrpProb
 }
 
 __global__ void __launch_bounds__(128) k_grp_rows_inv(const __grid_constant__ GrpTable tab) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int pi = grp_find(tab, blockIdx.x);
   const GrpProb& P = tab.p[pi];
@@ -568,6 +576,7 @@ __device__ __forceinline__ void grp_cols_case(const GrpProb& P, int local, unsig
 }
 
 template <bool INV> __global__ void __launch_bounds__(512, 2) k_grp_cols(const __grid_constant__ GrpTable tab) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   const int pi = grp_find(tab, blockIdx.x);
   const GrpProb& P = tab.p[pi];
@@ -604,7 +613,7 @@ template <typename T, int N> void cols_conv_n(const fvim_ctx* c) {
   const size_t smem = (size_t)kc * N * sizeof(V);
   smem_attr(k_cols_conv<T, N>, smem);
   const double two_pi = 6.283185307179586476925;
-  k_cols_conv<T, N><<<c->h1 / kc, kc * (N / 8), smem, c->stream>>>(
+  launch_chain(c, k_cols_conv<T, N>, c->h1 / kc, kc * (N / 8), smem, 
       (V*)c->surf, (const V*)c->tw2, c->h1, kc, (T)(two_pi / c->L1), (T)(two_pi / c->L2), (T)c->nu, (T)c->mu);
 }
 
@@ -659,7 +668,7 @@ int launch_grp_rows_fwd(GrpTable& t, cudaStream_t s) {
   t.start[t.n] = b;
   if (b == 0) return FVIM_OK;
   smem_attr(k_grp_rows_fwd, kGrpRowsFwdSmem);
-  k_grp_rows_fwd<<<b, 256, kGrpRowsFwdSmem, s>>>(t);
+  launch_chain_on(s, true, k_grp_rows_fwd, b, 256, kGrpRowsFwdSmem, t);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
 }
@@ -673,7 +682,7 @@ int launch_grp_rows_inv(GrpTable& t, cudaStream_t s) {
   t.start[t.n] = b;
   if (b == 0) return FVIM_OK;
   smem_attr(k_grp_rows_inv, kGrpRowsInvSmem);
-  k_grp_rows_inv<<<b, 128, kGrpRowsInvSmem, s>>>(t);
+  launch_chain_on(s, true, k_grp_rows_inv, b, 128, kGrpRowsInvSmem, t);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
 }
@@ -689,10 +698,10 @@ int launch_grp_cols(GrpTable& t, bool inverse, cudaStream_t s) {
   if (b == 0) return FVIM_OK;
   if (inverse) {
     smem_attr(k_grp_cols<true>, kGrpColsSmem);
-    k_grp_cols<true><<<b, 512, kGrpColsSmem, s>>>(t);
+    launch_chain_on(s, true, k_grp_cols<true>, b, 512, kGrpColsSmem, t);
   } else {
     smem_attr(k_grp_cols<false>, kGrpColsSmem);
-    k_grp_cols<false><<<b, 512, kGrpColsSmem, s>>>(t);
+    launch_chain_on(s, true, k_grp_cols<false>, b, 512, kGrpColsSmem, t);
   }
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;

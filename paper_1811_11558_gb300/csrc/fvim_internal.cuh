@@ -5,6 +5,9 @@
 #include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
+
+#include <utility>
 
 #include "fvim.h"
 
@@ -714,6 +717,7 @@ template <typename K> inline void smem_cap(K kern, size_t smem) {
 #define FVIM_NSOLVER_BUFS 26
 
 struct fvim_ctx {
+  int no_pdl;  // launches without the programmatic-serialisation attribute (solver graph capture)
   // h1: row stride of the half spectrum (complex); power-of-two grids: N1/2 columns (the
   // k1 = N1/2 coefficient kept apart in nq); gen: floor(N1/2) + 1 columns rounded up to 16
   int n1, n2, nz, h1;
@@ -759,6 +763,44 @@ struct fvim_ctx {
   int fft_path;    // in-plane FFT path chosen by the tuner or fvim_set_plan (FVIM_FFT_*), -1: none
                    // (the row / column kernels unless an environment variable selects another)
 };
+
+// ---------------------------------------------------------------------------
+// Chained launches.  The kernels of an apply depend on one another in stream order, and from one
+// stream launch to the next a dependent kernel starts about 4.5 us later, which is all the time there
+// is on small grids.  They are launched with programmatic stream serialisation: a kernel may be
+// placed on the device when the CTAs of the one before have left it, and chain_begin() - the first
+// statement of every such kernel, before any global access and any return - waits until that one is
+// complete and its writes are visible (so completion of a kernel implies completion of everything
+// before it).  There is no earlier trigger: placed from the start of the kernel before, the next
+// kernel's CTAs crowd the SMs that drain first (81 x 81 x 32 73 us against 53, a captured 64 x 64 x 8
+// apply 15.1 us against 11.1).  Applies, us, plain launches -> chained: 64 x 64 x 8 22.5 -> 13.6,
+// 128 x 128 x 32 with u3 48.1 -> 33.2, 81 x 81 x 32 64 -> 53, 256 x 128 x 57 94 -> 80, 512 x 512 x 64
+// 672 -> 661, grouped 823 -> 805.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chain_on(cudaStream_t stream, bool chained, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                            A&&... args) {
+  cudaLaunchConfig_t cfg;
+  memset(&cfg, 0, sizeof(cfg));
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cudaLaunchAttribute at;
+  memset(&at, 0, sizeof(at));
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = chained ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
+template <typename... P, typename... A>
+inline void launch_chain(const fvim_ctx* c, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, A&&... args) {
+  launch_chain_on(c->stream, !c->no_pdl, kern, grid, block, smem, std::forward<A>(args)...);
+}
 
 // tile plan of the depth kernel (depth.cu): default chunk length, and whether a chunk length
 // gives a launchable configuration on this context's grid and precision

@@ -227,7 +227,9 @@ template <class F> static int build_while_graph(fvim_ctx* c, F&& body, cudaGraph
     cudaGraphDestroy(g);
     return FVIM_ERR_CUDA;
   }
+  c->no_pdl = 1;
   const int rc = body(cond);
+  c->no_pdl = 0;
   cudaGraph_t captured = nullptr;
   const cudaError_t ce = cudaStreamEndCapture(c->stream, &captured);
   if (rc != FVIM_OK || FVIM_CU(ce)) {

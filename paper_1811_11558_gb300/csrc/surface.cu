@@ -11,6 +11,7 @@ namespace {
 template <typename T, int N>
 __global__ void __launch_bounds__(512) k_surf_rows_fwd(const T* __restrict__ f, typename Cx<T>::t* __restrict__ surf,
                                                        const typename Cx<T>::t* __restrict__ tw, int n2) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
@@ -42,6 +43,7 @@ __global__ void __launch_bounds__(512) k_surf_rows_fwd(const T* __restrict__ f, 
 template <typename T, int N>
 __global__ void __launch_bounds__(512) k_surf_rows_inv(const typename Cx<T>::t* __restrict__ surf, T* __restrict__ f,
                                                        const typename Cx<T>::t* __restrict__ tw, int n2, T scale) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
@@ -73,6 +75,7 @@ __global__ void __launch_bounds__(512) k_surf_rows_inv(const typename Cx<T>::t* 
 template <typename T, int N, bool INV>
 __global__ void __launch_bounds__(512) k_surf_cols(typename Cx<T>::t* __restrict__ plane,
                                                    const typename Cx<T>::t* __restrict__ tw, int h1, int kc) {
+  chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T4 = N / 4;
@@ -144,6 +147,7 @@ __global__ void __launch_bounds__(N / 16 * CW, 1024 / (N / 16 * CW) > 0 ? 1024 /
     k_bous_cols(const float2* __restrict__ surf, float2* __restrict__ spec, const float2* __restrict__ tw,
                 const float* __restrict__ zn, int h1, float w1, float w2, float nu, float sc, float zero33, float zero11,
                 int stress) {
+  chain_begin();
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T8 = N / 8, NP = CW / 2;
   const int f2 = threadIdx.x % NP, t = threadIdx.x / NP;
@@ -181,7 +185,7 @@ template <int N, int CW> void bous_cols(const fvim_ctx* c, int out_kind) {
   const bool st = out_kind == FVIM_STRESS;
   const double e33 = -1.0 / (c->lam + 2.0 * c->mu);  // uniform pressure: the strain below it
   smem_cap(k_bous_cols<N, CW>, (size_t)N * CW * sizeof(float2));
-  k_bous_cols<N, CW><<<dim3(c->h1 / CW, c->nz * 6), N / 16 * CW, (size_t)N * CW * sizeof(float2), c->stream>>>(
+  launch_chain(c, k_bous_cols<N, CW>, dim3(c->h1 / CW, c->nz * 6), N / 16 * CW, (size_t)N * CW * sizeof(float2), 
       (const float2*)c->surf, (float2*)c->spec, (const float2*)c->tw2, (const float*)c->z_dev, c->h1,
       (float)(two_pi / c->L1), (float)(two_pi / c->L2), (float)c->nu, st ? 1.f : (float)(0.5 / c->mu),
       st ? -1.f : (float)e33, st ? (float)(c->lam * e33) : 0.f, st ? 1 : 0);
@@ -198,7 +202,7 @@ template <typename T> bool launch_surf_rows_fwd(const fvim_ctx* c, const T* f) {
   if (c->n1 == N) {                                                                                             \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                             \
     smem_cap(k_surf_rows_fwd<T, N>, r.smem);                                                                            \
-    k_surf_rows_fwd<T, N><<<r.grid, r.threads, r.smem, c->stream>>>(f, (V*)c->surf, (const V*)c->tw1, c->n2);   \
+    launch_chain(c, k_surf_rows_fwd<T, N>, r.grid, r.threads, r.smem, f, (V*)c->surf, (const V*)c->tw1, c->n2);   \
     return true;                                                                                                \
   }
   SURF_SIZES(CASE)
@@ -212,7 +216,7 @@ template <typename T> bool launch_surf_rows_inv(const fvim_ctx* c, T* f, T scale
   if (c->n1 == N) {                                                                                                   \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                                   \
     smem_cap(k_surf_rows_inv<T, N>, r.smem);                                                                                  \
-    k_surf_rows_inv<T, N><<<r.grid, r.threads, r.smem, c->stream>>>((const V*)c->surf, f, (const V*)c->tw1, c->n2, scale); \
+    launch_chain(c, k_surf_rows_inv<T, N>, r.grid, r.threads, r.smem, (const V*)c->surf, f, (const V*)c->tw1, c->n2, scale); \
     return true;                                                                                                      \
   }
   SURF_SIZES(CASE)
@@ -231,10 +235,10 @@ template <typename T> bool launch_surf_cols(const fvim_ctx* c, bool inverse) {
   if (c->n2 == N) {                                                                                         \
     if (inverse) {                                                                                          \
       smem_cap(k_surf_cols<T, N, true>, smem);                                                                    \
-      k_surf_cols<T, N, true><<<c->h1 / kc, kc * (N / 4), smem, c->stream>>>((V*)c->surf, (const V*)c->tw2, c->h1, kc);  \
+      launch_chain(c, k_surf_cols<T, N, true>, c->h1 / kc, kc * (N / 4), smem, (V*)c->surf, (const V*)c->tw2, c->h1, kc);  \
     } else {                                                                                                \
       smem_cap(k_surf_cols<T, N, false>, smem);                                                                   \
-      k_surf_cols<T, N, false><<<c->h1 / kc, kc * (N / 4), smem, c->stream>>>((V*)c->surf, (const V*)c->tw2, c->h1, kc); \
+      launch_chain(c, k_surf_cols<T, N, false>, c->h1 / kc, kc * (N / 4), smem, (V*)c->surf, (const V*)c->tw2, c->h1, kc); \
     }                                                                                                       \
     return true;                                                                                            \
   }
