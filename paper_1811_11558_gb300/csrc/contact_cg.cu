@@ -113,44 +113,54 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
   V v[4];
   double sum[4] = {0, 0, 0, 0};
   int nol = 0;
-  auto value = [&](size_t i) -> T {
+  // the thread's eight points (four places in two rows), read together before anything is stored: with
+  // loads and stores in turn each point waited for memory by itself
+  auto at = [&](int e) { return i0 + (size_t)(e >> 1) * T4 + (size_t)(e & 1) * N; };
+  T a[8], b[8], c[8], d[8], x[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    a[e] = b[e] = c[e] = d[e] = x[e] = (T)0;
+    if (live) {
+      a[e] = p[at(e)];
+      if (MODE != FWD_INIT) b[e] = t[at(e)];
+      if (MODE == FWD_P) c[e] = g[at(e)];
+      if (MODE == FWD_T) {
+        c[e] = u[at(e)];
+        d[e] = h[at(e)];
+      }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    if (!live) break;
     if constexpr (MODE == FWD_INIT) {
-      const T x = start > 0 ? (T)(start * (double)p[i]) : (T)unif;
-      p[i] = x;
-      t[i] = (T)0;
-      return x;
+      x[e] = start > 0 ? (T)(start * (double)a[e]) : (T)unif;
+      p[at(e)] = x[e];
+      t[at(e)] = (T)0;
     } else if constexpr (MODE == FWD_P) {
-      const T po = p[i], ti = t[i], gi = g[i];
+      const T po = a[e], gi = c[e];
       T pn = (T)0;
-      if (po != (T)0 || ti != (T)0) {
-        const T x = axpy1(po, -tau, make_float2(-tau2.x, -tau2.y), ti);
-        pn = x > (T)0 ? x : (T)0;
+      if (po != (T)0 || b[e] != (T)0) {
+        const T y = axpy1(po, -tau, make_float2(-tau2.x, -tau2.y), b[e]);
+        pn = y > (T)0 ? y : (T)0;
       }
       if (pn == (T)0 && gi < (T)0) {
         pn = mul1(-tau, make_float2(-tau2.x, -tau2.y), gi);
         ++nol;
       }
-      pold[i] = po;
-      p[i] = pn;
+      pold[at(e)] = po;
+      p[at(e)] = pn;
       if (pn != (T)0) sum[0] += (double)pn;
-      return pn;
+      x[e] = pn;
     } else {
-      const T gi = gap1(u[i], h[i], gbar, gbar2);
-      g[i] = gi;
-      const T x = p[i] > (T)0 ? axpy1(gi, beta, beta2, t[i]) : (T)0;
-      t[i] = x;
-      return x;
-    }
-  };
-#pragma unroll
-  for (int m = 0; m < 4; ++m) {
-    v[m] = mk<V>(0, 0);
-    if (live) {
-      const size_t i = i0 + m * T4;
-      v[m].x = value(i);
-      v[m].y = value(i + N);
+      const T gi = gap1(c[e], d[e], gbar, gbar2);
+      g[at(e)] = gi;
+      x[e] = a[e] > (T)0 ? axpy1(gi, beta, beta2, b[e]) : (T)0;
+      t[at(e)] = x[e];
     }
   }
+#pragma unroll
+  for (int m = 0; m < 4; ++m) v[m] = mk<V>(x[2 * m], x[2 * m + 1]);
   SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
   fft4_ct<V, false, N, 1>(v, tt, sm, tw);
   // separation of the two rows: Z(N - k) of k = tt + m N/4, m < 2, is in another thread's upper half
@@ -235,6 +245,20 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   const bool live = pair < n2 / 2;
   T* p = static_cast<T*>(S->p);
   const T* h = static_cast<const T*>(S->h);
+  const size_t i0 = (size_t)(live ? 2 * pair : 0) * N + tt;
+  auto at = [&](int e) { return i0 + (size_t)(e >> 1) * T4 + (size_t)(e & 1) * N; };
+  // what the elementwise step needs at the thread's eight points, in flight during the transform
+  T fp[8], fa[8], fb[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    fp[e] = fa[e] = fb[e] = (T)0;
+    if (live) {
+      fp[e] = p[at(e)];
+      fa[e] = MODE == INV_R ? t[at(e)] : h[at(e)];
+      if (MODE == INV_R) fb[e] = g[at(e)];
+      if (MODE == INV_U) fb[e] = pold[at(e)];
+    }
+  }
   V v[4];
   const V* sa = surf + (size_t)(live ? 2 * pair : 0) * H1;
 #pragma unroll
@@ -248,44 +272,38 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   }
   const SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
   fft4_ct<V, true, N, 1>(v, tt, sm, tw);
-  const size_t i0 = (size_t)(live ? 2 * pair : 0) * N + tt;
   const double scl = S->s, gbar = S->gbar;
   const float2 scl2 = S->s2;
   double sum[4] = {0, 0, 0, 0};
   int nc = 0;
-  auto add = [&](size_t i, T x) {
+#pragma unroll
+  for (int e = 0; e < 8; ++e) {
+    if (!live) break;
+    const T x = ((e & 1) ? v[e >> 1].y : v[e >> 1].x) * scale;
     if constexpr (MODE == INV_R) {
-      if (p[i] > (T)0) {
-        const double xi = (double)x, ti = (double)t[i];
+      if (fp[e] > (T)0) {
+        const double xi = (double)x, ti = (double)fa[e];
         sum[0] += xi;
         sum[1] += ti;
-        sum[2] += (double)g[i] * ti;
+        sum[2] += (double)fb[e] * ti;
         sum[3] += xi * ti;
       }
     } else {
-      T pi = p[i];
+      T pi = fp[e];
       if constexpr (MODE == INV_U) {
-        const T po = pold[i];
         if (pi != (T)0) {
           pi = mul1(scl, scl2, pi);
-          p[i] = pi;
+          p[at(e)] = pi;
         }
-        if (pi != po) sum[2] += fabs((double)pi - (double)po);
+        if (pi != fb[e]) sum[2] += fabs((double)pi - (double)fb[e]);
       }
-      u[i] = x;
+      u[at(e)] = x;
       if (pi > (T)0) {
-        const double d = MODE == INV_U ? (double)x - (double)h[i] - gbar : (double)x - (double)h[i];
+        const double d = MODE == INV_U ? (double)x - (double)fa[e] - gbar : (double)x - (double)fa[e];
         sum[0] += d;
         if (MODE == INV_U) sum[1] += d * d;
         ++nc;
       }
-    }
-  };
-  if (live) {
-#pragma unroll
-    for (int m = 0; m < 4; ++m) {
-      add(i0 + m * T4, v[m].x * scale);
-      add(i0 + m * T4 + N, v[m].y * scale);
     }
   }
   if (MODE != INV_R) sum[3] = (double)nc;
