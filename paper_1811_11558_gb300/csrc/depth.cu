@@ -195,7 +195,7 @@ __device__ __forceinline__ ModeGeom<T> mode_geom(int k1, int k2, int n1, int n2,
 template <typename T> struct __align__(16) ColIn {
   T E, a, b0, b1, d0, d1;        // element coefficients of a uniform grid
   T c, s, cc, ss, cs2, cs, c2;   // rotation: cos, sin, cos^2, sin^2, 2 cos sin, cos sin, cos^2 - sin^2
-  T q, kind, pad;                // wavenumber; 0 recursion, 1 laminate (k = 0), 2 outside Z^2_N
+  T q, kind, EC;                 // wavenumber; 0 recursion, 1 laminate (k = 0), 2 outside Z^2_N; uniform: e^{-q C h}
   __device__ __forceinline__ El<T> el() const {
     El<T> e;
     e.E = E; e.a = a; e.b0 = b0; e.b1 = b1; e.d0 = d0; e.d1 = d1;
@@ -210,7 +210,7 @@ template <typename T> struct __align__(16) ColIn {
 // + n_P) added to 33, no pp component, all over 2 mu.  The constants of the rotation back are
 // folded into the combinations.
 template <typename T> struct __align__(16) ColOut {
-  T k11w, k22w, k12w, k11n, k22n, k12n, k11a, k12a, k33, cy, sy, cz, sz, pad[3];
+  T k11w, k22w, k12w, k11n, k22n, k12n, k11a, k12a, k33, cy, sy, cz, sz, EC1, pad[2];
 };
 template <typename T> struct __align__(16) Col {
   ColIn<T> in;
@@ -221,7 +221,7 @@ template <typename T> struct __align__(16) Col {
 // constants of column k1 of row k2 (uniform: with the element coefficients of spacing hz)
 template <typename T>
 __device__ __forceinline__ void col_put(Col<T>* p, int k1, int k2, int n1, int n2, int hs, T w1, T w2, const DepthMat<T>& m,
-                                        bool uniform, T hz) {
+                                        bool uniform, T hz, int C = 1, T d1 = 0) {
   const ModeGeom<T> g = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2);
   ColIn<T> i;
   El<T> e = {0, 0, 0, 0, 0, 0};
@@ -230,7 +230,7 @@ __device__ __forceinline__ void col_put(Col<T>* p, int k1, int k2, int n1, int n
   i.c = g.c; i.s = g.s; i.cc = g.c * g.c; i.ss = g.s * g.s; i.cs = g.c * g.s; i.cs2 = (T)2 * i.cs; i.c2 = i.cc - i.ss;
   i.q = g.q;
   i.kind = g.nyq ? (T)2 : (g.zero ? (T)1 : (T)0);
-  i.pad = 0;
+  i.EC = uniform ? dexp<T>(-g.q * hz * (T)C) : (T)0;
   p->in = i;
   const T kap = m.kap * g.q, q2 = m.hq * g.q, pp = m.p * kap;
   ColOut<T> o;
@@ -239,7 +239,8 @@ __device__ __forceinline__ void col_put(Col<T>* p, int k1, int k2, int n1, int n
   o.k11a = -q2 * i.cs2; o.k12a = q2 * i.c2;
   o.k33 = kap;
   o.cy = kap * g.c; o.sy = kap * g.s; o.cz = q2 * g.c; o.sz = q2 * g.s;
-  o.pad[0] = o.pad[1] = o.pad[2] = 0;
+  o.EC1 = uniform ? dexp<T>(-g.q * d1) : (T)0;  // propagator over the first chunk's nodes
+  o.pad[0] = o.pad[1] = 0;
   p->out = o;
 }
 
@@ -650,7 +651,7 @@ template <typename T, int KT, bool UNI>
 __device__ __forceinline__ void depth_prep(Col<T>* cols, T* el, const T* __restrict__ zn, int tid, int kblk, int k2, int nz,
                                            int C, int n1, int n2, int hs, T w1, T w2, const DepthMat<T>& m, T hz) {
   const int kt = tid & (KT - 1), k1 = kblk * KT + kt;
-  if (tid < KT) col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, UNI, hz);
+  if (tid < KT) col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, UNI, hz, C, zn[min(C - 1, nz - 1)] - zn[0]);
   if (!UNI) {
     const T q = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2).q;
     const int n0 = (tid / KT) * C, nend = min(n0 + C, nz);
@@ -742,8 +743,8 @@ __device__ __forceinline__ void depth_r_body(const typename Cx<T>::t* W, const X
   Br<V> cA = br_zero<V>(), cP = br_zero<V>(), im;
   if (!local) {
     if (!ghost)
-      chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, UNI ? dexp<T>(-g.q * hz * (T)C) : (T)0,
-                           UNI ? dexp<T>(-g.q * (zs[last] - zs[0])) : (T)0, !special,
+      chunk_carries<T, KT>(X, zs, tid, tt, C, nch, nz, g.q, UNI, hz, g.EC,
+                           cols[kt].out.EC1, !special,
                            want_u3 ? surf + (size_t)k2 * h1 + k1 : nullptr, m.iu);
     __syncthreads();
     if (!active) return;
