@@ -192,8 +192,8 @@ const char* fvim_last_cuda_error(void);
  * Tile plan of the per-wavevector depth kernel.  The paper has no counterpart: its depth
  * integral (Sec. 3.2) is evaluated here by exact O(Nz) exponential recursions whose depth
  * range is cut into chunks of depth_chunk nodes, one thread per chunk, the chunk carries
- * being combined by a log-depth scan.  Every launchable chunk length gives the same operator
- * up to the rounding order of that scan; the fastest one depends on the grid.
+ * being combined by a recurrence over the chunks.  Every launchable chunk length gives the same
+ * operator up to its rounding order; the fastest one depends on the grid.
  *   depth_chunk   chunk length in use (fvim_set_plan: 0 selects the default rule,
  *                 max(2, ceil(Nz / 16)))
  *   tuned         1 if depth_chunk came from a timing run (fvim_autotune) in this process
@@ -203,12 +203,12 @@ const char* fvim_last_cuda_error(void);
  *   depth_cutoff  eps_co of the FP32 register variant's chunk scan (the cutoff of Sec. 3.2,
  *                 restated for the exact recursion): a tile whose chunk spans all damp by
  *                 e^{-q span} < e^{-eps_co} takes each chunk's carry from its neighbour alone,
- *                 skipping the log-depth scan (the dropped terms are below e^{-eps_co} of the
+ *                 skipping that recurrence (the dropped terms are below e^{-eps_co} of the
  *                 moments).  Default FVIM_DEPTH_CUTOFF_DEFAULT = 18 (e^{-18} = 1.5e-8, below the
  *                 FP32 rounding unit); fvim_set_plan: 0 selects the exact scan.  Not used by
  *                 the shared-memory variant (FP64, deep grids), whose scan is sequential.
  *   depth_ctas    CTAs per SM the FP32 register variant of the depth kernel is compiled for:
- *                 2 (128 registers per thread, the default) or 3 (85 registers, chunk lengths
+ *                 2 (the default; chunks of 2 and 3 nodes run four and three) or 3 (80 registers, chunk lengths
  *                 4..8 whose tile fits three times in shared memory); 0 for the shared-memory
  *                 variant (FP64, deep grids), which has one launch shape per chunk length
  */

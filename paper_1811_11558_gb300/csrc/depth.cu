@@ -17,7 +17,7 @@
 //   (The generic form carries five rotated components and one contraction per branch, and
 //   evaluates the image field per node: 457 warp instructions per warp of nodes, measured on
 //   512 x 512 x 64 FP32, against 236 here.  Depth kernel, ms, generic form -> this one: 512 x
-//   512 x 64 FP32 0.204 -> 0.146, 1024 x 1024 x 32 (C = 2) 0.642 -> 0.339, 256 x 128 x 57
+//   512 x 64 FP32 0.204 -> 0.146, 1024 x 1024 x 32 (C = 2) 0.642 -> 0.336, 256 x 128 x 57
 //   refined 0.043 -> 0.028, 128 x 128 x 126 FP64 1.163 -> 0.355.)
 // * Depth integral: the g0/g1 kernels are exponentials exp(-q|y3 - x3|) times polynomials, so
 //   the moments follow from those of the neighbouring node by exact one-element steps,
@@ -191,7 +191,8 @@ __device__ __forceinline__ ModeGeom<T> mode_geom(int k1, int k2, int n1, int n2,
 // from shared memory by the column's chunk threads: evaluated by every thread they were half of
 // the instructions at two nodes per thread.  The trailing pad spreads the columns' 16-byte reads
 // over the banks.  (With this and the four-chunk read-ahead of the carries: C = 2 at 1024 x 1024 x
-// 32 0.465 -> 0.339 ms, FP64 128 x 128 x 126 0.385 -> 0.355.)
+// 32 0.465 -> 0.339 ms, FP64 128 x 128 x 126 0.385 -> 0.355; the exponentials of the carries among
+// them too: 0.341 -> 0.336.)
 template <typename T> struct __align__(16) ColIn {
   T E, a, b0, b1, d0, d1;        // element coefficients of a uniform grid
   T c, s, cc, ss, cs2, cs, c2;   // rotation: cos, sin, cos^2, sin^2, 2 cos sin, cos sin, cos^2 - sin^2
@@ -1118,7 +1119,7 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
       const size_t lim = (size_t)nz * 6 * 16 * sizeof(V) + (size_t)(2 * nchr) * 16 * kMom +
                          (size_t)3 * 16 * sizeof(V) + (((size_t)nz * sizeof(T) + 7) & ~(size_t)7) + 16;
       if (lim <= 227 * 1024 && 16 * nchr <= 256) {
-        // three CTAs per SM (85 registers): chunk lengths 4..8 whose tile fits three times
+        // three CTAs per SM (80 registers): chunk lengths 4..8 whose tile fits three times
         if (ctas == 3 && !(CR >= 4 && 3 * (lim + 1024) <= 228 * 1024)) return d;
         d = DepthCfg<T>{true, true, CR, nchr, 16, 16 * nchr, RegSmem<T, 16>::bytes(nz, nchr, c->uniform) + 16,
                         ctas == 3 ? 3 : 2};

@@ -805,7 +805,7 @@ inline void launch_chain(const fvim_ctx* c, void (*kern)(P...), dim3 grid, dim3 
 // tile plan of the depth kernel (depth.cu): default chunk length, and whether a chunk length
 // gives a launchable configuration on this context's grid and precision
 int depth_chunk_default(int nz);
-// ctas: CTAs per SM the FP32 register variant is compiled for (2 default, 3 with 85 registers)
+// ctas: CTAs per SM the FP32 register variant is compiled for (2 default, 3 with 80 registers)
 bool depth_chunk_ok(const fvim_ctx* c, int chunk, int ctas = 2);
 // CTAs per SM of the depth kernel's launch under the context's plan (0: shared-memory variant)
 int depth_launch_ctas(const fvim_ctx* c);

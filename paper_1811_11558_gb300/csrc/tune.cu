@@ -2,9 +2,9 @@
 // contracts in include/fvim.h).
 //
 // The depth range of every mode is cut into chunks of C nodes, one thread per chunk, whose
-// recursion carries are combined by a log-depth scan (depth.cu).  Short chunks give more
-// threads and a shorter serial recursion, long chunks fewer scan rounds and fewer threads
-// per tile; which one is fastest depends on the grid (small grids are latency bound, large
+// recursion carries are combined by a recurrence over the chunks (depth.cu).  Short chunks give
+// more threads and a shorter recursion in each, long chunks fewer carries and fewer threads per
+// tile; which one is fastest depends on the grid (small grids are latency bound, large
 // ones issue bound), so it is measured: every launchable C is timed on the context's own
 // stream and the fastest is kept in a process-wide table keyed by grid, precision and depth
 // spacing, so later contexts of that grid start with it.  The in-plane transforms have up to

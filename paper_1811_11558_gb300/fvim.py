@@ -62,7 +62,7 @@ class Plan(ctypes.Structure):
 
     def as_dict(self):
         """timings_ms: chunk length -> ms with the default register budget; timings_ms_3ctas:
-        the same with three CTAs per SM (85 registers), where built."""
+        the same with three CTAs per SM (80 registers), where built."""
         n = self.n_cand
         d = {"depth_chunk": self.depth_chunk, "depth_ctas": self.depth_ctas,
              "depth_cutoff": round(float(self.depth_cutoff), 6), "tuned": bool(self.tuned),
