@@ -14,7 +14,8 @@
 //   rowsU  inverse rows of u = K*p; p <- s p, change against the old pressure -> stop test; over
 //          the contact sums of d and d^2, d = u - h - (last gbar) -> gbar, G = sum of g^2 -> beta
 // (d is the gap up to the change of its mean, so G = sum d^2 - (sum d)^2 / n cancels nothing that
-// the iteration does not itself lose; the first G is summed from g.)  The sums are FP64, block
+// the iteration does not itself lose, unless a point whose depth dominated the mean has left the
+// contact: then the last block sums both again, gap_lost; the first G is summed from g.)  The sums are FP64, block
 // partials in block order added by the last block to finish, so results do not depend on timing.
 // Every scalar, the surface and pressure pointers, the load and the tolerance live in the device
 // state (PkState): one captured loop serves every call of a context.
@@ -65,6 +66,13 @@ __device__ __forceinline__ float gap1(float u, float h, double, float2 c) {
   return __fadd_rn(s, __fadd_rn(e2, __fsub_rn(e, c.y)));
 }
 __device__ __forceinline__ double gap1(double u, double h, double c, float2) { return u - h - c; }
+
+// Whether sums about the mean gap c have lost the new mean gb and G = sum g^2 over n points: c is far
+// above everything that is left (a point whose depth dominated the mean has gone out of contact).
+// Then both are summed again from the gaps themselves.
+__device__ __forceinline__ bool gap_lost(double c, double gb, double G, double n) {
+  return fabs(c) > 1e3 * (fabs(gb) + sqrt(G / n));
+}
 
 // state of a new solve, with the scale of the initial pressure from its sum (a guess without load
 // is replaced by the uniform pressure)
@@ -308,7 +316,46 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
     }
   }
   if (MODE != INV_R) sum[3] = (double)nc;
-  if (!grid_sum(sum, part, cnt)) return;
+  __shared__ int redo;
+  if (MODE == INV_U && threadIdx.x == 0) redo = 0;
+  if (MODE == INV_U && blockDim.x == 32) __threadfence();  // (more warps: the barriers of grid_sum before its fence)
+  const bool lead = grid_sum(sum, part, cnt);
+  if (MODE == INV_U) {
+    if (lead) {
+      const double mean = sum[0] / sum[3];
+      redo = sum[3] > 0 && isfinite(sum[0]) && gap_lost(gbar, gbar + mean, fmax(sum[1] - sum[0] * mean, 0.0), sum[3]);
+    }
+    __syncthreads();
+    if (redo) {  // the last block: every u and p of the pass is in memory
+      __shared__ double wsum[32];
+      __shared__ double mean;
+      double G = 0;
+      for (int pass = 0; pass < 2; ++pass) {
+        double a = 0;
+        for (size_t i = threadIdx.x; i < (size_t)N * n2; i += blockDim.x)
+          if (__ldcg(p + i) > (T)0) {
+            const double d = (double)__ldcg(u + i) - (double)h[i];
+            a += pass == 0 ? d : (d - mean) * (d - mean);
+          }
+        for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+        if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = a;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+          a = 0;
+          for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += wsum[w];
+          if (pass == 0) mean = a / sum[3];
+          else G = a;
+        }
+        __syncthreads();
+      }
+      if (lead) {  // as sums about the old mean whose difference is G
+        sum[0] = 0;
+        sum[1] = G;
+        S->gbar = mean;
+      }
+    }
+  }
+  if (!lead) return;
   if (MODE == INV_R) {
     // <g, t> / (<r, t> - rbar <t, 1>), rbar = sum r / nIc
     const double den = sum[3] * S->nIc - sum[0] * sum[1];
@@ -329,7 +376,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   if (!done && (!(sum[3] > 0) || !isfinite(sum[0]))) {
     bad = 1;
   } else {
-    const double mean = sum[0] / sum[3], gb = (MODE == INV_U ? gbar : 0.0) + mean;
+    const double mean = sum[0] / sum[3], gb = (MODE == INV_U ? (redo ? S->gbar : gbar) : 0.0) + mean;
     S->gbar = gb;
     S->gbar2 = pair_of(gb);
     if (MODE == INV_U) {
@@ -487,6 +534,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
   __shared__ PkState S;
   __shared__ double red[4][CL][4];        // partial sums of every CTA: start, tau, load, gap
   __shared__ double wsum[32 * 4];
+  __shared__ int redo;
 
   const int tid = threadIdx.x, nth = blockDim.x;
   T* pg = static_cast<T*>(init.p) + (size_t)rank * E;
@@ -747,22 +795,56 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
         if (err < S.tol || S.it >= S.max_it) done = 1;
         if (!isfinite(err)) bad = 1;
         S.nIc = n;
+        redo = 0;
         if (!done && (!(n > 0) || !isfinite(sd))) {
           bad = 1;
         } else {
-          const double mean = sd / n;
+          const double mean = sd / n, G = fmax(sdd - sd * mean, 0.0);
+          redo = !done && gap_lost(S.gbar, S.gbar + mean, G, n);
           S.gbar += mean;
           S.gbar2 = pair_of(S.gbar);
-          const double G = fmax(sdd - sd * mean, 0.0);
-          S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
-          S.beta2 = pair_of(S.beta);
-          S.G_old = G;
+          if (!redo) {
+            S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
+            S.beta2 = pair_of(S.beta);
+            S.G_old = G;
+          }
         }
         if (bad) S.bad = 1;
         S.done = done | bad;
       }
     }
     __syncthreads();
+    if (redo) {  // the same in every CTA
+      double a = 0;
+      for (int i = tid; i < E; i += nth)
+        if (p[i] > (T)0) a += (double)u[i] - (double)h[i];
+      send(1, a, 0, 0, 0);
+      cl.sync();
+      if (tid < 32) {
+        const double sum = value(total(1), 0);
+        if (tid == 0) S.gbar = sum / S.nIc;
+      }
+      __syncthreads();
+      const double gbar = S.gbar;
+      a = 0;
+      for (int i = tid; i < E; i += nth)
+        if (p[i] > (T)0) {
+          const double gi = (double)u[i] - (double)h[i] - gbar;
+          a += gi * gi;
+        }
+      send(2, a, 0, 0, 0);
+      cl.sync();
+      if (tid < 32) {
+        const double G = value(total(2), 0);
+        if (tid == 0) {
+          S.gbar2 = pair_of(gbar);
+          S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
+          S.beta2 = pair_of(S.beta);
+          S.G_old = G;
+        }
+      }
+      __syncthreads();
+    }
   }
   for (int i = tid; i < E; i += nth) pg[i] = p[i];
   if (rank == 0 && tid == 0) *out = S;

@@ -149,6 +149,27 @@ def test_contact_variants(n1, n2, prec):
     assert torch.equal(again, p)
 
 
+@pytest.mark.parametrize("hole", [1e6, 1e12, 1e20, 1e30])
+@pytest.mark.parametrize("n1,n2", [(16, 16), (64, 64), (64, 32), (256, 256)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_contact_with_a_masked_point(n1, n2, prec, hole):
+    """A point far below the surface dominates the first mean gap and never carries load: the
+    pressure is that of a hole just deep enough not to touch, whatever its depth."""
+    torch = require_gpu()
+    z = inputs.uniform_depth(2, 0.1)
+    h = inputs.hertz_profile(n1, n2, 1.0, 1.0, 0.5)
+    W = 2e-2 * ES * (np.pi / 4) ** 2
+    h[1, 2] = -10.0
+    ref, _ = C.polonsky_keer(h, W, 1.0, 1.0, E, NU, tol=1e-13)
+    assert ref[1, 2] == 0
+    h[1, 2] = -hole
+    ctx = _ctx(n1, n2, z, prec)
+    opts = ctx.default_opts(cg_tol=1e-13) if prec == "fp64" else ctx.default_opts()
+    p = torch.zeros(ctx.surf_shape, dtype=ctx.dtype, device="cuda")
+    ctx.elastic_contact(to_dev(torch, h, ctx.dtype), W, p, opts)
+    assert rel_l2(p.cpu().numpy(), ref) < (1e-9 if prec == "fp64" else 2e-5)
+
+
 @pytest.mark.parametrize("prec", ["fp64", "fp32"])
 def test_contact_loop_equals_batches(prec, monkeypatch):
     """The six-kernel iteration as one WHILE graph and as host-driven batches: the same bits, for two
