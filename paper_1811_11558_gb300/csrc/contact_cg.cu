@@ -26,8 +26,8 @@
 // updates in two-float arithmetic, rounded once as the FP64 expression is; FP64 only in the sums,
 // and there only at points that carry pressure; a warp's sums of several values reduced together.
 // us per iteration, fourteen kernels -> seven with eight values per thread and FP64 updates -> this
-// (with all of a thread's points read before the first store): 256^2 83 -> 44, 512^2 132 -> 75 ->
-// 51, 1024^2 206 -> 156 -> 113 (smaller squares: the cluster kernel below).
+// (with all of a thread's points read before the first store): 256^2 83 -> 46, 512^2 132 -> 75 ->
+// 53, 1024^2 206 -> 156 -> 115 (smaller squares: the cluster kernel below).
 #include <cooperative_groups.h>
 
 #include <algorithm>
