@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
                                                       unsigned* cnt) {
   typedef typename Cx<T>::t V;
   if (MODE != FWD_INIT && S->done) return;
+  if (MODE == FWD_T && blockIdx.x == 0 && threadIdx.x == 0) S->passes += 1;
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
   const int r = threadIdx.x / T4, tt = threadIdx.x % T4;
@@ -247,6 +248,10 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
     if (MODE == INV_U && use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
     return;
   }
+  // the pass cap does not wait for the sums: the first block ends the loop there by itself, and the last
+  // block never asks for another pass beyond it
+  const bool cap = MODE == INV_U && S->passes >= S->max_it;
+  if (cap && use_cond && blockIdx.x == 0 && threadIdx.x == 0) cudaGraphSetConditional(cond, 0u);
   extern __shared__ __align__(16) unsigned char smraw[];
   constexpr int T4 = N / 4, H1 = N / 2, LD = SurfSm<V, N>::LD;
   const int r = threadIdx.x / T4, tt = threadIdx.x % T4;
@@ -389,7 +394,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   }
   if (bad) S->bad = 1;
   S->done = done | bad;
-  if (MODE == INV_U && use_cond) cudaGraphSetConditional(cond, (done | bad) ? 0u : 1u);
+  if (MODE == INV_U && use_cond) cudaGraphSetConditional(cond, (done | bad) || cap ? 0u : 1u);
 }
 
 // G = sum over the contact of g^2, g = u - h - gbar, of the first iteration

@@ -920,6 +920,7 @@ struct PkState {
   const void* h;
   void* p;
   int done, it, bad, max_it;
+  int passes;  // iterations begun, counted apart from the sums: the loop ends at max_it whatever they do
 };
 static_assert(sizeof(PkState) <= 256, "pinned copy of the contact state");
 struct PkfArgs {

@@ -53,8 +53,7 @@ template <typename T> int ensure_ws(fvim_ctx* c) {
   if (FVIM_CU(cudaMalloc(&c->sv[V_WZ], (size_t)c->nz * sizeof(double)))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_PKS], kScalarBlock))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMalloc(&c->sv[V_DFS], kDfsBytes))) return FVIM_ERR_OOM;
-  if (FVIM_CU(cudaMalloc(&c->sv[V_PKF], kPkfBytes)) || FVIM_CU(cudaMemset(c->sv[V_PKF], 0, kPkfBytes)))
-    return FVIM_ERR_OOM;
+  if (FVIM_CU(cudaMalloc(&c->sv[V_PKF], kPkfBytes))) return FVIM_ERR_OOM;
   if (FVIM_CU(cudaMallocHost(&c->h_part, (size_t)RMAXB * NVMAX * sizeof(double) + 256 + kDfsBytes))) {
     c->h_part = nullptr;
     return FVIM_ERR_OOM;
@@ -735,6 +734,8 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
     if (err_out) *err_out = sh->err;
     return sh->err < o->cg_tol ? FVIM_OK : FVIM_ERR_NOT_CONVERGED;
   }
+  // the arrival counter of the sums, whatever an earlier solve left in it
+  if (FVIM_CU(cudaMemsetAsync(a.cnt, 0, sizeof(unsigned), c->stream))) return FVIM_ERR_CUDA;
   if ((rc = pkf_begin<T>(a, s0))) return rc;
   SolverRT* srt = rt(c);
   bool ran_device = false;

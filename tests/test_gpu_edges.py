@@ -1,0 +1,48 @@
+"""Limits of the solvers and operators that the oracle comparisons do not reach: iteration caps,
+non-finite input, deep grids, launch plans and selection switches."""
+import numpy as np
+import pytest
+
+from oracle import tensors as T
+from paper_1811_11558_gb300 import inputs
+
+from gpu_util import rel_l2, require_gpu, to_dev
+
+pytestmark = pytest.mark.gpu
+
+E, NU = 1.0, 0.3
+ES = T.e_star(E, NU)
+
+
+def _ctx(n1, n2, z, prec, **kw):
+    from paper_1811_11558_gb300 import Context
+
+    kw = {"E": E, "nu": NU, **kw}
+    return Context(n1, n2, z, 1.0, 1.0, precision=prec, **kw)
+
+
+def _hertz(torch, ctx, R=0.5):
+    h = to_dev(torch, inputs.hertz_profile(ctx.n1, ctx.n2, 1.0, 1.0, R), ctx.dtype)
+    return h, 2e-2 * ES * (np.pi / 4) ** 2
+
+
+@pytest.mark.parametrize("loop", ["1", "0"])
+def test_contact_loop_ends_at_the_iteration_cap(loop, monkeypatch):
+    """The loop of a power-of-two surface stops after cg_max_iter passes with that count, also after a
+    refused solve, and on a side stream from a context's first solve on (the arrival counter of its sums is
+    cleared by every solve on the solver's own stream)."""
+    torch = require_gpu()
+    monkeypatch.setenv("FVIM_DEVICE_CG", loop)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        ctx = _ctx(256, 64, inputs.uniform_depth(2, 0.1), "fp32")
+        h, W = _hertz(torch, ctx)
+        bad = h.clone()
+        bad[3, 5] = float("nan")
+        for cap in (1, 2, 5, 3):
+            it, err = ctx.elastic_contact(h, W, torch.zeros_like(h), ctx.default_opts(cg_tol=1e-30, cg_max_iter=cap),
+                                          allow_not_converged=True)
+            assert it == cap and np.isfinite(err)
+            with pytest.raises(Exception):
+                ctx.elastic_contact(bad, W, torch.zeros_like(h), ctx.default_opts(cg_max_iter=cap))
+    side.synchronize()
