@@ -947,7 +947,8 @@ struct DFS {
   void* pF[2];        // their residuals
   double f, nF0, fmax, eta, ap, am, fp, fm, best_old, tol_abs, tol_rel, gamma, smin, smax, tmin, tmax;
   double hist[32];    // ring of the accepted residuals, hist[i & 31] for i < len
-  int len, k, bt, phase, done, conv, bad, cur, trials, max_iter, max_trials, evals;
+  int len, k, bt, phase, done, conv, bad, cur, max_iter, max_trials, evals;
+  int passes;         // trials begun, counted apart from the sums: the loop ends at max_trials whatever they do
   double sigma;       // spectral step
   double coef;        // step of the current trial: -ap sigma (phase 0) or am sigma (phase 1)
   float coef32;       // the same, rounded once
@@ -961,10 +962,11 @@ constexpr int kDfsM = 10, kDfsStag = 30;
 // the increment of cumulated plastic strain, and notes the layer range of the flowing voxels.
 // The loop leaves d_ep out: the solve recomputes the return map of its final point.
 template <typename T>
-__global__ void k_dfd_trial_rmap(const DFS* __restrict__ s, const T* __restrict__ sig_n, const T* __restrict__ ep, T* __restrict__ d_eps_p,
+__global__ void k_dfd_trial_rmap(DFS* __restrict__ s, const T* __restrict__ sig_n, const T* __restrict__ ep, T* __restrict__ d_eps_p,
                                  T* __restrict__ d_ep, size_t nxy, size_t nvox, T lam, T mu, T sy, T Eh,
                                  int* __restrict__ zr) {
   const size_t v = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (v == 0) s->passes += 1;
   if (v >= nvox) return;
   const int cur = s->cur;
   const T* a = static_cast<const T*>(s->px[cur]);
@@ -995,7 +997,6 @@ __device__ void dfd_decide(DFS* s, double ft, double ss, double sy, cudaGraphCon
   // largest and smallest of non-negative values by their bit patterns (an FP64 comparison costs 64
   // cycles; the history is up to thirty values long)
   auto bits = [](double x) { return __double_as_longlong(x); };
-  s->trials += 1;
   s->evals += 1;
   int done = s->done;
   bool acc = false;
@@ -1062,7 +1063,7 @@ __device__ void dfd_decide(DFS* s, double ft, double ss, double sy, cudaGraphCon
       }
     }
   }
-  if (s->trials >= s->max_trials) done = 1;
+  if (s->passes >= s->max_trials) done = 1;
   const double coef = (s->phase == 0 ? -s->ap : s->am) * s->sigma;
   s->coef = coef;
   s->coef32 = (float)coef;
@@ -1078,6 +1079,8 @@ template <typename T>
 __global__ void __launch_bounds__(RT) k_dfd_res_sy(DFS* s, const T* __restrict__ b, const T* __restrict__ tmp,
                                                    const double* __restrict__ wz, int lgxy, size_t n, int per_plane,
                                                    double* part, unsigned* cnt, int* zr, cudaGraphConditionalHandle cond) {
+  // the trial cap does not wait for the sums: the first block ends the loop there by itself
+  if (blockIdx.x == 0 && threadIdx.x == 0 && s->passes >= s->max_trials) cudaGraphSetConditional(cond, 0u);
   const int cur = s->cur;
   const T* x = static_cast<const T*>(s->px[cur]);
   const T* F = static_cast<const T*>(s->pF[cur]);

@@ -46,3 +46,31 @@ def test_contact_loop_ends_at_the_iteration_cap(loop, monkeypatch):
             with pytest.raises(Exception):
                 ctx.elastic_contact(bad, W, torch.zeros_like(h), ctx.default_opts(cg_max_iter=cap))
     side.synchronize()
+
+
+def test_dfsane_loop_ends_at_its_caps():
+    """The device loop of a plastic increment stops after df_max_iter accepted points, reported as not
+    converged, and a later solve through the same context is that of a fresh one."""
+    torch = require_gpu()
+    from paper_1811_11558_gb300 import FvimError
+
+    z = inputs.uniform_depth(6, 0.4)
+    sy = 0.05 * ES
+    x = (np.arange(32) + 0.5) / 32 - 0.5
+    p = 0.15 * ES * np.sqrt(np.maximum(0.0, 1.0 - (x[None, :] ** 2 + x[:, None] ** 2) / 0.09))
+
+    def solve(ctx, **kw):
+        out = [torch.empty(s, dtype=ctx.dtype, device="cuda") for s in (ctx.vol_shape, ctx.vol_shape, ctx.scal_shape)]
+        rep = ctx.plasticity_solve(to_dev(torch, p, ctx.dtype), *out, ctx.default_opts(**kw))
+        torch.cuda.synchronize()
+        return rep, out
+
+    for prec in ("fp32", "fp64"):
+        ctx = _ctx(32, 32, z, prec, sigma_y=sy, E_h=0.1)
+        full, ref = solve(ctx)
+        for cap in (1, 2):
+            assert cap < full[0]
+            with pytest.raises(FvimError, match="not converged"):
+                solve(ctx, df_max_iter=cap)
+        again, out = solve(ctx)
+        assert again == full and all(torch.equal(a, b) for a, b in zip(out, ref))
