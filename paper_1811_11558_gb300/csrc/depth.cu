@@ -438,6 +438,14 @@ __device__ __forceinline__ void chunk_carries(const Xch<typename Cx<T>::t, KT>& 
 // Bound by the FP64 pipe in FP64 (two multiply-adds per clock and SM): 1163 -> 355 us at
 // 128 x 128 x 126 when the moments went from six to three per branch.
 // ----------------------------------------------------------------------------------
+// Gap behind each chunk's rows in shared memory: rows shorter than 128 bytes go an odd number apart from
+// chunk to chunk, or the warp's chunks would meet on the same banks (an even number of nodes per chunk).
+// 128 x 128 FP32 refined, us per apply, without the gaps -> with them (and every thread copying its own
+// nodes, without the index divisions of a shared copy loop): 192 layers 234 -> 173, 256 324 -> 254, 288
+// 400 -> 336; FP64 128 x 128 x 126 refined 1602 -> 1581.
+__host__ __device__ inline int chunk_gap(int rows, int kt, int row_bytes) {
+  return row_bytes < 128 && rows % 2 == 0 ? kt : 0;
+}
 template <typename T, int KT, bool LS>
 __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __restrict__ spec, typename Cx<T>::t* __restrict__ surf,
                                 const T* __restrict__ zn, int nz, int n1, int n2, int hs, int h1, int C, int nch, T w1,
@@ -447,13 +455,16 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   typedef typename Cx<T>::t V;
   constexpr int SL = LS ? 6 : 9, CM = LS ? 8 : 1;
   extern __shared__ __align__(128) unsigned char smraw[];  // one alignment for every kernel of this file
-  V* W = reinterpret_cast<V*>(smraw);                      // [nz][SL][KT]
-  V* xbase = W + (size_t)nz * SL * KT;
+  const int gw = chunk_gap(C * SL, KT, KT * sizeof(V)), ge = chunk_gap(C * EL_N, KT, KT * sizeof(T)),
+            gp = chunk_gap(C, KT, KT * sizeof(T));
+  V* W = reinterpret_cast<V*>(smraw);                      // [nz][SL][KT], chunks gw apart
+  V* xbase = W + (size_t)nz * SL * KT + (size_t)nch * gw;
   const Xch<V, KT> X(xbase, nch);
   Col<T>* cols = reinterpret_cast<Col<T>*>(xbase + Xch<V, KT>::count(nch));  // [KT]
-  T* el = reinterpret_cast<T*>(cols + KT);                 // [uniform ? 0 : nz][6][KT]
-  T* pr = el + (size_t)(uniform ? 0 : nz) * EL_N * KT;     // [uniform ? C : nz][KT] propagators within a chunk
-  T* zs = pr + (size_t)(uniform ? C : nz) * KT;            // [nz] depth nodes
+  T* el = reinterpret_cast<T*>(cols + KT);                 // refined: [nz][6][KT], chunks ge apart
+  // propagators within a chunk: uniform [C][KT], refined [nz][KT], chunks gp apart
+  T* pr = el + (uniform ? (size_t)0 : (size_t)nz * EL_N * KT + (size_t)nch * ge);
+  T* zs = pr + (uniform ? (size_t)C * KT : (size_t)nz * KT + (size_t)nch * gp);  // [nz] depth nodes
   const int kt = threadIdx.x & (KT - 1);
   const int ch = threadIdx.x / KT;
   const int k1 = blockIdx.x * KT + kt;
@@ -461,21 +472,28 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   const size_t plane = (size_t)n2 * h1;
   const size_t colofs = (size_t)k2 * h1 + blockIdx.x * KT;
 
-  // 1. load the tile (coalesced KT-wide rows, every copy in flight before one wait) and
-  //    the depth nodes
-  // (layers outside zr hold no input: their spectrum was not computed and reads as zero)
-  const int zlo = zr ? zr[0] : 0, zhi = zr ? zr[1] : nz;
-  for (int idx = threadIdx.x; idx < nz * 6 * KT; idx += blockDim.x) {
-    const int zc = idx / KT, j = idx & (KT - 1);
-    const int zl = zc / 6;
-    V* dst = W + ((size_t)zl * SL + (zc - zl * 6)) * KT + j;
-    if (zl >= zlo && zl < zhi) cp_async_cx(dst, spec + (size_t)zc * plane + colofs + j);
-    else *dst = mk<V>(0, 0);
-  }
-  for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
   const int n0 = ch * C;
   const int nend = min(n0 + C, nz);
   const bool active = n0 < nz;
+  // the thread's column in its own chunk: node i at own + i SL KT, elements and propagators likewise
+  V* own = W + (size_t)ch * gw + kt;
+  T* elc = el + ch * ge + kt;
+  T* prc = pr + (uniform ? 0 : ch * gp) + kt;
+
+  // 1. load the tile (every thread its own nodes, KT-wide rows, every copy in flight before one wait)
+  //    and the depth nodes
+  // (layers outside zr hold no input: their spectrum was not computed and reads as zero)
+  const int zlo = zr ? zr[0] : 0, zhi = zr ? zr[1] : nz;
+  const V* src = spec + (size_t)n0 * 6 * plane + colofs + kt;
+  for (int i = n0; i < nend; ++i, src += 6 * plane) {
+    V* dst = own + (size_t)i * SL * KT;
+#pragma unroll
+    for (int cc = 0; cc < 6; ++cc) {
+      if (i >= zlo && i < zhi) cp_async_cx(dst + cc * KT, src + cc * plane);
+      else dst[cc * KT] = mk<V>(0, 0);
+    }
+  }
+  for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
   // column constants while the tile is in flight, and on a uniform grid the powers E^0 .. E^(C-1) of
   // its propagator, for distances within a chunk; on a refined grid the coefficients of element e
   // below node e (none, zero, below the last node).  Longer distances take an exponential each (one
@@ -495,7 +513,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     for (int e = n0; e < nend; ++e) {
       El<T> c = {0, 0, 0, 0, 0, 0};
       if (e + 1 < nz) c = elem_coef<T>(q, zn[e + 1] - zn[e]);
-      el_put<T, KT>(el + (size_t)e * EL_N * KT + kt, c);
+      el_put<T, KT>(elc + e * EL_N * KT, c);
     }
   }
   cp_async_wait_all();
@@ -511,7 +529,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   if (work) {
     Br<V> s = br_zero<V>();
     auto fwd = [&](int i, V* Li) {
-      V* w = W + (size_t)i * SL * KT + kt;
+      V* w = own + (size_t)i * SL * KT;
       V x[6];
 #pragma unroll
       for (int cc = 0; cc < 6; ++cc) x[cc] = w[cc * KT];
@@ -523,9 +541,9 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
         br_put<V, KT>(w, s);
         br_leave(s, ec, o.nA, o.m, o.aA);
       } else {
-        if (i > 0) br_arrive(s, el_get<T, KT>(el + (size_t)(i - 1) * EL_N * KT + kt), o.nA, o.m, o.aA);
+        if (i > 0) br_arrive(s, el_get<T, KT>(elc + (i - 1) * EL_N * KT - (i == n0 ? ge : 0)), o.nA, o.m, o.aA);
         br_put<V, KT>(w, s);
-        br_leave(s, el_get<T, KT>(el + (size_t)i * EL_N * KT + kt), o.nA, o.m, o.aA);
+        br_leave(s, el_get<T, KT>(elc + i * EL_N * KT), o.nA, o.m, o.aA);
       }
       w[3 * KT] = o.nP;
       w[4 * KT] = o.m;
@@ -539,24 +557,25 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
       for (int i = n0; i < nend; ++i) {
         fwd(i, L[0]);
 #pragma unroll
-        for (int j = 0; j < 3; ++j) W[((size_t)i * SL + 6 + j) * KT + kt] = L[0][j];
+        for (int j = 0; j < 3; ++j) own[((size_t)i * SL + 6 + j) * KT] = L[0][j];
       }
     }
     br_put<V, KT>(X.A + (size_t)ch * 3 * KT + kt, s);
     s = br_zero<V>();
     T ep = 1;  // propagator from node i to the chunk's last node
     for (int i = nend - 1; i >= n0; --i) {
-      V* w = W + (size_t)i * SL * KT + kt;
+      V* w = own + (size_t)i * SL * KT;
       const V sn = w[3 * KT], sm = w[4 * KT], sa = w[5 * KT];
       if (!uniform) {
-        ec = el_get<T, KT>(el + (size_t)i * EL_N * KT + kt);
+        ec = el_get<T, KT>(elc + i * EL_N * KT);
         if (i + 1 < nend) ep *= ec.E;
-        pr[i * KT + kt] = ep;
+        prc[i * KT] = ep;
       }
       if (i + 1 < nz) br_arrive(s, ec, sn, sm, sa);
       br_put<V, KT>(w + 3 * KT, s);
       if (i == 0) br_put<V, KT>(X.R + kt, s);
-      if (!uniform) ec = el_get<T, KT>(el + (size_t)max(i - 1, 0) * EL_N * KT + kt);
+      // (the element above the chunk's first node is the last one of the chunk above)
+      if (!uniform) ec = el_get<T, KT>(elc + max(i - 1, 0) * EL_N * KT - (i == n0 && i > 0 ? ge : 0));
       br_leave(s, ec, sn, sm, sa);
     }
     br_put<V, KT>(X.P + (size_t)ch * 3 * KT + kt, s);
@@ -580,7 +599,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     for (int i = n0; i < nend; ++i, out += 6 * plane) {
       V w[6], o[6];
 #pragma unroll
-      for (int cc = 0; cc < 6; ++cc) w[cc] = W[((size_t)i * SL + cc) * KT + kt];
+      for (int cc = 0; cc < 6; ++cc) w[cc] = own[((size_t)i * SL + cc) * KT];
       if (ein) hooke_mode(w, m.lam, m.mu);
       node_special(o, w, g.kind == (T)2, m);
 #pragma unroll
@@ -598,19 +617,19 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   const int last = n0 + C - 1;  // node the P carry arrives at (a ragged last chunk has none: zero)
   T EA = 1;
   auto fin = [&](int i, const V* Li) {
-    V* w = W + (size_t)i * SL * KT + kt;
+    V* w = own + (size_t)i * SL * KT;
     Br<V> A = br_get<V, KT>(w), P = br_get<V, KT>(w + 3 * KT);
     T xA, xP, EP;
     if (uniform) {
       xA = ec.a * (T)(i - n0);
       xP = ec.a * (T)(last - i);
-      EA = pr[(i - n0) * KT + kt];
-      EP = pr[(last - i) * KT + kt];
+      EA = prc[(i - n0) * KT];
+      EP = prc[(last - i) * KT];
     } else {
       xA = g.q * (zs[i] - zs[n0]);
       xP = g.q * (zs[nend - 1] - zs[i]);
-      if (i > n0) EA *= el[((size_t)(i - 1) * EL_N) * KT + kt];
-      EP = pr[i * KT + kt];
+      if (i > n0) EA *= elc[(i - 1) * EL_N * KT];
+      EP = prc[i * KT];
     }
     br_add_prop(A, cA, EA, xA * EA);
     br_add_prop(P, cP, EP, xP * EP);
@@ -627,7 +646,7 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
   } else {
     for (int i = n0; i < nend; ++i) {
 #pragma unroll
-      for (int j = 0; j < 3; ++j) L[0][j] = W[((size_t)i * SL + 6 + j) * KT + kt];
+      for (int j = 0; j < 3; ++j) L[0][j] = own[((size_t)i * SL + 6 + j) * KT];
       fin(i, L[0]);
     }
   }
@@ -1137,8 +1156,11 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   d.ok = lim_of(KT) <= 227 * 1024 && KT * nch <= 256;
   // tile width of the launch: as wide as fits twice on an SM, and at least one 32-byte sector
   auto smem_of = [&](int kt) {
-    const size_t vals = (size_t)nz * (C <= 8 ? 6 : 9) * kt + 6 * (size_t)(nch + 1) * kt;
-    const size_t reals = (size_t)(c->uniform ? 0 : nz) * EL_N * kt + (size_t)(c->uniform ? C : nz) * kt + nz;
+    const int sl = C <= 8 ? 6 : 9, rb = kt * (int)sizeof(T);
+    const size_t vals = (size_t)nz * sl * kt + (size_t)nch * chunk_gap(C * sl, kt, 2 * rb) + 6 * (size_t)(nch + 1) * kt;
+    const size_t reals = (c->uniform ? (size_t)C * kt
+                                     : (size_t)nz * (EL_N + 1) * kt +
+                                           (size_t)nch * (chunk_gap(C * EL_N, kt, rb) + chunk_gap(C, kt, rb))) + nz;
     return vals * sizeof(V) + kt * sizeof(Col<T>) + reals * sizeof(T);
   };
   const int kmin = 32 / (int)sizeof(V);

@@ -101,3 +101,32 @@ def test_deep_uniform_grids_propagate_without_drift(n1, nz):
     bar = (C + -(-nz // C) + 10) * 2.0 ** -24
     last = slice(nz - C, nz)
     assert rel_l2(out["fp32"][last], out["fp64"][last]) < bar
+
+
+@pytest.mark.parametrize("n1,n2,nz", [(16, 8, 37), (4, 4, 23), (64, 4, 150)])
+@pytest.mark.parametrize("refined", [False, True])
+def test_chunk_lengths_agree_in_the_shared_memory_kernel(n1, n2, nz, refined):
+    """Every accepted chunk length, odd and even, with a ragged last chunk and tiles of every width: the
+    same operator to the rounding of FP64 (1e-13 of it), and FP32 within the operator's bar of FP64."""
+    torch = require_gpu()
+    from paper_1811_11558_gb300 import FvimError
+
+    z = 0.3 * np.linspace(0.0, 1.0, nz) ** (1.5 if refined else 1.0)
+    ep = inputs.plastic_strain_field(n1, n2, z, seed=48)
+    ref = None
+    for prec, chunks in (("fp64", range(2, 20)), ("fp32", range(9, 20))):
+        ctx = _ctx(n1, n2, z, prec)
+        d = to_dev(torch, ep, ctx.dtype)
+        ran = []
+        for C in chunks:
+            try:
+                ctx.set_plan(C)
+            except FvimError:
+                continue
+            u3 = torch.empty(ctx.surf_shape, dtype=ctx.dtype, device="cuda")
+            out = [t.cpu().numpy().astype(np.float64) for t in (ctx.apply_mindlin(d, u3=u3), u3)]
+            if ref is None:
+                ref = out
+            assert all(rel_l2(a, b) < (1e-13 if prec == "fp64" else 2e-5) for a, b in zip(out, ref)), (prec, C)
+            ran.append(C)
+        assert len(ran) > 6
