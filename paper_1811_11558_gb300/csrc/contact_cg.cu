@@ -41,29 +41,33 @@ enum { INV_U0 = 0, INV_U, INV_R };
 
 // ---- elementwise updates with FP64 scalars, rounded once to the path's precision ------------
 // FP32: the scalar as a float pair, products and sums as exact pairs (to about 2^-46 of the result
-// before its one rounding)
+// before its one rounding).  A leading sum that is not finite is the result: the rounding error taken
+// from it would be a NaN.  (For the same reason a scalar beyond FP32 is its largest value.)
 __device__ __forceinline__ float2 pair_of(double x) {
-  const float h = (float)x;
+  float h = (float)x;
+  if (isinf(h)) h = copysignf(3.402823466e+38f, h), x = (double)h;
   return make_float2(h, isfinite(h) ? (float)(x - (double)h) : 0.f);
 }
 // a + k x
 __device__ __forceinline__ float axpy1(float a, double, float2 k, float x) {
   const float p = __fmul_rn(k.x, x), pl = __fmaf_rn(k.x, x, -p);
   const float s = __fadd_rn(a, p), e = two_sum_err(a, p, s);
-  return __fadd_rn(s, __fadd_rn(e, __fmaf_rn(k.y, x, pl)));
+  const float r = __fadd_rn(s, __fadd_rn(e, __fmaf_rn(k.y, x, pl)));
+  return isfinite(s) ? r : s;
 }
 __device__ __forceinline__ double axpy1(double a, double k, float2, double x) { return a + k * x; }
 // k x
 __device__ __forceinline__ float mul1(double, float2 k, float x) {
-  const float p = __fmul_rn(k.x, x);
-  return __fadd_rn(p, __fmaf_rn(k.y, x, __fmaf_rn(k.x, x, -p)));
+  const float p = __fmul_rn(k.x, x), r = __fadd_rn(p, __fmaf_rn(k.y, x, __fmaf_rn(k.x, x, -p)));
+  return isfinite(p) ? r : p;
 }
 __device__ __forceinline__ double mul1(double k, float2, double x) { return k * x; }
 // u - h - c
 __device__ __forceinline__ float gap1(float u, float h, double, float2 c) {
   const float d = __fsub_rn(u, h), e = two_sum_err(u, -h, d);
   const float s = __fsub_rn(d, c.x), e2 = two_sum_err(d, -c.x, s);
-  return __fadd_rn(s, __fadd_rn(e2, __fsub_rn(e, c.y)));
+  const float r = __fadd_rn(s, __fadd_rn(e2, __fsub_rn(e, c.y)));
+  return isfinite(s) ? r : s;
 }
 __device__ __forceinline__ double gap1(double u, double h, double c, float2) { return u - h - c; }
 
@@ -75,14 +79,15 @@ __device__ __forceinline__ bool gap_lost(double c, double gb, double G, double n
 }
 
 // state of a new solve, with the scale of the initial pressure from its sum (a guess without load
-// is replaced by the uniform pressure)
+// is replaced by the uniform pressure, scale -1; one of infinite load scales to nothing, and the empty
+// contact that leaves is refused)
 template <typename T>
 __global__ void __launch_bounds__(256) k_pkf_begin(PkState* S, const T* __restrict__ p, size_t n, PkState init, double* part,
                                                    unsigned* cnt) {
   double v[4] = {0, 0, 0, 0};
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) v[0] += (double)p[i];
   if (grid_sum(v, part, cnt)) {
-    init.start = v[0] > 0 ? init.W / (init.dA * v[0]) : 0.0;
+    init.start = v[0] > 0 ? init.W / (init.dA * v[0]) : -1.0;
     *S = init;
   }
 }
@@ -144,7 +149,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
   for (int e = 0; e < 8; ++e) {
     if (!live) break;
     if constexpr (MODE == FWD_INIT) {
-      x[e] = start > 0 ? (T)(start * (double)a[e]) : (T)unif;
+      x[e] = start >= 0 ? (T)(start * (double)a[e]) : (T)unif;
       p[at(e)] = x[e];
       t[at(e)] = (T)0;
     } else if constexpr (MODE == FWD_P) {
@@ -634,11 +639,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
     cl.sync();
     if (tid < 32) {
       const double sum = value(total(0), 0);
-      if (tid == 0) S.start = sum > 0 ? S.W / (S.dA * sum) : 0.0;
+      if (tid == 0) S.start = sum > 0 ? S.W / (S.dA * sum) : -1.0;
     }
     __syncthreads();
     const double start = S.start, unif = S.unif;
-    for (int i = tid; i < E; i += nth) p[i] = start > 0 ? (T)(start * (double)p[i]) : (T)unif;
+    for (int i = tid; i < E; i += nth) p[i] = start >= 0 ? (T)(start * (double)p[i]) : (T)unif;
     __syncthreads();
     rows_fwd(p);
     cl.sync();

@@ -914,7 +914,7 @@ template <typename T> bool launch_rows_inv6_ct(const fvim_ctx* c, T* out, T nq_s
 // device state of one contact solve
 struct PkState {
   double nIc, gbar, G_old, beta, delta, tau, s, err;  // scalars of the iteration
-  double start, unif;                                  // scale of the initial pressure (0: uniform), uniform pressure
+  double start, unif;                                  // scale of the initial pressure (negative: uniform), uniform pressure
   double W, dA, dA_W, tol;                             // dA_W = dA / W
   float2 gbar2, beta2, tau2, s2;                       // the scalars of the elementwise steps as float pairs
   const void* h;

@@ -130,3 +130,34 @@ def test_chunk_lengths_agree_in_the_shared_memory_kernel(n1, n2, nz, refined):
             assert all(rel_l2(a, b) < (1e-13 if prec == "fp64" else 2e-5) for a, b in zip(out, ref)), (prec, C)
             ran.append(C)
         assert len(ran) > 6
+
+
+@pytest.mark.parametrize("n1,n2", [(64, 64), (64, 32)])       # one cluster; six kernels
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_contact_refuses_infinite_input(n1, n2, prec):
+    """An infinite height above a point without starting pressure re-enters the contact with an infinite
+    pressure, an infinite starting pressure leaves no contact: both are refused.  An infinite depth below
+    such a point is a hole like any other."""
+    torch = require_gpu()
+    from paper_1811_11558_gb300 import FvimError
+
+    ctx = _ctx(n1, n2, inputs.uniform_depth(2, 0.1), prec)
+    h, W = _hertz(torch, ctx)
+    guess = torch.ones_like(h)
+    guess[1, 2] = 0
+    up = h.clone()
+    up[1, 2] = float("inf")
+    with pytest.raises(FvimError, match="non-finite"):
+        ctx.elastic_contact(up, W, guess.clone())
+    inf = guess.clone()
+    inf[n2 // 2, n1 // 2] = float("inf")
+    with pytest.raises(FvimError, match="non-finite"):
+        ctx.elastic_contact(h, W, inf)
+    res = []
+    for depth in (float("-inf"), -10.0):
+        down, p = h.clone(), guess.clone()
+        down[1, 2] = depth
+        ctx.elastic_contact(down, W, p)
+        assert p[1, 2] == 0
+        res.append(p.cpu().numpy().astype(np.float64))
+    assert rel_l2(res[0], res[1]) < (1e-9 if prec == "fp64" else 2e-5)
