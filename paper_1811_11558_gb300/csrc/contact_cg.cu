@@ -23,7 +23,7 @@
 // What bounds it: an FP64 instruction holds its pipe for 64 cycles per warp here (a conversion
 // counts as one), so a kernel's time is its FP64 instructions per warp and the dependent chain of
 // its sums.  So: four complex values per thread (more warps with less each); elementwise FP32
-// updates in two-float arithmetic, rounded once as the FP64 expression is; FP64 only in the sums,
+// updates in words of FP32, rounded once as the FP64 expression is; FP64 only in the sums,
 // and there only at points that carry pressure; a warp's sums of several values reduced together.
 // us per iteration, fourteen kernels -> seven with eight values per thread and FP64 updates -> this
 // (with all of a thread's points read before the first store): 256^2 83 -> 46, 512^2 132 -> 75 ->
@@ -40,36 +40,61 @@ enum { FWD_INIT = 0, FWD_P, FWD_T };
 enum { INV_U0 = 0, INV_U, INV_R };
 
 // ---- elementwise updates with FP64 scalars, rounded once to the path's precision ------------
-// FP32: the scalar as a float pair, products and sums as exact pairs (to about 2^-46 of the result
-// before its one rounding).  A leading sum that is not finite is the result: the rounding error taken
-// from it would be a NaN.  (For the same reason a scalar beyond FP32 is its largest value.)
-__device__ __forceinline__ float2 pair_of(double x) {
-  float h = (float)x;
-  if (isinf(h)) h = copysignf(3.402823466e+38f, h), x = (double)h;
-  return make_float2(h, isfinite(h) ? (float)(x - (double)h) : 0.f);
+// FP32: the scalar's 53 bits in three words and a power of two, products and sums error-free in two
+// words, a third for what they leave.  Over 2^21 draws each, the result is the exact value's rounding
+// wherever the FP64 expression's is; where a sum cancels to its last bits the FP64 expression is off in
+// 3.3e-2 of the draws and this in 2.9e-5 (the scalar in two floats only: 2.1e-1).  A leading sum that is not
+// finite is the result: the rounding error taken from it would be a NaN.
+
+// x = (x + y + z) w, the words of a number in [1, 2) with x's sign; integer operations, for an FP64
+// conversion holds the pipe as long as an addition
+__device__ __forceinline__ float4 words_of(double x) {
+  const long long u = __double_as_longlong(x);
+  const int ex = (int)(u >> 52) & 0x7ff;
+  const float one = u < 0 ? -1.f : 1.f;
+  if (ex > 1023 - 126 && ex < 1023 + 127) {
+    const long long m = (u & 0xfffffffffffffll) | 0x10000000000000ll;
+    return make_float4(one * (float)(int)(m >> 29) * 0x1p-23f, one * (float)((int)(m >> 5) & 0xffffff) * 0x1p-47f,
+                       one * (float)((int)m & 31) * 0x1p-52f, __int_as_float((ex - 1023 + 127) << 23));
+  }
+  if (x == 0) return make_float4(0.f, 0.f, 0.f, 1.f);
+  // beyond FP32's exponents (or not finite): the nearest scale, the largest value where that is too little
+  const float w = ex < 1023 ? 0x1p-126f : 0x1p127f;
+  const double r = ex < 1023 ? x * 0x1p126 : x * 0x1p-127;
+  float a = (float)r;
+  if (isinf(a) && ex != 0x7ff) a = one * 3.402823466e+38f;
+  return make_float4(a, 0.f, 0.f, w);
+}
+__device__ __forceinline__ float4 words_neg(float4 k) { return make_float4(-k.x, -k.y, -k.z, k.w); }
+// s + (t + lo) rounded once
+__device__ __forceinline__ float three_sum(float s, float t, float lo) {
+  const float r = __fadd_rn(s, t), v = __fadd_rn(r, __fadd_rn(two_sum_err(s, t, r), lo));
+  return isfinite(s) ? v : s;
 }
 // a + k x
-__device__ __forceinline__ float axpy1(float a, double, float2 k, float x) {
-  const float p = __fmul_rn(k.x, x), pl = __fmaf_rn(k.x, x, -p);
-  const float s = __fadd_rn(a, p), e = two_sum_err(a, p, s);
-  const float r = __fadd_rn(s, __fadd_rn(e, __fmaf_rn(k.y, x, pl)));
-  return isfinite(s) ? r : s;
+__device__ __forceinline__ float axpy1(float a, double, float4 k, float x) {
+  x = __fmul_rn(x, k.w);
+  const float p = __fmul_rn(k.x, x), pl = __fmaf_rn(k.x, x, -p), q = __fmul_rn(k.y, x);
+  const float r = __fmaf_rn(k.z, x, __fmaf_rn(k.y, x, -q));
+  const float s = __fadd_rn(a, p), e = two_sum_err(a, p, s), t = __fadd_rn(e, pl), u = __fadd_rn(t, q);
+  return three_sum(s, u, __fadd_rn(__fadd_rn(two_sum_err(e, pl, t), two_sum_err(t, q, u)), r));
 }
-__device__ __forceinline__ double axpy1(double a, double k, float2, double x) { return a + k * x; }
+__device__ __forceinline__ double axpy1(double a, double k, float4, double x) { return a + k * x; }
 // k x
-__device__ __forceinline__ float mul1(double, float2 k, float x) {
-  const float p = __fmul_rn(k.x, x), r = __fadd_rn(p, __fmaf_rn(k.y, x, __fmaf_rn(k.x, x, -p)));
-  return isfinite(p) ? r : p;
+__device__ __forceinline__ float mul1(double, float4 k, float x) {
+  x = __fmul_rn(x, k.w);
+  const float p = __fmul_rn(k.x, x), pl = __fmaf_rn(k.x, x, -p), q = __fmul_rn(k.y, x);
+  const float r = __fmaf_rn(k.z, x, __fmaf_rn(k.y, x, -q)), t = __fadd_rn(pl, q);
+  return three_sum(p, t, __fadd_rn(two_sum_err(pl, q, t), r));
 }
-__device__ __forceinline__ double mul1(double k, float2, double x) { return k * x; }
+__device__ __forceinline__ double mul1(double k, float4, double x) { return k * x; }
 // u - h - c
-__device__ __forceinline__ float gap1(float u, float h, double, float2 c) {
-  const float d = __fsub_rn(u, h), e = two_sum_err(u, -h, d);
-  const float s = __fsub_rn(d, c.x), e2 = two_sum_err(d, -c.x, s);
-  const float r = __fadd_rn(s, __fadd_rn(e2, __fsub_rn(e, c.y)));
-  return isfinite(s) ? r : s;
+__device__ __forceinline__ float gap1(float u, float h, double, float4 c) {
+  const float d = __fsub_rn(u, h), e = two_sum_err(u, -h, d), c0 = c.x * c.w, c1 = c.y * c.w, c2 = c.z * c.w;
+  const float s = __fsub_rn(d, c0), e2 = two_sum_err(d, -c0, s), t = __fadd_rn(e2, e), v = __fsub_rn(t, c1);
+  return three_sum(s, v, __fsub_rn(__fadd_rn(two_sum_err(e2, e, t), two_sum_err(t, -c1, v)), c2));
 }
-__device__ __forceinline__ double gap1(double u, double h, double c, float2) { return u - h - c; }
+__device__ __forceinline__ double gap1(double u, double h, double c, float4) { return u - h - c; }
 
 // Whether sums about the mean gap c have lost the new mean gb and G = sum g^2 over n points: c is far
 // above everything that is left (a point whose depth dominated the mean has gone out of contact).
@@ -124,7 +149,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
   const T* h = static_cast<const T*>(S->h);
   const size_t i0 = (size_t)(live ? 2 * pair : 0) * N + tt;
   const double start = S->start, unif = S->unif, tau = S->tau, gbar = S->gbar, beta = S->beta;
-  const float2 tau2 = S->tau2, gbar2 = S->gbar2, beta2 = S->beta2;
+  const float4 tauw = S->tauw, gbarw = S->gbarw, betaw = S->betaw;
   V v[4];
   double sum[4] = {0, 0, 0, 0};
   int nol = 0;
@@ -156,11 +181,11 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
       const T po = a[e], gi = c[e];
       T pn = (T)0;
       if (po != (T)0 || b[e] != (T)0) {
-        const T y = axpy1(po, -tau, make_float2(-tau2.x, -tau2.y), b[e]);
+        const T y = axpy1(po, -tau, words_neg(tauw), b[e]);
         pn = y > (T)0 ? y : (T)0;
       }
       if (pn == (T)0 && gi < (T)0) {
-        pn = mul1(-tau, make_float2(-tau2.x, -tau2.y), gi);
+        pn = mul1(-tau, words_neg(tauw), gi);
         ++nol;
       }
       pold[at(e)] = po;
@@ -168,9 +193,9 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
       if (pn != (T)0) sum[0] += (double)pn;
       x[e] = pn;
     } else {
-      const T gi = gap1(c[e], d[e], gbar, gbar2);
+      const T gi = gap1(c[e], d[e], gbar, gbarw);
       g[at(e)] = gi;
-      x[e] = a[e] > (T)0 ? axpy1(gi, beta, beta2, b[e]) : (T)0;
+      x[e] = a[e] > (T)0 ? axpy1(gi, beta, betaw, b[e]) : (T)0;
       t[at(e)] = x[e];
     }
   }
@@ -203,7 +228,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_fwd(PkState* S, const T* __res
       } else {
         const double x = S->W / (S->dA * sum[0]);
         S->s = x;
-        S->s2 = pair_of(x);
+        S->sw = words_of(x);
       }
     }
   }
@@ -225,7 +250,7 @@ __global__ void __launch_bounds__(512) k_pkf_cols(const PkState* S, typename Cx<
   V* col = plane + at;
   V v[4];
   const double scl = SCALE ? S->s : 1.0;
-  const float2 scl2 = S->s2;
+  const float4 sclw = S->sw;
   T f0[4];
 #pragma unroll
   for (int m = 0; m < 4; ++m) {
@@ -235,7 +260,7 @@ __global__ void __launch_bounds__(512) k_pkf_cols(const PkState* S, typename Cx<
   const SurfColSm<V> sm{reinterpret_cast<V*>(smraw), kc, f};
   fft4_ct<V, false, N, 1>(v, t, sm, tw);
 #pragma unroll
-  for (int m = 0; m < 4; ++m) v[m] = cscale(v[m], SCALE ? mul1(scl, scl2, f0[m]) : f0[m]);
+  for (int m = 0; m < 4; ++m) v[m] = cscale(v[m], SCALE ? mul1(scl, sclw, f0[m]) : f0[m]);
   fft4_ct<V, true, N, 1>(v, t, sm, tw);
 #pragma unroll
   for (int m = 0; m < 4; ++m) col[(size_t)(t + m * T4) * h1] = v[m];
@@ -292,7 +317,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   const SurfSm<V, N> sm{reinterpret_cast<V*>(smraw) + (size_t)r * LD};
   fft4_ct<V, true, N, 1>(v, tt, sm, tw);
   const double scl = S->s, gbar = S->gbar;
-  const float2 scl2 = S->s2;
+  const float4 sclw = S->sw;
   double sum[4] = {0, 0, 0, 0};
   int nc = 0;
 #pragma unroll
@@ -311,7 +336,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
       T pi = fp[e];
       if constexpr (MODE == INV_U) {
         if (pi != (T)0) {
-          pi = mul1(scl, scl2, pi);
+          pi = mul1(scl, sclw, pi);
           p[at(e)] = pi;
         }
         if (pi != fb[e]) sum[2] += fabs((double)pi - (double)fb[e]);
@@ -371,7 +396,7 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
     const double den = sum[3] * S->nIc - sum[0] * sum[1];
     const double tau = den != 0 ? sum[2] * S->nIc / den : 0.0;
     S->tau = tau;
-    S->tau2 = pair_of(tau);
+    S->tauw = words_of(tau);
     return;
   }
   int done = 0, bad = 0;
@@ -388,12 +413,12 @@ __global__ void __launch_bounds__(512) k_pkf_rows_inv(PkState* S, const T* __res
   } else {
     const double mean = sum[0] / sum[3], gb = (MODE == INV_U ? (redo ? S->gbar : gbar) : 0.0) + mean;
     S->gbar = gb;
-    S->gbar2 = pair_of(gb);
+    S->gbarw = words_of(gb);
     if (MODE == INV_U) {
       // (a gap that vanishes to the last bit restarts the direction)
       const double G = fmax(sum[1] - sum[0] * mean, 0.0), beta = S->G_old > 0 ? S->delta * (G / S->G_old) : 0.0;
       S->beta = beta;
-      S->beta2 = pair_of(beta);
+      S->betaw = words_of(beta);
       S->G_old = G;
     }
   }
@@ -597,10 +622,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
   // this CTA's columns: transform, compliance (times the load scale), inverse, rows to their owners
   auto cols = [&](bool scaled) {
     const double s = scaled ? S.s : 1.0;
-    const float2 s2 = scaled ? S.s2 : make_float2(1.f, 0.f);
+    const float4 sw = scaled ? S.sw : make_float4(1.f, 0.f, 0.f, 1.f);
     cl_fft<T, N, false>(
         xch, tw, [&](int f, int i) { return colb[f * N + i]; },
-        [&](int f, int i, V x) { colb[f * N + i] = cscale(x, scaled ? mul1(s, s2, green[f * N + i]) : green[f * N + i]); });
+        [&](int f, int i, V x) { colb[f * N + i] = cscale(x, scaled ? mul1(s, sw, green[f * N + i]) : green[f * N + i]); });
     __syncthreads();
     cl_fft<T, N, true>(
         xch, tw, [&](int f, int i) { return colb[f * N + i]; },
@@ -667,7 +692,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
           S.done = 1;
         } else {
           S.gbar = sum / n;
-          S.gbar2 = pair_of(S.gbar);
+          S.gbarw = words_of(S.gbar);
         }
       }
     }
@@ -692,11 +717,11 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
     // g, conjugate direction
     {
       const double gbar = S.gbar, beta = S.beta;
-      const float2 gbar2 = S.gbar2, beta2 = S.beta2;
+      const float4 gbarw = S.gbarw, betaw = S.betaw;
       for (int i = tid; i < E; i += nth) {
-        const T gi = gap1(u[i], h[i], gbar, gbar2);
+        const T gi = gap1(u[i], h[i], gbar, gbarw);
         g[i] = gi;
-        t[i] = p[i] > (T)0 ? axpy1(gi, beta, beta2, t[i]) : (T)0;
+        t[i] = p[i] > (T)0 ? axpy1(gi, beta, betaw, t[i]) : (T)0;
       }
     }
     __syncthreads();
@@ -724,14 +749,14 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
       if (tid == 0) {
         const double den = srt * S.nIc - sr * st;
         S.tau = den != 0 ? sgt * S.nIc / den : 0.0;
-        S.tau2 = pair_of(S.tau);
+        S.tauw = words_of(S.tau);
       }
     }
     __syncthreads();
     // pressure step
     {
       const double tau = S.tau;
-      const float2 mt = make_float2(-S.tau2.x, -S.tau2.y);
+      const float4 mt = words_neg(S.tauw);
       double a = 0;
       int nol = 0;
       for (int i = tid; i < E; i += nth) {
@@ -763,7 +788,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
           S.done = 1;
         } else {
           S.s = S.W / (S.dA * sum);
-          S.s2 = pair_of(S.s);
+          S.sw = words_of(S.s);
         }
       }
     }
@@ -775,13 +800,13 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
     // load scale, change, mean gap and G
     {
       const double s = S.s, gbar = S.gbar;
-      const float2 s2 = S.s2;
+      const float4 sw = S.sw;
       double a = 0, b = 0, c = 0;
       int n = 0;
       for (int i = tid; i < E; i += nth) {
         T pi = p[i];
         if (pi != (T)0) {
-          pi = mul1(s, s2, pi);
+          pi = mul1(s, sw, pi);
           p[i] = pi;
         }
         if (pi != po[i]) c += fabs((double)pi - (double)po[i]);
@@ -812,10 +837,10 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
           const double mean = sd / n, G = fmax(sdd - sd * mean, 0.0);
           redo = !done && gap_lost(S.gbar, S.gbar + mean, G, n);
           S.gbar += mean;
-          S.gbar2 = pair_of(S.gbar);
+          S.gbarw = words_of(S.gbar);
           if (!redo) {
             S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
-            S.beta2 = pair_of(S.beta);
+            S.betaw = words_of(S.beta);
             S.G_old = G;
           }
         }
@@ -847,9 +872,9 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(ClCfg<T, N>::BT)
       if (tid < 32) {
         const double G = value(total(2), 0);
         if (tid == 0) {
-          S.gbar2 = pair_of(gbar);
+          S.gbarw = words_of(gbar);
           S.beta = S.G_old > 0 ? S.delta * (G / S.G_old) : 0.0;
-          S.beta2 = pair_of(S.beta);
+          S.betaw = words_of(S.beta);
           S.G_old = G;
         }
       }

@@ -916,7 +916,7 @@ struct PkState {
   double nIc, gbar, G_old, beta, delta, tau, s, err;  // scalars of the iteration
   double start, unif;                                  // scale of the initial pressure (negative: uniform), uniform pressure
   double W, dA, dA_W, tol;                             // dA_W = dA / W
-  float2 gbar2, beta2, tau2, s2;                       // the scalars of the elementwise steps as float pairs
+  float4 gbarw, betaw, tauw, sw;                       // the scalars of the elementwise steps in words of FP32
   const void* h;
   void* p;
   int done, it, bad, max_it;

@@ -712,7 +712,7 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
   memset(&s0, 0, sizeof(s0));
   s0.G_old = 1.0;
   s0.s = 1.0;
-  s0.s2 = make_float2(1.f, 0.f);
+  s0.sw = make_float4(1.f, 0.f, 0.f, 1.f);
   s0.err = INFINITY;
   s0.unif = W / (c->L1 * c->L2);
   s0.W = W;
