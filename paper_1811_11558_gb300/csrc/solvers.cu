@@ -681,9 +681,18 @@ static bool device_cg_enabled() {
   return !(e && e[0] == '0');
 }
 
-// The fused iteration (contact_cg.cu): one WHILE graph per context, whatever the surface, pressure,
-// load and tolerance (all in the device state), one read of the state per solve; with
-// FVIM_DEVICE_CG=0, graphs off or while kernels are timed, batches of iterations with one read each.
+// small square surfaces take the cluster kernel unless FVIM_CONTACT_CLUSTER=0 (read on every solve)
+static bool contact_cluster_enabled() {
+  const char* e = getenv("FVIM_CONTACT_CLUSTER");
+  return !(e && e[0] == '0');
+}
+
+// The fused iteration (contact_cg.cu).  Small square surfaces: the whole solve as one cluster launch,
+// which is no graph and no loop of the host's (FVIM_DEVICE_CG, FVIM_SOLVER_GRAPHS and profiling do not
+// change it).  Others, and those where the launch is refused or switched off: one WHILE graph per context,
+// whatever the surface, pressure, load and tolerance (all in the device state), one read of the state
+// per solve; with FVIM_DEVICE_CG=0, graphs off or while kernels are timed, batches of iterations with
+// one read each.
 template <typename T>
 int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_opts* o, int* iters, double* err_out) {
   const size_t n = (size_t)c->n1 * c->n2;
@@ -724,15 +733,17 @@ int elastic_contact_fused(fvim_ctx* c, const T* h, double W, T* p, const fvim_op
   s0.max_it = o->cg_max_iter;
   PkState* sh = reinterpret_cast<PkState*>(c->h_part + (size_t)RMAXB * NVMAX);  // pinned
   int rc;
-  if (pkf_small(c)) {
-    if ((rc = pkf_solve_small<T>(a, s0))) return rc;
-    if (FVIM_CU(cudaMemcpyAsync(sh, a.S, sizeof(PkState), cudaMemcpyDeviceToHost, c->stream)) ||
-        FVIM_CU(cudaStreamSynchronize(c->stream)))
-      return FVIM_ERR_CUDA;
-    if (sh->bad) return FVIM_ERR_NONFINITE;
-    if (iters) *iters = sh->it;
-    if (err_out) *err_out = sh->err;
-    return sh->err < o->cg_tol ? FVIM_OK : FVIM_ERR_NOT_CONVERGED;
+  if (pkf_small(c) && contact_cluster_enabled()) {
+    if (pkf_solve_small<T>(a, s0) == FVIM_OK) {
+      if (FVIM_CU(cudaMemcpyAsync(sh, a.S, sizeof(PkState), cudaMemcpyDeviceToHost, c->stream)) ||
+          FVIM_CU(cudaStreamSynchronize(c->stream)))
+        return FVIM_ERR_CUDA;
+      if (sh->bad) return FVIM_ERR_NONFINITE;
+      if (iters) *iters = sh->it;
+      if (err_out) *err_out = sh->err;
+      return sh->err < o->cg_tol ? FVIM_OK : FVIM_ERR_NOT_CONVERGED;
+    }
+    cudaGetLastError();  // the cluster launch was refused (nothing ran): the six kernels below
   }
   // the arrival counter of the sums, whatever an earlier solve left in it
   if (FVIM_CU(cudaMemsetAsync(a.cnt, 0, sizeof(unsigned), c->stream))) return FVIM_ERR_CUDA;

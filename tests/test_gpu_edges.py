@@ -161,3 +161,23 @@ def test_contact_refuses_infinite_input(n1, n2, prec):
         assert p[1, 2] == 0
         res.append(p.cpu().numpy().astype(np.float64))
     assert rel_l2(res[0], res[1]) < (1e-9 if prec == "fp64" else 2e-5)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_small_contact_without_the_cluster(prec, monkeypatch):
+    """The six kernels take over on the surfaces of the cluster kernel (FVIM_CONTACT_CLUSTER=0, or a refused
+    launch): the same pressure at the bar of the contact solve, not the same bits (the sums add up in
+    another order)."""
+    torch = require_gpu()
+    ctx = _ctx(64, 64, inputs.uniform_depth(2, 0.1), prec)
+    h = to_dev(torch, inputs.self_affine_surface(64, 1.0, 0.8, 4, 8, 16, 0.1, seed=7), ctx.dtype)
+    W = 2e-2 * ES * 0.1
+    opts = ctx.default_opts(cg_tol=1e-13) if prec == "fp64" else ctx.default_opts()
+    p = {}
+    for mode in ("1", "0"):
+        monkeypatch.setenv("FVIM_CONTACT_CLUSTER", mode)
+        p[mode] = torch.zeros_like(h)
+        ctx.elastic_contact(h, W, p[mode], opts)
+    assert not torch.equal(p["0"], p["1"])
+    a, b = (p[m].cpu().numpy().astype(np.float64) for m in "01")
+    assert rel_l2(a, b) < (1e-9 if prec == "fp64" else 2e-5)
