@@ -716,8 +716,10 @@ size_t fvim_footprint(int n1, int n2, int nz, int precision) {
   const size_t h = (size_t)spec_stride(n1, n2);
   const size_t spec = (size_t)nz * 6 * n2 * h * 2 * es + (size_t)nz * 6 * n2 * es;
   const size_t state = nv * 6 * es * 2 + nv * es + ns * es;
-  const size_t solver = 8 * nv * 6 * es + nv * es + 13 * ns * es + 64 * 1024;
-  return spec + state + solver + (size_t)(n1 + n2) * 2 * es + (size_t)n2 * h * 2 * es;
+  // (twelve surface arrays, and one for the captured solver loops)
+  const size_t solver = 8 * nv * 6 * es + nv * es + 13 * ns * es + (size_t)nz * sizeof(double) + kPartBytes +
+                        kScalarBlock + kDfsBytes + kPkfBytes;
+  return spec + state + solver + (size_t)(n1 + n2) * 2 * es + (size_t)n2 * h * 2 * es + (size_t)(n2 + nz) * es + 16;
 }
 
 int fvim_sync(fvim_ctx* c) {

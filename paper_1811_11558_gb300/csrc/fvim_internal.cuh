@@ -716,6 +716,13 @@ template <typename K> inline void smem_cap(K kern, size_t smem) {
 // ---------------------------------------------------------------------------
 #define FVIM_NSOLVER_BUFS 26
 
+// fixed parts of the solver workspace, bytes
+constexpr int kDfsBlocks = 4096;  // blocks of the DF-SANE residual pass (at least one per plane, 3072 planes)
+constexpr size_t kPartBytes = (size_t)kDfsBlocks * 4 * sizeof(double);  // block partials, up to four values each
+constexpr size_t kScalarBlock = 256;  // scalars of the solver loops (V_PKS)
+constexpr size_t kDfsBytes = 1024;    // device DF-SANE state (V_DFS)
+constexpr size_t kPkfBytes = 512;     // fused contact iteration (V_PKF): PkState, arrival counter at byte 256
+
 struct fvim_ctx {
   int no_pdl;  // launches without the programmatic-serialisation attribute (solver graph capture)
   // h1: row stride of the half spectrum (complex); power-of-two grids: N1/2 columns (the

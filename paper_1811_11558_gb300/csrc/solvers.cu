@@ -27,11 +27,6 @@ namespace {
 constexpr int RT = 256;       // threads of a reduction block
 constexpr int RMAXB = 1024;   // blocks of a reduction grid
 constexpr int NVMAX = 3;      // values reduced per pass
-constexpr int DFS_BLOCKS = 4096;  // blocks of the DF-SANE residual pass (at least one per plane, 3072 planes)
-constexpr size_t kPartBytes = (size_t)DFS_BLOCKS * 4 * sizeof(double);  // block partials, up to four values each
-constexpr size_t kScalarBlock = 256;  // bytes of the solver's device scalar block (V_PKS)
-constexpr size_t kDfsBytes = 1024;     // bytes of the device DF-SANE state (V_DFS)
-constexpr size_t kPkfBytes = 512;      // fused contact iteration (V_PKF): PkState, arrival counter at byte 256
 
 // surface buffers [N2][N1]
 enum { S_P = 0, S_POLD, S_T, S_G, S_U, S_R, S_H, S_H0, S_DU, S_DUPREV, S_TPREV, S_DT, S_NSURF };
@@ -1195,12 +1190,12 @@ template <typename T> int build_dfloop(fvim_ctx* c, SolverRT* r, size_t n, int g
             (T)c->lam, (T)c->mu, (T)c->sigma_y, (T)c->E_h, flow_range(c));
         FVIM_CUDA_CHECK_LAUNCH();
         if ((e = apply_mindlin_t<T>(c, S<T>(c, V_DEP), S<T>(c, V_TMP), FVIM_STRAIN, nullptr, flow_range(c)))) return e;
-        // FP32 planes of a power of two: whole blocks per plane, about DFS_BLOCKS / 4 in all
+        // FP32 planes of a power of two: whole blocks per plane, about kDfsBlocks / 4 in all
         const size_t nxy = (size_t)c->n1 * c->n2;
         const bool by_plane = sizeof(T) == 4 && nxy == (size_t)1 << lgxy && lgxy >= 2;
         const int planes = c->nz * 6;
         const int per_plane =
-            by_plane ? (int)std::min<size_t>((nxy / 4 + RT - 1) / RT, std::max(1, DFS_BLOCKS / 4 / planes)) : 0;
+            by_plane ? (int)std::min<size_t>((nxy / 4 + RT - 1) / RT, std::max(1, kDfsBlocks / 4 / planes)) : 0;
         const int g = by_plane ? planes * per_plane : grd;
         k_dfd_res_sy<T><<<g, RT, 0, c->stream>>>(dfs, S<T>(c, V_B), S<T>(c, V_TMP), (const double*)c->sv[V_WZ], lgxy, n,
                                                  per_plane, (double*)c->sv[V_PART], dfs_count(c), flow_range(c), cond);

@@ -144,3 +144,19 @@ def test_no_cpu_fallback():
     if not torch.cuda.is_available():
         with pytest.raises(RuntimeError):
             fvim.Context(8, 8, np.array([0.0, 0.1]))
+
+
+@pytest.mark.parametrize("n1,n2,nz", [(32, 32, 2), (64, 64, 8), (16, 4, 512), (81, 27, 5)])
+def test_footprint_covers_what_a_context_allocates(n1, n2, nz):
+    """The reported device bytes are at least the sum of a context's allocations once its solvers have
+    run: scratch, plastic state, and the solver workspace with its 128 KB of block partials."""
+    from paper_1811_11558_gb300 import fvim
+
+    h = n1 // 2 if not (n1 & 1 or n2 & 1) else (n1 // 2 + 16) // 16 * 16
+    ns, nv = n1 * n2, n1 * n2 * nz
+    for prec, es in ((fvim.FVIM_FP32, 4), (fvim.FVIM_FP64, 8)):
+        scratch = nz * 6 * n2 * h * 2 * es + nz * 6 * n2 * es + n2 * h * 2 * es + n2 * es
+        tables = (n1 + n2) * 2 * es + nz * es + 16
+        state = 13 * nv * es + ns * es
+        work = 12 * ns * es + 8 * 6 * nv * es + nv * es + nz * 8 + 4096 * 4 * 8 + 256 + 1024 + 512
+        assert fvim.lib().fvim_footprint(n1, n2, nz, prec) >= scratch + tables + state + work
