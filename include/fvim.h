@@ -209,7 +209,8 @@ const char* fvim_last_cuda_error(void);
  *                 the shared-memory variant (FP64, deep grids), whose scan is sequential.
  *   depth_ctas    CTAs per SM the FP32 register variant of the depth kernel is compiled for:
  *                 2 (the default; chunks of 2 and 3 nodes run four and three) or 3 (80 registers, chunk lengths
- *                 4..8 whose tile fits three times in shared memory); 0 for the shared-memory
+ *                 4..8 whose tile fits three times in shared memory; where the element table of a refined
+ *                 grid leaves no room for that, a plan of 3 runs, and reports, 2); 0 for the shared-memory
  *                 variant (FP64, deep grids), which has one launch shape per chunk length
  */
 #define FVIM_PLAN_MAX_CAND 16
@@ -256,6 +257,7 @@ int fvim_autotune(fvim_ctx* ctx, int reps, fvim_plan* out);
  * (n1, n2, nz, precision as in fvim_create), in timing order: chunk lengths in chunks[0..] and
  * the register budget of each (CTAs per SM, 2 or 3; 0 for the shared-memory variant) in
  * ctas[0..] (host arrays, at most max_chunks entries; ctas may be NULL); returns their number.
+ * On refined depth nodes the tuner leaves out the three-CTA shapes whose tile does not fit thrice.
  * Host computation only (no device, no context).  FVIM_ERR_ARG on a grid fvim_create refuses
  * or a bad output array. */
 int fvim_plan_candidates(int n1, int n2, int nz, int precision, int* chunks, int* ctas, int max_chunks);

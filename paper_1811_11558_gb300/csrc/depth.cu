@@ -1111,7 +1111,7 @@ template <typename T> struct DepthCfg {
   bool reg;       // FP32 register variant
   int C, nch, KT, threads;
   size_t smem;
-  int mb;         // register variant: CTAs per SM it is compiled for (2: 128 registers, 3: 85)
+  int mb;         // register variant: register budget (2: 128 registers, 3: 80, for three CTAs per SM)
 };
 
 int depth_chunk_default(int nz) {
@@ -1125,8 +1125,9 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   const int nz = c->nz, h1 = c->h1;
   d.ok = false;
   if (C < 2 || C > nz) return d;
-  // the launch limits of a plan: 16-column tiles of [Nz][6] values and 12 values per chunk (register
-  // variant) or per node (shared-memory variant), which every layout below stays within
+  // the launch limits of a plan (what fvim_set_plan accepts): 16-column tiles of [Nz][6] values and 12
+  // values per chunk (register variant) or per node (shared-memory variant).  A refined grid's element
+  // table comes on top of them: what is launched is sized by its own layout below
   constexpr size_t kMom = 6 * sizeof(V);
   if constexpr (sizeof(T) == 4) {
     // FP32, 16-column tiles, at most 8 nodes per chunk: the register variant (C rounded up
@@ -1137,10 +1138,13 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
       const size_t lim = (size_t)nz * 6 * 16 * sizeof(V) + (size_t)(2 * nchr) * 16 * kMom +
                          (size_t)3 * 16 * sizeof(V) + (((size_t)nz * sizeof(T) + 7) & ~(size_t)7) + 16;
       if (lim <= 227 * 1024 && 16 * nchr <= 256) {
-        // three CTAs per SM (80 registers): chunk lengths 4..8 whose tile fits three times
+        // three CTAs per SM (80 registers): chunk lengths 4..8; accepted by the limits, launched where the
+        // tile itself fits three times (64 refined layers in chunks of 4 take 89 KB and run the 128-register
+        // build, as two CTAs)
         if (ctas == 3 && !(CR >= 4 && 3 * (lim + 1024) <= 228 * 1024)) return d;
-        d = DepthCfg<T>{true, true, CR, nchr, 16, 16 * nchr, RegSmem<T, 16>::bytes(nz, nchr, c->uniform) + 16,
-                        ctas == 3 ? 3 : 2};
+        const size_t bytes = RegSmem<T, 16>::bytes(nz, nchr, c->uniform) + 16;
+        d = DepthCfg<T>{true, true, CR, nchr, 16, 16 * nchr, bytes,
+                        ctas == 3 && 3 * (bytes + 1024) <= 228 * 1024 ? 3 : 2};
         return d;
       }
     }
@@ -1174,11 +1178,14 @@ template <typename T> DepthCfg<T> depth_cfg(const fvim_ctx* c, int C, int ctas) 
   return d;
 }
 
-int depth_launch_ctas(const fvim_ctx* c) {
-  const int C = c->depth_chunk > 0 ? c->depth_chunk : depth_chunk_default(c->nz);
+int depth_shape_ctas(const fvim_ctx* c, int chunk, int ctas) {
   if (c->prec == FVIM_FP64) return 0;
-  const DepthCfg<float> d = depth_cfg<float>(c, C, c->depth_ctas);
+  const DepthCfg<float> d = depth_cfg<float>(c, chunk, ctas);
   return d.ok && d.reg ? d.mb : 0;
+}
+
+int depth_launch_ctas(const fvim_ctx* c) {
+  return depth_shape_ctas(c, c->depth_chunk > 0 ? c->depth_chunk : depth_chunk_default(c->nz), c->depth_ctas);
 }
 
 bool depth_chunk_ok(const fvim_ctx* c, int C, int ctas) {

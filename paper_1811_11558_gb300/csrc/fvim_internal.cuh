@@ -814,7 +814,9 @@ inline void launch_chain(const fvim_ctx* c, void (*kern)(P...), dim3 grid, dim3 
 int depth_chunk_default(int nz);
 // ctas: CTAs per SM the FP32 register variant is compiled for (2 default, 3 with 80 registers)
 bool depth_chunk_ok(const fvim_ctx* c, int chunk, int ctas = 2);
-// CTAs per SM of the depth kernel's launch under the context's plan (0: shared-memory variant)
+// CTAs per SM the depth kernel is launched for with a chunk length and register budget, and under the
+// context's plan (0: shared-memory variant; a budget of 3 whose tile does not fit three times gives 2)
+int depth_shape_ctas(const fvim_ctx* c, int chunk, int ctas);
 int depth_launch_ctas(const fvim_ctx* c);
 // process-wide plan table (tune.cu): the tuned chunk length of a grid, or 0; its tuned FFT
 // path, or -1

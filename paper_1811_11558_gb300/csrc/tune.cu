@@ -40,7 +40,7 @@ PlanKey key_of(const fvim_ctx* c) { return PlanKey(c->prec, c->n1, c->n2, c->nz,
 
 // candidate launch shapes (chunk length, CTAs per SM): the instantiated register-variant
 // lengths, two longer ones and the default rule, each with the default register budget, then
-// the lengths that also build for three CTAs per SM
+// the lengths that also run three CTAs per SM
 struct Cand {
   int C, ctas;
   bool operator==(const Cand& o) const { return C == o.C && ctas == o.ctas; }
@@ -51,7 +51,8 @@ std::vector<Cand> candidates(const fvim_ctx* c) {
   for (int ctas : {2, 3})
     for (int C : base) {
       const Cand k{C, ctas};
-      if (depth_chunk_ok(c, C, ctas) && std::find(v.begin(), v.end(), k) == v.end()) v.push_back(k);
+      if (depth_chunk_ok(c, C, ctas) && (ctas == 2 || depth_shape_ctas(c, C, 3) == 3) &&
+          std::find(v.begin(), v.end(), k) == v.end()) v.push_back(k);
     }
   if ((int)v.size() > FVIM_PLAN_MAX_CAND) v.resize(FVIM_PLAN_MAX_CAND);
   return v;
@@ -227,9 +228,11 @@ int fvim_autotune(fvim_ctx* c, int reps, fvim_plan* out) {
 int fvim_plan_candidates(int n1, int n2, int nz, int precision, int* chunks, int* ctas, int max_chunks) {
   if (!grid_ok(n1, n2) || nz < 2 || nz > 512) return FVIM_ERR_ARG;
   if ((precision != FVIM_FP32 && precision != FVIM_FP64) || !chunks || max_chunks < 1) return FVIM_ERR_ARG;
-  // the launch rules need the grid and precision only: a host-side description of the grid
+  // a host-side description of the grid, with uniform depth nodes (refined ones leave some of the
+  // three-CTA shapes out)
   fvim_ctx g;
   memset(&g, 0, sizeof(g));
+  g.uniform = 1;
   g.n1 = n1;
   g.n2 = n2;
   g.nz = nz;

@@ -181,3 +181,22 @@ def test_small_contact_without_the_cluster(prec, monkeypatch):
     assert not torch.equal(p["0"], p["1"])
     a, b = (p[m].cpu().numpy().astype(np.float64) for m in "01")
     assert rel_l2(a, b) < (1e-9 if prec == "fp64" else 2e-5)
+
+
+def test_three_cta_plans_run_where_their_tile_fits_thrice():
+    """A plan for three CTAs per SM is accepted on refined nodes as on uniform ones; where the element
+    table of the refined grid takes the room, it runs and reports two, and the tuner does not time it."""
+    torch = require_gpu()
+    uni = inputs.uniform_depth(64, 0.4)
+    ref = 0.4 * np.linspace(0.0, 1.0, 64) ** 1.5
+    short = 0.4 * np.linspace(0.0, 1.0, 32) ** 1.5
+    for z, ctas in ((uni, 3), (ref, 2), (short, 3)):
+        ctx = _ctx(128, 32, z, "fp32")
+        d = to_dev(torch, inputs.plastic_strain_field(128, 32, z, seed=47), torch.float32)
+        ctx.set_plan(4, depth_ctas=2)
+        two = ctx.apply_mindlin(d).cpu().numpy()
+        ctx.set_plan(4, depth_ctas=3)
+        assert ctx.plan["depth_ctas"] == ctas
+        three = ctx.apply_mindlin(d).cpu().numpy()
+        assert rel_l2(three, two) < 1e-6
+        assert (4 in ctx.autotune(reps=3).get("timings_ms_3ctas", {})) == (ctas == 3)
