@@ -85,7 +85,8 @@ template <int CW> struct ColPairSm {
 };
 
 }  // namespace
-// 1024-point columns, 8 per CTA: 361 -> 339 us per direction at 1024 x 1024 x 32
+// 1024-point columns, 8 per CTA: fewer table reads than the products apart; apply at 1024 x 1024 x 32
+// 1591 -> 1547 us
 template <> struct UseBf2<float2, 1024, ColPairSm<8>> {
   static constexpr bool v = true;
 };
