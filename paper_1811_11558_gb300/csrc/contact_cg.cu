@@ -447,14 +447,12 @@ __global__ void __launch_bounds__(256) k_pkf_gap(PkState* S, const T* __restrict
 template <typename T, int N, int MODE> void rows_fwd(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
   const SurfRowCfg r = surf_row_cfg<T, N>(a.n2);
-  surf_row_smem_cap(k_pkf_rows_fwd<T, N, MODE>, r.smem);
   k_pkf_rows_fwd<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(a.S, (const T*)a.u, (T*)a.g, (T*)a.t, (T*)a.pold,
                                                                    (V*)a.surf, (const V*)a.tw1, a.n2, a.part, a.cnt);
 }
 template <typename T, int N, int MODE> void rows_inv(const PkfArgs& a) {
   typedef typename Cx<T>::t V;
   const SurfRowCfg r = surf_row_cfg<T, N>(a.n2);
-  surf_row_smem_cap(k_pkf_rows_inv<T, N, MODE>, r.smem);
   k_pkf_rows_inv<T, N, MODE><<<r.grid, r.threads, r.smem, a.stream>>>(
       a.S, (const T*)a.g, (const T*)a.t, (const T*)a.pold, (T*)a.u, (const V*)a.surf, (const V*)a.tw1, a.n2,
       (T)(1.0 / ((double)N * (double)a.n2)), a.part, a.cnt, a.cond, a.use_cond);

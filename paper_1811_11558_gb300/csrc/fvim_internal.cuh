@@ -578,7 +578,9 @@ template <typename V> struct SurfColSm {
   __device__ __forceinline__ V get(int p) const { return buf[p * kc + f]; }
 };
 
-// CTA of a row pass: about one transform pair per CTA and SM, whole warps
+// CTA of a row pass: about one transform pair per CTA and SM, whole warps.  At most 512 threads, each
+// with four values and their padding: 36 KB of dynamic shared memory in FP64, below the 48 KB that need
+// a raised limit, also beside the static arrays of the contact kernels.
 struct SurfRowCfg {
   int grid, threads;
   size_t smem;
@@ -590,6 +592,7 @@ template <typename T, int N> inline SurfRowCfg surf_row_cfg(int n2) {
   while (slots * 2 * 128 <= pairs && slots * 2 * T4 <= 512) slots *= 2;
   const int threads = slots * T4 > 32 ? slots * T4 : 32;
   slots = threads / T4;
+  static_assert((size_t)512 / T4 * SurfSm<V, N>::LD * sizeof(V) <= 36 * 1024, "row CTAs need no shared-memory opt-in");
   return SurfRowCfg{(pairs + slots - 1) / slots, threads, (size_t)slots * SurfSm<V, N>::LD * sizeof(V)};
 }
 
@@ -698,13 +701,6 @@ inline int smem_optin_max() {
   }();
   return v;
 }
-// dynamic shared memory cap of the row kernels (at most four FP64 transforms of 1024 points; they
-// hold static shared memory too, so not the whole opt-in maximum); the same value on every call
-template <typename K> inline void surf_row_smem_cap(K kern, size_t smem) {
-  if (smem <= 40 * 1024) return;
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
-}
-
 // multiprocessors of the current device
 inline int sm_count() {
   static const int v = [] {

@@ -201,7 +201,6 @@ template <typename T> bool launch_surf_rows_fwd(const fvim_ctx* c, const T* f) {
 #define CASE(N)                                                                                                 \
   if (c->n1 == N) {                                                                                             \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                             \
-    smem_cap(k_surf_rows_fwd<T, N>, r.smem);                                                                            \
     launch_chain(c, k_surf_rows_fwd<T, N>, r.grid, r.threads, r.smem, f, (V*)c->surf, (const V*)c->tw1, c->n2);   \
     return true;                                                                                                \
   }
@@ -215,7 +214,6 @@ template <typename T> bool launch_surf_rows_inv(const fvim_ctx* c, T* f, T scale
 #define CASE(N)                                                                                                       \
   if (c->n1 == N) {                                                                                                   \
     const SurfRowCfg r = surf_row_cfg<T, N>(c->n2);                                                                   \
-    smem_cap(k_surf_rows_inv<T, N>, r.smem);                                                                                  \
     launch_chain(c, k_surf_rows_inv<T, N>, r.grid, r.threads, r.smem, (const V*)c->surf, f, (const V*)c->tw1, c->n2, scale); \
     return true;                                                                                                      \
   }
