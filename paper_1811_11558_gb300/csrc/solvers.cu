@@ -1243,10 +1243,8 @@ int plasticity_t(fvim_ctx* c, const T* dT, T* dE, T* deps_p, T* dep, const fvim_
   const int M = 10;
   const double gamma = 1e-4, smin = 1e-10, smax = 1e10, tmin = 0.1, tmax = 0.5;
   std::vector<double> hist(1, f);
-  // the spectral step lives on the device (after the plasticity state block)
+  // the host loop's spectral step lives on the device (after the plasticity state block)
   double* dsig = reinterpret_cast<double*>(static_cast<char*>(c->sv[V_PKS]) + 128);
-  k_set_double<<<1, 1, 0, c->stream>>>(dsig, 1.0);
-  FVIM_CUDA_CHECK_LAUNCH();
   int k = 0;
   bool conv_ok = false;
   // stagnation at the rounding floor of the path precision: the best residual of the
@@ -1312,6 +1310,10 @@ int plasticity_t(fvim_ctx* c, const T* dT, T* dE, T* deps_p, T* dep, const fvim_
     c->sv[V_XT] = xt;
     c->sv[V_F] = F;
     c->sv[V_FT] = Ft;
+  }
+  if (!ran_device) {
+    k_set_double<<<1, 1, 0, c->stream>>>(dsig, 1.0);
+    FVIM_CUDA_CHECK_LAUNCH();
   }
   for (k = ran_device ? k : 0; !ran_device && k < o->df_max_iter; ++k) {
     if (!isfinite(f)) return FVIM_ERR_NONFINITE;
