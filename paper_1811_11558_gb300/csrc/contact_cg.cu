@@ -916,13 +916,17 @@ inline int flat_grid(size_t n) { return (int)std::min<size_t>((n + 255) / 256, 2
 
 }  // namespace
 
-bool pkf_small(const fvim_ctx* c) { return !c->gen && c->n1 == c->n2 && c->n1 >= 16 && c->n1 <= 128; }
+// (FP64 at 128^2: eight SMs hold too few FP64 pipes, 120 us an iteration there against 66 in six kernels)
+bool pkf_small(const fvim_ctx* c) {
+  return !c->gen && c->n1 == c->n2 && c->n1 >= 16 && c->n1 <= (c->prec == FVIM_FP64 ? 64 : 128);
+}
 
 template <typename T> int pkf_solve_small(const PkfArgs& a, const PkState& init) {
   if (a.n1 == 16) return cluster_solve<T, 16>(a, init);
   if (a.n1 == 32) return cluster_solve<T, 32>(a, init);
   if (a.n1 == 64) return cluster_solve<T, 64>(a, init);
-  if (a.n1 == 128) return cluster_solve<T, 128>(a, init);
+  if constexpr (sizeof(T) == 4)
+    if (a.n1 == 128) return cluster_solve<T, 128>(a, init);
   return FVIM_ERR_UNSUPPORTED;
 }
 
