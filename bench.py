@@ -375,7 +375,41 @@ def run_gpu(args):
         pg.barrier()
         pg.destroy_process_group()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        # the per-problem and per-increment records go to stderr: the line stays short enough to be read
+        # from the tail of a captured output
+        print(json.dumps({"detail": line}), file=sys.stderr, flush=True)
+        print(json.dumps(short_line(line)), flush=True)
+
+
+LINE_MAX = 8000  # characters of the result line
+
+
+def short_line(line):
+    """The result line without the records of single problems, requests and increments: inside the
+    metrics of whole workloads, lists that hold records or more than eight values are left out, and
+    numbers keep six digits; if the line is still longer than LINE_MAX, the largest of those metrics go."""
+    def cut(x):
+        if isinstance(x, dict):
+            y = {k: cut(v) for k, v in x.items()}
+            return {k: v for k, v in y.items() if v is not None or x[k] is None}
+        if isinstance(x, (list, tuple)):
+            if len(x) > 8 or any(isinstance(v, (dict, list, tuple)) for v in x):
+                return None
+            return [cut(v) for v in x]
+        return float("%.6g" % x) if isinstance(x, float) else x
+
+    sections = [k for k in ("solves", "scaling_sweep", "group_apply") if k in line]
+    out = {k: cut(v) if k in sections else v for k, v in line.items()}
+    while len(json.dumps(out)) > LINE_MAX and sections:
+        big = max(sections, key=lambda k: len(json.dumps(out[k])))
+        if isinstance(out[big], dict) and len(out[big]) > 1:
+            sub = dict(out[big])
+            sub.pop(max(sub, key=lambda k: len(json.dumps(sub[k]))))
+            out[big] = sub
+        else:
+            out.pop(big)
+            sections.remove(big)
+    return out
 
 
 def hertz_case():

@@ -78,3 +78,25 @@ def test_batch_runs_every_problem_with_the_carried_relaxation():
     for pb in bench.batch_problems(64, 1814):
         assert pb["relax_mode"] == 1
         assert pb["relax"] == (0.3 if pb["rough"] else 0.5)
+
+
+def test_result_line_is_short_and_keeps_the_contract():
+    """The line printed on stdout stays below bench.LINE_MAX characters with every workload's metrics in
+    it (a 23 KB line did not survive a captured output's tail); contract keys pass unchanged."""
+    import json
+
+    keys = {"metric": bench.METRIC, "value": 1.25e10, "unit": bench.UNIT, "n_gpus": 1, "steps": 20, "warmup": 5,
+            "ms_per_step": 0.65123456789, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
+            "dtype": "f32", "data": "synthetic", "gpu_launches": 100, "config": {"workload": "w", "n1": 512},
+            "e2e": {"value": 6.5e9, "h2d_bytes_per_step": 402653184, "d2h_bytes_per_step": 402653184},
+            "clocks": {"sm_mhz": 2070.0, "sm_max_mhz": 2070.0, "reasons": []}}
+    rec = [{"n": 512, "nz": 32, "ms": 3444.142112000, "iters": [3, 13, 24, 30, 30]} for _ in range(64)]
+    big = dict(keys, solves={"batch": {"solves_per_s": 1.23456789, "per_problem": rec, "grids": [64, 128, 256, 512]}},
+               scaling_sweep={"ms": {"fp32_%d" % n: 0.1234567891 for n in (4, 8, 16)}})
+    out = bench.short_line(big)
+    assert {k: out[k] for k in keys} == keys
+    assert out["solves"]["batch"] == {"solves_per_s": 1.23457, "grids": [64, 128, 256, 512]}
+    assert out["scaling_sweep"]["ms"]["fp32_8"] == 0.123457
+    many = dict(big, solves={"m%d" % i: {"x%d" % j: 0.123456789 for j in range(40)} for i in range(40)})
+    assert len(json.dumps(bench.short_line(many))) <= bench.LINE_MAX
+    assert {k: bench.short_line(many)[k] for k in keys} == keys
