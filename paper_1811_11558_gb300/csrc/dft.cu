@@ -14,21 +14,28 @@
 //   X(k), X(N - k) = a(0) + C(k) -+ i S(k),  C = sum (a(n) + a(N - n)) cos,  S = sum (a(n) - a(N - n)) sin
 // (plus (-1)^k a(N/2) on an even side), and likewise for the inverse rows: half the terms, and two
 // outputs from each column sum.  The inner loops keep one twiddle for several rows or columns per
-// thread (eight rows, four complex columns), read as broadcast vectors: what bounded the plain form
+// thread (FP32: eight rows, four complex columns), read as broadcast vectors: what bounded the plain form
 // was two shared-memory reads per multiply-add.  81 x 81 x 32 FP32, us: rows 39 -> 14, columns 33 ->
 // 18, inverse rows 37 -> 16 (event-bracketed launches); apply 143 -> 64.
 #include "fvim_internal.cuh"
 
 namespace {
 
-constexpr int RB = 32;    // rows per CTA (row kernels)
-constexpr int RT = 8;     // rows per thread
-constexpr int CT = 16;    // columns per CTA (column kernel)
-constexpr int CC = 4;     // columns per thread
+// Rows per thread RT (row kernels, four times as many per CTA), columns per CTA and thread CT, CC (column
+// kernel).  FP32: several per thread, which share a twiddle.  FP64 sums are bound by the FP64 pipe, one per
+// scheduler, whatever they read, so there one each, for the most warps: eight rows and four columns per
+// thread left 8 CTAs for the rows of 256 x 5 x 8.  Applies with u3, us, plain sums -> several -> one: 256 x
+// 5 x 8 418 -> 938 -> 155, 255 x 64 x 8 2026 -> 994 -> 613, 81 x 81 x 32 2377 -> 674 -> 563.
+template <typename T> struct Dft {
+  static constexpr int RT = sizeof(T) == 4 ? 8 : 1, RB = 4 * RT, CT = sizeof(T) == 4 ? 16 : 2, CC = sizeof(T) == 4 ? 4 : 1;
+  static constexpr int LD = RB + 16 / (int)sizeof(T);  // row stride of the folded tables (the fill walks them along n)
+};
 
 // RT consecutive values of T at a 16-byte boundary
-template <typename T> __device__ __forceinline__ void ld_rows(T (&v)[RT], const T* p) {
-  if constexpr (sizeof(T) == 4) {
+template <typename T, int RT> __device__ __forceinline__ void ld_rows(T (&v)[RT], const T* p) {
+  if constexpr (RT == 1) {
+    v[0] = p[0];
+  } else if constexpr (sizeof(T) == 4) {
 #pragma unroll
     for (int q = 0; q < RT; q += 4) {
       const float4 a = *reinterpret_cast<const float4*>(p + q);
@@ -43,8 +50,8 @@ template <typename T> __device__ __forceinline__ void ld_rows(T (&v)[RT], const 
   }
 }
 // CC complex columns at a 16-byte boundary
-template <typename V> __device__ __forceinline__ void ld_cols(V (&v)[CC], const V* p) {
-  if constexpr (sizeof(V) == 8) {
+template <typename V, int CC> __device__ __forceinline__ void ld_cols(V (&v)[CC], const V* p) {
+  if constexpr (sizeof(V) == 8 && CC % 2 == 0) {
 #pragma unroll
     for (int q = 0; q < CC; q += 2) {
       const float4 a = *reinterpret_cast<const float4*>(p + q);
@@ -56,10 +63,6 @@ template <typename V> __device__ __forceinline__ void ld_cols(V (&v)[CC], const 
     for (int q = 0; q < CC; ++q) v[q] = p[q];
   }
 }
-// row stride of the folded tables: RB values and 16 bytes (the fill walks them along n)
-template <typename T> struct RowLd {
-  static constexpr int v = RB + 16 / (int)sizeof(T);
-};
 
 // forward row DFTs of real rows: src [rows][n1] -> dst [rows][ldh] (k1 < hs, zeros above)
 template <typename T>
@@ -69,7 +72,7 @@ __global__ void __launch_bounds__(256) k_dft_rows_fwd(const T* __restrict__ src,
   chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int LD = RowLd<T>::v;
+  constexpr int LD = Dft<T>::LD, RT = Dft<T>::RT, RB = Dft<T>::RB;
   const int H = n1 / 2, J = (n1 - 1) / 2;             // folded terms n = 1 .. J
   T* P = reinterpret_cast<T*>(smraw);                 // [H + 1][LD] sums; row 0: a(0), row H of an even side: a(N/2)
   T* Q = P + (size_t)(H + 1) * LD;                    // [H + 1][LD] differences
@@ -131,6 +134,7 @@ __global__ void __launch_bounds__(256) k_dft_cols(typename Cx<T>::t* __restrict_
   chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
+  constexpr int CT = Dft<T>::CT, CC = Dft<T>::CC;
   const int H = n2 / 2, J = (n2 - 1) / 2;
   V* P = reinterpret_cast<V*>(smraw);       // [H + 1][CT] sums; row 0: a(0), row H of an even side: a(N/2)
   V* Q = P + (size_t)(H + 1) * CT;          // [H + 1][CT] differences
@@ -198,7 +202,7 @@ __global__ void __launch_bounds__(256) k_dft_rows_inv(const typename Cx<T>::t* _
   chain_begin();
   typedef typename Cx<T>::t V;
   extern __shared__ __align__(16) unsigned char smraw[];
-  constexpr int LD = RowLd<T>::v;
+  constexpr int LD = Dft<T>::LD, RT = Dft<T>::RT, RB = Dft<T>::RB;
   const int H = n1 / 2, J = (n1 - 1) / 2;
   T* P = reinterpret_cast<T*>(smraw);                 // [H + 1][LD] real parts (H = hs - 1)
   T* Q = P + (size_t)(H + 1) * LD;                    // [H + 1][LD] imaginary parts
@@ -263,9 +267,9 @@ inline int dft_threads(int items) {
 
 template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, void* dst, size_t rows) {
   typedef typename Cx<T>::t V;
-  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
+  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * Dft<T>::LD * sizeof(T);
   smem_cap(k_dft_rows_fwd<T>, smem);
-  launch_chain(c, k_dft_rows_fwd<T>, (unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * c->h1), smem, src, (V*)dst, (const V*)c->tw1, c->n1,
+  launch_chain(c, k_dft_rows_fwd<T>, (unsigned)((rows + Dft<T>::RB - 1) / Dft<T>::RB), dft_threads(4 * c->h1), smem, src, (V*)dst, (const V*)c->tw1, c->n1,
                                                                                 c->hs, c->h1, rows);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;
@@ -273,6 +277,7 @@ template <typename T> int launch_dft_rows_fwd(const fvim_ctx* c, const T* src, v
 
 template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void* planes, int nplanes) {
   typedef typename Cx<T>::t V;
+  constexpr int CT = Dft<T>::CT, CC = Dft<T>::CC;
   const size_t smem = (size_t)c->n2 * sizeof(V) + (size_t)2 * (c->n2 / 2 + 1) * CT * sizeof(V);
   const int threads = dft_threads(CT / CC * (c->n2 / 2 + 1));
   dim3 grid(c->h1 / CT, nplanes);
@@ -289,9 +294,9 @@ template <typename T> int launch_dft_cols(const fvim_ctx* c, bool inverse, void*
 
 template <typename T> int launch_dft_rows_inv(const fvim_ctx* c, const void* src, T* dst, size_t rows, T scale) {
   typedef typename Cx<T>::t V;
-  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * RowLd<T>::v * sizeof(T);
+  const size_t smem = (size_t)c->n1 * sizeof(V) + (size_t)2 * (c->n1 / 2 + 1) * Dft<T>::LD * sizeof(T);
   smem_cap(k_dft_rows_inv<T>, smem);
-  launch_chain(c, k_dft_rows_inv<T>, (unsigned)((rows + RB - 1) / RB), dft_threads(RB / RT * (c->n1 / 2 + 1)), smem, (const V*)src, dst, (const V*)c->tw1,
+  launch_chain(c, k_dft_rows_inv<T>, (unsigned)((rows + Dft<T>::RB - 1) / Dft<T>::RB), dft_threads(4 * (c->n1 / 2 + 1)), smem, (const V*)src, dst, (const V*)c->tw1,
                                                                                 c->n1, c->hs, c->h1, rows, scale);
   FVIM_CUDA_CHECK_LAUNCH();
   return FVIM_OK;

@@ -200,3 +200,25 @@ def test_three_cta_plans_run_where_their_tile_fits_thrice():
         three = ctx.apply_mindlin(d).cpu().numpy()
         assert rel_l2(three, two) < 1e-6
         assert (4 in ctx.autotune(reps=3).get("timings_ms_3ctas", {})) == (ctas == 3)
+
+
+@pytest.mark.parametrize("n1,n2,nz", [(3, 3, 2), (255, 2, 2), (256, 3, 2), (3, 256, 2), (4, 255, 2), (33, 7, 3)])
+@pytest.mark.parametrize("prec", ["fp64", "fp32"])
+def test_direct_transforms_at_their_limits(n1, n2, nz, prec):
+    """Direct DFTs of the shortest and longest sides next to short ones (few rows, columns and CTAs), through
+    the operator and the surface convolution, at the operators' bars."""
+    torch = require_gpu()
+    from oracle import operators as op
+
+    z = inputs.uniform_depth(nz, 0.02)
+    ep = inputs.plastic_strain_field(n1, n2, z, seed=49)
+    p = np.abs(inputs.random_field((n2, n1), seed=50)) + 0.5
+    ref, u3_ref = op.mindlin_apply(ep, z, 1.0, 1.0, E, NU, "stress", with_surface=True)
+    ctx = _ctx(n1, n2, z, prec)
+    u3 = torch.empty(ctx.surf_shape, dtype=ctx.dtype, device="cuda")
+    out = ctx.apply_mindlin(to_dev(torch, ep, ctx.dtype), u3=u3)
+    bu = torch.empty_like(u3)
+    ctx.apply_boussinesq(to_dev(torch, p, ctx.dtype), u3=bu)
+    tol = 1e-10 if prec == "fp64" else 2e-5
+    assert rel_l2(out.cpu().numpy(), ref) < tol and rel_l2(u3.cpu().numpy(), u3_ref) < tol
+    assert rel_l2(bu.cpu().numpy(), op.boussinesq_apply(p, z, 1.0, 1.0, E, NU, "stress")[0]) < tol
