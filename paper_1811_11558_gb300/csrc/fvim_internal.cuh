@@ -657,11 +657,33 @@ __device__ __forceinline__ float two_sum_err(float a, float b, float s) {  // a 
   const float bb = __fsub_rn(s, a);
   return __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
 }
-// running sum of FP32 values as an exact pair
-__device__ __forceinline__ void pair_add(float2& a, float x) {
-  const float s = __fadd_rn(a.x, x);
-  a.y = __fadd_rn(a.y, two_sum_err(a.x, x, s));
-  a.x = s;
+// Running sum of FP32 values in three words: the rounding of each word goes to the next, only the
+// last word's is lost (below 2^-70 of the sum; an FP64 sum loses 2^-53 at every addition).
+struct Sum3 {
+  float a, b, c;
+};
+__device__ __forceinline__ void sum3_add(Sum3& s, float x) {
+  const float a = __fadd_rn(s.a, x), e = two_sum_err(s.a, x, a);
+  const float b = __fadd_rn(s.b, e);
+  s.c = __fadd_rn(s.c, two_sum_err(s.b, e, b));
+  s.a = a;
+  s.b = b;
+}
+// Three such sums in FP64, by a whole warp.  The third words, zero up to two values per sum, are added
+// only where a lane has one, and by a call: FP64 instructions under a predicate hold the pipe all the same.
+static __device__ __noinline__ double sum3_third(double v, float c) { return v + (double)c; }
+__device__ __forceinline__ void sum3_values(const Sum3& x, const Sum3& y, const Sum3& z, double& vx, double& vy, double& vz) {
+  vx = (double)x.b;
+  vy = (double)y.b;
+  vz = (double)z.b;
+  if (__any_sync(0xffffffffu, x.c != 0.f || y.c != 0.f || z.c != 0.f)) {
+    vx = sum3_third(vx, x.c);
+    vy = sum3_third(vy, y.c);
+    vz = sum3_third(vz, z.c);
+  }
+  vx += (double)x.a;
+  vy += (double)y.a;
+  vz += (double)z.a;
 }
 
 // ---------------------------------------------------------------------------

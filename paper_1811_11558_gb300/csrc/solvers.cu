@@ -1110,22 +1110,22 @@ __global__ void __launch_bounds__(RT) k_dfd_res_sy(DFS* s, const T* __restrict__
       sy = s0 * y0 + s1 * y1 + s2 * y2 + s3 * y3;
     };
     if (per_plane > 0) {
-      // per_plane blocks per plane: one weight per block, the thread's sums as exact FP32 pairs (an
-      // FP64 multiply-add per four values held the FP64 pipe as long as the memory traffic took)
+      // per_plane blocks per plane: one weight per block, the thread's sums in three FP32 words, which
+      // lose less than FP64 ones (an FP64 multiply-add per four values held the FP64 pipe as long as the
+      // memory traffic took)
       const unsigned zc = blockIdx.x / per_plane, sub = blockIdx.x - zc * per_plane;
       const size_t n4 = (size_t)1 << (lgxy - 2), base = (size_t)zc * n4;
-      float2 a0 = make_float2(0.f, 0.f), a1 = a0, a2 = a0;
+      Sum3 a0 = {0.f, 0.f, 0.f}, a1 = a0, a2 = a0;
       for (size_t j = sub * (size_t)RT + threadIdx.x; j < n4; j += (size_t)per_plane * RT) {
         float ff, ss, sy;
         four(base + j, ff, ss, sy);
-        pair_add(a0, ff);
-        pair_add(a1, ss);
-        pair_add(a2, sy);
+        sum3_add(a0, ff);
+        sum3_add(a1, ss);
+        sum3_add(a2, sy);
       }
       const double w = plane_weight(wz, zc);
-      v[0] = w * ((double)a0.x + (double)a0.y);
-      v[1] = w * ((double)a1.x + (double)a1.y);
-      v[2] = w * ((double)a2.x + (double)a2.y);
+      sum3_values(a0, a1, a2, v[0], v[1], v[2]);
+      for (int q = 0; q < 3; ++q) v[q] *= w;
     } else {
       const size_t n4 = n >> 2;
       const int lg4 = lgxy - 2;
