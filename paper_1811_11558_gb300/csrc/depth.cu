@@ -494,19 +494,24 @@ __global__ void __launch_bounds__(256) k_mindlin_depth(typename Cx<T>::t* __rest
     }
   }
   for (int i = threadIdx.x; i < nz; i += blockDim.x) zs[i] = zn[i];
-  // column constants while the tile is in flight, and on a uniform grid the powers E^0 .. E^(C-1) of
-  // its propagator, for distances within a chunk; on a refined grid the coefficients of element e
-  // below node e (none, zero, below the last node).  Longer distances take an exponential each (one
-  // per thread and two per column): a power carries the rounding of E as many times as there are
-  // elements.  Error of the operator on a smooth strain, powers over the whole depth -> this: FP32 512
-  // layers 6.1e-6 -> 9.3e-7, FP64 126 layers 1.9e-15 -> 6.5e-16; 128 x 128 x 126 FP64 1320.6 -> 1322.9 us.
+  // column constants while the tile is in flight; on a refined grid the coefficients of element e below
+  // node e (none, zero, below the last node); on a uniform grid the propagators over 0 .. C - 1 elements,
+  // for distances within a chunk: FP64 as powers (an exponential costs eighteen multiplications), FP32 by
+  // an exponential each, as longer distances in both (one per thread and two per column): a power carries
+  // the rounding of E as many times as there are elements.  Error of the operator on a smooth strain,
+  // powers over the whole depth -> this: FP32 512 layers 6.1e-6 -> 5.4e-7 (powers within chunks: 8.5e-7),
+  // FP64 126 layers 1.9e-15 -> 6.5e-16; 128 x 128 x 126 FP64 1320.6 -> 1322.9 us.
   if (threadIdx.x < KT) {
     col_put<T>(cols + kt, k1, k2, n1, n2, hs, w1, w2, m, uniform != 0, hz, C, zn[min(C - 1, nz - 1)] - zn[0]);
-    if (uniform) {
+    if (uniform && sizeof(T) == 8) {
       T p = 1;
       const T E = cols[kt].in.E;
       for (int k = 0; k < C; ++k, p *= E) pr[k * KT + kt] = p;
     }
+  }
+  if (uniform && sizeof(T) == 4) {
+    const T a = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2).q * hz;
+    for (int k = ch; k < C; k += nch) pr[k * KT + kt] = dexp<T>(-a * (T)k);
   }
   if (!uniform) {
     const T q = mode_geom<T>(k1, k2, n1, n2, hs, w1, w2).q;
