@@ -289,14 +289,16 @@ const char* fvim_profile_name(int slot);
 
 /* ------------------------------------------------------------------------------------
  * Solvers.  Vectors live on the device in the context's precision; every reduction
- * (dot products, norms, the total load) is accumulated in FP64 in a fixed order (block
- * partials summed in block order by the last block to finish), so repeated runs give
- * bitwise identical results.  The iteration logic runs on the device: the contact CG's
+ * (dot products, norms, the total load) is accumulated in a fixed order (block partials
+ * summed in block order by the last block to finish), in FP64 or, inside a thread of the FP32
+ * path, in three FP32 words that lose less than FP64 does, so repeated runs give bitwise
+ * identical results.  The iteration logic runs on the device: the contact CG's
  * scalars (step, conjugation, rigid shift, load scaling, stop test) are kept in device
  * memory; the CG iterations and DF-SANE's iterations with its line search each run inside
  * one captured CUDA graph (a device-side WHILE loop), and the host reads their state once
  * per solve (batches of captured CG iterations with one status read per batch when
- * FVIM_DEVICE_CG=0).  Every loop has an iteration cap, enforced on the device.
+ * FVIM_DEVICE_CG=0; small square surfaces run the whole contact solve as one cluster kernel
+ * unless FVIM_CONTACT_CLUSTER=0).  Every loop has an iteration cap, enforced on the device.
  * ------------------------------------------------------------------------------------ */
 #define FVIM_MAX_INCREMENTS 64
 

@@ -27,7 +27,7 @@
 // and there only at points that carry pressure; a warp's sums of several values reduced together.
 // us per iteration, fourteen kernels -> seven with eight values per thread and FP64 updates -> this
 // (with all of a thread's points read before the first store): 256^2 83 -> 46, 512^2 132 -> 75 ->
-// 53, 1024^2 206 -> 156 -> 115 (smaller squares: the cluster kernel below).
+// 53, 1024^2 206 -> 156 -> 118 (smaller squares: the cluster kernel below).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -475,8 +475,8 @@ template <typename T, int N, bool SCALE> void cols(const PkfArgs& a) {
 // back, and sums are exchanged the same way, each CTA adding the eight partials in rank order (the
 // same value everywhere, so every decision is the same everywhere).  Six cluster barriers per
 // iteration (about 350 cycles each); the loop ends at the stop test or the iteration cap.
-// us per iteration, six kernels -> this: FP64 32^2 56 -> 22, FP32 32^2 41 -> 13, 64^2 42 -> 21, 128^2
-// 47 -> 33 (256^2 does not fit).
+// us per iteration, six kernels -> this: FP64 32^2 55 -> 22, 64^2 57 -> 36, FP32 32^2 35 -> 12, 64^2 37 -> 20,
+// 128^2 45 -> 31 (256^2 does not fit).
 constexpr int CL = 8;
 
 // Stockham stages of radix 2 on two values per thread (FP64: the pipes are idle but for the few

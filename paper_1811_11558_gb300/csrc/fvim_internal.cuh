@@ -787,7 +787,7 @@ struct fvim_ctx {
   void* srt;       // solver runtime (solvers.cu): own stream, events, captured CUDA graphs
   int depth_chunk; // depth nodes per chunk thread of the depth kernel; 0: depth_chunk_default
   int plan_tuned;  // depth_chunk came from a timing run (fvim_autotune) in this process
-  int depth_ctas;  // CTAs per SM of the FP32 register depth kernel: 0 or 2 (128 registers), 3 (85)
+  int depth_ctas;  // CTAs per SM of the FP32 register depth kernel: 0 or 2 (128 registers), 3 (80)
   float depth_cut; // chunk-scan cutoff eps_co of the FP32 register depth kernel (0: exact scan)
   void* tmap;      // CUtensorMap (host, 64-byte aligned) over the spectrum for the depth tile, or NULL
   int tma_rows;    // rows (z, component) per tensor-copy box of the depth tile; 0: no tensor copies

@@ -333,8 +333,9 @@ template <typename T> __global__ void k_count_pos(const T* __restrict__ a, size_
 // Plane zc = (z, c) of the volume has the trapezoid weight dA w_z, doubled for the three
 // shear components.  N1 N2 is a power of two, so the plane of an index is a shift.  FP32
 // vectors are processed four values at a time: the four products are summed in FP32 and
-// the partial is accumulated in FP64 (one FP64 multiply-add per four values); FP64
-// vectors keep every operation in FP64.
+// the partial is accumulated in FP64 (one FP64 multiply-add per four values), in the device
+// loop's pass over whole planes in three FP32 words (k_dfd_res_sy); FP64 vectors keep every
+// operation in FP64.
 __device__ __forceinline__ double plane_weight(const double* wz, unsigned zc) {
   return wz[zc / 6] * ((zc % 6) < 3 ? 1.0 : 2.0);
 }
