@@ -66,6 +66,8 @@ template <typename T> int ensure_ws(fvim_ctx* c) {
   for (int i = 0; i < V_PART; ++i)
     if (FVIM_CU(cudaMemset(c->sv[i], 0, (i < S_NSURF ? ns : (i == V_EP ? nv : nv * 6)) * sizeof(T))))
       return FVIM_ERR_CUDA;
+  // the fills and the copy run on the legacy stream, which the solvers' non-blocking stream does not wait for
+  if (FVIM_CU(cudaStreamSynchronize(cudaStreamLegacy))) return FVIM_ERR_CUDA;
   return FVIM_OK;
 }
 

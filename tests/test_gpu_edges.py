@@ -222,3 +222,23 @@ def test_direct_transforms_at_their_limits(n1, n2, nz, prec):
     tol = 1e-10 if prec == "fp64" else 2e-5
     assert rel_l2(out.cpu().numpy(), ref) < tol and rel_l2(u3.cpu().numpy(), u3_ref) < tol
     assert rel_l2(bu.cpu().numpy(), op.boussinesq_apply(p, z, 1.0, 1.0, E, NU, "stress")[0]) < tol
+
+
+def test_first_solve_on_a_side_stream():
+    """A context's first solve fills its workspace; on a stream that does not wait for the legacy one it gives
+    the bits of a later solve."""
+    torch = require_gpu()
+    z = inputs.uniform_depth(24, 0.3)
+    sy = 0.05 * ES
+    x = (np.arange(256) + 0.5) / 256 - 0.5
+    p = 0.13 * ES * np.sqrt(np.maximum(0.0, 1.0 - (x[None, :] ** 2 + x[:, None] ** 2) / 0.06))
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        ctx = _ctx(256, 256, z, "fp32", sigma_y=sy, E_h=0.1)
+        d = to_dev(torch, p, torch.float32)
+        res = []
+        for _ in range(2):
+            out = [torch.empty(s, dtype=ctx.dtype, device="cuda") for s in (ctx.vol_shape, ctx.vol_shape, ctx.scal_shape)]
+            res.append((ctx.plasticity_solve(d, *out), out))
+    side.synchronize()
+    assert res[0][0] == res[1][0] and all(torch.equal(a, b) for a, b in zip(res[0][1], res[1][1]))
